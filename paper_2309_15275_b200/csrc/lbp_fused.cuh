@@ -1,4 +1,4 @@
-// Declarations of the persistent products + expansion kernel (bf16, r <= 16).
+// Declarations of the persistent products + expansion kernel (bf16 data).
 #pragma once
 
 #include <cuda.h>
@@ -9,43 +9,43 @@
 
 namespace lbp {
 
-// Highest rank the persistent products kernel takes: a 128-row group must hold
-// several blocks, and the tensor-pipe projection must produce that many rows
-// per block (orders 8 and 16: up to 48, which covers LP_L1-6, LP_L1-7 and LP_L1-8
-// of the paper's tables; order 4: all 16).
+// Highest rank the persistent products kernel takes: the tensor-pipe projection must
+// produce that many rows per block (orders 8 and 16: up to 48, which covers LP_L1-6,
+// LP_L1-7 and LP_L1-8 of the paper's tables; order 4: all 16).
 inline int fused_max_rank(int k) { return k == 4 ? 16 : 48; }
 
 // Scaling inside the products path.  Eq. 6-7 put 1/k on either side of the
 // products; all of it is powers of two, so it can sit anywhere without changing
 // a bit of the results.  Here g_y_hat carries 1/k^2 and x_hat none: g_W =
 // g_y_hat^T x_hat comes out right, and g_x_hat = g_y_hat W already holds the 1/k
-// of the reverse projection, which then only adds, subtracts and rounds.
-inline float fused_scale_gy(int k) { return 1.0f / static_cast<float>(k * k); }
+// of the reverse projection, which then only adds, subtracts and rounds.  Where
+// x_hat was taken at forward time (orthonormal coefficients) g_y_hat carries 1/k
+// too and the expansion multiplies by the other 1/k.
+inline float fused_scale_gy(int k, bool x_hat_given) {
+  return 1.0f / static_cast<float>(x_hat_given ? k : k * k);
+}
 inline float fused_scale_x(int) { return 1.0f; }
 
 struct FusedParams {
-  // token grid and low-rank row layout: block blk of group g = blk / bpt owns rows
-  // g * 128 + (blk % bpt) * r ... + r - 1 of x_hat / g_y_hat; the other rows of a
-  // group are zero
-  int32_t nb, Hb, Wb, H, W, r, bpt, G;
+  // token grid and low-rank rows: block blk owns rows blk * r .. blk * r + r - 1 of
+  // x_hat / g_y_hat (dense); nb = 0: no grid, only tokens that take Eq. 2
+  int32_t nb, Hb, Wb, H, W, r;
   int32_t Cin, Cout;
-  // products
-  int32_t BNx, n_tx, num_kb_x;            // GX: column tile, tiles per row group, k-blocks (Cout / 64)
-  int32_t BNw, mt_w, nt_w, num_kb_w;      // GW: 128 x BNw tiles, k-blocks (G * 2)
+  // GX: tiles of 128 channels per CTA x BNx low-rank rows; a tile's rows are those of
+  // bpt whole blocks (what BNx leaves over is multiplied and dropped)
+  int32_t BNx, bpt, n_ct, n_rt, num_kb_x;   // channel tiles, row tiles, k-blocks (Cout / 64)
+  // GW: 128 rows of g_W per CTA x BNw columns; k-blocks of the low-rank rows, then of
+  // the tokens outside the grid
+  int32_t BNw, mt_w, nt_w, kb_lr, num_kb_w;
   int32_t n_gx_tiles, n_gw_tiles;         // n_gw_tiles counts K slices: mt_w * nt_w * gw_splits
   int32_t gw_splits, kb_per_split_w;      // K slices of a GW tile (fp32 planes, reduced afterwards)
   float* gw_planes;                       // [gw_splits][Cout][Cin] when gw_splits > 1
   int32_t gw_bf16;
-  int32_t lb_kernel, n_extra;             // epilogue core size and bases added token by token (host dispatch)
-  __nv_bfloat16* x_hat;
-  __nv_bfloat16* gy_hat;
-  __nv_bfloat16* g_x;
+  float beta;                             // g_W <- beta * g_W + ... (0: overwritten, not read)
+  float gx_scale;                         // factor of g_x_hat ahead of the expansion (a power of two)
+  int32_t n_extra;                        // tokens outside the grid (Eq. 2): GX tiles behind the grid's
   void* g_W;
   uint32_t* status;
-  // element strides of x, g_y (read by the projection's tensor maps) and of g_x
-  // (the expansion's stores); dense tensors: (H*W*C, W*C, C)
-  lbp_view vx, vgy, vgx;
-  int32_t gx_image8;   // vgx.image / 8 (a multiple of 8 elements: 16 bytes of bf16)
   // failure-injection hook of the test suite (lbp_test_stall_products): the TMA
   // producers issue no load, so every other role runs into its bounded wait
   int32_t test_stall;
@@ -57,7 +57,7 @@ struct FusedParams {
 // Which unit (a CTA, or a CTA pair) works on which tiles, in which order: planned
 // on the host (lbp_fused_plan.cu) and handed to the kernel as a launch
 // parameter.  Tile ids: [0, n_gw_tiles) are the GW tiles (id = tile * gw_splits +
-// K slice), then the GX tiles (row group (pair), column tile).
+// K slice), then the GX tiles (row tile, channel tile).
 constexpr int kSchedMaxItems = 1536;
 constexpr int kSchedMaxUnits = 160;
 struct FusedSchedule {
@@ -66,10 +66,10 @@ struct FusedSchedule {
   uint16_t ids[kSchedMaxItems];
 };
 
-// One tile of work as the kernels see it.
+// One tile of work as the kernel sees it.
 struct WorkTile {
   int is_gw;
-  int a, b;        // GW: (row tile i, column tile j) ; GX: (row group (pair) m, column tile n)
+  int a, b;        // GW: (row tile i, column tile j) ; GX: (row tile m, channel tile n); m >= n_rt: extra tokens
   int kb0, n_kb;   // k-block range (a K slice for GW)
   int slice;
 };
@@ -81,16 +81,18 @@ __device__ __forceinline__ WorkTile unit_tile(const FusedParams& p, const FusedS
                                               int units, int nth);
 #endif
 
-constexpr int kFusedMaxExtra = 2;
-
+// How the expansion finds a block's coefficients: natural-order LB x LB position ->
+// accumulator column inside the block's columns, and what to AND the value with
+// (all ones, or zero where the basis is not selected; col is 0 there).  Forms with
+// an 8 x 8 array keep it as four 4 x 4 quadrants (see Expand).
 struct FusedBasis {
-  int16_t qmap[64];   // natural-order LB x LB position -> basis slot, -1 unused
-  // Bases outside the LB x LB core (kernels instantiated with extras only): the
-  // epilogue adds them token by token.  ex_q: slot, -1 = none; bit u of ex_mu /
-  // bit v of ex_mv is set where the Walsh row along H / W is -1.
-  int16_t ex_q[kFusedMaxExtra];
-  uint16_t ex_mu[kFusedMaxExtra];
-  uint16_t ex_mv[kFusedMaxExtra];
+  int32_t col[64];
+  uint32_t keep[64];
+  int32_t has_hh;            // 8 x 8: some basis has both indices of 4 or more
+  // sparse form: the one basis with i >= 4 (side 0) and the one with j >= 4 (side 1)
+  int32_t ex_col[2];
+  uint32_t ex_keep[2];
+  uint32_t ex_sign[2][16];   // sign bit of that basis on the 4 x 4 patches
 };
 
 // Builds with -DLBP_ROLE_TRACE carry a per-CTA role timeline (diagnostics) in
@@ -105,7 +107,6 @@ constexpr size_t kFusedTraceBytes = 0;
 
 struct FusedLayout {
   size_t x_hat, gy_hat, planes, planes_bytes, trace, total;
-  int G, bpt;
 };
 
 // Side-stream mode of one call (set per thread by lbp_backward_batch): the
@@ -147,19 +148,9 @@ __device__ __forceinline__ WorkTile unit_tile(const FusedParams& p, const FusedS
   if (sc.listed) {
     id = sc.ids[sc.first[unit] + nth];
   } else {
-    const int total = p.n_gw_tiles + p.n_gx_tiles;
-    int seen = 0;
-    for (int round = 0; round * units < total; ++round) {
-      const int pos = (round & 1) ? (units - 1 - unit) : unit;
-      const int t = round * units + pos;
-      if (t < total) {
-        if (seen == nth) {
-          id = t;
-          break;
-        }
-        ++seen;
-      }
-    }
+    // every pass of the snake gives a unit one tile, the last one perhaps none
+    const int pos = (nth & 1) ? (units - 1 - unit) : unit;
+    id = nth * units + pos;
   }
   WorkTile tl;
   if (id < p.n_gw_tiles) {
@@ -175,8 +166,8 @@ __device__ __forceinline__ WorkTile unit_tile(const FusedParams& p, const FusedS
     id -= p.n_gw_tiles;
     tl.is_gw = 0;
     tl.slice = 0;
-    tl.a = id / p.n_tx;
-    tl.b = id - tl.a * p.n_tx;
+    tl.a = id / p.n_ct;
+    tl.b = id - tl.a * p.n_ct;
     tl.kb0 = 0;
     tl.n_kb = p.num_kb_x;
   }
@@ -185,14 +176,20 @@ __device__ __forceinline__ WorkTile unit_tile(const FusedParams& p, const FusedS
 #endif
 
 // ---- host-side tile plan (lbp_fused_plan.cu) ----
+// GW tiles: row_tile x BNw pieces of a gw_rows x gw_cols matrix, num_kb_w k-blocks
+// deep, possibly in K slices.  GX tiles: row_tile of the fixed side (gx_side) x BNx of
+// the other, num_kb_x k-blocks deep; the other side is made of `blocks` indivisible
+// pieces of `piece` columns, plus `n_extra` single columns in tiles of their own.  A
+// unit is a CTA (row_tile 128) or a CTA pair (256).
 struct PlanShape {
-  int Cin, Cout;
-  int G;            // 128-row groups of low-rank rows
-  int bpt, k;       // blocks per group, transform order (size of a group's expansion)
-  int units;        // CTAs, or CTA pairs
-  int pair;         // 1: a unit is a CTA pair working on 256-row tiles
-  int max_splits;   // K slices of g_W the scratch has planes for
-  int epi_kind;     // expansion variant: 0 core butterfly, 1 core + extra bases, 2 8 x 8 core
+  int gw_rows, gw_cols;
+  int gx_side;
+  int blocks, piece, n_extra;
+  int units, pair;
+  int bnw_step, bnx_step, bn_max;   // column tiles: multiples of the step up to bn_max
+  int max_splits;                   // K slices of g_W the scratch has planes for
+  int expand_bytes;                 // what the epilogue of a GX tile writes per piece and channel
+  int epi_kind;                     // expansion: 0 up to a 4 x 4 core, 1 sparse 8 x 8, 2 8 x 8 core
   int num_kb_w, num_kb_x;
 };
 struct TilePlan {
@@ -213,16 +210,22 @@ size_t fused_scratch_bytes(const lbp_layer& L, int r, FusedLayout* lay);
 struct CallViews {
   lbp_view x, gy, gx;
 };
+// What lbp_extras adds to the products kernel: accumulation into g_W and the
+// tokens outside the grid (pitches in elements, 0: dense).
+struct FusedExtras {
+  float beta;
+  int n_extra;
+  const void* x;
+  const void* gy;
+  void* gx;
+  long long x_pitch, gy_pitch, gx_pitch;
+};
 // Exactly one of x / x_hat_dense is given; x_hat_dense are coefficients p(x)
 // taken earlier, stored densely (blocks * r, Cin).  views: null = all dense.
 int launch_fused(const void* x, const void* x_hat_dense, const void* g_y, const void* W, void* g_x,
                  void* g_W, const lbp_layer& L, const BasisPlan& bp, uint8_t* scratch,
                  uint32_t* status, cudaStream_t stream, FusedPhaseHook hook, void* hook_arg,
-                 const CallViews* views = nullptr);
-// Algorithm 1, steps 1-2 for the products kernel: g_y_hat (and x_hat, from x or
-// from dense coefficients) with rows padded to 128-row groups.
-int fused_project(const void* x, const void* x_hat_dense, const void* g_y, const lbp_layer& L,
-                  const BasisPlan& bp, const FusedParams& p, uint32_t* status, cudaStream_t stream);
+                 const CallViews* views = nullptr, const FusedExtras* extras = nullptr);
 
 // Modelled time (microseconds) of the products kernel of this layer on `pairs`
 // CTA pairs, and of its projection kernel on `ctas` SMs (both from B200
@@ -231,12 +234,8 @@ int fused_project(const void* x, const void* x_hat_dense, const void* g_y, const
 double fused_products_model_us(const lbp_layer& L, const BasisPlan& bp, int pairs);
 double fused_projection_model_us(const lbp_layer& L, const BasisPlan& bp, int ctas);
 
-// CTA-pair variant (tcgen05 cta_group::2): used when Cin >= 128 and the SM count is even.
+// Whether the products kernel runs on CTA pairs (tcgen05 cta_group::2): Cin >= 128
+// and an even SM count.
 bool fused_pair_supported(const lbp_layer& L, int sms);
-int launch_fused_pair(const void* x, const void* x_hat_dense, const void* g_y, const void* W,
-                      void* g_W, const lbp_layer& L,
-                      const BasisPlan& bp, FusedParams p, const FusedBasis& fb,
-                      const FusedLayout& lay, int sms, uint32_t* status, cudaStream_t stream,
-                      FusedPhaseHook hook, void* hook_arg);
 
 }  // namespace lbp

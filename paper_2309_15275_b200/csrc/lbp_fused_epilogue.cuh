@@ -1,19 +1,26 @@
-// Epilogue of one accumulator tile of the products kernels, shared by the
-// one-CTA and the CTA-pair variants: a GW tile is written to g_W (or to an fp32
-// K-slice plane); a GX tile is expanded with the transposed bases (Eq. 7) and
-// written to g_x, so g_x_hat never leaves the chip.
+// Epilogue of one accumulator tile of the products kernel: a GW tile is written
+// to g_W (or to an fp32 K-slice plane); a GX tile is expanded with the transposed
+// bases (Eq. 7) and written to g_x, so g_x_hat never leaves the chip.
 //
-// Four warps (one per TMEM lane quarter) form a group; group `eg` takes the
-// 32-column chunks eg, eg + kEGroups, ... of the tile.  A chunk goes TMEM ->
-// registers -> swizzled shared staging (row = low-rank row, 32 columns); then
-// every thread owns NCH channels of one block, gathers that block's r
-// coefficients, runs the LB x LB butterfly and stores the k x k tokens.
+// Four warps (one per TMEM lane quarter) form a group.
+//
+// GX: the accumulator holds g_x_hat transposed, one channel per TMEM lane and one
+// low-rank row per column, so a thread reads all coefficients of a block for its
+// channel with tcgen05.ld and needs no other thread's data: butterfly in
+// registers, one bf16 per distinct token value into a shared-memory tile of
+// T x T tokens x 128 channels, and TMA stores from there, issued by a warp of their own
+// (one per group), so that the four warps never wait for one another.  A Walsh row
+// of sequency below LB is constant on runs of K / LB tokens; the repetition over
+// tokens is left to the TMA: the tile is stored S x S times, each time through a
+// tensor map that addresses every S-th token (S = K / T), which writes each distinct
+// value to shared memory once instead of S * S times and clips what hangs over the
+// grid.  What bounds it: an SM's stores.  TMA stores of 256-byte rows move 51 GB/s
+// from one SM and 5.3-5.8 TB/s from all (128-byte rows: 26 and 3.5; a warp's 8-byte
+// stores to four 64-byte pieces, the earlier form of this epilogue, 34 and 4.3).
 #pragma once
 
 #include <cuda_bf16.h>
 #include <stdint.h>
-
-#include <type_traits>
 
 #include "lbp_fused.cuh"
 #include "ptx_sm100.cuh"
@@ -23,9 +30,42 @@ namespace lbp {
 namespace fused {
 
 constexpr int BM = 128;
-constexpr int kEStride = 32;   // fp32 words per staged row; 16-byte chunk c of row i sits at chunk c ^ (i & 7)
-constexpr int kEBytes = (BM + 1) * kEStride * 4;   // 128 staged rows + one row of zeros
-constexpr int kEGroups = 2;                        // epilogue groups of 4 warps
+constexpr int kEGroups = 2;            // epilogue groups of 4 warps
+constexpr int kFillBytes = 8192;       // what a group hands to the TMA at a time
+constexpr int kFillBufs = 4;           // such buffers per group
+constexpr int kGroupBytes = kFillBufs * kFillBytes;
+constexpr int kGwStageBytes = BM * 32 * 4;   // a 32-column chunk of a GW tile: half of the group's buffers
+static_assert(2 * kGwStageBytes == kGroupBytes, "two GW chunks fill a group's buffers");
+constexpr int kStoreMapsMax = 16;
+
+// Forms of the expansion (template CORE): 2, 4: a 2 x 2 / 4 x 4 array of
+// coefficients.  8: an 8 x 8 array as four 4 x 4 quadrants: with u = 2 a + d, v = 2 b
+// + e, natural row index 2 m + h, the Walsh sign factors into that of (m, a) and
+// (-1)^(h d), and h = 1 exactly where the sequency is 4 or more, so
+//   value(u, v) = Q00[a][b] + (-1)^d Q10[a][b] + (-1)^e Q01[a][b] + (-1)^(d+e) Q11[a][b]
+// with Qhh' the 4 x 4 transform of a quadrant; Q11 is empty for every LP_L1 set of
+// the paper and then skipped.  6: the same with at most one basis in Q10 and one in
+// Q01 (PREFIX sets of rank 14-16): their quadrants are a sign times one coefficient,
+// and an 8 x 8 block costs 16 + 2 loads and 160 additions instead of 64 and 384.
+constexpr int kCoreSparse = 6;
+
+template <int K, int CORE>
+struct Expand {
+  static constexpr int LB = CORE == kCoreSparse ? 8 : CORE;
+  static constexpr int T = LB <= 4 ? 4 : 8;   // side of the stored tile
+  static constexpr int S = K / T;             // token stride of a store
+  static constexpr int kMaps = S * S;
+  static constexpr int kBlockBytes = T * T * 256;
+  static constexpr int kBlocksPerFill = kBlockBytes < kFillBytes ? kFillBytes / kBlockBytes : 1;
+  static constexpr int kFillsPerBlock = kBlockBytes > kFillBytes ? kBlockBytes / kFillBytes : 1;
+  static constexpr int kBoxRows = T / kFillsPerBlock;   // token rows of one store
+  static_assert(K % T == 0 && kMaps <= kStoreMapsMax && kBoxRows == 4, "store geometry");
+};
+
+struct StoreMaps {
+  CUtensorMap m[kStoreMapsMax];
+  CUtensorMap extra;   // g_x of the tokens outside the grid: boxes of 32 tokens x 128 channels
+};
 
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
@@ -47,290 +87,379 @@ __device__ __forceinline__ bool named_bar_or(int id, int nthreads, bool pred) {
   return any != 0;
 }
 
-__device__ __forceinline__ int blocks_in_group(const FusedParams& p, int g) {
-  const int left = p.nb - g * p.bpt;
-  return left < p.bpt ? left : p.bpt;
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap* m, const void* smem_src, int32_t c0,
+                                             int32_t c1, int32_t c2, int32_t c3) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(
+          reinterpret_cast<uint64_t>(m)),
+      "r"(ptx::smem_u32(smem_src)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+      : "memory");
 }
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// at most N of this thread's latest store groups have not yet read their source
+template <int N>
+__device__ __forceinline__ void bulk_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // What the epilogue needs to know about the accumulator it drains.
 struct DrainTile {
-  int is_gw;
-  int row_base;       // GW: first g_W row of these 128 accumulator rows
-  int group;          // GX: 128-row group of low-rank rows
-  int col_base;       // first output column (channel) of the tile
-  int bn;             // accumulator columns in use
+  int row_base;       // GW: first g_W row of these 128 accumulator rows; GX: first channel of the 128 lanes
+  int row_tile;       // GX: row tile
+  int col_base;       // GW: first g_W column
   int slice;          // GW: K slice (plane index when gw_splits > 1)
   uint32_t tmem_acc;  // TMEM address of column 0, lane 0 of the accumulator
 };
 
-// `release()` is called by lane 0 of every warp once the warp has read its last
-// accumulator column (the tensor core may then overwrite the slot).
-template <int K, int LB, int NEX, class Release>
-__device__ __forceinline__ void drain_tile(const FusedParams& p, const FusedBasis& fb,
-                                           const DrainTile& t, float* Eg, int bar_id, int eg,
-                                           int etid, int quarter, int lane, Release release) {
+// A warp has read its last accumulator column of the tile.
+template <class Release>
+__device__ __forceinline__ void release_slot(int lane, Release release) {
+  ptx::tc_fence_before_sync();
+  __syncwarp();
+  if (lane == 0) release();
+}
+
+// ---- GW tile: g_W[row_base + row, col_base + col] ----
+// A chunk of 32 columns is staged in shared memory and written out with eight
+// lanes along a row, so that a store instruction covers whole 128-byte pieces of
+// four rows.  Two stages, used alternately: one barrier per chunk.
+template <class Release>
+__device__ __forceinline__ void drain_gw(const FusedParams& p, const DrainTile& t, uint8_t* buf,
+                                         int bar_id, int eg, int etid, int quarter, int lane,
+                                         Release release) {
+  constexpr int kStride = 32;   // fp32 words per staged row; 16-byte piece c of row i sits at piece c ^ (i & 7)
+  const uint32_t lane_bits = static_cast<uint32_t>(quarter * 32) << 16;
+  const int ew = etid >> 5;
+  const bool planes = p.gw_splits > 1;
+  bool released = false;
+  int stage = 0;
+  for (int c0 = eg * 32; c0 < p.BNw; c0 += 32 * kEGroups) {
+    uint32_t v[32];
+    ptx::tmem_ld_32x32(t.tmem_acc + lane_bits + c0, v);
+    ptx::tmem_ld_wait();
+    if (c0 + 32 * kEGroups >= p.BNw) {
+      released = true;
+      release_slot(lane, release);
+    }
+    float* const E = reinterpret_cast<float*>(buf + stage * kGwStageBytes);
+    stage ^= 1;
+    const int erow_i = quarter * 32 + lane;
+    uint4* erow = reinterpret_cast<uint4*>(E + erow_i * kStride);
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      erow[q ^ (erow_i & 7)] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    named_bar_sync(bar_id, 128);
+    if (planes || !p.gw_bf16) {
+      // fp32 g_W, or a K slice: fp32 partial plane, summed by the reduce kernel that follows
+      float* dst = planes ? p.gw_planes + static_cast<long long>(t.slice) * p.Cout * p.Cin
+                          : static_cast<float*>(p.g_W);
+      const bool add = !planes && p.beta != 0.f;
+      const int o = lane & 7, rs = lane >> 3;
+      const int col = t.col_base + c0 + o * 4;
+#pragma unroll
+      for (int it = 0; it < 8; ++it) {
+        const int row = it * 16 + ew * 4 + rs;
+        const long long grow = static_cast<long long>(t.row_base) + row;
+        if (grow < p.Cout && col < p.Cin) {
+          float4 f = *reinterpret_cast<const float4*>(E + row * kStride + ((o ^ (row & 7)) << 2));
+          float4* at = reinterpret_cast<float4*>(dst + grow * p.Cin + col);
+          if (add) {
+            const float4 old = *at;
+            f.x = fmaf(p.beta, old.x, f.x);
+            f.y = fmaf(p.beta, old.y, f.y);
+            f.z = fmaf(p.beta, old.z, f.z);
+            f.w = fmaf(p.beta, old.w, f.w);
+          }
+          *at = f;
+        }
+      }
+    } else {
+      __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(p.g_W);
+      const int o = lane & 3, rs = lane >> 2;
+      const int col = t.col_base + c0 + o * 8;
+#pragma unroll
+      for (int it = 0; it < 4; ++it) {
+        const int row = it * 32 + ew * 8 + rs;
+        const long long grow = static_cast<long long>(t.row_base) + row;
+        if (grow < p.Cout && col < p.Cin) {
+          float4 f0 =
+              *reinterpret_cast<const float4*>(E + row * kStride + (((2 * o) ^ (row & 7)) << 2));
+          float4 f1 =
+              *reinterpret_cast<const float4*>(E + row * kStride + (((2 * o + 1) ^ (row & 7)) << 2));
+          uint4* at = reinterpret_cast<uint4*>(dst + grow * p.Cin + col);
+          if (p.beta != 0.f) {
+            const uint4 old = *at;
+            f0.x = fmaf(p.beta, bf16_lo(old.x), f0.x);
+            f0.y = fmaf(p.beta, bf16_hi(old.x), f0.y);
+            f0.z = fmaf(p.beta, bf16_lo(old.y), f0.z);
+            f0.w = fmaf(p.beta, bf16_hi(old.y), f0.w);
+            f1.x = fmaf(p.beta, bf16_lo(old.z), f1.x);
+            f1.y = fmaf(p.beta, bf16_hi(old.z), f1.y);
+            f1.z = fmaf(p.beta, bf16_lo(old.w), f1.z);
+            f1.w = fmaf(p.beta, bf16_hi(old.w), f1.w);
+          }
+          *at = make_uint4(pack_bf16x2(f0.x, f0.y), pack_bf16x2(f0.z, f0.w), pack_bf16x2(f1.x, f1.y),
+                           pack_bf16x2(f1.z, f1.w));
+        }
+      }
+    }
+  }
+  if (!released) release_slot(lane, release);   // this group had no chunk of the tile
+}
+
+// A group's buffers on their way from the epilogue warps to the warp that issues
+// their TMA stores.  `count` runs over all fills of the group; fill n lies in buffer
+// n % kFillBufs.  full[b]: the four warps have written it; empty[b]: its stores have
+// read it.
+struct Fills {
+  uint8_t* buf;
+  uint64_t* full;    // [kFillBufs]
+  uint64_t* empty;   // [kFillBufs]
+  uint32_t* status;
+  uint32_t count;
+  bool held;         // store warp: the stores of fill count - 1 may still read their buffer
+  __device__ __forceinline__ uint8_t* at(uint32_t n) const { return buf + (n % kFillBufs) * kFillBytes; }
+  // writers: the buffer of fill n may be written
+  __device__ __forceinline__ bool wait_empty(uint32_t n) const {
+    return ptx::mbar_wait(&empty[n % kFillBufs], ((n / kFillBufs) + 1) & 1u, status, (5u << 16) | 6u);
+  }
+  // writers: this warp's part of fill `count` is written
+  __device__ __forceinline__ void written(int lane) {
+    ptx::fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) ptx::mbar_arrive(&full[count % kFillBufs]);
+    ++count;
+  }
+  // store warp: give back the buffer of fill n; at most N later ones may still be read
+  template <int N>
+  __device__ __forceinline__ void give_back(uint32_t n, int lane) {
+    bulk_wait_read<N>();
+    __syncwarp();
+    if (held && lane == 0) ptx::mbar_arrive(&empty[n % kFillBufs]);
+  }
+};
+
+// ---- GX tile of tokens outside the grid: g_x[token, channel], no expansion ----
+// The drains of GX tiles return false when a wait expired.
+template <class Release>
+__device__ __forceinline__ bool drain_gx_extra(const FusedParams& p, const DrainTile& t, Fills& fills,
+                                               int eg, int quarter, int lane, Release release) {
   const uint32_t lane_bits = static_cast<uint32_t>(quarter * 32) << 16;
   bool released = false;
+  for (int c0 = eg * 32; c0 < p.BNx; c0 += 32 * kEGroups) {
+    uint32_t v[32];
+    ptx::tmem_ld_32x32(t.tmem_acc + lane_bits + c0, v);
+    ptx::tmem_ld_wait();
+    if (c0 + 32 * kEGroups >= p.BNx) {
+      released = true;
+      release_slot(lane, release);
+    }
+    if (!__all_sync(0xffffffffu, fills.wait_empty(fills.count))) return false;
+    uint16_t* const o = reinterpret_cast<uint16_t*>(fills.at(fills.count)) + quarter * 32 + lane;
+#pragma unroll
+    for (int j = 0; j < 32; j += 2) {
+      const uint32_t pk = pack_bf16x2(__uint_as_float(v[j]), __uint_as_float(v[j + 1]));
+      o[j * 128] = static_cast<uint16_t>(pk);
+      o[(j + 1) * 128] = static_cast<uint16_t>(pk >> 16);
+    }
+    fills.written(lane);
+  }
+  if (!released) release_slot(lane, release);
+  return true;
+}
 
-  if (t.is_gw) {
-    // ---- GW tile: g_W[128 i + row, BNw j + col] ----
-    // A chunk is staged like a GX chunk and written out with eight lanes along a
-    // row, so that a store instruction covers whole 128-byte pieces of four rows.
-    const int ew = etid >> 5;
-    for (int c0 = eg * 32; c0 < t.bn; c0 += 32 * kEGroups) {
-      uint32_t v[32];
-      ptx::tmem_ld_32x32(t.tmem_acc + lane_bits + c0, v);
+// N x N coefficients of a block (positions pos0 ..) from the accumulator columns at `at`.
+// Unselected positions read column 0 of the block and drop it (mask_transform): a
+// branch around a tcgen05.ld costs more than the load.
+template <int N>
+__device__ __forceinline__ void read_coeffs(uint32_t at, const FusedBasis& fb, int pos0,
+                                            float (&q)[N][N][1]) {
+#pragma unroll
+  for (int a = 0; a < N; ++a)
+#pragma unroll
+    for (int b = 0; b < N; ++b)
+      q[a][b][0] = __uint_as_float(ptx::tmem_ld_x1(at + fb.col[pos0 + a * N + b]));
+}
+template <int N>
+__device__ __forceinline__ void mask_transform(const FusedBasis& fb, int pos0, float scale,
+                                               float (&q)[N][N][1]) {
+#pragma unroll
+  for (int a = 0; a < N; ++a)
+#pragma unroll
+    for (int b = 0; b < N; ++b)
+      q[a][b][0] = __uint_as_float(__float_as_uint(q[a][b][0]) & fb.keep[pos0 + a * N + b]);
+  if (scale != 1.f) {
+#pragma unroll
+    for (int a = 0; a < N; ++a)
+#pragma unroll
+      for (int b = 0; b < N; ++b) q[a][b][0] *= scale;
+  }
+  hadamard_rows<N, 1>(q);
+  hadamard_cols<N, 1>(q);
+}
+
+// ---- GX tile: expand g_x_hat (128 channels x BNx low-rank rows) into g_x ----
+template <int K, int CORE, class Release>
+__device__ __forceinline__ bool drain_gx(const FusedParams& p, const FusedBasis& fb, const DrainTile& t,
+                                         Fills& fills, int eg, int quarter, int lane, Release release) {
+  using X = Expand<K, CORE>;
+  constexpr int FB = X::kBlocksPerFill;
+  const uint32_t acc0 = t.tmem_acc + (static_cast<uint32_t>(quarter * 32) << 16);
+  const int blk0 = t.row_tile * p.bpt;
+  const int n_blocks = p.nb - blk0 < p.bpt ? p.nb - blk0 : p.bpt;
+  const bool live = t.row_base + quarter * 32 < p.Cin;   // some of this warp's channels exist
+  bool released = false;
+  auto release_after = [&](int next_j0) {
+    if (next_j0 >= n_blocks) {
+      released = true;
+      release_slot(lane, release);
+    }
+  };
+
+  if constexpr (X::LB <= 4) {
+    constexpr int LB = X::LB, REP = X::T / LB;
+    for (int j0 = eg * FB; j0 < n_blocks; j0 += FB * kEGroups) {
+      float q[FB][LB][LB][1];
+#pragma unroll
+      for (int j = 0; j < FB; ++j)   // a fill may end with a block that does not exist: read twice, not stored
+        read_coeffs<LB>(acc0 + (j0 + j < n_blocks ? j0 + j : j0) * p.r, fb, 0, q[j]);
       ptx::tmem_ld_wait();
-      if (c0 + 32 * kEGroups >= t.bn) {
-        released = true;
-        ptx::tc_fence_before_sync();
-        __syncwarp();
-        if (lane == 0) release();
+      release_after(j0 + FB * kEGroups);
+      if (live) {
+#pragma unroll
+        for (int j = 0; j < FB; ++j) mask_transform<LB>(fb, 0, p.gx_scale, q[j]);
       }
-      const int erow_i = quarter * 32 + lane;
-      uint4* erow = reinterpret_cast<uint4*>(Eg + erow_i * kEStride);
+      if (!__all_sync(0xffffffffu, fills.wait_empty(fills.count))) return false;
+      uint8_t* const dst = fills.at(fills.count);
+      if (live) {
 #pragma unroll
-      for (int q = 0; q < 8; ++q)
-        erow[q ^ (erow_i & 7)] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-      named_bar_sync(bar_id, 128);
-      if (p.gw_splits > 1 || !p.gw_bf16) {
-        // fp32 g_W, or a K slice: fp32 partial plane, summed by the reduce kernel that follows
-        float* dst = p.gw_splits > 1
-                         ? p.gw_planes + static_cast<long long>(t.slice) * p.Cout * p.Cin
-                         : static_cast<float*>(p.g_W);
-        const int o = lane & 7, rs = lane >> 3;
-        const int col = t.col_base + c0 + o * 4;
+        for (int j = 0; j < FB; ++j) {
+          uint16_t* const o = reinterpret_cast<uint16_t*>(dst + j * X::kBlockBytes) + quarter * 32 + lane;
 #pragma unroll
-        for (int it = 0; it < 8; ++it) {
-          const int row = it * 16 + ew * 4 + rs;
-          const long long grow = static_cast<long long>(t.row_base) + row;
-          if (grow < p.Cout && col < p.Cin)
-            *reinterpret_cast<uint4*>(dst + grow * p.Cin + col) =
-                *reinterpret_cast<const uint4*>(Eg + row * kEStride + ((o ^ (row & 7)) << 2));
-        }
-      } else {
-        __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(p.g_W);
-        const int o = lane & 3, rs = lane >> 2;
-        const int col = t.col_base + c0 + o * 8;
+          for (int u = 0; u < X::T; ++u)
 #pragma unroll
-        for (int it = 0; it < 4; ++it) {
-          const int row = it * 32 + ew * 8 + rs;
-          const long long grow = static_cast<long long>(t.row_base) + row;
-          if (grow < p.Cout && col < p.Cin) {
-            const float4 f0 = *reinterpret_cast<const float4*>(
-                Eg + row * kEStride + (((2 * o) ^ (row & 7)) << 2));
-            const float4 f1 = *reinterpret_cast<const float4*>(
-                Eg + row * kEStride + (((2 * o + 1) ^ (row & 7)) << 2));
-            uint4 pk;
-            pk.x = pack_bf16x2(f0.x, f0.y);
-            pk.y = pack_bf16x2(f0.z, f0.w);
-            pk.z = pack_bf16x2(f1.x, f1.y);
-            pk.w = pack_bf16x2(f1.z, f1.w);
-            *reinterpret_cast<uint4*>(dst + grow * p.Cin + col) = pk;
-          }
+            for (int b = 0; b < LB; b += 2) {
+              const uint32_t pk = pack_bf16x2(q[j][u / REP][b][0], q[j][u / REP][b + 1][0]);
+#pragma unroll
+              for (int d = 0; d < REP; ++d) {
+                o[(u * X::T + b * REP + d) * 128] = static_cast<uint16_t>(pk);
+                o[(u * X::T + (b + 1) * REP + d) * 128] = static_cast<uint16_t>(pk >> 16);
+              }
+            }
         }
       }
-      named_bar_sync(bar_id, 128);
+      fills.written(lane);
     }
   } else {
-    // ---- GX tile: expand g_x_hat (128 rows x BNx columns) into g_x ----
-    const int m = t.group;
-    const int bg = blocks_in_group(p, m);
-    // channels per thread: an 8 x 8 coefficient array leaves registers for two
-    constexpr int NCH = LB <= 4 ? 4 : 2;
-    constexpr int RUN = K / LB;
-    constexpr int CPT = 32 / NCH;       // threads across one 32-column chunk
-    constexpr int BSLOTS = 128 / CPT;   // blocks expanded concurrently
-    const int cc = etid % CPT, bs = etid / CPT;
-    // element offsets of a token inside a block fit 32 bits (checked on the host)
-    const int tok_stride = static_cast<int>(p.vgx.token), row_stride = static_cast<int>(p.vgx.row);
-    // first token of block bl of this group (channel 0) and how many of its K x K
-    // tokens lie on the grid
-    auto block_origin = [&](int bl, __nv_bfloat16** o, int* ulim, int* vlim) {
-      const int blk = m * p.bpt + bl;
-      const int bw = blk % p.Wb, t2 = blk / p.Wb, bh = t2 % p.Hb, b = t2 / p.Hb;
-      // the offset inside one image fits 32 bits (checked on the host)
-      *o = p.g_x + (static_cast<long long>(b) * p.gx_image8 * 8 +
-                   (bh * K * row_stride + bw * K * tok_stride));
-      *ulim = p.H - bh * K < K ? p.H - bh * K : K;
-      *vlim = p.W - bw * K < K ? p.W - bw * K : K;
-    };
-    // the first block a thread expands is the same for every chunk of the tile
-    __nv_bfloat16* o_first = p.g_x;
-    int ulim_first = K, vlim_first = K;
-    if (bs < bg) {
-      block_origin(bs, &o_first, &ulim_first, &vlim_first);
-      o_first += t.col_base + cc * NCH;
-    }
-    for (int c0 = eg * 32; c0 < t.bn; c0 += 32 * kEGroups) {
-      uint32_t v[32];
-      ptx::tmem_ld_32x32(t.tmem_acc + lane_bits + c0, v);
-      ptx::tmem_ld_wait();
-      if (c0 + 32 * kEGroups >= t.bn) {
-        released = true;
-        ptx::tc_fence_before_sync();
-        __syncwarp();
-        if (lane == 0) release();
+    for (int j0 = eg; j0 < n_blocks; j0 += kEGroups) {
+      const uint32_t at = acc0 + j0 * p.r;
+      float q00[4][4][1], q10[4][4][1], q01[4][4][1], q11[4][4][1];
+      read_coeffs<4>(at, fb, 0, q00);
+      if constexpr (CORE == kCoreSparse) {
+        q10[0][0][0] = __uint_as_float(ptx::tmem_ld_x1(at + fb.ex_col[0]));
+        q01[0][0][0] = __uint_as_float(ptx::tmem_ld_x1(at + fb.ex_col[1]));
+      } else {
+        read_coeffs<4>(at, fb, 16, q10);
+        read_coeffs<4>(at, fb, 32, q01);
+        if (fb.has_hh) read_coeffs<4>(at, fb, 48, q11);
       }
-      const int erow_i = quarter * 32 + lane;
-      uint4* erow = reinterpret_cast<uint4*>(Eg + erow_i * kEStride);
+      ptx::tmem_ld_wait();
+      release_after(j0 + kEGroups);
+      if (live) {
+        mask_transform<4>(fb, 0, p.gx_scale, q00);
+        if constexpr (CORE == kCoreSparse) {
+          const uint32_t e0 = __float_as_uint(q10[0][0][0] * p.gx_scale) & fb.ex_keep[0];
+          const uint32_t e1 = __float_as_uint(q01[0][0][0] * p.gx_scale) & fb.ex_keep[1];
 #pragma unroll
-      for (int q = 0; q < 8; ++q)
-        erow[q ^ (erow_i & 7)] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-      named_bar_sync(bar_id, 128);
-      const int ch = t.col_base + c0 + cc * NCH;
-      if (ch < p.Cin) {
-        for (int bl = bs; bl < bg; bl += BSLOTS) {
-          float acc[LB][LB][NCH];
-          const int row_b = bl * p.r;
-#pragma unroll
-          for (int a = 0; a < LB; ++a) {
-#pragma unroll
-            for (int b = 0; b < LB; ++b) {
-              const int q = fb.qmap[a * LB + b];
-              const int row_q = q >= 0 ? row_b + q : BM;
-              if constexpr (NCH == 4) {
-                const float4 f =
-                    *reinterpret_cast<const float4*>(Eg + row_q * kEStride + ((cc ^ (row_q & 7)) << 2));
-                acc[a][b][0] = f.x;
-                acc[a][b][1] = f.y;
-                acc[a][b][2] = f.z;
-                acc[a][b][3] = f.w;
-              } else if constexpr (NCH == 2) {
-                const float2 f = *reinterpret_cast<const float2*>(
-                    Eg + row_q * kEStride + (((cc >> 1) ^ (row_q & 7)) << 2) + (cc & 1) * 2);
-                acc[a][b][0] = f.x;
-                acc[a][b][1] = f.y;
-              } else {
-                acc[a][b][0] = Eg[row_q * kEStride + (((cc >> 2) ^ (row_q & 7)) << 2) + (cc & 3)];
-              }
-            }
+          for (int i = 0; i < 16; ++i) {
+            q10[i >> 2][i & 3][0] = __uint_as_float(e0 ^ fb.ex_sign[0][i]);
+            q01[i >> 2][i & 3][0] = __uint_as_float(e1 ^ fb.ex_sign[1][i]);
           }
-          hadamard_rows<LB, NCH>(acc);
-          hadamard_cols<LB, NCH>(acc);
-          __nv_bfloat16* o;
-          int ulim, vlim;
-          if (bl == bs) {
-            o = o_first + (ch - t.col_base - cc * NCH);
-            ulim = ulim_first;
-            vlim = vlim_first;
+        } else {
+          mask_transform<4>(fb, 16, p.gx_scale, q10);
+          mask_transform<4>(fb, 32, p.gx_scale, q01);
+          if (fb.has_hh) {
+            mask_transform<4>(fb, 48, p.gx_scale, q11);
           } else {
-            block_origin(bl, &o, &ulim, &vlim);
-            o += ch;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) q11[i >> 2][i & 3][0] = 0.f;
           }
-          // Stores of one expanded block.  RAGGED: the block reaches past the grid
-          // (a side that is no multiple of K) and every token is checked; all other
-          // blocks take the unchecked form.  The 1/k of Eq. 7 is already in the
-          // coefficients (g_y_hat carries 1/k^2), so a value is rounded as it is.
-          auto emit = [&](auto ragged) {
-            constexpr bool RAGGED = decltype(ragged)::value;
-            if constexpr (NEX > 0) {
-              // Bases outside the LB x LB core: B_{i,j}[u][v] = s_i(u) s_j(v) with
-              // s = +-1, so each adds +-coefficient to every token.  The row sign is
-              // folded into the coefficient once per token row, the column sign is
-              // a +-1.0 factor of an FMA.
-              static_assert(NCH == 4, "extras go with four channels per thread");
-              float ce[NEX][NCH];
-              uint32_t mu[NEX], mv[NEX];
-#pragma unroll
-              for (int x = 0; x < NEX; ++x) {
-                const int q = fb.ex_q[x];
-                const int row_q = q >= 0 ? row_b + q : BM;
-                const float4 f =
-                    *reinterpret_cast<const float4*>(Eg + row_q * kEStride + ((cc ^ (row_q & 7)) << 2));
-                ce[x][0] = f.x;
-                ce[x][1] = f.y;
-                ce[x][2] = f.z;
-                ce[x][3] = f.w;
-                mu[x] = fb.ex_mu[x];
-                mv[x] = fb.ex_mv[x];
-              }
-#pragma unroll
-              for (int a = 0; a < LB; ++a) {
-#pragma unroll 1
-                for (int du = 0; du < RUN; ++du) {
-                  const int u = a * RUN + du;
-                  if (RAGGED && u >= ulim) break;
-                  float ceu[NEX][NCH];
-#pragma unroll
-                  for (int x = 0; x < NEX; ++x) {
-                    const float su = __uint_as_float(0x3f800000u | (((mu[x] >> u) & 1u) << 31));
-#pragma unroll
-                    for (int c = 0; c < NCH; ++c) ceu[x][c] = ce[x][c] * su;
-                  }
-                  __nv_bfloat16* orow = o + u * row_stride;
-#pragma unroll
-                  for (int v = 0; v < K; ++v) {
-                    float val[NCH];
-#pragma unroll
-                    for (int c = 0; c < NCH; ++c) val[c] = acc[a][v / RUN][c];
-#pragma unroll
-                    for (int x = 0; x < NEX; ++x) {
-                      const float sv = __uint_as_float(0x3f800000u | ((mv[x] << (31 - v)) & 0x80000000u));
-#pragma unroll
-                      for (int c = 0; c < NCH; ++c) val[c] = fmaf(sv, ceu[x][c], val[c]);
-                    }
-                    uint2 pk;
-                    pk.x = pack_bf16x2(val[0], val[1]);
-                    pk.y = pack_bf16x2(val[2], val[3]);
-                    if (!RAGGED || v < vlim) *reinterpret_cast<uint2*>(orow + v * tok_stride) = pk;
-                  }
-                }
-              }
-            } else {
-              // each of the LB x LB values covers a RUN x RUN patch of tokens: round
-              // and pack once, store RUN * RUN times
-#pragma unroll
-              for (int a = 0; a < LB; ++a) {
-#pragma unroll
-                for (int b2 = 0; b2 < LB; ++b2) {
-                  if constexpr (NCH == 4) {
-                    uint2 pk;
-                    pk.x = pack_bf16x2(acc[a][b2][0], acc[a][b2][1]);
-                    pk.y = pack_bf16x2(acc[a][b2][2], acc[a][b2][3]);
-#pragma unroll
-                    for (int du = 0; du < RUN; ++du)
-#pragma unroll
-                      for (int dv = 0; dv < RUN; ++dv)
-                        if (!RAGGED || (a * RUN + du < ulim && b2 * RUN + dv < vlim))
-                          *reinterpret_cast<uint2*>(o + (a * RUN + du) * row_stride +
-                                                    (b2 * RUN + dv) * tok_stride) = pk;
-                  } else if constexpr (NCH == 1) {
-                    const __nv_bfloat16 hv = __float2bfloat16_rn(acc[a][b2][0]);
-#pragma unroll
-                    for (int du = 0; du < RUN; ++du)
-#pragma unroll
-                      for (int dv = 0; dv < RUN; ++dv)
-                        if (!RAGGED || (a * RUN + du < ulim && b2 * RUN + dv < vlim))
-                          o[(a * RUN + du) * row_stride + (b2 * RUN + dv) * tok_stride] = hv;
-                  } else {
-                    const uint32_t pk = pack_bf16x2(acc[a][b2][0], acc[a][b2][1]);
-#pragma unroll
-                    for (int du = 0; du < RUN; ++du)
-#pragma unroll
-                      for (int dv = 0; dv < RUN; ++dv)
-                        if (!RAGGED || (a * RUN + du < ulim && b2 * RUN + dv < vlim))
-                          *reinterpret_cast<uint32_t*>(o + (a * RUN + du) * row_stride +
-                                                       (b2 * RUN + dv) * tok_stride) = pk;
-                  }
-                }
-              }
-            }
-          };
-          if (ulim == K && vlim == K)
-            emit(std::false_type{});
-          else
-            emit(std::true_type{});
         }
       }
-      named_bar_sync(bar_id, 128);
+#pragma unroll
+      for (int part = 0; part < 2; ++part) {
+        if (!__all_sync(0xffffffffu, fills.wait_empty(fills.count))) return false;
+        uint8_t* const dst = fills.at(fills.count);
+        if (live) {
+          uint16_t* const o = reinterpret_cast<uint16_t*>(dst) + quarter * 32 + lane;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int a = 2 * part + (i >> 2), b = i & 3;
+            const float sp = q00[a][b][0] + q10[a][b][0], sm = q00[a][b][0] - q10[a][b][0];
+            float tp = q01[a][b][0], tm = q01[a][b][0];
+            if constexpr (CORE != kCoreSparse) {
+              tp += q11[a][b][0];
+              tm -= q11[a][b][0];
+            }
+            const uint32_t row0 = pack_bf16x2(sp + tp, sp - tp), row1 = pack_bf16x2(sm + tm, sm - tm);
+            uint16_t* const at2 = o + ((2 * (i >> 2)) * 8 + 2 * b) * 128;
+            at2[0] = static_cast<uint16_t>(row0);
+            at2[128] = static_cast<uint16_t>(row0 >> 16);
+            at2[8 * 128] = static_cast<uint16_t>(row1);
+            at2[9 * 128] = static_cast<uint16_t>(row1 >> 16);
+          }
+        }
+        fills.written(lane);
+      }
     }
   }
-  if (!released) {   // this group had no chunk of the tile
-    ptx::tc_fence_before_sync();
-    __syncwarp();
-    if (lane == 0) release();
+  if (!released) release_slot(lane, release);   // this group had no block of the tile
+  return true;
+}
+
+// ---- the store warp of a group: the TMA stores of a GX tile's fills ----
+// A lane issues one store of a fill (FB * kMaps of them) and waits for its own.
+template <int K, int CORE>
+__device__ __forceinline__ bool store_gx(const FusedParams& p, const StoreMaps& maps, const DrainTile& t,
+                                         Fills& fills, int eg, int lane) {
+  using X = Expand<K, CORE>;
+  constexpr int FB = X::kBlocksPerFill;
+  static_assert(FB * X::kMaps <= 32, "one store per lane");
+  const bool extra = t.row_tile >= p.n_rt;
+  const int blk0 = t.row_tile * p.bpt;
+  const int n_blocks = p.nb - blk0 < p.bpt ? p.nb - blk0 : p.bpt;
+  const int first = extra ? eg * 32 : eg * FB, step = extra ? 32 * kEGroups : FB * kEGroups;
+  const int end = extra ? p.BNx : n_blocks, parts = extra ? 1 : X::kFillsPerBlock;
+  const int j = lane / X::kMaps, m = lane % X::kMaps;
+  for (int i = first; i < end; i += step) {
+    // the box starts at token (y, x) of image b; boxes that hang over the grid are
+    // clipped, those that lie outside are not issued
+    const int blk = blk0 + i + j;
+    const int bw = blk % p.Wb, t2 = blk / p.Wb, bh = t2 % p.Hb, b = t2 / p.Hb;
+    for (int part = 0; part < parts; ++part) {
+      const uint32_t n = fills.count;
+      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&fills.full[n % kFillBufs], (n / kFillBufs) & 1u,
+                                                  p.status, (5u << 16) | 7u)))
+        return false;
+      const uint8_t* src = fills.at(n);
+      if (extra) {
+        const int row = (t.row_tile - p.n_rt) * p.BNx + i;
+        if (lane == 0 && t.row_base < p.Cin && row < p.n_extra)
+          tma_store_4d(&maps.extra, src, t.row_base, row, 0, 0);
+      } else {
+        const int y = bh * K + part * X::kBoxRows * X::S + m / X::S, x = bw * K + m % X::S;
+        if (j < FB && i + j < n_blocks && t.row_base < p.Cin && y < p.H && x < p.W)
+          tma_store_4d(&maps.m[m], src + j * X::kBlockBytes, t.row_base, bw * X::T,
+                       bh * X::T + part * X::kBoxRows, b);
+      }
+      bulk_commit();
+      fills.give_back<1>(n - 1, lane);
+      fills.held = true;
+      ++fills.count;
+    }
   }
+  return true;
 }
 
 }  // namespace fused
