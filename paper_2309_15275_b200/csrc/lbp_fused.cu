@@ -417,3 +417,406 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 }  // namespace fused
+
+// --------------------------------------------------------------- launcher ----
+static thread_local const FusedOverlap* g_overlap = nullptr;
+void set_fused_overlap(const FusedOverlap* ov) { g_overlap = ov; }
+const FusedOverlap* fused_overlap() { return g_overlap; }
+
+static thread_local bool g_test_stall = false;
+void set_test_stall(bool on) { g_test_stall = on; }
+bool test_stall() { return g_test_stall; }
+static thread_local bool g_test_stall_projection = false;
+void set_test_stall_projection(bool on) { g_test_stall_projection = on; }
+bool test_stall_projection() { return g_test_stall_projection; }
+
+static long long grid_blocks(const lbp_layer& L) {
+  return static_cast<long long>(L.B) * blocks_along(L.H, L.k) * blocks_along(L.W, L.k);
+}
+
+bool fused_supported(const lbp_layer& L, const BasisPlan& bp) {
+  return L.dtype == LBP_BF16 && grid_blocks(L) * bp.r < (1ll << 31) - 256 &&
+         (L.k == 4 || L.k == 8 || L.k == 16) && bp.r <= fused_max_rank(L.k) && bp.LB <= 8 && bp.LB <= L.k;
+}
+
+bool fused_pair_supported(const lbp_layer& L, int sms) {
+  if (!tune_options().pair) return false;
+  return L.Cin >= 128 && sms >= 2 && (sms % 2) == 0;
+}
+
+size_t fused_scratch_bytes(const lbp_layer& L, int r, FusedLayout* lay) {
+  const long long rows = grid_blocks(L) * r;
+  FusedLayout l;
+  size_t off = 0;
+  l.x_hat = off;
+  off += static_cast<size_t>(rows) * L.Cin * 2;
+  off = (off + 1023) / 1024 * 1024;
+  l.gy_hat = off;
+  off += static_cast<size_t>(rows) * L.Cout * 2;
+  off = (off + 1023) / 1024 * 1024;
+  // fp32 planes for K slices of g_W: only layers with few GW tiles slice, and
+  // slices * tiles stays below the SM count (bounded here for up to 256 SMs)
+  l.planes = off;
+  {
+    const long long tiles_min = ((L.Cout + 127) / 128) * ((L.Cin + 255) / 256);
+    long long s_cap = tiles_min >= 96 ? 1 : 192 / tiles_min;
+    const long long kbs = (rows + fused::BK - 1) / fused::BK;
+    if (s_cap > kbs) s_cap = kbs;
+    l.planes_bytes = s_cap > 1 ? static_cast<size_t>(s_cap) * L.Cout * L.Cin * 4 : 0;
+    const size_t cap = 48u << 20;
+    if (l.planes_bytes > cap) l.planes_bytes = cap;
+  }
+  off += l.planes_bytes;
+  off = (off + 1023) / 1024 * 1024;
+  l.trace = off;
+  off += kFusedTraceBytes;
+  l.total = (off + 1023) / 1024 * 1024;
+  if (lay) *lay = l;
+  return l.total;
+}
+
+// The form of the expansion a basis plan takes (see Expand): rank 1 is a 2 x 2 array
+// with three empty places.
+static int expand_core(const BasisPlan& bp) {
+  if (bp.LB < 8) return bp.LB < 2 ? 2 : bp.LB;
+  int hl = 0, lh = 0, hh = 0;
+  for (int q = 0; q < bp.r; ++q) {
+    const bool hi = bp.seq_i[q] >= 4, hj = bp.seq_j[q] >= 4;
+    hl += hi && !hj;
+    lh += hj && !hi;
+    hh += hi && hj;
+  }
+  return hh == 0 && hl <= 1 && lh <= 1 ? fused::kCoreSparse : 8;
+}
+
+static FusedBasis make_fused_basis(const BasisPlan& bp, int core) {
+  FusedBasis fb{};
+  if (core <= 4) {
+    for (int a = 0; a < bp.LB; ++a)
+      for (int b = 0; b < bp.LB; ++b) {
+        const int q = bp.qmap[a * bp.LB + b];
+        fb.col[a * core + b] = q >= 0 ? q : 0;
+        fb.keep[a * core + b] = q >= 0 ? 0xffffffffu : 0u;
+      }
+    return fb;
+  }
+  for (int a = 0; a < 8; ++a)
+    for (int b = 0; b < 8; ++b) {
+      const int q = bp.qmap[a * 8 + b];
+      if (q < 0) continue;
+      // bit 0 of a natural index is set exactly where the sequency is 4 or more
+      const int quad = 2 * (b & 1) + (a & 1), pos = (a >> 1) * 4 + (b >> 1);
+      if (quad == 3) fb.has_hh = 1;
+      if (core == fused::kCoreSparse && quad != 0) {
+        const int side = quad - 1;
+        fb.ex_col[side] = q;
+        fb.ex_keep[side] = 0xffffffffu;
+        for (int i = 0; i < 16; ++i) {
+          const int par = __builtin_popcount((a >> 1) & (i >> 2)) + __builtin_popcount((b >> 1) & (i & 3));
+          fb.ex_sign[side][i] = static_cast<uint32_t>(par & 1) << 31;
+        }
+      } else {
+        fb.col[quad * 16 + pos] = q;
+        fb.keep[quad * 16 + pos] = 0xffffffffu;
+      }
+    }
+  return fb;
+}
+
+// blocks * piece low-rank rows; blocks = 0: exact backpropagation on n_extra tokens
+static PlanShape plan_shape(const lbp_layer& L, long long blocks, int piece, int core, int n_extra,
+                            size_t planes_bytes, int units, bool pair) {
+  PlanShape s{};
+  s.gw_rows = L.Cout;
+  s.gw_cols = L.Cin;
+  s.gx_side = L.Cin;
+  s.blocks = static_cast<int>(blocks);
+  s.piece = piece;
+  s.n_extra = n_extra;
+  s.units = units;
+  s.pair = pair ? 1 : 0;
+  s.bnw_step = pair ? 128 : 64;
+  s.bnx_step = 32;
+  s.bn_max = pair ? 256 : 128;
+  s.max_splits = static_cast<int>(planes_bytes / (static_cast<size_t>(L.Cout) * L.Cin * 4));
+  s.expand_bytes = blocks > 0 ? L.k * L.k * 2 : 2;
+  s.epi_kind = core == 8 ? 2 : core == fused::kCoreSparse ? 1 : 0;
+  s.num_kb_w = static_cast<int>((blocks * piece + fused::BK - 1) / fused::BK) +
+               (n_extra + fused::BK - 1) / fused::BK;
+  s.num_kb_x = (L.Cout + fused::BK - 1) / fused::BK;
+  return s;
+}
+
+double fused_products_model_us(const lbp_layer& L, const BasisPlan& bp, int pairs) {
+  FusedLayout lay;
+  fused_scratch_bytes(L, bp.r, &lay);
+  // measured times sit about a third above the model (the stages of a unit share
+  // its path to L2), plus the launch and the first operand tiles
+  return 1.35 * plan_products(plan_shape(L, grid_blocks(L), bp.r, expand_core(bp), 0, lay.planes_bytes,
+                                         pairs, true))
+                    .model_us +
+         4.0;
+}
+
+double fused_projection_model_us(const lbp_layer& L, const BasisPlan& bp, int ctas) {
+  const double T = static_cast<double>(L.B) * L.H * L.W;
+  const double nb = static_cast<double>(grid_blocks(L));
+  const double bytes = 2.0 * (T + nb * bp.r) * (L.Cin + L.Cout);
+  // one SM streams about 70 GB/s through its tile ring; the chip about 5.2 TB/s
+  const double rate = ctas * 70e3 < 5.2e6 ? ctas * 70e3 : 5.2e6;   // bytes per microsecond
+  return bytes / rate + 5.0;
+}
+
+// Algorithm 1, steps 1-2: x_hat and g_y_hat (g_y_hat alone when x_hat is given).
+static int fused_project(const void* x, void* x_hat, const void* g_y, void* gy_hat, const lbp_layer& L,
+                         const BasisPlan& bp, const CallViews* views, uint32_t* status,
+                         cudaStream_t stream) {
+  const RowMap dense{1, bp.r};
+  const FusedOverlap* ov = fused_overlap();
+  cudaStream_t ps = ov != nullptr ? ov->proj_stream : stream;
+  if (ov != nullptr) set_projection_launch(ProjLaunch{ov->proj_ctas, ov->proj_ctas > 0, false});
+  const float sgy = fused_scale_gy(L.k, x == nullptr);
+  int e = LBP_OK;
+  if (x != nullptr)
+    e = launch_project2(g_y, gy_hat, L.Cout, x, x_hat, L.Cin, LBP_BF16, L.B, L.H, L.W, bp, dense, status,
+                        ps, sgy, fused_scale_x(L.k), views ? &views->gy : nullptr,
+                        views ? &views->x : nullptr);
+  else
+    e = launch_project(g_y, gy_hat, LBP_BF16, L.B, L.H, L.W, L.Cout, bp, dense, status, ps, sgy,
+                       views ? &views->gy : nullptr);
+  if (ov != nullptr) {
+    set_projection_launch(ProjLaunch{0, false, true});
+    if (e != LBP_OK) return e;
+    LBP_CUDA_TRY(cudaEventRecord(ov->proj_done, ps));
+    LBP_CUDA_TRY(cudaStreamWaitEvent(stream, ov->proj_done, 0));
+  }
+  return e;
+}
+
+// Maps of the expansion's stores: map du * S + dv addresses the tokens (S u + du,
+// S v + dv) of every image, so that its extents clip exactly at the grid's edge.
+// Maps of offsets a small grid does not have are never used (copies of the first).
+static int encode_store_maps(fused::StoreMaps* sm, void* g_x, const lbp_layer& L, int S, int T,
+                             const lbp_view& v) {
+  for (int du = 0; du < S; ++du)
+    for (int dv = 0; dv < S; ++dv) {
+      if (du >= L.H || dv >= L.W) {
+        sm->m[du * S + dv] = sm->m[0];
+        continue;
+      }
+      const lbp_view s{v.image, v.row * S, v.token * S};
+      __nv_bfloat16* base = static_cast<__nv_bfloat16*>(g_x) + du * v.row + dv * v.token;
+      if (int e = encode_box_tensor_map(&sm->m[du * S + dv], base, LBP_BF16, L.B, (L.H - du + S - 1) / S,
+                                        (L.W - dv + S - 1) / S, L.Cin, 128, T, 4, false, &s))
+        return e;
+    }
+  return LBP_OK;
+}
+
+// One launch of the products kernel.
+struct ProductsCall {
+  const lbp_layer* L;
+  // the grid's part; blocks = 0: none
+  long long blocks;
+  int r, core;
+  const void *gy_hat, *x_hat;
+  void* g_x;
+  lbp_view gx_view;
+  float gx_scale;
+  FusedBasis fb;
+  // the tokens outside the grid; ex.n_extra = 0: none
+  FusedExtras ex;
+  const void* W;
+  void* g_W;
+  float* planes;
+  size_t planes_bytes;
+  uint32_t* status;
+#ifdef LBP_ROLE_TRACE
+  unsigned long long* trace;
+#endif
+};
+
+template <int K, int CORE, bool PAIR>
+static int launch_kernel(const cudaLaunchConfig_t& cfg, int dev, const fused::OperandMaps& tm,
+                         const fused::StoreMaps& sm, const FusedParams& p, const FusedBasis& fb,
+                         const FusedSchedule& sc) {
+  auto kern = fused::lbp_products_kernel<K, CORE, PAIR>;
+  static std::atomic<uint64_t> configured{0};   // one bit per device
+  const uint64_t bit = 1ull << (dev & 63);
+  if (dev > 63 || (configured.load(std::memory_order_relaxed) & bit) == 0) {
+    LBP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, fused::kSmemBytes));
+    configured.fetch_or(bit, std::memory_order_relaxed);
+  }
+  LBP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, tm, sm, p, fb, sc));
+  count_launch();
+  return LBP_OK;
+}
+
+static int launch_products(const ProductsCall& c, cudaStream_t stream) {
+  using namespace fused;
+  const lbp_layer& L = *c.L;
+  const int K = L.k, n_extra = c.ex.n_extra;
+  int dev = 0, sms = 0;
+  LBP_CUDA_TRY(cudaGetDevice(&dev));
+  LBP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const bool pair = fused_pair_supported(L, sms);
+  const FusedOverlap* ov = fused_overlap();
+  int units = pair ? sms / 2 : sms;
+  if (pair && ov != nullptr && ov->prod_units > 0 && ov->prod_units < units) units = ov->prod_units;
+
+  const TilePlan& plan =
+      plan_products(plan_shape(L, c.blocks, c.r, c.core, n_extra, c.planes_bytes, units, pair));
+  const int ctas = pair ? 2 : 1;
+  FusedParams p{};
+  p.nb = static_cast<int32_t>(c.blocks);
+  p.Hb = blocks_along(L.H, K);
+  p.Wb = blocks_along(L.W, K);
+  p.H = L.H;
+  p.W = L.W;
+  p.r = c.r;
+  p.Cin = L.Cin;
+  p.Cout = L.Cout;
+  p.BNx = plan.BNx;
+  p.bpt = plan.BNx / c.r;
+  p.n_ct = (L.Cin + ctas * BM - 1) / (ctas * BM);
+  p.n_rt = (p.nb + p.bpt - 1) / p.bpt;
+  p.num_kb_x = (L.Cout + BK - 1) / BK;
+  p.n_gx_tiles = p.n_ct * (p.n_rt + (n_extra + p.BNx - 1) / p.BNx);
+  const long long rows = c.blocks * c.r;
+  p.BNw = plan.BNw;
+  p.mt_w = (L.Cout + ctas * BM - 1) / (ctas * BM);
+  p.nt_w = (L.Cin + p.BNw - 1) / p.BNw;
+  p.kb_lr = static_cast<int>((rows + BK - 1) / BK);
+  p.num_kb_w = p.kb_lr + (n_extra + BK - 1) / BK;
+  p.gw_splits = plan.splits;
+  p.kb_per_split_w = plan.kbps;
+  p.n_gw_tiles = p.mt_w * p.nt_w * p.gw_splits;
+  p.gw_planes = c.planes;
+  p.gw_bf16 = L.gw_dtype == LBP_BF16 ? 1 : 0;
+  p.beta = c.ex.beta;
+  p.gx_scale = c.gx_scale;
+  p.n_extra = n_extra;
+  p.g_W = c.g_W;
+  p.status = c.status;
+  p.test_stall = test_stall() ? 1 : 0;
+#ifdef LBP_ROLE_TRACE
+  p.trace = c.trace;
+  if (p.trace != nullptr) LBP_CUDA_TRY(cudaMemsetAsync(p.trace, 0, kFusedTraceBytes, stream));
+#endif
+
+  OperandMaps tm;
+  StoreMaps sm;
+  const int T = c.core <= 4 ? 4 : 8;
+  if (int e = encode_matrix_tensor_map(&tm.w, c.W, L.Cout, L.Cin, BK)) return e;
+  if (rows > 0) {
+    if (int e = encode_matrix_tensor_map(&tm.gyhat_k, c.gy_hat, rows, L.Cout, p.BNx / ctas)) return e;
+    if (int e = encode_matrix_tensor_map(&tm.gyhat_mn, c.gy_hat, rows, L.Cout, BK)) return e;
+    if (int e = encode_matrix_tensor_map(&tm.xhat, c.x_hat, rows, L.Cin, BK)) return e;
+    if (int e = encode_store_maps(&sm, c.g_x, L, K / T, T, c.gx_view)) return e;
+  }
+  if (n_extra > 0) {
+    if (int e = encode_matrix_tensor_map(&tm.gye_k, c.ex.gy, n_extra, L.Cout, p.BNx / ctas, c.ex.gy_pitch)) return e;
+    if (int e = encode_matrix_tensor_map(&tm.gye_mn, c.ex.gy, n_extra, L.Cout, BK, c.ex.gy_pitch)) return e;
+    if (int e = encode_matrix_tensor_map(&tm.xe, c.ex.x, n_extra, L.Cin, BK, c.ex.x_pitch)) return e;
+    const int64_t pitch = c.ex.gx_pitch > 0 ? c.ex.gx_pitch : L.Cin;
+    const lbp_view rows_view{pitch * n_extra, pitch * n_extra, pitch};
+    if (int e = encode_box_tensor_map(&sm.extra, c.ex.gx, LBP_BF16, 1, 1, n_extra, L.Cin, 128, 32, 1, false,
+                                      &rows_view))
+      return e;
+  } else {
+    tm.gye_k = tm.gyhat_k;
+    tm.gye_mn = tm.gyhat_mn;
+    tm.xe = tm.xhat;
+    sm.extra = sm.m[0];
+  }
+  if (rows == 0) {
+    tm.gyhat_k = tm.gye_k;
+    tm.gyhat_mn = tm.gye_mn;
+    tm.xhat = tm.xe;
+    for (CUtensorMap& m : sm.m) m = sm.extra;
+  }
+
+  const int total_tiles = p.n_gw_tiles + p.n_gx_tiles;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas * (total_tiles < units ? total_tiles : units));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  unsigned n_attr = 0;
+  if (pair) {
+    attr[n_attr].id = cudaLaunchAttributeClusterDimension;
+    attr[n_attr].val.clusterDim.x = 2;
+    attr[n_attr].val.clusterDim.y = 1;
+    attr[n_attr++].val.clusterDim.z = 1;
+  }
+  // Beside a projection on another stream the kernel is launched in plain stream
+  // order: launched early, its CTAs would sit on the SMs that projection is
+  // meant to get while they wait for the kernel ahead.
+  if (ov == nullptr) {
+    attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n_attr++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = n_attr;
+  int e = LBP_ERR_BASIS;
+#define LBP_CASE(KK, CC)                                                                          \
+  case KK * 100 + CC:                                                                             \
+    e = pair ? launch_kernel<KK, CC, true>(cfg, dev, tm, sm, p, c.fb, plan.sched)                 \
+             : launch_kernel<KK, CC, false>(cfg, dev, tm, sm, p, c.fb, plan.sched);               \
+    break
+  switch (K * 100 + c.core) {
+    LBP_CASE(4, 2);
+    LBP_CASE(4, 4);
+    LBP_CASE(8, 2);
+    LBP_CASE(8, 4);
+    LBP_CASE(8, 6);
+    LBP_CASE(8, 8);
+    LBP_CASE(16, 2);
+    LBP_CASE(16, 4);
+    LBP_CASE(16, 6);
+    LBP_CASE(16, 8);
+  }
+#undef LBP_CASE
+  if (e != LBP_OK) return e;
+  if (p.gw_splits > 1)
+    return launch_splitk_reduce(p.gw_planes, c.g_W, static_cast<long long>(L.Cout) * L.Cin, p.gw_splits,
+                                p.gw_bf16 != 0, p.beta, stream);
+  return LBP_OK;
+}
+
+int launch_fused(const void* x, const void* x_hat_dense, const void* g_y, const void* W, void* g_x,
+                 void* g_W, const lbp_layer& L, const BasisPlan& bp, uint8_t* scratch,
+                 uint32_t* status, cudaStream_t stream, FusedPhaseHook hook, void* hook_arg,
+                 const CallViews* views, const FusedExtras* extras) {
+  FusedLayout lay;
+  fused_scratch_bytes(L, bp.r, &lay);
+  void* x_hat = scratch + lay.x_hat;
+  void* gy_hat = scratch + lay.gy_hat;
+  if (int e = fused_project(x, x_hat, g_y, gy_hat, L, bp, views, status, stream)) return e;
+  if (hook != nullptr)
+    if (int e = hook(hook_arg, stream)) return e;
+  ProductsCall c{};
+  c.L = &L;
+  c.blocks = grid_blocks(L);
+  c.r = bp.r;
+  c.core = expand_core(bp);
+  c.gy_hat = gy_hat;
+  c.x_hat = x_hat_dense != nullptr ? x_hat_dense : x_hat;
+  c.g_x = g_x;
+  c.gx_view = resolve_view(views ? &views->gx : nullptr, L.H, L.W, L.Cin);
+  c.gx_scale = x_hat_dense != nullptr ? 1.0f / static_cast<float>(L.k) : 1.0f;
+  c.fb = make_fused_basis(bp, c.core);
+  if (extras != nullptr) c.ex = *extras;
+  c.W = W;
+  c.g_W = g_W;
+  c.planes = reinterpret_cast<float*>(scratch + lay.planes);
+  c.planes_bytes = lay.planes_bytes;
+  c.status = status;
+#ifdef LBP_ROLE_TRACE
+  c.trace = reinterpret_cast<unsigned long long*>(scratch + lay.trace);
+#endif
+  return launch_products(c, stream);
+}
+
+}  // namespace lbp
