@@ -15,6 +15,7 @@
 
 #include "lbp_internal.h"
 #include "ptx_sm100.cuh"
+#include "wht_device.cuh"
 
 namespace lbp {
 
@@ -196,10 +197,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-// Sum fp32 partial tiles [splits][M*N] and write D (fp32 or bf16).
+// Sum fp32 partial tiles [splits][M*N] and write D (fp32 or bf16); beta != 0 adds
+// beta * D.
 __global__ void __launch_bounds__(256)
     splitk_reduce_kernel(const float* __restrict__ part, void* __restrict__ D, long long mn,
-                         int splits, int d_bf16) {
+                         int splits, int d_bf16, float beta) {
   const long long i4 = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) * 4;
   if (i4 >= mn) return;
   float4 acc = *reinterpret_cast<const float4*>(part + i4);
@@ -211,14 +213,25 @@ __global__ void __launch_bounds__(256)
     acc.w += v.w;
   }
   if (d_bf16) {
-    __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x, acc.y);
-    __nv_bfloat162 hi = __floats2bfloat162_rn(acc.z, acc.w);
-    uint2 o;
-    o.x = *reinterpret_cast<uint32_t*>(&lo);
-    o.y = *reinterpret_cast<uint32_t*>(&hi);
-    *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(D) + i4) = o;
+    uint2* const d = reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(D) + i4);
+    if (beta != 0.f) {
+      const uint2 old = *d;
+      acc.x = fmaf(beta, bf16_lo(old.x), acc.x);
+      acc.y = fmaf(beta, bf16_hi(old.x), acc.y);
+      acc.z = fmaf(beta, bf16_lo(old.y), acc.z);
+      acc.w = fmaf(beta, bf16_hi(old.y), acc.w);
+    }
+    *d = make_uint2(pack_bf16x2(acc.x, acc.y), pack_bf16x2(acc.z, acc.w));
   } else {
-    *reinterpret_cast<float4*>(static_cast<float*>(D) + i4) = acc;
+    float4* const d = reinterpret_cast<float4*>(static_cast<float*>(D) + i4);
+    if (beta != 0.f) {
+      const float4 old = *d;
+      acc.x = fmaf(beta, old.x, acc.x);
+      acc.y = fmaf(beta, old.y, acc.y);
+      acc.z = fmaf(beta, old.z, acc.z);
+      acc.w = fmaf(beta, old.w, acc.w);
+    }
+    *d = acc;
   }
 }
 
@@ -286,10 +299,10 @@ int launch_gemm_fp32(const float* A, bool a_mn_major, const float* Bm, float* D,
                      long long N, long long K, cudaStream_t stream);
 
 int launch_splitk_reduce(const float* planes, void* D, long long mn, int splits, bool d_bf16,
-                         cudaStream_t stream) {
+                         float beta, cudaStream_t stream) {
   const long long threads = (mn + 3) / 4;
   splitk_reduce_kernel<<<static_cast<unsigned>((threads + 255) / 256), 256, 0, stream>>>(
-      planes, D, mn, splits, d_bf16 ? 1 : 0);
+      planes, D, mn, splits, d_bf16 ? 1 : 0, beta);
   count_launch();
   LBP_CUDA_TRY(cudaGetLastError());
   return LBP_OK;
@@ -375,14 +388,8 @@ int launch_gemm(const void* A, bool a_mn_major, const void* Bm, void* D, int in_
   count_launch();
   LBP_CUDA_TRY(cudaGetLastError());
 
-  if (t.splits > 1) {
-    const long long mn = M * N;
-    const long long threads = (mn + 3) / 4;
-    splitk_reduce_kernel<<<static_cast<unsigned>((threads + 255) / 256), 256, 0, stream>>>(
-        splitk_ws, D, mn, t.splits, d_dtype == LBP_BF16 ? 1 : 0);
-    count_launch();
-    LBP_CUDA_TRY(cudaGetLastError());
-  }
+  if (t.splits > 1)
+    return launch_splitk_reduce(splitk_ws, D, M * N, t.splits, d_dtype == LBP_BF16, 0.f, stream);
   return LBP_OK;
 }
 

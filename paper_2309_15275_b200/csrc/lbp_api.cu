@@ -97,11 +97,11 @@ int encode_box_tensor_map(CUtensorMap* map, const void* base, int dtype, int B, 
 }
 
 int encode_matrix_tensor_map(CUtensorMap* map, const void* base, long long rows, long long cols,
-                             int box_rows) {
+                             int box_rows, long long pitch) {
   EncodeTiledFn enc;
   if (int e = get_encode_fn(&enc)) return e;
   const cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
-  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(cols) * 2};
+  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(pitch > 0 ? pitch : cols) * 2};
   const cuuint32_t box[2] = {64u, static_cast<cuuint32_t>(box_rows)};
   const cuuint32_t estr[2] = {1u, 1u};
   const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims,
@@ -409,12 +409,13 @@ static int plan_batch(int n, const lbp_layer* layers, const lbp_basis* set, int 
   struct Key {
     int n, r, sms, want;
     lbp_layer layers[8];
-    lbp_basis set[16];
+    lbp_basis set[48];   // r <= 48 here
     BatchPlan plan;
   };
   static thread_local Key cache[8];
   static thread_local int cache_n = 0, cache_next = 0;
-  const bool keyed = n <= 8;
+  const char* env_order = std::getenv("LBP_BATCH_ORDER");   // tuning override: "1,3,2,0"
+  const bool keyed = n <= 8 && env_order == nullptr;
   auto same = [&](const Key& k) {
     if (k.n != n || k.r != r || k.sms != sms || k.want != want) return false;
     for (int i = 0; i < n; ++i)
@@ -486,7 +487,7 @@ static int plan_batch(int n, const lbp_layer* layers, const lbp_basis* set, int 
         fprintf(stderr, "\n");
       }
     }
-    if (const char* e = std::getenv("LBP_BATCH_ORDER")) {   // tuning override: "1,3,2,0"
+    if (const char* e = env_order) {
       int o[6] = {0, 1, 2, 3, 4, 5};
       bool seen[6] = {};
       bool ok = std::sscanf(e, "%d,%d,%d,%d,%d,%d", &o[0], &o[1], &o[2], &o[3], &o[4], &o[5]) >= n;
@@ -541,15 +542,20 @@ int lbp_test_tile_plan(int Cin, int Cout, int G, int bpt, int k, int units, int 
   if (Cin < 1 || Cout < 1 || G < 1 || bpt < 1 || units < 1 || units > kSchedMaxUnits ||
       epi_kind < 0 || epi_kind > 2)
     return LBP_ERR_SHAPE;
+  // the planner's core on a geometry whose GX tiles have 128 or 256 low-rank rows on
+  // the fixed side and columns of W on the other
   PlanShape s{};
-  s.Cin = Cin;
-  s.Cout = Cout;
-  s.G = G;
-  s.bpt = bpt;
-  s.k = k;
+  s.gw_rows = Cout;
+  s.gw_cols = Cin;
+  s.gx_side = G * 128;
+  s.blocks = Cin;
+  s.piece = 1;
   s.units = units;
   s.pair = pair ? 1 : 0;
+  s.bnw_step = s.bnx_step = pair ? 128 : 64;
+  s.bn_max = 256;
   s.max_splits = max_splits;
+  s.expand_bytes = bpt * k * k * 2 / 128;
   s.epi_kind = epi_kind;
   s.num_kb_w = G * 2;
   s.num_kb_x = (Cout + 63) / 64;
@@ -692,29 +698,30 @@ struct CoefLoc {
   double dc_to_sum;   // token sum of a block = dc_to_sum * its (0,0) coefficient as stored
 };
 
+// Whether a low-rank call runs on the persistent products kernel.
+static bool runs_fused(const lbp_layer& L, const BasisPlan& plan) {
+  return fused_enabled() && fused_supported(L, plan);
+}
+
 // Algorithm 1 after validation.  Exactly one of x / x_hat is given: x_hat are the
 // dense coefficients p(x), (blocks * r, Cin), taken earlier (Eq. 3).
-// views: strides of x, g_y, g_x when they are not dense (low-rank paths only).
+// views: strides of x, g_y, g_x when they are not dense (low-rank paths only);
+// extras: what the persistent products kernel takes in itself (runs_fused only).
 static int run_core(const void* x, const void* x_hat_in, const void* g_y, const void* W, void* g_x,
                     void* g_W, const lbp_layer& L, const BasisPlan& plan, const Layout& lay,
                     uint8_t* wsb, cudaStream_t st, CoefLoc* gy_loc,
-                    const CallViews* views = nullptr) {
+                    const CallViews* views = nullptr, const FusedExtras* extras = nullptr) {
   const int r = plan.r;
   gy_loc->ptr = nullptr;
   if (r == L.k * L.k && x_hat_in == nullptr) return run_fullrank(x, g_y, W, g_x, g_W, L, wsb, st);
 
   uint32_t* status = reinterpret_cast<uint32_t*>(wsb);
-  // the expansion of the products kernel addresses the tokens of an image with
-  // 32-bit offsets (dense tensors: checked by fused_supported)
-  const bool span_ok = views == nullptr || is_dense(&views->gx) ||
-                       (views->gx.row * L.H + views->gx.token * L.W < (1ll << 31) &&
-                        views->gx.image / 8 < (1ll << 31));
-  if (fused_enabled() && fused_supported(L, plan) && span_ok) {
+  if (runs_fused(L, plan)) {
     FusedLayout fl;
     fused_scratch_bytes(L, r, &fl);
     gy_loc->ptr = wsb + lay.fused + fl.gy_hat;
-    gy_loc->rows = RowMap{fl.bpt, 128};
-    gy_loc->dc_to_sum = 1.0 / static_cast<double>(fused_scale_gy(L.k));
+    gy_loc->rows = RowMap{1, r};
+    gy_loc->dc_to_sum = 1.0 / static_cast<double>(fused_scale_gy(L.k, x_hat_in != nullptr));
     // projection kernel, then one persistent kernel for both products with the
     // expansion fused into the g_x_hat epilogue
     if (int e = mark_phase(0, st)) return e;
@@ -723,7 +730,7 @@ static int run_core(const void* x, const void* x_hat_in, const void* g_y, const 
       return mark_phase(2, s);
     };
     if (int e = launch_fused(x, x_hat_in, g_y, W, g_x, g_W, L, plan, wsb + lay.fused, status, st,
-                             after_projection, nullptr, views))
+                             after_projection, nullptr, views, extras))
       return e;
     for (int ph = 3; ph <= 5; ++ph)
       if (int e = mark_phase(ph, st)) return e;
@@ -818,6 +825,8 @@ static int run_backward_ex(const void* x, const void* x_hat, const void* g_y, co
 
   CallViews cv{ex->x_view, ex->gy_view, ex->gx_view};
   const bool strided = !is_dense(&cv.x) || !is_dense(&cv.gy) || !is_dense(&cv.gx);
+  // the persistent products kernel adds to g_W and takes the tokens outside the grid itself
+  const bool fused = (plan.r < L.k * L.k || x_hat != nullptr) && runs_fused(L, plan);
   const bool accumulate = ex->beta != 0.f || ex->n_extra > 0;
   if (!accumulate && ex->g_bias == nullptr && !strided)
     return run_core(x, x_hat, g_y, W, g_x, g_W, L, plan, lay, wsb, st, &gy_loc);
@@ -829,8 +838,8 @@ static int run_backward_ex(const void* x, const void* x_hat, const void* g_y, co
   float* sk = reinterpret_cast<float*>(wsb + lay.splitk);
   const long long T = static_cast<long long>(L.B) * L.H * L.W;
   lbp_layer Lg = L;
-  if (accumulate) Lg.gw_dtype = LBP_F32;   // this call's term in fp32, added below
-  void* gw_core = accumulate ? static_cast<void*>(gw0) : g_W;
+  if (accumulate && !fused) Lg.gw_dtype = LBP_F32;   // this call's term in fp32, added below
+  void* gw_core = accumulate && !fused ? static_cast<void*>(gw0) : g_W;
 
   // g_y as the bias gradient reads it when no coefficients serve
   const void* gy_tokens = g_y;
@@ -860,12 +869,14 @@ static int run_backward_ex(const void* x, const void* x_hat, const void* g_y, co
       if (int e = launch_copy_tokens(gxd, g_x, false, T, L.Cin, L.dtype, token_map(cv.gx, L.H, L.W), st))
         return e;
   } else {
+    const FusedExtras fe{ex->beta,     ex->n_extra,       ex->x_extra,        ex->gy_extra,
+                         ex->gx_extra, ex->x_extra_pitch, ex->gy_extra_pitch, ex->gx_extra_pitch};
     if (int e = run_core(x, x_hat, g_y, W, g_x, gw_core, Lg, plan, lay, wsb, st, &gy_loc,
-                         strided ? &cv : nullptr))
+                         strided ? &cv : nullptr, fused ? &fe : nullptr))
       return e;
   }
   const TokenMap gye_map{1, 1, pitched(ex->gy_extra_pitch, L.Cout) ? ex->gy_extra_pitch : L.Cout, 0, 0};
-  if (ex->n_extra > 0) {
+  if (ex->n_extra > 0 && !fused) {
     // tokens outside the grid (a class token): Eq. 2 exactly, on dense rows
     const void* xe = ex->x_extra;
     const void* gye = ex->gy_extra;
@@ -893,7 +904,7 @@ static int run_backward_ex(const void* x, const void* x_hat, const void* g_y, co
                                      TokenMap{1, 1, ex->gx_extra_pitch, 0, 0}, st))
         return e;
   }
-  if (accumulate)
+  if (accumulate && !fused)
     if (int e = launch_gw_combine(g_W, L.gw_dtype == LBP_BF16, gw0, ex->n_extra > 0 ? gw1 : nullptr,
                                   ex->beta, static_cast<long long>(L.Cout) * L.Cin, st))
       return e;

@@ -1,6 +1,6 @@
 // Small kernels around Algorithm 1 that a ViT layer needs and the paper leaves
-// out: accumulation into g_W, the bias gradient, and the row layout change for
-// coefficients x_hat that were taken at forward time.
+// out: accumulation into g_W (outside the products kernel), the bias gradient, and
+// dense copies of strided token tensors.
 #include <cuda_bf16.h>
 
 #include "lbp_internal.h"
@@ -102,38 +102,6 @@ __global__ void __launch_bounds__(256)
   g_bias[c] = static_cast<float>(s);
 }
 
-__device__ __forceinline__ uint32_t scale_bf16x2(uint32_t w, float f) {
-  return pack_bf16x2(bf16_lo(w) * f, bf16_hi(w) * f);
-}
-
-// Dense bf16 coefficient rows (block blk, slot q at row blk * r + q) -> rows
-// padded to groups: (blk / bpt) * tile_rows + (blk % bpt) * r + q; rows no block
-// owns are zero.  Values are multiplied by `factor`, a power of two (exact).
-// One thread moves 16 bytes.
-__global__ void __launch_bounds__(256)
-    regroup_rows_kernel(const uint4* __restrict__ dense, uint4* __restrict__ grouped, int nb, int r,
-                        int bpt, int tile_rows, int row_vec /* 16-byte pieces per row */,
-                        long long n_vec /* groups * tile_rows * row_vec */, float factor) {
-  const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= n_vec) return;
-  const long long row = i / row_vec;
-  const int piece = static_cast<int>(i - row * row_vec);
-  const long long g = row / tile_rows;
-  const int j = static_cast<int>(row - g * tile_rows);
-  const long long blk = g * bpt + j / r;
-  uint4 v = make_uint4(0u, 0u, 0u, 0u);
-  if (j < bpt * r && blk < nb) {
-    v = dense[(blk * r + j % r) * row_vec + piece];
-    if (factor != 1.f) {
-      v.x = scale_bf16x2(v.x, factor);
-      v.y = scale_bf16x2(v.y, factor);
-      v.z = scale_bf16x2(v.z, factor);
-      v.w = scale_bf16x2(v.w, factor);
-    }
-  }
-  grouped[i] = v;
-}
-
 // Moves n_tok tokens of C channels between a tensor laid out as `tm` says and a
 // dense (n_tok, C) matrix; one thread moves 16 bytes.  Strides in 16-byte units.
 __global__ void __launch_bounds__(256)
@@ -204,19 +172,6 @@ int launch_bias_finish(float* g_bias, int C, float beta, const double* a, int sl
                        const double* b, int slabs_b, cudaStream_t stream) {
   bias_finish_kernel<<<(C + 255) / 256, 256, 0, stream>>>(g_bias, C, beta, a, slabs_a, scale_a, b,
                                                          slabs_b);
-  count_launch();
-  LBP_CUDA_TRY(cudaGetLastError());
-  return LBP_OK;
-}
-
-int launch_regroup_rows(const void* dense, void* grouped, int nb, int r, RowMap rows, int C,
-                        float factor, cudaStream_t stream) {
-  const int row_vec = C * 2 / 16;
-  const long long groups = (static_cast<long long>(nb) + rows.bpt - 1) / rows.bpt;
-  const long long n_vec = groups * rows.tile_rows * row_vec;
-  regroup_rows_kernel<<<static_cast<unsigned>((n_vec + 255) / 256), 256, 0, stream>>>(
-      static_cast<const uint4*>(dense), static_cast<uint4*>(grouped), nb, r, rows.bpt,
-      rows.tile_rows, row_vec, n_vec, factor);
   count_launch();
   LBP_CUDA_TRY(cudaGetLastError());
   return LBP_OK;

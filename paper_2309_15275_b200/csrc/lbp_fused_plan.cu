@@ -7,7 +7,7 @@
 // order, and two accumulator slots let tile i + 1 be multiplied while tile i is
 // drained (tile i + 2 has to wait for tile i's slot).  The stages cost very
 // different amounts per tile kind:
-//   GX tile (g_x_hat = g_y_hat W, expanded by Eq. 7 in the epilogue): short
+//   GX tile (g_x_hat^T = W^T g_y_hat^T, expanded by Eq. 7 in the epilogue): short
 //           product (K = Cout), long epilogue (writes k*k / r times its size);
 //   GW tile (g_W = g_y_hat^T x_hat): long product (K = all low-rank rows), short
 //           epilogue.
@@ -29,9 +29,9 @@ namespace {
 // Operand delivery from L2 bounds the products: about 110 GB/s per SM.
 constexpr double kFeedBytesPerUs = 110e3;
 constexpr double kTileFixedUs = 0.3;
-// The expansion writes g_x at about 34 GB/s per SM (core butterfly); the forms
-// with extra bases or an 8 x 8 core are slower per byte.
-constexpr double kExpandBytesPerUs[3] = {34e3, 21e3, 12e3};
+// The expansion writes g_x at about 45 GB/s per SM (TMA stores, up to a 4 x 4
+// core); an 8 x 8 core is bound by the epilogue warps.
+constexpr double kExpandBytesPerUs[3] = {45e3, 30e3, 15e3};
 constexpr double kGwStoreBytesPerUs = 30e3;
 // K slices of g_W go through fp32 planes and one more kernel.
 constexpr double kReduceFixedUs = 3.0;
@@ -49,7 +49,7 @@ Costs tile_costs(const PlanShape& s, int bnw, int bnx, int kbps) {
   c.mma_w = kTileFixedUs + kbps * (a_bytes + bw) / kFeedBytesPerUs;
   c.mma_x = kTileFixedUs + s.num_kb_x * (a_bytes + bx) / kFeedBytesPerUs;
   c.epi_w = kTileFixedUs + 128.0 * bnw * 4 / kGwStoreBytesPerUs;
-  c.epi_x = 0.5 + static_cast<double>(s.bpt) * s.k * s.k * bnx * 2 / kExpandBytesPerUs[s.epi_kind];
+  c.epi_x = 0.5 + static_cast<double>(bnx / s.piece) * s.expand_bytes * 128.0 / kExpandBytesPerUs[s.epi_kind];
   return c;
 }
 
@@ -99,9 +99,21 @@ double simulate(int units, int n_gx, int n_gw, const Costs& c, std::vector<int>*
 }
 
 bool same_shape(const PlanShape& a, const PlanShape& b) {
-  return a.Cin == b.Cin && a.Cout == b.Cout && a.G == b.G && a.bpt == b.bpt && a.k == b.k &&
-         a.units == b.units && a.pair == b.pair && a.max_splits == b.max_splits &&
+  return a.gw_rows == b.gw_rows && a.gw_cols == b.gw_cols && a.gx_side == b.gx_side &&
+         a.blocks == b.blocks && a.piece == b.piece && a.n_extra == b.n_extra && a.units == b.units &&
+         a.pair == b.pair && a.bnw_step == b.bnw_step && a.bnx_step == b.bnx_step &&
+         a.bn_max == b.bn_max && a.max_splits == b.max_splits && a.expand_bytes == b.expand_bytes &&
          a.epi_kind == b.epi_kind && a.num_kb_w == b.num_kb_w && a.num_kb_x == b.num_kb_x;
+}
+
+int ceil_div(int a, int b) { return (a + b - 1) / b; }
+
+// Tiles of this shape under given column tiles.
+int count_gx(const PlanShape& s, int row_tile, int bnx) {
+  return ceil_div(s.gx_side, row_tile) * (ceil_div(s.blocks, bnx / s.piece) + ceil_div(s.n_extra, bnx));
+}
+int count_gw(const PlanShape& s, int row_tile, int bnw, int splits) {
+  return ceil_div(s.gw_rows, row_tile) * ceil_div(s.gw_cols, bnw) * splits;
 }
 
 struct Cached {
@@ -118,32 +130,31 @@ const TilePlan& plan_products(const PlanShape& s) {
     if (same_shape(c.shape, s)) return c.plan;
 
   const int row_tile = s.pair ? 256 : 128;
-  const int mt_w = (s.Cout + row_tile - 1) / row_tile;
-  const int gx_rows = s.pair ? (s.G + 1) / 2 : s.G;
-  const int bn_step = s.pair ? 128 : 64;
-  const int cin_pad = (s.Cin + bn_step - 1) / bn_step * bn_step;
+  const int bnw_top = ceil_div(s.gw_cols, s.bnw_step) * s.bnw_step;   // no column tile wider than the matrix
   static const int kSplitChoices[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192};
 
   TilePlan best{};
   double best_t = -1.0;
   const TuneOptions& tune = tune_options();
-  for (int bnw = bn_step; bnw <= 256; bnw += bn_step) {
-    for (int bnx = bn_step; bnx <= 256; bnx += bn_step) {
-      if (bnw > cin_pad || bnx > cin_pad) continue;
+  for (int bnw = s.bnw_step; bnw <= s.bn_max && bnw <= bnw_top; bnw += s.bnw_step) {
+    for (int bnx = s.bnx_step; bnx <= s.bn_max; bnx += s.bnx_step) {
+      if (bnx < s.piece) continue;
+      // no wider than all pieces (or all single columns) together need
+      const int less = bnx - s.bnx_step;
+      if (less >= s.piece && less / s.piece >= s.blocks && less >= s.n_extra) continue;
       for (int want : kSplitChoices) {
         if (want > 1 && (want > s.max_splits || want > s.num_kb_w / 4)) continue;
         if (tune.has_tiles &&
             (bnw != tune.tiles_bnw || bnx != tune.tiles_bnx || want != tune.tiles_splits))
           continue;
-        const int kbps = (s.num_kb_w + want - 1) / want;
-        const int splits = (s.num_kb_w + kbps - 1) / kbps;
-        const int nt_w = (s.Cin + bnw - 1) / bnw, n_tx = (s.Cin + bnx - 1) / bnx;
-        const int n_gw = mt_w * nt_w * splits, n_gx = gx_rows * n_tx;
+        const int kbps = ceil_div(s.num_kb_w, want);
+        const int splits = ceil_div(s.num_kb_w, kbps);
+        const int n_gw = count_gw(s, row_tile, bnw, splits), n_gx = count_gx(s, row_tile, bnx);
         const Costs c = tile_costs(s, bnw, bnx, kbps);
         const int units = n_gw + n_gx < s.units ? n_gw + n_gx : s.units;
         double t = simulate(units, n_gx, n_gw, c, nullptr);
         if (splits > 1)
-          t += kReduceFixedUs + (splits + 1.0) * s.Cout * static_cast<double>(s.Cin) * 4 / kReduceBytesPerUs;
+          t += kReduceFixedUs + (splits + 1.0) * s.gw_rows * static_cast<double>(s.gw_cols) * 4 / kReduceBytesPerUs;
         if (best_t < 0 || t < best_t - 1e-9) {
           best_t = t;
           best.BNw = bnw;
@@ -156,14 +167,15 @@ const TilePlan& plan_products(const PlanShape& s) {
   }
   best.model_us = best_t;
   if (best_t < 0) {   // an override that fits nothing: the widest tiles, no slices
-    best.BNw = best.BNx = cin_pad < 256 ? cin_pad : 256;
+    best.BNw = bnw_top < s.bn_max ? bnw_top : s.bn_max;
+    best.BNx = s.bn_max;
     best.splits = 1;
     best.kbps = s.num_kb_w;
   }
 
   // per-unit tile lists of the chosen plan
-  const int nt_w = (s.Cin + best.BNw - 1) / best.BNw, n_tx = (s.Cin + best.BNx - 1) / best.BNx;
-  const int n_gw = mt_w * nt_w * best.splits, n_gx = gx_rows * n_tx;
+  const int n_gw = count_gw(s, row_tile, best.BNw, best.splits);
+  const int n_gx = count_gx(s, row_tile, best.BNx);
   const int units = n_gw + n_gx < s.units ? n_gw + n_gx : s.units;
   FusedSchedule& sc = best.sched;
   sc.listed = 0;
@@ -183,9 +195,9 @@ const TilePlan& plan_products(const PlanShape& s) {
     sc.listed = 1;
   }
   if (tune.verbose)
-    fprintf(stderr, "lbp products plan (%s): G=%d BNw=%d BNx=%d gw_splits=%d kb/split=%d tiles=%d+%d "
+    fprintf(stderr, "lbp products plan (%s): BNw=%d BNx=%d gw_splits=%d kb/split=%d tiles=%d+%d "
                     "units=%d listed=%d model=%.1f us\n",
-            s.pair ? "CTA pairs" : "CTAs", s.G, best.BNw, best.BNx, best.splits, best.kbps, n_gx, n_gw,
+            s.pair ? "CTA pairs" : "CTAs", best.BNw, best.BNx, best.splits, best.kbps, n_gx, n_gw,
             units, sc.listed, best_t);
 
   if (cache.capacity() < 128) cache.reserve(128);

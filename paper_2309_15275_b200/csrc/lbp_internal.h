@@ -88,9 +88,9 @@ inline lbp_view resolve_view(const lbp_view* v, int H, int W, int C) {
 }
 inline bool is_dense(const lbp_view* v) { return v == nullptr || v->token == 0; }
 // 2-D row-major bf16 matrix (rows, cols): box = box_rows x 64 columns (128 B),
-// 128-byte swizzle.
+// 128-byte swizzle.  pitch: elements between rows (0: dense).
 int encode_matrix_tensor_map(CUtensorMap* map, const void* base, long long rows, long long cols,
-                             int box_rows);
+                             int box_rows, long long pitch = 0);
 
 // ---- kernel launchers (each returns an lbp_status) ------------------------
 // Row q of block blk of a projected tensor lives at
@@ -155,9 +155,10 @@ int launch_gemm(const void* A, bool a_mn_major, const void* Bm, void* D, int in_
                 long long M, long long N, long long K, float* splitk_ws, size_t splitk_ws_bytes,
                 uint32_t* status, cudaStream_t stream);
 size_t gemm_splitk_ws_bytes(long long M, long long N, long long K, int in_dtype);
-// D[i] = sum over `splits` fp32 planes of mn elements each (mn a multiple of 4), in plane order.
+// D[i] = beta * D[i] + sum over `splits` fp32 planes of mn elements each (mn a multiple
+// of 4), in plane order; D is not read when beta is 0.
 int launch_splitk_reduce(const float* planes, void* D, long long mn, int splits, bool d_bf16,
-                         cudaStream_t stream);
+                         float beta, cudaStream_t stream);
 
 int check_device_arch();
 
@@ -195,11 +196,6 @@ int launch_copy_tokens(const void* src, void* dst, bool to_dense, long long n_to
 // g_bias[c] <- beta * g_bias[c] + scale_a * (sum of the slabs of a) + (sum of the slabs of b)
 int launch_bias_finish(float* g_bias, int C, float beta, const double* a, int slabs_a, double scale_a,
                        const double* b, int slabs_b, cudaStream_t stream);
-// Dense coefficient rows (blocks * r, C) -> rows padded to groups under `rows`
-// (rows no block owns are zero), every bf16 value multiplied by `factor` (a power of two).
-int launch_regroup_rows(const void* dense, void* grouped, int nb, int r, RowMap rows, int C,
-                        float factor, cudaStream_t stream);
-
 // Tuning switches, read from the environment once (first use):
 //   LBP_FUSED=0          separate product and expansion kernels instead of the
 //                        persistent products kernel
