@@ -696,6 +696,7 @@ struct CoefLoc {
   const void* ptr;
   RowMap rows;
   double dc_to_sum;   // token sum of a block = dc_to_sum * its (0,0) coefficient as stored
+  int dc_slot;        // slot of that coefficient; -1: basis (0,0) is not selected
 };
 
 // Whether a low-rank call runs on the persistent products kernel.
@@ -730,7 +731,7 @@ static int run_core(const void* x, const void* x_hat_in, const void* g_y, const 
       return mark_phase(2, s);
     };
     if (int e = launch_fused(x, x_hat_in, g_y, W, g_x, g_W, L, plan, wsb + lay.fused, status, st,
-                             after_projection, nullptr, views, extras))
+                             after_projection, nullptr, views, extras, &gy_loc->dc_slot))
       return e;
     for (int ph = 3; ph <= 5; ++ph)
       if (int e = mark_phase(ph, st)) return e;
@@ -744,6 +745,9 @@ static int run_core(const void* x, const void* x_hat_in, const void* g_y, const 
   gy_loc->ptr = gy_hat;
   gy_loc->rows = dense;
   gy_loc->dc_to_sum = static_cast<double>(L.k);   // orthonormal: coefficient = block sum / k
+  gy_loc->dc_slot = -1;
+  for (int q = 0; q < r; ++q)
+    if (plan.seq_i[q] == 0 && plan.seq_j[q] == 0) gy_loc->dc_slot = q;
 
   if (int e = mark_phase(0, st)) return e;
   if (x_hat_in != nullptr) {
@@ -914,15 +918,12 @@ static int run_backward_ex(const void* x, const void* x_hat, const void* g_y, co
     // otherwise g_y is read once more.
     double* pa = reinterpret_cast<double*>(wsb + el.bias_a);
     double* pb = reinterpret_cast<double*>(wsb + el.bias_b);
-    int q_dc = -1;
-    for (int q = 0; q < plan.r; ++q)
-      if (plan.seq_i[q] == 0 && plan.seq_j[q] == 0) q_dc = q;
     long long n_a;
     double scale_a;
-    if (gy_loc.ptr != nullptr && q_dc >= 0) {
+    if (gy_loc.ptr != nullptr && gy_loc.dc_slot >= 0) {
       n_a = static_cast<long long>(L.B) * blocks_along(L.H, L.k) * blocks_along(L.W, L.k);
       scale_a = gy_loc.dc_to_sum;
-      if (int e = launch_column_sum(gy_loc.ptr, L.dtype, n_a, L.Cout, gy_loc.rows, plan.r, q_dc, pa, st))
+      if (int e = launch_column_sum(gy_loc.ptr, L.dtype, n_a, L.Cout, gy_loc.rows, plan.r, gy_loc.dc_slot, pa, st))
         return e;
     } else {
       n_a = T;

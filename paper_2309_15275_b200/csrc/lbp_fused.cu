@@ -25,7 +25,7 @@
 //
 // Warp roles: warp 0 TMA producer, warp 1 TMEM owner and tcgen05 issuer (the
 // leader CTA's of a pair), warps 2 and 3 the TMA stores of the two epilogue groups,
-// warps 4-11 epilogue in two groups of four that take turns on the blocks (GX) or
+// warps 4-19 epilogue in two groups of eight that take turns on the blocks (GX) or
 // 32-column chunks (GW) of a tile, while the tensor core already works on the next
 // tile (two accumulator slots in TMEM, used alternately).
 // All roles walk the same tile list.  Barriers:
@@ -53,17 +53,15 @@ namespace lbp {
 namespace fused {
 
 constexpr int BK = 64;
-constexpr int kStages = 5;
 constexpr int kABytes = BM * BK * 2;             // 16 KB: this CTA's 128 rows of A
 constexpr int kBBytes = 128 * BK * 2;            // 16 KB: this CTA's half of B (a pair's), or up to 128 columns
 constexpr int kStageBytes = kABytes + kBBytes;   // 32 KB
 constexpr int kChunkBytes = 64 * BK * 2;         // 8 KB: one 64-wide chunk of an MN-major tile
 // warps 0-3: TMA producer, tensor-core issuer, a store warp per epilogue group; then those groups
-constexpr int kThreads = (4 + 4 * kEGroups) * 32;
-constexpr int kOffE = kStages * kStageBytes;
-constexpr int kOffBar = kOffE + kEGroups * kGroupBytes;
-constexpr int kSmemBytes = kOffBar + 320 + 1024;
-static_assert((2 * kStages + 4 + 2 * kEGroups * kFillBufs) * 8 + 8 <= 320, "barriers");
+constexpr int kThreads = (4 + 8 * kEGroups) * 32;
+constexpr int kStages = 5;
+constexpr int kOffBar = kStages * kStageBytes + kEGroups * kGroupBytes;   // ring, buffers, then the barriers
+constexpr int kSmemBytes = kOffBar + 384 + 1024;
 static_assert(kSmemBytes <= 227 * 1024, "shared memory budget of one CTA exceeded");
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kSlotCols = 256;   // two accumulator slots; tile number t of a unit uses slot t & 1
@@ -158,6 +156,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     lbp_products_kernel(const __grid_constant__ OperandMaps tm, const __grid_constant__ StoreMaps sm,
                         const __grid_constant__ FusedParams p, const __grid_constant__ FusedBasis fb,
                         const __grid_constant__ FusedSchedule sc) {
+  using X = Expand<K, CORE>;
+  constexpr int kBufs = X::kBufs;
+  static_assert((2 * kStages + 4 + 2 * kEGroups * kBufs) * 8 + 8 <= 384, "barriers");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -165,9 +166,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* empty_bar = full_bar + kStages;
   uint64_t* acc_full = empty_bar + kStages;                   // [2]
   uint64_t* acc_empty = acc_full + 2;                         // [2], the leader's are used
-  uint64_t* fill_full = acc_empty + 2;                        // [kEGroups][kFillBufs]
-  uint64_t* fill_empty = fill_full + kEGroups * kFillBufs;    // [kEGroups][kFillBufs]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fill_empty + kEGroups * kFillBufs);
+  uint64_t* fill_full = acc_empty + 2;                        // [kEGroups][kBufs]
+  uint64_t* fill_empty = fill_full + kEGroups * kBufs;    // [kEGroups][kBufs]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fill_empty + kEGroups * kBufs);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   constexpr int kCtas = PAIR ? 2 : 1;   // CTAs of a unit
@@ -182,10 +183,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int s = 0; s < 2; ++s) {
       ptx::mbar_init(&acc_full[s], 1);
-      ptx::mbar_init(&acc_empty[s], kCtas * 4 * kEGroups);   // epilogue warps of all CTAs of the unit
+      ptx::mbar_init(&acc_empty[s], kCtas * 8 * kEGroups);   // epilogue warps of all CTAs of the unit
     }
-    for (int s = 0; s < kEGroups * kFillBufs; ++s) {
-      ptx::mbar_init(&fill_full[s], 4);    // the warps of the group
+    for (int s = 0; s < kEGroups * kBufs; ++s) {
+      ptx::mbar_init(&fill_full[s], 8);    // the warps of the group
       ptx::mbar_init(&fill_empty[s], 1);   // its store warp
     }
     ptx::mbar_fence_init();
@@ -331,15 +332,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       trace_mark(p, 3);
     }
   } else {
-    // ============ epilogue (each CTA its own 128 lanes): two groups of four warps (from
+    // ============ epilogue (each CTA its own 128 lanes): two groups of eight warps (from
     // warp 4 on), each with a store warp (warps 2 and 3) ============
     const bool stores = warp < 4;
-    const int eg = stores ? warp - 2 : (warp - 4) >> 2;
+    const int eg = stores ? warp - 2 : (warp - 4) >> 3;
+    const int sub = (warp >> 2) & 1 ? 0 : 1;             // half of the group (warps 4-7 and 12-15: 0)
     const int quarter = warp & 3;                        // TMEM lane quarter this warp may read
-    const int etid = quarter * 32 + lane;                // 0..127 within the group
-    const int bar_id = 1 + eg;
-    Fills fills{smem + kOffE + eg * kGroupBytes, fill_full + eg * kFillBufs, fill_empty + eg * kFillBufs,
-                p.status, 0u, false};
+    const bool first = sub == 0 && quarter == 0 && lane == 0;   // one thread of the group
+    const int bar_id = 1 + eg;                           // the group; its halves: 3 + 2 eg + sub
+    Fills<X> fills{smem + kStages * kStageBytes + eg * kGroupBytes, fill_full + eg * kBufs,
+                       fill_empty + eg * kBufs, p.status, 0u, 0u};
     bool alive = true;
     for (int ti = 0; ti < my_tiles && alive; ++ti) {
       const WorkTile tl = unit_tile(p, sc, unit, units, ti);
@@ -353,26 +355,24 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (stores) {
         if (!tl.is_gw) alive = store_gx<K, CORE>(p, sm, dt, fills, eg, lane);
         // before a GW tile, which uses the buffers its own way: everything has been read
-        if (alive && !tl.is_gw && ti + 1 < my_tiles && unit_tile(p, sc, unit, units, ti + 1).is_gw) {
-          fills.give_back<0>(fills.count - 1, lane);
-          fills.held = false;
-        }
+        if (alive && !tl.is_gw && ti + 1 < my_tiles && unit_tile(p, sc, unit, units, ti + 1).is_gw)
+          fills.flush(lane);
         continue;
       }
       bool ok = ptx::mbar_wait(&acc_full[slot], static_cast<uint32_t>(ti >> 1) & 1u, p.status, (5u << 16) | 5u);
       // a GW tile stages its chunks in the buffers: the stores of every fill have been read
       if (tl.is_gw)
-        for (int b = 0; b < kFillBufs && ok; ++b) ok = fills.wait_empty(fills.count + b);
+        for (int b = 0; b < kBufs && ok; ++b) ok = fills.wait_empty(fills.count + b);
       // One answer for the whole group: a thread that saw its own wait expire, or
-      // the flag another role raised, takes the other 127 threads with it (read
+      // the flag another role raised, takes the other 255 threads with it (read
       // one by one after the barrier, the flag could split the group, and the
       // threads left inside the tile would wait on a barrier that never fills).
-      if (named_bar_or(bar_id, 128, !ok || *abort_flag != 0)) {
-        if (etid == 0) *abort_flag = 1;
+      if (named_bar_or(bar_id, 256, !ok || *abort_flag != 0)) {
+        if (first) *abort_flag = 1;
         break;
       }
       ptx::tc_fence_after_sync();
-      if (etid == 0 && ti < 15) trace_mark(p, 8 + 8 * ti + 2 + 2 * eg);
+      if (first && ti < 15) trace_mark(p, 8 + 8 * ti + 2 + 2 * eg);
       uint64_t* const mine = &acc_empty[slot];
       auto release = [mine]() {
         if constexpr (PAIR)
@@ -382,13 +382,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       };
       bool drained = true;
       if (tl.is_gw)
-        drain_gw(p, dt, fills.buf, bar_id, eg, etid, quarter, lane, release);
+        drain_gw(p, dt, reinterpret_cast<float*>(fills.buf + sub * kGwStageBytes), 3 + 2 * eg + sub,
+                 2 * eg + sub, quarter, lane, release);
       else if (tl.a >= p.n_rt)
-        drained = drain_gx_extra(p, dt, fills, eg, quarter, lane, release);
+        drained = drain_gx_extra(p, dt, fills, eg, sub, quarter, lane, release);
       else
-        drained = drain_gx<K, CORE>(p, fb, dt, fills, eg, quarter, lane, release);
+        drained = drain_gx<K, CORE>(p, fb, dt, fills, eg, sub, quarter, lane, release);
       if (!drained) *abort_flag = 1;   // the group leaves together at the next tile
-      if (etid == 0 && ti < 15) {
+      if (first && ti < 15) {
         trace_mark(p, 8 + 8 * ti + 3 + 2 * eg);
 #ifdef LBP_ROLE_TRACE
         if (eg == 0 && p.trace != nullptr)
@@ -401,7 +402,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!alive) *abort_flag = 1;
       bulk_wait_all();   // this warp's stores are complete before the CTA leaves
     }
-    if (etid == 0 && !stores) trace_mark(p, 4);   // latest of the groups
+    if (first && !stores) trace_mark(p, 4);   // latest of the groups
   }
 
   ptx::tc_fence_before_sync();
@@ -486,11 +487,48 @@ static int expand_core(const BasisPlan& bp) {
     lh += hj && !hi;
     hh += hi && hj;
   }
-  return hh == 0 && hl <= 1 && lh <= 1 ? fused::kCoreSparse : 8;
+  if (hh > 0) return 8;
+  return hl <= 1 && lh <= 1 ? fused::kCoreSparse : fused::kCoreNoHH;
 }
 
-static FusedBasis make_fused_basis(const BasisPlan& bp, int core) {
+// The same bases with their slots ordered by rows (i, then j).  Only where every row
+// holds j = 0 .. n_i - 1 (true of every set that contains, with a basis, all those of
+// lower frequency along W: the LP_L1, LP_Linf and PREFIX sets): the expansion then
+// reads a row with one load.  False: bp is not changed.
+static bool order_by_rows(BasisPlan* bp) {
+  int slot_of[8][8], n[8] = {};
+  for (auto& row : slot_of)
+    for (int& q : row) q = -1;
+  for (int q = 0; q < bp->r; ++q) {
+    if (bp->seq_i[q] >= 8 || bp->seq_j[q] >= 8) return false;
+    slot_of[bp->seq_i[q]][bp->seq_j[q]] = q;
+    ++n[bp->seq_i[q]];
+  }
+  for (int i = 0; i < 8; ++i)
+    for (int j = 0; j < n[i]; ++j)
+      if (slot_of[i][j] < 0) return false;
+  const BasisPlan old = *bp;
+  int16_t new_slot[kMaxRank];
+  int q = 0;
+  for (int i = 0; i < 8; ++i)
+    for (int j = 0; j < n[i]; ++j, ++q) {
+      const int from = slot_of[i][j];
+      new_slot[from] = static_cast<int16_t>(q);
+      bp->nat_i[q] = old.nat_i[from];
+      bp->nat_j[q] = old.nat_j[from];
+      bp->seq_i[q] = old.seq_i[from];
+      bp->seq_j[q] = old.seq_j[from];
+    }
+  for (int p = 0; p < bp->LB * bp->LB; ++p)
+    if (old.qmap[p] >= 0) bp->qmap[p] = new_slot[old.qmap[p]];
+  return true;
+}
+
+static FusedBasis make_fused_basis(const BasisPlan& bp, int core, bool by_rows) {
   FusedBasis fb{};
+  fb.by_rows = by_rows ? 1 : 0;
+  if (by_rows)
+    for (int q = bp.r - 1; q >= 0; --q) fb.row[bp.seq_i[q]] = q;
   if (core <= 4) {
     for (int a = 0; a < bp.LB; ++a)
       for (int b = 0; b < bp.LB; ++b) {
@@ -506,14 +544,13 @@ static FusedBasis make_fused_basis(const BasisPlan& bp, int core) {
       if (q < 0) continue;
       // bit 0 of a natural index is set exactly where the sequency is 4 or more
       const int quad = 2 * (b & 1) + (a & 1), pos = (a >> 1) * 4 + (b >> 1);
-      if (quad == 3) fb.has_hh = 1;
       if (core == fused::kCoreSparse && quad != 0) {
         const int side = quad - 1;
         fb.ex_col[side] = q;
         fb.ex_keep[side] = 0xffffffffu;
         for (int i = 0; i < 16; ++i) {
           const int par = __builtin_popcount((a >> 1) & (i >> 2)) + __builtin_popcount((b >> 1) & (i & 3));
-          fb.ex_sign[side][i] = static_cast<uint32_t>(par & 1) << 31;
+          fb.ex_sign[side][i] = (par & 1) != 0 ? -1.f : 1.f;
         }
       } else {
         fb.col[quad * 16 + pos] = q;
@@ -540,7 +577,7 @@ static PlanShape plan_shape(const lbp_layer& L, long long blocks, int piece, int
   s.bn_max = pair ? 256 : 128;
   s.max_splits = static_cast<int>(planes_bytes / (static_cast<size_t>(L.Cout) * L.Cin * 4));
   s.expand_bytes = blocks > 0 ? L.k * L.k * 2 : 2;
-  s.epi_kind = core == 8 ? 2 : core == fused::kCoreSparse ? 1 : 0;
+  s.epi_kind = blocks == 0 ? -1 : core <= 4 ? 0 : core == fused::kCoreSparse ? 1 : 2;
   s.num_kb_w = static_cast<int>((blocks * piece + fused::BK - 1) / fused::BK) +
                (n_extra + fused::BK - 1) / fused::BK;
   s.num_kb_x = (L.Cout + fused::BK - 1) / fused::BK;
@@ -596,7 +633,7 @@ static int fused_project(const void* x, void* x_hat, const void* g_y, void* gy_h
 // Maps of the expansion's stores: map du * S + dv addresses the tokens (S u + du,
 // S v + dv) of every image, so that its extents clip exactly at the grid's edge.
 // Maps of offsets a small grid does not have are never used (copies of the first).
-static int encode_store_maps(fused::StoreMaps* sm, void* g_x, const lbp_layer& L, int S, int T,
+static int encode_store_maps(fused::StoreMaps* sm, void* g_x, const lbp_layer& L, int S, int T, int box_rows,
                              const lbp_view& v) {
   for (int du = 0; du < S; ++du)
     for (int dv = 0; dv < S; ++dv) {
@@ -607,7 +644,7 @@ static int encode_store_maps(fused::StoreMaps* sm, void* g_x, const lbp_layer& L
       const lbp_view s{v.image, v.row * S, v.token * S};
       __nv_bfloat16* base = static_cast<__nv_bfloat16*>(g_x) + du * v.row + dv * v.token;
       if (int e = encode_box_tensor_map(&sm->m[du * S + dv], base, LBP_BF16, L.B, (L.H - du + S - 1) / S,
-                                        (L.W - dv + S - 1) / S, L.Cin, 128, T, 4, false, &s))
+                                        (L.W - dv + S - 1) / S, L.Cin, 128, T, box_rows, false, &s))
         return e;
     }
   return LBP_OK;
@@ -712,7 +749,7 @@ static int launch_products(const ProductsCall& c, cudaStream_t stream) {
     if (int e = encode_matrix_tensor_map(&tm.gyhat_k, c.gy_hat, rows, L.Cout, p.BNx / ctas)) return e;
     if (int e = encode_matrix_tensor_map(&tm.gyhat_mn, c.gy_hat, rows, L.Cout, BK)) return e;
     if (int e = encode_matrix_tensor_map(&tm.xhat, c.x_hat, rows, L.Cin, BK)) return e;
-    if (int e = encode_store_maps(&sm, c.g_x, L, K / T, T, c.gx_view)) return e;
+    if (int e = encode_store_maps(&sm, c.g_x, L, K / T, T, 4, c.gx_view)) return e;
   }
   if (n_extra > 0) {
     if (int e = encode_matrix_tensor_map(&tm.gye_k, c.ex.gy, n_extra, L.Cout, p.BNx / ctas, c.ex.gy_pitch)) return e;
@@ -771,10 +808,12 @@ static int launch_products(const ProductsCall& c, cudaStream_t stream) {
     LBP_CASE(8, 2);
     LBP_CASE(8, 4);
     LBP_CASE(8, 6);
+    LBP_CASE(8, 7);
     LBP_CASE(8, 8);
     LBP_CASE(16, 2);
     LBP_CASE(16, 4);
     LBP_CASE(16, 6);
+    LBP_CASE(16, 7);
     LBP_CASE(16, 8);
   }
 #undef LBP_CASE
@@ -786,13 +825,17 @@ static int launch_products(const ProductsCall& c, cudaStream_t stream) {
 }
 
 int launch_fused(const void* x, const void* x_hat_dense, const void* g_y, const void* W, void* g_x,
-                 void* g_W, const lbp_layer& L, const BasisPlan& bp, uint8_t* scratch,
+                 void* g_W, const lbp_layer& L, const BasisPlan& list, uint8_t* scratch,
                  uint32_t* status, cudaStream_t stream, FusedPhaseHook hook, void* hook_arg,
-                 const CallViews* views, const FusedExtras* extras) {
+                 const CallViews* views, const FusedExtras* extras, int* dc_slot) {
   FusedLayout lay;
-  fused_scratch_bytes(L, bp.r, &lay);
+  fused_scratch_bytes(L, list.r, &lay);
   void* x_hat = scratch + lay.x_hat;
   void* gy_hat = scratch + lay.gy_hat;
+  // the slots of a block may lie in any order as long as x_hat and g_y_hat agree;
+  // coefficients handed in keep the caller's
+  BasisPlan bp = list;
+  const bool by_rows = x_hat_dense == nullptr && order_by_rows(&bp);
   if (int e = fused_project(x, x_hat, g_y, gy_hat, L, bp, views, status, stream)) return e;
   if (hook != nullptr)
     if (int e = hook(hook_arg, stream)) return e;
@@ -806,7 +849,12 @@ int launch_fused(const void* x, const void* x_hat_dense, const void* g_y, const 
   c.g_x = g_x;
   c.gx_view = resolve_view(views ? &views->gx : nullptr, L.H, L.W, L.Cin);
   c.gx_scale = x_hat_dense != nullptr ? 1.0f / static_cast<float>(L.k) : 1.0f;
-  c.fb = make_fused_basis(bp, c.core);
+  c.fb = make_fused_basis(bp, c.core, by_rows);
+  if (dc_slot != nullptr) {
+    *dc_slot = -1;
+    for (int q = 0; q < bp.r; ++q)
+      if (bp.seq_i[q] == 0 && bp.seq_j[q] == 0) *dc_slot = q;
+  }
   if (extras != nullptr) c.ex = *extras;
   c.W = W;
   c.g_W = g_W;

@@ -88,11 +88,14 @@ __device__ __forceinline__ WorkTile unit_tile(const FusedParams& p, const FusedS
 struct FusedBasis {
   int32_t col[64];
   uint32_t keep[64];
-  int32_t has_hh;            // 8 x 8: some basis has both indices of 4 or more
+  // 1: the slots of a block are ordered by rows (i, then j) and every row holds j = 0 ..
+  // n_i - 1 only: row i starts at column row[i] and is read with one wide load
+  int32_t by_rows;
+  int32_t row[8];
   // sparse form: the one basis with i >= 4 (side 0) and the one with j >= 4 (side 1)
   int32_t ex_col[2];
   uint32_t ex_keep[2];
-  uint32_t ex_sign[2][16];   // sign bit of that basis on the 4 x 4 patches
+  float ex_sign[2][16];      // +-1: sign of that basis on the 4 x 4 patches
 };
 
 // Builds with -DLBP_ROLE_TRACE carry a per-CTA role timeline (diagnostics) in
@@ -189,7 +192,7 @@ struct PlanShape {
   int bnw_step, bnx_step, bn_max;   // column tiles: multiples of the step up to bn_max
   int max_splits;                   // K slices of g_W the scratch has planes for
   int expand_bytes;                 // what the epilogue of a GX tile writes per piece and channel
-  int epi_kind;                     // expansion: 0 up to a 4 x 4 core, 1 sparse 8 x 8, 2 8 x 8 core
+  int epi_kind;                     // expansion: 0 up to a 4 x 4 array, 1 sparse 8 x 8, 2 8 x 8; -1 none
   int num_kb_w, num_kb_x;
 };
 struct TilePlan {
@@ -222,10 +225,12 @@ struct FusedExtras {
 };
 // Exactly one of x / x_hat_dense is given; x_hat_dense are coefficients p(x)
 // taken earlier, stored densely (blocks * r, Cin).  views: null = all dense.
+// dc_slot: receives the slot of basis (0, 0) in g_y_hat, -1 = not selected.
 int launch_fused(const void* x, const void* x_hat_dense, const void* g_y, const void* W, void* g_x,
                  void* g_W, const lbp_layer& L, const BasisPlan& bp, uint8_t* scratch,
                  uint32_t* status, cudaStream_t stream, FusedPhaseHook hook, void* hook_arg,
-                 const CallViews* views = nullptr, const FusedExtras* extras = nullptr);
+                 const CallViews* views = nullptr, const FusedExtras* extras = nullptr,
+                 int* dc_slot = nullptr);
 
 // Modelled time (microseconds) of the products kernel of this layer on `pairs`
 // CTA pairs, and of its projection kernel on `ctas` SMs (both from B200

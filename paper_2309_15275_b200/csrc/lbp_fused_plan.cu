@@ -29,9 +29,10 @@ namespace {
 // Operand delivery from L2 bounds the products: about 110 GB/s per SM.
 constexpr double kFeedBytesPerUs = 110e3;
 constexpr double kTileFixedUs = 0.3;
-// The expansion writes g_x at about 45 GB/s per SM (TMA stores, up to a 4 x 4
-// core); an 8 x 8 core is bound by the epilogue warps.
-constexpr double kExpandBytesPerUs[3] = {45e3, 30e3, 15e3};
+// The expansion writes g_x at about 45 GB/s per SM (bound by the stores in flight, up
+// to a 4 x 4 array); with an 8 x 8 array the epilogue warps bind.  It takes four blocks
+// at a time.
+constexpr double kExpandBytesPerUs[3] = {45e3, 30e3, 20e3};
 constexpr double kGwStoreBytesPerUs = 30e3;
 // K slices of g_W go through fp32 planes and one more kernel.
 constexpr double kReduceFixedUs = 3.0;
@@ -49,7 +50,8 @@ Costs tile_costs(const PlanShape& s, int bnw, int bnx, int kbps) {
   c.mma_w = kTileFixedUs + kbps * (a_bytes + bw) / kFeedBytesPerUs;
   c.mma_x = kTileFixedUs + s.num_kb_x * (a_bytes + bx) / kFeedBytesPerUs;
   c.epi_w = kTileFixedUs + 128.0 * bnw * 4 / kGwStoreBytesPerUs;
-  c.epi_x = 0.5 + static_cast<double>(bnx / s.piece) * s.expand_bytes * 128.0 / kExpandBytesPerUs[s.epi_kind];
+  c.epi_x = 0.5 + (s.epi_kind < 0 ? bnx : (bnx / s.piece + 3) / 4 * 4) * s.expand_bytes * 128.0 /
+                    kExpandBytesPerUs[s.epi_kind < 0 ? 0 : s.epi_kind];
   return c;
 }
 
