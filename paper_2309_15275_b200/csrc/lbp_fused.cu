@@ -587,9 +587,9 @@ static PlanShape plan_shape(const lbp_layer& L, long long blocks, int piece, int
 double fused_products_model_us(const lbp_layer& L, const BasisPlan& bp, int pairs) {
   FusedLayout lay;
   fused_scratch_bytes(L, bp.r, &lay);
-  // measured times sit about a third above the model (the stages of a unit share
-  // its path to L2), plus the launch and the first operand tiles
-  return 1.35 * plan_products(plan_shape(L, grid_blocks(L), bp.r, expand_core(bp), 0, lay.planes_bytes,
+  // measured times sit a little above the model, plus the launch and the first
+  // operand tiles
+  return 1.1 * plan_products(plan_shape(L, grid_blocks(L), bp.r, expand_core(bp), 0, lay.planes_bytes,
                                          pairs, true))
                     .model_us +
          4.0;

@@ -26,14 +26,15 @@ namespace lbp {
 namespace {
 
 // ---- cost model (microseconds) ----
-// Operand delivery from L2 bounds the products: about 110 GB/s per SM.
-constexpr double kFeedBytesPerUs = 110e3;
+// Operand delivery from L2 bounds the products: per SM about 95 GB/s to a GX tile, 76
+// GB/s to a GW tile (all SMs at work: 11 TB/s).
+constexpr double kFeedGxBytesPerUs = 95e3, kFeedGwBytesPerUs = 76e3;
 constexpr double kTileFixedUs = 0.3;
-// The expansion writes g_x at about 45 GB/s per SM (bound by the stores in flight, up
+// The expansion writes g_x at about 43 GB/s per SM (bound by the stores in flight, up
 // to a 4 x 4 array); with an 8 x 8 array the epilogue warps bind.  It takes four blocks
 // at a time.
-constexpr double kExpandBytesPerUs[3] = {45e3, 30e3, 20e3};
-constexpr double kGwStoreBytesPerUs = 30e3;
+constexpr double kExpandBytesPerUs[3] = {43e3, 26e3, 18e3};
+constexpr double kGwStoreBytesPerUs = 45e3;
 // K slices of g_W go through fp32 planes and one more kernel.
 constexpr double kReduceFixedUs = 3.0;
 constexpr double kReduceBytesPerUs = 4e6;
@@ -47,8 +48,8 @@ Costs tile_costs(const PlanShape& s, int bnw, int bnx, int kbps) {
   const double bw = (s.pair ? bnw / 2 : bnw) * 64.0 * 2;       // its share of B
   const double bx = (s.pair ? bnx / 2 : bnx) * 64.0 * 2;
   Costs c;
-  c.mma_w = kTileFixedUs + kbps * (a_bytes + bw) / kFeedBytesPerUs;
-  c.mma_x = kTileFixedUs + s.num_kb_x * (a_bytes + bx) / kFeedBytesPerUs;
+  c.mma_w = kTileFixedUs + kbps * (a_bytes + bw) / kFeedGwBytesPerUs;
+  c.mma_x = kTileFixedUs + s.num_kb_x * (a_bytes + bx) / kFeedGxBytesPerUs;
   c.epi_w = kTileFixedUs + 128.0 * bnw * 4 / kGwStoreBytesPerUs;
   c.epi_x = 0.5 + (s.epi_kind < 0 ? bnx : (bnx / s.piece + 3) / 4 * 4) * s.expand_bytes * 128.0 /
                     kExpandBytesPerUs[s.epi_kind < 0 ? 0 : s.epi_kind];
