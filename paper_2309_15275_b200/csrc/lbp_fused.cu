@@ -599,8 +599,8 @@ double fused_projection_model_us(const lbp_layer& L, const BasisPlan& bp, int ct
   const double T = static_cast<double>(L.B) * L.H * L.W;
   const double nb = static_cast<double>(grid_blocks(L));
   const double bytes = 2.0 * (T + nb * bp.r) * (L.Cin + L.Cout);
-  // one SM streams about 70 GB/s through its tile ring; the chip about 5.2 TB/s
-  const double rate = ctas * 70e3 < 5.2e6 ? ctas * 70e3 : 5.2e6;   // bytes per microsecond
+  // one SM moves about 80 GB/s in and out, the chip about 5.3 TB/s
+  const double rate = ctas * 80e3 < 5.3e6 ? ctas * 80e3 : 5.3e6;   // bytes per microsecond
   return bytes / rate + 5.0;
 }
 

@@ -106,6 +106,7 @@ int launch_project(const void* t, void* t_hat, int dtype, int B, int H, int W, i
                    float scale = 0.f, const lbp_view* view = nullptr);
 
 // Per-thread switch read by the projection launchers (see ProjParams::defer_wait).
+bool test_stall_projection();   // test hook (lbp_fused.cu)
 void set_projection_defer_wait(bool on);
 bool projection_defer_wait();
 

@@ -296,29 +296,9 @@ int launch_project2(const void* t0, void* out0, int C0, const void* t1, void* ou
   LBP_CUDA_TRY(cudaGetDevice(&dev));
   LBP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
 
-  // The tcgen05 kernel works on four 64-channel chunks of a block at a time: with
-  // channel counts that leave many of those places empty (48 and 192 channels:
-  // half of them) the warp-level kernel is the faster one.
-  const int chunks_all = p.n_chunks[0] + (t1 ? p.n_chunks[1] : 0);
-  const int places_all = 4 * ((p.n_chunks[0] + 3) / 4 + (t1 ? (p.n_chunks[1] + 3) / 4 : 0));
-  if (dtype == LBP_BF16 && tune_options().umma && project_umma_supported(K, bp.r) &&
-      5 * chunks_all >= 4 * places_all) {
-    // orders 8 and 16 at low rank: tcgen05 kernel, an item is a block x four 64-channel chunks
-    CUtensorMap qm[2];
-    // a box is 64 tokens: the block at order 8, four of its token rows at order 16
-    const int box_h = 64 / K;
-    if (int e = encode_box_tensor_map(&qm[0], t0, dtype, B, H, W, C0, box_c, K, box_h, true, view0)) return e;
-    qm[1] = qm[0];
-    if (t1 != nullptr)
-      if (int e = encode_box_tensor_map(&qm[1], t1, dtype, B, H, W, C1, box_c, K, box_h, true, view1)) return e;
-    ProjParams pq = p;
-    pq.n_chunks[0] = (p.n_chunks[0] + 3) / 4;
-    pq.n_chunks[1] = t1 ? (p.n_chunks[1] + 3) / 4 : 1;
-    pq.n_items0 = static_cast<uint32_t>(static_cast<long long>(p.nb) * pq.n_chunks[0]);
-    pq.n_items = pq.n_items0 + (t1 ? static_cast<uint32_t>(static_cast<long long>(p.nb) * pq.n_chunks[1]) : 0u);
-    return launch_project_umma(qm, static_cast<__nv_bfloat16*>(out0), static_cast<__nv_bfloat16*>(out1),
-                               pq, bp, sms, stream);
-  }
+  if (dtype == LBP_BF16 && tune_options().umma && project_umma_supported(K, bp.r) && rows.bpt == 1)
+    return launch_project_umma(t0, out0, C0, view0, t1, out1, C1, view1, B, H, W, bp, p.scale[0], p.scale[1],
+                               sms, status, stream);
   if (dtype == LBP_BF16 && project_mma_supported(K, bp.r)) {
     // bf16 data at moderate rank: the +-1 basis matrix is applied on the tensor pipe
     CUtensorMap sw[2];

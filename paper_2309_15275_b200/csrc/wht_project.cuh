@@ -44,11 +44,13 @@ bool project_mma_supported(int k, int r);
 bool project_mma_strips(int k, int r);
 int launch_project_mma(const CUtensorMap* tmaps, __nv_bfloat16* out0, __nv_bfloat16* out1,
                        const ProjParams& p, const BasisPlan& bp, int sms, cudaStream_t stream);
-// Orders 8 and 16, r <= 48 on the tcgen05 tensor cores (boxes of 64 tokens; in the
-// parameters n_chunks counts items of four 64-channel chunks per block).
+// tcgen05 tensor cores (bf16): orders 8 and 16 at r <= 48, order 4 at every rank.
+// Coefficients are written densely (block blk: rows blk * r ..); t1 may be null.
 bool project_umma_supported(int k, int r);
-int launch_project_umma(const CUtensorMap* tmaps, __nv_bfloat16* out0, __nv_bfloat16* out1,
-                        const ProjParams& p, const BasisPlan& bp, int sms, cudaStream_t stream);
+int launch_project_umma(const void* t0, void* out0, int C0, const lbp_view* view0, const void* t1,
+                        void* out1, int C1, const lbp_view* view1, int B, int H, int W,
+                        const BasisPlan& bp, float scale0, float scale1, int sms, uint32_t* status,
+                        cudaStream_t stream);
 // Grid size and launch attributes of a projection launch under the per-thread
 // launch shape (see ProjLaunch): `want` CTAs at most.
 int projection_grid(uint32_t want, int sms, cudaLaunchAttribute* attr, unsigned* n_attr);
