@@ -13,15 +13,17 @@
 // same input took 8 times the tensor-core work at r <= 16, about as much as the
 // products of the layer themselves (and power is what bounds long runs).
 //
-// An item is two slots; a slot is a block x 128 channels of one of the two tensors.
+// The chunks (a block x 64 channels) of both tensors are numbered through; an item is
+// four consecutive ones, whatever block or tensor they belong to, so that narrow layers
+// (48 channels: one chunk per block) fill the ring like wide ones.
 //   order 8   a block is one box (8 x 8 tokens);
 //   order 16  four parts of 64 tokens (four token rows each), every part a stage of its
 //             own against its own 64 columns of the basis matrix, accumulating;
 //   order 4   a "block" here is a strip of four along W (a box of 4 x 16 tokens); the
 //             basis matrix holds the bases of the four blocks one after the other.
 // The accumulator holds one channel per TMEM lane and one coefficient per column: a
-// thread reads its r columns, rounds them and stores them to r rows of 128 channels in
-// shared memory, from where one TMA store per slot writes them as rows of 256 bytes.
+// thread reads its r columns, rounds them and stores them to r rows of 64 channels in
+// shared memory, from where one TMA store per chunk writes them.
 //
 // Roles: warps 0-3 TMA producers (one 64-channel chunk of an item each), warp 4 MMA
 // issuer, warps 8-23 four epilogue warpgroups that take turns on the items (an item's
@@ -42,7 +44,7 @@ namespace lbp {
 namespace umma {
 
 constexpr int kTileBytes = 64 * 128;             // 64 tokens x 64 channels of bf16
-constexpr int kStageBytes = 4 * kTileBytes;      // 32 KB: two slots
+constexpr int kStageBytes = 4 * kTileBytes;      // 32 KB: an item, or a quarter of one at order 16
 constexpr int kProducers = 4;
 constexpr int kMaxGroups = 4;                    // epilogue warpgroups
 constexpr int kThreads = (8 + 4 * kMaxGroups) * 32;
@@ -53,16 +55,16 @@ constexpr uint32_t kTmemCols = 512;
 constexpr int kSlots = 4;                        // accumulator slots (items in flight)
 constexpr uint32_t kSlotCols = kTmemCols / kSlots, kHalfCols = kSlotCols / 2;
 
-// Steps between a cursor's consecutive slots, so that it moves without divisions.
+// Steps between a cursor's consecutive chunks, so that it moves without divisions.
 struct Steps {
-  uint32_t pair, bw, bh, b;
+  uint32_t col, bw, bh, b;
 };
 struct Params {
   int32_t Hb, Wb;                // blocks (order 4: strips) of an image
   int32_t Wblocks, per_strip;    // blocks along W; blocks per cursor step along W (order 4: 4, else 1)
   int32_t r;
-  int32_t C[2], pairs[2];        // channels; 128-channel pairs of chunks
-  uint32_t n_slots0, n_slots;    // slots of tensor 0, of both
+  int32_t C[2], cols[2];         // channels; chunks per block
+  uint32_t n_chunks0, n_chunks;  // chunks of tensor 0, of both
   uint32_t* status;
   float scale[2];
   int32_t defer_wait, test_stall;
@@ -70,34 +72,34 @@ struct Params {
   Steps step[2];
 };
 
-// Slot number -> tensor, block and channel pair.  The position is decoded once, then
+// Chunk number -> tensor, block and column.  The position is decoded once, then
 // moved by precomputed steps with carries.
 struct Cursor {
-  uint32_t slot, which, pair, bw, bh, b;
+  uint32_t chunk, which, col, bw, bh, b;
   __device__ __forceinline__ void decode(const Params& p, uint32_t s) {
-    slot = s;
-    which = s >= p.n_slots0 ? 1u : 0u;
-    const uint32_t local = s - (which ? p.n_slots0 : 0u);
-    const uint32_t np = static_cast<uint32_t>(p.pairs[which]);
+    chunk = s;
+    which = s >= p.n_chunks0 ? 1u : 0u;
+    const uint32_t local = s - (which ? p.n_chunks0 : 0u);
+    const uint32_t np = static_cast<uint32_t>(p.cols[which]);
     const uint32_t blk = local / np;
-    pair = local - blk * np;
+    col = local - blk * np;
     const uint32_t t2 = blk / p.Wb;
     bw = blk - t2 * p.Wb;
     b = t2 / p.Hb;
     bh = t2 - b * p.Hb;
   }
   __device__ __forceinline__ void advance(const Params& p, uint32_t stride) {
-    const uint32_t next = slot + stride;
-    if (which == 0u && next >= p.n_slots0) {   // into the second tensor: once per cursor
+    const uint32_t next = chunk + stride;
+    if (which == 0u && next >= p.n_chunks0) {   // into the second tensor: once per cursor
       decode(p, next);
       return;
     }
-    slot = next;
+    chunk = next;
     const Steps& st = p.step[which];
-    const uint32_t np = static_cast<uint32_t>(p.pairs[which]);
-    pair += st.pair;
-    uint32_t carry = pair >= np ? 1u : 0u;
-    pair -= carry ? np : 0u;
+    const uint32_t np = static_cast<uint32_t>(p.cols[which]);
+    col += st.col;
+    uint32_t carry = col >= np ? 1u : 0u;
+    col -= carry ? np : 0u;
     bw += st.bw + carry;
     carry = bw >= static_cast<uint32_t>(p.Wb) ? 1u : 0u;
     bw -= carry ? p.Wb : 0u;
@@ -136,7 +138,7 @@ __device__ __forceinline__ bool group_or(int id, bool pred) {
   return any != 0;
 }
 
-// Output maps of one tensor: boxes of the rows of a whole "block" (order 4: of the
+// Output maps of the tensors: boxes of the rows of a whole "block" (order 4: of the
 // four blocks of a strip) and, order 4, of the last strip of a row of blocks.
 struct OutMaps {
   CUtensorMap full[2], tail[2];
@@ -157,9 +159,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint8_t* sB = smem + p.stages * kStageBytes;
   uint8_t* sOut = sB + kParts * kPanelBytes;
-  const int rows = p.r * p.per_strip;             // coefficient rows of a slot
-  const int half_bytes = rows * 256;
-  uint64_t* full_bar = reinterpret_cast<uint64_t*>(sOut + 2 * p.groups * half_bytes);   // [kMaxStages]
+  const int rows = p.r * p.per_strip;             // coefficient rows of a chunk
+  const int out_bytes = rows * 128;
+  uint64_t* full_bar = reinterpret_cast<uint64_t*>(sOut + 4 * p.groups * out_bytes);   // [kMaxStages]
   uint64_t* empty_bar = full_bar + kMaxStages;
   uint64_t* acc_full = empty_bar + kMaxStages;   // [kSlots]
   uint64_t* acc_empty = acc_full + kSlots;       // [kSlots]
@@ -224,9 +226,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (!p.defer_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
 
   // items dealt to the CTAs round robin
-  const uint32_t n_items = (p.n_slots + 1) / 2;
+  const uint32_t n_items = (p.n_chunks + 3) / 4;
   const uint32_t my_items = blockIdx.x < n_items ? (n_items - blockIdx.x + gridDim.x - 1) / gridDim.x : 0u;
-  const uint32_t slot_stride = 2u * gridDim.x;   // slots between a CTA's consecutive items
+  const uint32_t stride = 4u * gridDim.x;   // chunks between a CTA's consecutive items
 
   if (warp < kProducers) {
     // =========================== TMA producers ===========================
@@ -236,15 +238,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       // x and g_y are read exactly once: they should not push the coefficients
       // just written (read back from L2 by the next kernel) out of L2
       const uint64_t stream_once = ptx::l2_policy_evict_first();
-      const uint32_t half = static_cast<uint32_t>(warp) >> 1;
       Cursor c;
-      c.decode(p, 2 * blockIdx.x + half);
+      c.decode(p, 4 * blockIdx.x + warp);
       bool ok = true;
       int s = 0;
       uint32_t phase = 0;
       for (uint32_t n = 0; n < my_items && !p.test_stall && ok; ++n) {
-        const int ch = static_cast<int>(c.pair) * 128 + (warp & 1) * 64;
-        const bool have = c.slot < p.n_slots && ch < p.C[c.which];
+        const int ch = static_cast<int>(c.col) * 64;
+        const bool have = c.chunk < p.n_chunks;
         for (int part = 0; part < kParts; ++part) {
           if (!ptx::mbar_wait(&empty_bar[s], phase ^ 1u, p.status, (6u << 16) | 1u)) {
             ok = false;
@@ -265,7 +266,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             phase ^= 1u;
           }
         }
-        if (ok && n + 1 < my_items) c.advance(p, slot_stride);
+        if (ok && n + 1 < my_items) c.advance(p, stride);
       }
       if (!ok) *abort_flag = 1;
     }
@@ -279,7 +280,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t phase = 0;
       for (uint32_t n = 0; n < my_items && ok; ++n) {
         const int slot = static_cast<int>(n % kSlots);
-        const bool second = 2 * (blockIdx.x + n * gridDim.x) + 1 < p.n_slots;
+        const bool second = 4 * (blockIdx.x + n * gridDim.x) + 2 < p.n_chunks;   // of the two halves of an item
         if (!ptx::mbar_wait(&acc_empty[slot], ((n / kSlots) + 1) & 1u, p.status, (6u << 16) | 2u)) {
           ok = false;
           break;
@@ -319,7 +320,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int g = (warp - 8) >> 2, quarter = warp & 3;
     const bool first = quarter == 0 && lane == 0;
     const uint64_t keep = ptx::l2_policy_evict_last();   // read back from L2 by the next kernel
-    uint8_t* const out = sOut + g * 2 * half_bytes;
+    uint8_t* const out = sOut + g * 4 * out_bytes;
     for (uint32_t n = g < p.groups ? g : my_items; n < my_items; n += p.groups) {
       const int slot = static_cast<int>(n % kSlots);
       const bool ok = ptx::mbar_wait(&acc_full[slot], (n / kSlots) & 1u, p.status, (6u << 16) | 4u);
@@ -331,13 +332,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         break;
       }
       ptx::tc_fence_after_sync();
-      const uint32_t slot0 = 2 * (blockIdx.x + n * gridDim.x);
-      const int halves = slot0 + 1 < p.n_slots ? 2 : 1;
+      const uint32_t chunk0 = 4 * (blockIdx.x + n * gridDim.x);
+      const int chunks = p.n_chunks - chunk0 < 4u ? static_cast<int>(p.n_chunks - chunk0) : 4;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        if (h < halves) {
-          const float sc = p.scale[slot0 + h >= p.n_slots0 ? 1 : 0];
-          uint16_t* const o = reinterpret_cast<uint16_t*>(out + h * half_bytes) + quarter * 32 + lane;
+        if (2 * h < chunks) {
+          // lanes 0-63 of the accumulator are the first chunk of the half, 64-127 the second
+          const int i = 2 * h + (quarter >> 1);
+          const float sc = p.scale[chunk0 + i >= p.n_chunks0 ? 1 : 0];
+          uint16_t* const o = reinterpret_cast<uint16_t*>(out + i * out_bytes) + (quarter & 1) * 32 + lane;
 #pragma unroll
           for (int nb = 0; nb < NB; ++nb) {
             uint32_t v[16];
@@ -348,8 +351,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int q = 0; q < 16; q += 2) {
               const uint32_t pk = pack_bf16x2(__uint_as_float(v[q]) * sc, __uint_as_float(v[q + 1]) * sc);
-              if (nb * 16 + q < rows) o[(nb * 16 + q) * 128] = static_cast<uint16_t>(pk);
-              if (nb * 16 + q + 1 < rows) o[(nb * 16 + q + 1) * 128] = static_cast<uint16_t>(pk >> 16);
+              if (nb * 16 + q < rows) o[(nb * 16 + q) * 64] = static_cast<uint16_t>(pk);
+              if (nb * 16 + q + 1 < rows) o[(nb * 16 + q + 1) * 64] = static_cast<uint16_t>(pk >> 16);
             }
           }
         }
@@ -359,13 +362,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&acc_empty[slot]);   // the slot may be overwritten
       group_sync(1 + g);
-      if (quarter == 0 && lane < halves) {
+      if (quarter == 0 && lane < chunks) {
         Cursor c;
-        c.decode(p, slot0 + lane);
+        c.decode(p, chunk0 + lane);
         const long long blk = (static_cast<long long>(c.b) * p.Hb + c.bh) * p.Wblocks + c.bw * p.per_strip;
         const bool tail = K == 4 && static_cast<int>(c.bw * 4 + 4) > p.Wblocks;
-        tma_store_4d_hint(tail ? &om.tail[c.which] : &om.full[c.which], out + lane * half_bytes,
-                          static_cast<int32_t>(c.pair) * 128, static_cast<int32_t>(blk * p.r), keep);
+        tma_store_4d_hint(tail ? &om.tail[c.which] : &om.full[c.which], out + lane * out_bytes,
+                          static_cast<int32_t>(c.col) * 64, static_cast<int32_t>(blk * p.r), keep);
       }
       if (quarter == 0) bulk_commit();
     }
@@ -401,15 +404,15 @@ int launch_project_umma(const void* t0, void* out0, int C0, const lbp_view* view
   p.r = r;
   p.C[0] = C0;
   p.C[1] = t1 != nullptr ? C1 : C0;
-  p.pairs[0] = (C0 + 127) / 128;
-  p.pairs[1] = (p.C[1] + 127) / 128;
+  p.cols[0] = (C0 + 63) / 64;
+  p.cols[1] = (p.C[1] + 63) / 64;
   const long long cells = static_cast<long long>(B) * p.Hb * p.Wb;
-  const long long n0 = cells * p.pairs[0], n1 = t1 != nullptr ? cells * p.pairs[1] : 0;
-  // slot numbers, and one stride past the last, fit 32 bits
+  const long long n0 = cells * p.cols[0], n1 = t1 != nullptr ? cells * p.cols[1] : 0;
+  // chunk numbers, and one stride past the last, fit 32 bits
   if (n0 + n1 >= (1ll << 31) || static_cast<long long>(B) * p.Hb * p.Wblocks * r >= (1ll << 31))
     return LBP_ERR_SHAPE;
-  p.n_slots0 = static_cast<uint32_t>(n0);
-  p.n_slots = static_cast<uint32_t>(n0 + n1);
+  p.n_chunks0 = static_cast<uint32_t>(n0);
+  p.n_chunks = static_cast<uint32_t>(n0 + n1);
   p.status = status;
   p.scale[0] = scale0;
   p.scale[1] = scale1;
@@ -426,13 +429,13 @@ int launch_project_umma(const void* t0, void* out0, int C0, const lbp_view* view
   const int tail_blocks = p.Wblocks % p.per_strip;
   auto maps = [&](int i, const void* t, void* out, int C, const lbp_view* view) -> int {
     if (int e = encode_box_tensor_map(&in[i], t, LBP_BF16, B, H, W, C, 64, box_w, box_h, true, view)) return e;
-    // the coefficient matrix: boxes of a slot's rows x 128 channels
+    // the coefficient matrix: boxes of a chunk's rows x 64 channels
     const int rows = static_cast<int>(static_cast<long long>(B) * p.Hb * p.Wblocks * r);
-    if (int e = encode_box_tensor_map(&om.full[i], out, LBP_BF16, 1, 1, rows, C, 128, r * p.per_strip, 1, false))
+    if (int e = encode_box_tensor_map(&om.full[i], out, LBP_BF16, 1, 1, rows, C, 64, r * p.per_strip, 1, false))
       return e;
     om.tail[i] = om.full[i];
     if (tail_blocks > 0)
-      if (int e = encode_box_tensor_map(&om.tail[i], out, LBP_BF16, 1, 1, rows, C, 128, r * tail_blocks, 1, false))
+      if (int e = encode_box_tensor_map(&om.tail[i], out, LBP_BF16, 1, 1, rows, C, 64, r * tail_blocks, 1, false))
         return e;
     return LBP_OK;
   };
@@ -447,22 +450,22 @@ int launch_project_umma(const void* t0, void* out0, int C0, const lbp_view* view
 
   const int rows = r * p.per_strip, nb = (rows + 15) / 16, parts = K == 16 ? 4 : 1;
   const int fixed = 1024 + kBarBytes + parts * nb * 2048;
-  auto ring = [&](int groups) { return (kSmemMax - fixed - 2 * groups * rows * 256) / kStageBytes; };
+  auto ring = [&](int groups) { return (kSmemMax - fixed - 4 * groups * rows * 128) / kStageBytes; };
   p.groups = kMaxGroups;
   while (p.groups > 2 && ring(p.groups) < 4) --p.groups;
   p.stages = ring(p.groups) < kMaxStages ? ring(p.groups) : kMaxStages;
-  const int smem_bytes = fixed + p.stages * kStageBytes + 2 * p.groups * rows * 256;
+  const int smem_bytes = fixed + p.stages * kStageBytes + 4 * p.groups * rows * 128;
 
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
-  // Alone on the chip the kernel is bound by HBM long before it runs out of SMs,
-  // and on three quarters of them it is about 5 % faster than on all (fewer
-  // requests in flight against one another); beside a products kernel the
-  // caller's launch shape says how many it gets.
-  const int sms_alone = projection_launch().max_ctas > 0 ? sms : (3 * sms + 3) / 4;
-  const int grid = projection_grid((p.n_slots + 1) / 2, sms_alone, attr, &cfg.numAttrs);
+  // Alone on the chip the kernel is bound by HBM before it runs out of SMs: 201 MB in 43
+  // us on 96 to 128 of 148 SMs and 45 on all, 77 MB of 14 x 14 or 56 x 56 grids in 24.6
+  // us on 112, 22.6 on 128, 22.8 on all.  Beside a products kernel the caller's launch
+  // shape says how many it gets.
+  const int sms_alone = projection_launch().max_ctas > 0 ? sms : (7 * sms + 7) / 8;
+  const int grid = projection_grid((p.n_chunks + 3) / 4, sms_alone, attr, &cfg.numAttrs);
   for (int w = 0; w < 2; ++w) {
-    const uint32_t stride = 2u * static_cast<uint32_t>(grid), np = static_cast<uint32_t>(p.pairs[w]);
+    const uint32_t stride = 4u * static_cast<uint32_t>(grid), np = static_cast<uint32_t>(p.cols[w]);
     const uint32_t blk = stride / np, t2 = blk / p.Wb;
     p.step[w] = Steps{stride - blk * np, blk % p.Wb, t2 % p.Hb, t2 / p.Hb};
   }
