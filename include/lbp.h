@@ -216,7 +216,7 @@ typedef struct {
   /* g_W <- beta * g_W + (g_W of this call); 0 overwrites.  beta = 1 adds a
    * micro-batch to an accumulated gradient.  g_bias follows the same rule. */
   float beta;
-  /* NULL, or fp32[Cout]: gradient of a bias added to y, the sum of g_y over all
+  /* NULL, or an array of Cout (g_bias_dtype): gradient of a bias added to y, the sum of g_y over all
    * tokens (grid and extra).  With the basis (0,0) in the list this is k times
    * the sum of the DC coefficients of g_y_hat (exact in exact arithmetic: that
    * basis is the block sum scaled by 1/k); otherwise g_y is read once more. */
@@ -245,6 +245,8 @@ typedef struct {
    * same rules as a view's strides.  With one class token per image in a
    * (B, 1 + H*W, C) sequence this is (1 + H*W) * C. */
   int64_t x_extra_pitch, gy_extra_pitch, gx_extra_pitch;
+  /* lbp_dtype of g_bias: LBP_F32 (0), or LBP_BF16 with bf16 data. */
+  int32_t g_bias_dtype;
 } lbp_extras;
 
 /* Scratch for lbp_backward_ex (>= lbp_workspace_bytes; 0 = invalid arguments). */

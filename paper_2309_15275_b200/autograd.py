@@ -1,8 +1,9 @@
 """`torch.autograd` front end of the C ABI: a linear layer whose backward pass is
 Algorithm 1 (low-rank backpropagation on the selected Walsh-Hadamard bases).
 
-Only the backward pass is the library's: the forward product `y = x W^T` is a
-plain matrix product and is left to torch.  The layer takes the token grid
+Only the backward pass is the library's: the forward product `y = x W^T + b` is a
+plain matrix product and is left to torch (one call: the bias is added in the product's
+epilogue instead of in a pass over y of its own).  The layer takes the token grid
 explicit, x of shape (B, H, W, Cin), or, with `grid=(H, W)`, a token sequence
 (B, n + H*W, Cin) whose first n tokens (class tokens) are not part of the grid:
 those take exact backpropagation (Eq. 2), and the grid tokens are handed to the
@@ -37,8 +38,7 @@ class LbpLinearFunction(torch.autograd.Function):
                 raise ValueError("with a grid, x must be (B, n + H*W, Cin)")
             ctx.grid, ctx.projected = (H, W), False
             ctx.save_for_backward(x, weight)
-            y = torch.matmul(x, weight.t())
-            return y if bias is None else y + bias
+            return torch.nn.functional.linear(x, weight, bias)
         if x.dim() != 4:
             raise ValueError("x must be (B, H, W, Cin)")
         ctx.projected = bool(save_projected) and x.is_cuda
@@ -46,13 +46,12 @@ class LbpLinearFunction(torch.autograd.Function):
             ctx.save_for_backward(_b.lbp_project(x.contiguous(), ctx.k, ctx.bases), weight)
         else:
             ctx.save_for_backward(x, weight)
-        y = torch.matmul(x, weight.t())
-        return y if bias is None else y + bias
+        return torch.nn.functional.linear(x, weight, bias)
 
     @staticmethod
     def backward(ctx, g_y: torch.Tensor):
         saved, weight = ctx.saved_tensors
-        g_b = (torch.empty(weight.shape[0], dtype=torch.float32, device=g_y.device)
+        g_b = (torch.empty(weight.shape[0], dtype=weight.dtype, device=g_y.device)
                if ctx.has_bias else None)
         if ctx.grid is not None:
             return LbpLinearFunction._backward_sequence(ctx, saved, weight, g_y, g_b)
@@ -61,7 +60,7 @@ class LbpLinearFunction(torch.autograd.Function):
         g_x, g_W = _b.lbp_backward_ex(None if ctx.projected else saved.contiguous(), g_y,
                                       weight.contiguous(), ctx.k, ctx.bases, g_bias=g_b,
                                       gw_dtype=weight.dtype, **kw)
-        return g_x, g_W, (None if g_b is None else g_b.to(weight.dtype)), None, None, None, None
+        return g_x, g_W, g_b, None, None, None, None
 
     @staticmethod
     def _backward_sequence(ctx, x, weight, g_y, g_b):
@@ -82,7 +81,7 @@ class LbpLinearFunction(torch.autograd.Function):
                                     gw_dtype=weight.dtype, g_x=g_x[:, n:].unflatten(1, (H, W)), **kw)
         if n > 1:
             g_x[:, :n] = gx_cls.view(B, n, Cin)
-        return g_x, g_W, (None if g_b is None else g_b.to(weight.dtype)), None, None, None, None
+        return g_x, g_W, g_b, None, None, None, None
 
 
 class LbpLinear(torch.nn.Module):

@@ -50,7 +50,7 @@ class Extras(C.Structure):
                 ("x_extra", C.c_void_p), ("gy_extra", C.c_void_p), ("gx_extra", C.c_void_p),
                 ("x_view", View), ("gy_view", View), ("gx_view", View),
                 ("x_extra_pitch", C.c_int64), ("gy_extra_pitch", C.c_int64),
-                ("gx_extra_pitch", C.c_int64)]
+                ("gx_extra_pitch", C.c_int64), ("g_bias_dtype", C.c_int32)]
 
 
 _LIB = None
@@ -378,9 +378,10 @@ def _extras(g_y, Cin, beta, g_bias, x_extra, gy_extra, gx_extra):
     ex = Extras()
     ex.beta = float(beta)
     if g_bias is not None:
-        if g_bias.dtype != torch.float32 or tuple(g_bias.shape) != (Cout,):
-            raise ValueError("g_bias must be fp32 of shape (Cout,)")
+        if g_bias.dtype not in (torch.float32, g_y.dtype) or tuple(g_bias.shape) != (Cout,):
+            raise ValueError("g_bias must be fp32, or of the layer's dtype, of shape (Cout,)")
         ex.g_bias = _dev(g_bias, "g_bias")
+        ex.g_bias_dtype = _dtype_code(g_bias.dtype)
     n = 0
     if x_extra is not None or gy_extra is not None:
         if x_extra is None or gy_extra is None or gx_extra is None:

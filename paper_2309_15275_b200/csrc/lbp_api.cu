@@ -142,14 +142,13 @@ struct Layout {
 
 // Scratch of lbp_backward_ex beyond `Layout::total`: two fp32 (Cout, Cin)
 // matrices (this call's g_W before it is added to the caller's, the term of the
-// tokens outside the grid) and the fp64 column-sum partials of the bias gradient.
+// tokens outside the grid).
 struct ExtrasLayout {
-  size_t gw0, gw1, bias_a, bias_b, total;
+  size_t gw0, gw1, total;
   // dense copies of tensors given as views, where a kernel wants dense operands
   // (0: not needed): the token tensors in the full-rank mode, the extra tokens
   size_t pack_x, pack_gy, pack_gx, ex_x, ex_gy, ex_gx;
 };
-constexpr int kBiasSlabsMax = 64;
 
 static bool pitched(int64_t pitch, int C) { return pitch != 0 && pitch != C; }
 
@@ -161,11 +160,6 @@ static ExtrasLayout plan_extras(const lbp_layer& L, size_t base_total, int r, co
   off = align_up(off + gw, 1024);
   e.gw1 = off;
   off = align_up(off + gw, 1024);
-  const size_t part = static_cast<size_t>(kBiasSlabsMax) * L.Cout * 8;
-  e.bias_a = off;
-  off = align_up(off + part, 1024);
-  e.bias_b = off;
-  off = align_up(off + part, 1024);
   if (ex != nullptr) {
     const size_t es = static_cast<size_t>(elem_size(L.dtype));
     auto take = [&](size_t* where, size_t bytes) {
@@ -694,7 +688,6 @@ namespace lbp {
 // the full-rank mode and materialised nothing.
 struct CoefLoc {
   const void* ptr;
-  RowMap rows;
   double dc_to_sum;   // token sum of a block = dc_to_sum * its (0,0) coefficient as stored
   int dc_slot;        // slot of that coefficient; -1: basis (0,0) is not selected
 };
@@ -721,7 +714,6 @@ static int run_core(const void* x, const void* x_hat_in, const void* g_y, const 
     FusedLayout fl;
     fused_scratch_bytes(L, r, &fl);
     gy_loc->ptr = wsb + lay.fused + fl.gy_hat;
-    gy_loc->rows = RowMap{1, r};
     gy_loc->dc_to_sum = 1.0 / static_cast<double>(fused_scale_gy(L.k, x_hat_in != nullptr));
     // projection kernel, then one persistent kernel for both products with the
     // expansion fused into the g_x_hat epilogue
@@ -743,7 +735,6 @@ static int run_core(const void* x, const void* x_hat_in, const void* g_y, const 
   float* sk = reinterpret_cast<float*>(wsb + lay.splitk);
   const RowMap dense{1, r};
   gy_loc->ptr = gy_hat;
-  gy_loc->rows = dense;
   gy_loc->dc_to_sum = static_cast<double>(L.k);   // orthonormal: coefficient = block sum / k
   gy_loc->dc_slot = -1;
   for (int q = 0; q < r; ++q)
@@ -814,6 +805,8 @@ static int check_extras(const lbp_extras* ex, const lbp_layer* L) {
     if (int e = check_pitch(ex->gx_extra_pitch, L->Cin, es)) return e;
   }
   if (ex->g_bias != nullptr && !aligned16(ex->g_bias)) return LBP_ERR_ALIGN;
+  if (ex->g_bias_dtype != LBP_F32 && (ex->g_bias_dtype != LBP_BF16 || L->dtype != LBP_BF16))
+    return LBP_ERR_DTYPE;
   if (int e = check_view(ex->x_view, L->Cin, es)) return e;
   if (int e = check_view(ex->gy_view, L->Cout, es)) return e;
   if (int e = check_view(ex->gx_view, L->Cin, es)) return e;
@@ -916,27 +909,12 @@ static int run_backward_ex(const void* x, const void* x_hat, const void* g_y, co
     // Sum of g_y over all tokens.  With the DC basis (0,0) selected that is k times
     // the sum of the DC coefficients of g_y_hat, which the call has just produced;
     // otherwise g_y is read once more.
-    double* pa = reinterpret_cast<double*>(wsb + el.bias_a);
-    double* pb = reinterpret_cast<double*>(wsb + el.bias_b);
-    long long n_a;
-    double scale_a;
-    if (gy_loc.ptr != nullptr && gy_loc.dc_slot >= 0) {
-      n_a = static_cast<long long>(L.B) * blocks_along(L.H, L.k) * blocks_along(L.W, L.k);
-      scale_a = gy_loc.dc_to_sum;
-      if (int e = launch_column_sum(gy_loc.ptr, L.dtype, n_a, L.Cout, gy_loc.rows, plan.r, gy_loc.dc_slot, pa, st))
-        return e;
-    } else {
-      n_a = T;
-      scale_a = 1.0;
-      if (int e = launch_column_sum(gy_tokens, L.dtype, n_a, L.Cout, RowMap{1, 1}, 0, 0, pa, st, &gy_map))
-        return e;
-    }
-    if (ex->n_extra > 0)
-      if (int e = launch_column_sum(ex->gy_extra, L.dtype, ex->n_extra, L.Cout, RowMap{1, 1}, 0, 0, pb,
-                                    st, &gye_map))
-        return e;
-    if (int e = launch_bias_finish(static_cast<float*>(ex->g_bias), L.Cout, ex->beta, pa,
-                                   bias_slabs(n_a), scale_a, pb, bias_slabs(ex->n_extra), st))
+    const bool dc = gy_loc.ptr != nullptr && gy_loc.dc_slot >= 0;
+    const long long blocks = static_cast<long long>(L.B) * blocks_along(L.H, L.k) * blocks_along(L.W, L.k);
+    if (int e = launch_bias_grad(dc ? gy_loc.ptr : gy_tokens, dc ? blocks : T, dc ? plan.r : 0,
+                                 dc ? gy_loc.dc_slot : 0, gy_map, dc ? gy_loc.dc_to_sum : 1.0, ex->gy_extra,
+                                 ex->n_extra, gye_map, L.Cout, L.dtype, ex->g_bias,
+                                 ex->g_bias_dtype == LBP_BF16, ex->beta, st))
       return e;
   }
   return LBP_OK;

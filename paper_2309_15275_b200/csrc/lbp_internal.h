@@ -182,21 +182,18 @@ struct TokenMap {
 inline TokenMap token_map(const lbp_view& v, int H, int W) {
   return TokenMap{H * W, W, v.image, v.row, v.token};
 }
-// Column sums in fp64 of n_sel selected rows of a matrix of `dtype`, as
-// bias_slabs(n_sel) partial rows of C doubles.  r == 0: tokens 0..n_sel-1 under
-// `tokens` (null: a dense (n_sel, C) matrix); r > 0: the row of slot q of block i
-// of a dense coefficient matrix under the row map `rows`.
-int bias_slabs(long long n_sel);
-int launch_column_sum(const void* m, int dtype, long long n_sel, int C, RowMap rows, int r, int q,
-                      double* partial, cudaStream_t stream, const TokenMap* tokens = nullptr);
 // Gathers (to_dense) or scatters n_tok tokens of C channels between a tensor
 // laid out as `tm` says (element strides, multiples of 16 bytes) and a dense
 // (n_tok, C) matrix.
 int launch_copy_tokens(const void* src, void* dst, bool to_dense, long long n_tok, int C, int dtype,
                        TokenMap tm, cudaStream_t stream);
-// g_bias[c] <- beta * g_bias[c] + scale_a * (sum of the slabs of a) + (sum of the slabs of b)
-int launch_bias_finish(float* g_bias, int C, float beta, const double* a, int slabs_a, double scale_a,
-                       const double* b, int slabs_b, cudaStream_t stream);
+// g_bias <- beta * g_bias + scale * (sum of n_a rows of a) + (sum of n_b rows of b), fp64
+// sums.  r > 0: the rows of a are the coefficients of slot q of its blocks (dense, r
+// per block); r == 0: tokens under `ta`.  b: tokens under `tb`.  g_bias is fp32 or bf16.
+int launch_bias_grad(const void* a, long long n_a, int r, int q, TokenMap ta, double scale,
+                     const void* b, long long n_b, TokenMap tb, int C, int dtype, void* g_bias,
+                     bool out_bf16, float beta, cudaStream_t stream);
+
 // Tuning switches, read from the environment once (first use):
 //   LBP_FUSED=0          separate product and expansion kernels instead of the
 //                        persistent products kernel
