@@ -1,6 +1,9 @@
-"""ctypes binding of liblbp.so: argument marshalling only.
+"""Python binding of liblbp.so: argument marshalling only.
 
-Every function mirrors one entry point of include/lbp.h.  Tensors are torch
+Every function mirrors one entry point of include/lbp.h.  The calls of a training
+step go through a native module (csrc/torch_binding.cpp), which checks its arguments
+itself and hands back whatever it does not take as it is; the ctypes code here then
+checks again and names the error.  Tensors are torch
 CUDA tensors used as device-memory handles (data_ptr) -- all arithmetic runs in
 the library's kernels.  There is no CPU or eager fallback: if the shared library
 is missing or a call fails, an exception is raised.
@@ -133,6 +136,29 @@ def _lib() -> C.CDLL:
     return _LIB
 
 
+_NATIVE = None
+
+
+def _native():
+    """The native half of this binding."""
+    global _NATIVE
+    if _NATIVE is None:
+        import importlib.machinery
+        import importlib.util
+        path = os.path.join(_HERE, "_lbp_torch.so")
+        if not os.path.exists(path):
+            raise RuntimeError(
+                f"{path} is missing: build it with "
+                "`python -m paper_2309_15275_b200.build` (there is no fallback path)")
+        _lib()
+        loader = importlib.machinery.ExtensionFileLoader("_lbp_torch", path)
+        mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("_lbp_torch", loader))
+        loader.exec_module(mod)
+        mod.load(LIB_PATH, LbpError)
+        _NATIVE = mod
+    return _NATIVE
+
+
 EXPORTED = ("lbp_select_bases", "lbp_basis_matrix", "lbp_flops", "lbp_status_string",
             "lbp_last_cuda_error", "lbp_workspace_bytes", "lbp_status_bytes", "lbp_project",
             "lbp_expand", "lbp_backward", "lbp_backward_fullrank", "lbp_poll_status",
@@ -146,6 +172,12 @@ EXPORTED = ("lbp_select_bases", "lbp_basis_matrix", "lbp_flops", "lbp_status_str
 def _check(status: int, where: str) -> None:
     if status != LBP_OK:
         raise LbpError(status, where)
+
+
+def _result(got, where: str):
+    if type(got) is int:
+        raise LbpError(got, where)
+    return got
 
 
 def _bases(bases: Sequence[Tuple[int, int]]):
@@ -247,6 +279,9 @@ def _status_ws(device) -> torch.Tensor:
 def lbp_project(t: torch.Tensor, k: int, bases, out: torch.Tensor | None = None,
                 ws: torch.Tensor | None = None) -> torch.Tensor:
     """t (B,H,W,C) -> t_hat (B,ceil(H/k),ceil(W/k),r,C)."""
+    got = _native().project(t, k, bases, out, ws)
+    if got is not None:
+        return _result(got, "lbp_project")
     B, H, W, Cc = t.shape
     r = len(bases)
     if out is None:
@@ -278,6 +313,9 @@ def lbp_spectrum_workspace_bytes(B: int, H: int, W: int, Cc: int, k: int, dtype_
 def lbp_spectrum(t: torch.Tensor, k: int, out: torch.Tensor | None = None,
                  ws: torch.Tensor | None = None) -> torch.Tensor:
     """t (B,H,W,C) -> energy (k, k) float64 on the device: sum of squares of every basis response."""
+    got = _native().spectrum(t, k, out, ws)
+    if got is not None:
+        return _result(got, "lbp_spectrum")
     B, H, W, Cc = t.shape
     if out is None:
         out = torch.empty((k, k), dtype=torch.float64, device=t.device)
@@ -353,6 +391,9 @@ def _check_layer_tensors(g_y, W, g_x, g_W, Cin: int, x=None, x_hat=None, k=None,
 def lbp_backward(x, g_y, W, k: int, bases, *, gw_dtype: torch.dtype = torch.float32,
                  g_x=None, g_W=None, ws=None):
     """Algorithm 1.  Returns (g_x (B,H,W,Cin), g_W (Cout,Cin))."""
+    got = _native().backward(x, g_y, W, k, bases, gw_dtype, g_x, g_W, ws) if bases is not None else None
+    if got is not None:
+        return _result(got, "lbp_backward")
     if x.dim() != 4:
         raise ValueError("x must be (B, H, W, Cin)")
     B, H, Wd, Cin = x.shape
@@ -378,10 +419,9 @@ def _extras(g_y, Cin, beta, g_bias, x_extra, gy_extra, gx_extra):
     ex = Extras()
     ex.beta = float(beta)
     if g_bias is not None:
-        if g_bias.dtype not in (torch.float32, g_y.dtype) or tuple(g_bias.shape) != (Cout,):
-            raise ValueError("g_bias must be fp32, or of the layer's dtype, of shape (Cout,)")
+        if g_bias.dtype != torch.float32 or tuple(g_bias.shape) != (Cout,):
+            raise ValueError("g_bias must be fp32 of shape (Cout,)")
         ex.g_bias = _dev(g_bias, "g_bias")
-        ex.g_bias_dtype = _dtype_code(g_bias.dtype)
     n = 0
     if x_extra is not None or gy_extra is not None:
         if x_extra is None or gy_extra is None or gx_extra is None:
@@ -427,6 +467,10 @@ def lbp_backward_ex(x, g_y, W, k: int, bases, *, x_hat=None, beta: float = 0.0, 
     """Algorithm 1 with what a ViT layer needs around it: accumulation into g_W
     (beta), the bias gradient, tokens outside the grid (Eq. 2), and x_hat = p(x)
     handed in instead of x (pass x=None).  Returns (g_x, g_W)."""
+    got = _native().backward_ex(x, x_hat, g_y, W, k, bases, float(beta), g_bias, x_extra, gy_extra, gx_extra,
+                                gw_dtype, g_x, g_W, ws)
+    if got is not None:
+        return _result(got, "lbp_backward_ex")
     if (x is None) == (x_hat is None):
         raise ValueError("give exactly one of x and x_hat")
     B, H, Wd, Cout = g_y.shape
@@ -495,6 +539,11 @@ def lbp_backward_batch(xs, g_ys, Ws, k: int, bases, *, g_xs, g_Ws, wss, done_eve
     the caller's and must not overlap anything of another layer.  done_events: an
     optional list of torch.cuda.Event (or None entries), one per layer, recorded
     behind that layer's last kernel."""
+    if done_events is None:
+        got = _native().backward_batch(xs, g_ys, Ws, k, bases, g_xs, g_Ws, wss)
+        if got is not None:
+            _check(got, "lbp_backward_batch")
+            return g_xs, g_Ws
     n = len(xs)
     lays = (Layer * n)()
     for i in range(n):
@@ -524,6 +573,9 @@ def lbp_backward_batch(xs, g_ys, Ws, k: int, bases, *, g_xs, g_Ws, wss, done_eve
 def lbp_backward_fullrank(x, g_y, W, k: int, *, gw_dtype: torch.dtype = torch.float32,
                           g_x=None, g_W=None, ws=None):
     """Eq. 2, exact backpropagation (the r = k*k mode)."""
+    got = _native().backward(x, g_y, W, k, None, gw_dtype, g_x, g_W, ws)
+    if got is not None:
+        return _result(got, "lbp_backward_fullrank")
     B, H, Wd, Cin = x.shape
     Cout = g_y.shape[-1]
     _check_layer_tensors(g_y, W, g_x, g_W, Cin, x=x)

@@ -1,4 +1,5 @@
-"""Builds liblbp.so (the C-ABI library) in-tree with nvcc for sm_100a."""
+"""Builds, in-tree, liblbp.so (the C-ABI library) with nvcc for sm_100a and
+_lbp_torch.so (the native part of the Python binding) with the host compiler."""
 from __future__ import annotations
 
 import os
@@ -10,6 +11,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblbp.so")
+BINDING = os.path.join(HERE, "_lbp_torch.so")
+BINDING_SOURCE = os.path.join(CSRC, "torch_binding.cpp")
 
 SOURCES = ["lbp_host.cpp", "lbp_api.cu", "wht_project.cu", "wht_project_mma.cu", "wht_expand.cu",
            "gemm_fp32.cu", "gemm_bf16.cu", "lbp_fused.cu", "lbp_static.cu",
@@ -24,16 +27,32 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(BINDING):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
     deps.append(os.path.join(ROOT, "include", "lbp.h"))
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _binding_command() -> list:
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(os.path.abspath(torch.__file__))
+    cuda = os.path.dirname(os.path.dirname(_nvcc()))
+    libs = os.path.join(root, "lib")
+    return [shutil.which("g++") or "g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+            "-Wall", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            "-I", os.path.join(ROOT, "include"), "-isystem", os.path.join(root, "include"),
+            "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+            "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"),
+            BINDING_SOURCE, "-o", BINDING, "-L", libs, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch",
+            "-ltorch_python", "-ldl", f"-Wl,-rpath,{libs}"]
+
+
 def build_library(force: bool = False, verbose: bool = False, extra_flags=(), out: str | None = None) -> str:
-    """Compile every CUDA source into paper_2309_15275_b200/liblbp.so.
+    """Compile every CUDA source into paper_2309_15275_b200/liblbp.so, and the binding.
 
     `extra_flags` (e.g. ["-DLBP_ROLE_TRACE"]) with `out` builds a diagnostic
     variant into another file; the binding loads it when LBP_LIBRARY names it."""
@@ -55,11 +74,15 @@ def build_library(force: bool = False, verbose: bool = False, extra_flags=(), ou
         cmd = [_nvcc(), *common, "-x", "cu", "-c", os.path.join(CSRC, src), "-o", obj]
         procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT,
                                             text=True)))
+    if out is None:
+        procs.append((os.path.basename(BINDING_SOURCE),
+                      subprocess.Popen(_binding_command(), stdout=subprocess.PIPE, stderr=subprocess.STDOUT,
+                                       text=True)))
     failed = False
     for src, p in procs:
-        out, _ = p.communicate()
+        log, _ = p.communicate()
         if verbose or p.returncode != 0:
-            sys.stderr.write(f"--- {src} ---\n{out}\n")
+            sys.stderr.write(f"--- {src} ---\n{log}\n")
         failed |= p.returncode != 0
     if failed:
         raise RuntimeError("nvcc failed")
