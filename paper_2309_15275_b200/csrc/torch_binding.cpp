@@ -18,6 +18,7 @@
 #include <torch/csrc/Dtype.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/custom_function.h>
+#include <torch/csrc/autograd/python_cpp_function.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <torch/csrc/utils/pybind.h>
 
@@ -535,6 +536,33 @@ PyObject* py_linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
   END_HANDLE_TH_ERRORS
 }
 
+// What a Python autograd function shows of the node: y.grad_fn.saved_tensors.
+PyObject* node_saved_tensors(PyObject* self, void*) {
+  HANDLE_TH_ERRORS
+  using Node = torch::autograd::CppNode<LinearFunction>;
+  auto* node = dynamic_cast<Node*>(reinterpret_cast<torch::autograd::THPCppFunction*>(self)->cdata.get());
+  if (node == nullptr) {
+    PyErr_SetString(PyExc_RuntimeError, "saved_tensors: not a node of LbpLinear");
+    return nullptr;
+  }
+  const auto vars = node->ctx_.get_saved_variables();
+  PyObject* t = PyTuple_New(static_cast<Py_ssize_t>(vars.size()));
+  if (t == nullptr) return nullptr;
+  for (size_t i = 0; i < vars.size(); ++i) PyTuple_SET_ITEM(t, i, THPVariable_Wrap(vars[i]));
+  return t;
+  END_HANDLE_TH_ERRORS
+}
+void register_node_type() {
+  using namespace torch::autograd;
+  static PyTypeObject type;
+  static PyGetSetDef properties[] = {
+      {const_cast<char*>("saved_tensors"), node_saved_tensors, nullptr, nullptr, nullptr},
+      THP_FUNCTION_DEFAULT_PROPERTIES,
+      {nullptr, nullptr, nullptr, nullptr, nullptr}};
+  torch::autograd::_initFunctionPyTypeObject(type, "LbpLinearBackward", properties, nullptr);
+  torch::autograd::registerCppFunction(typeid(torch::autograd::CppNode<LinearFunction>), &type);
+}
+
 // load(path of liblbp.so, LbpError)
 PyObject* py_load(PyObject*, PyObject* args) {
   const char* path = nullptr;
@@ -558,6 +586,7 @@ PyObject* py_load(PyObject*, PyObject* args) {
     PyErr_Format(PyExc_RuntimeError, "%s does not export what this binding calls", path);
     return nullptr;
   }
+  if (error_type == nullptr) register_node_type();
   Py_INCREF(err);
   Py_XSETREF(error_type, err);
   Py_RETURN_NONE;
