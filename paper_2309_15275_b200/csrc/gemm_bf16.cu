@@ -295,9 +295,6 @@ Tiling choose_tiling(long long M, long long N, long long K, int sms) {
 
 }  // namespace
 
-int launch_gemm_fp32(const float* A, bool a_mn_major, const float* Bm, float* D, long long M,
-                     long long N, long long K, cudaStream_t stream);
-
 int launch_splitk_reduce(const float* planes, void* D, long long mn, int splits, bool d_bf16,
                          float beta, cudaStream_t stream) {
   const long long threads = (mn + 3) / 4;
@@ -329,8 +326,9 @@ int launch_gemm(const void* A, bool a_mn_major, const void* Bm, void* D, int in_
                 uint32_t* status, cudaStream_t stream) {
   if (in_dtype == LBP_F32) {
     if (d_dtype != LBP_F32) return LBP_ERR_DTYPE;
-    return launch_gemm_fp32(static_cast<const float*>(A), a_mn_major, static_cast<const float*>(Bm),
-                            static_cast<float*>(D), M, N, K, stream);
+    const GemmFp32 job{static_cast<const float*>(A), static_cast<const float*>(Bm), static_cast<float*>(D), M, N, K,
+                       a_mn_major};
+    return launch_gemm_fp32(&job, 1, stream);
   }
   int dev = 0, sms = 0;
   LBP_CUDA_TRY(cudaGetDevice(&dev));

@@ -233,6 +233,16 @@ static int mark_phase(int i, cudaStream_t stream) {
   return LBP_OK;
 }
 
+// Both fp32 products of a layer, g_W = gy^T xs over `rows` rows and gx = gy W, in one launch.
+static int run_products_fp32(const void* xs, const void* gy, const void* W, void* gx, void* g_W,
+                             const lbp_layer& L, long long rows, cudaStream_t stream) {
+  const float* g = static_cast<const float*>(gy);
+  const GemmFp32 jobs[2] = {
+      {g, static_cast<const float*>(W), static_cast<float*>(gx), rows, L.Cin, L.Cout, false},
+      {g, static_cast<const float*>(xs), static_cast<float*>(g_W), L.Cout, L.Cin, rows, true}};
+  return launch_gemm_fp32(jobs, 2, stream);
+}
+
 static int run_fullrank(const void* x, const void* g_y, const void* W, void* g_x, void* g_W,
                         const lbp_layer& L, uint8_t* ws, cudaStream_t stream) {
   const Layout lay = plan_layout(L, L.k * L.k);
@@ -240,6 +250,11 @@ static int run_fullrank(const void* x, const void* g_y, const void* W, void* g_x
   uint32_t* status = reinterpret_cast<uint32_t*>(ws);
   float* sk = reinterpret_cast<float*>(ws + lay.splitk);
   if (int e = mark_phase(0, stream)) return e;
+  if (L.dtype == LBP_F32) {   // Eq. 2, both products
+    if (int e = run_products_fp32(x, g_y, W, g_x, g_W, L, T, stream)) return e;
+    if (int e = mark_phase(3, stream)) return e;
+    return mark_phase(4, stream);
+  }
   // Eq. 2: g_W = g_y^T x
   if (int e = launch_gemm(g_y, /*a_mn_major=*/true, x, g_W, L.dtype, L.gw_dtype, L.Cout, L.Cin, T,
                           sk, lay.splitk_bytes, status, stream))
@@ -755,6 +770,16 @@ static int run_core(const void* x, const void* x_hat_in, const void* g_y, const 
   }
   if (int e = mark_phase(1, st)) return e;
   if (int e = mark_phase(2, st)) return e;
+  if (L.dtype == LBP_F32) {
+    // steps 3 and 4
+    if (int e = run_products_fp32(x_hat, gy_hat, W, gx_hat, g_W, L, lay.rows, st)) return e;
+    if (int e = mark_phase(3, st)) return e;
+    if (int e = mark_phase(4, st)) return e;
+    if (int e = launch_expand(gx_hat, /*in_f32=*/true, g_x, L.dtype, L.B, L.H, L.W, L.Cin, plan, dense, st,
+                              views ? &views->gx : nullptr))
+      return e;
+    return mark_phase(5, st);
+  }
   // step 3: g_W = g_y_hat^T x_hat
   if (int e = launch_gemm(gy_hat, /*a_mn_major=*/true, x_hat, g_W, L.dtype, L.gw_dtype, L.Cout,
                           L.Cin, lay.rows, sk, lay.splitk_bytes, status, st))

@@ -155,6 +155,15 @@ int launch_expand(const void* t_hat, bool in_f32, void* t, int dtype, int B, int
 int launch_gemm(const void* A, bool a_mn_major, const void* Bm, void* D, int in_dtype, int d_dtype,
                 long long M, long long N, long long K, float* splitk_ws, size_t splitk_ws_bytes,
                 uint32_t* status, cudaStream_t stream);
+// fp32 products (gemm_fp32.cu): one or two independent ones in one launch; M (when
+// a_mn), K (when not) and N are multiples of 4, operands 16-byte aligned.
+struct GemmFp32 {
+  const float *A, *B;
+  float* D;
+  long long M, N, K;
+  bool a_mn;
+};
+int launch_gemm_fp32(const GemmFp32* jobs, int n, cudaStream_t stream);
 size_t gemm_splitk_ws_bytes(long long M, long long N, long long K, int in_dtype);
 // D[i] = beta * D[i] + sum over `splits` fp32 planes of mn elements each (mn a multiple
 // of 4), in plane order; D is not read when beta is 0.
