@@ -255,6 +255,11 @@ static int run_fullrank(const void* x, const void* g_y, const void* W, void* g_x
     if (int e = mark_phase(3, stream)) return e;
     return mark_phase(4, stream);
   }
+  if (fused_enabled()) {   // Eq. 2, both products
+    if (int e = launch_exact(x, g_y, W, g_x, g_W, L, T, sk, lay.splitk_bytes, status, stream)) return e;
+    if (int e = mark_phase(3, stream)) return e;
+    return mark_phase(4, stream);
+  }
   // Eq. 2: g_W = g_y^T x
   if (int e = launch_gemm(g_y, /*a_mn_major=*/true, x, g_W, L.dtype, L.gw_dtype, L.Cout, L.Cin, T,
                           sk, lay.splitk_bytes, status, stream))

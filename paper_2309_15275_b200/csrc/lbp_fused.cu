@@ -867,4 +867,27 @@ int launch_fused(const void* x, const void* x_hat_dense, const void* g_y, const 
   return launch_products(c, stream);
 }
 
+int launch_exact(const void* x, const void* g_y, const void* W, void* g_x, void* g_W, const lbp_layer& L,
+                 long long tokens, float* planes, size_t planes_bytes, uint32_t* status,
+                 cudaStream_t stream) {
+  if (tokens >= (1ll << 31) - 256) return LBP_ERR_SHAPE;
+  ProductsCall c{};
+  lbp_layer Le = L;
+  Le.k = 8;   // no grid: any instance of the kernel serves
+  c.L = &Le;
+  c.r = 1;
+  c.core = 4;
+  c.gx_scale = 1.f;
+  c.ex.n_extra = static_cast<int>(tokens);
+  c.ex.x = x;
+  c.ex.gy = g_y;
+  c.ex.gx = g_x;
+  c.W = W;
+  c.g_W = g_W;
+  c.planes = planes;
+  c.planes_bytes = planes_bytes;
+  c.status = status;
+  return launch_products(c, stream);
+}
+
 }  // namespace lbp

@@ -232,6 +232,12 @@ int launch_fused(const void* x, const void* x_hat_dense, const void* g_y, const 
                  const CallViews* views = nullptr, const FusedExtras* extras = nullptr,
                  int* dc_slot = nullptr);
 
+// Eq. 2 (exact backpropagation, bf16) over `tokens` dense tokens: both products in one
+// launch of the products kernel, every token outside the grid.  planes: scratch for K
+// slices of g_W.
+int launch_exact(const void* x, const void* g_y, const void* W, void* g_x, void* g_W, const lbp_layer& L,
+                 long long tokens, float* planes, size_t planes_bytes, uint32_t* status, cudaStream_t stream);
+
 // Modelled time (microseconds) of the products kernel of this layer on `pairs`
 // CTA pairs, and of its projection kernel on `ctas` SMs (both from B200
 // measurements); lbp_backward_batch balances the two when it runs the
