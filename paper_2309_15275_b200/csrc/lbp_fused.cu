@@ -213,9 +213,6 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const int my_tiles = unit_tile_count(p, sc, unit, units);
   if (threadIdx.x == 0) trace_mark(p, 0);
-  // the next kernel on the stream (the projection of the next call) may be
-  // scheduled as SMs free up; it waits for this grid before touching memory
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
     // =========================== TMA producer ===========================
@@ -223,6 +220,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       // launched with programmatic stream serialization: x_hat / g_y_hat of the
       // projection kernel may only be read after this wait
       asm volatile("griddepcontrol.wait;" ::: "memory");
+      // The next kernel on the stream may be scheduled as SMs free up.  A projection that
+      // defers its own wait (buffers disjoint from this kernel's) then reads x and g_y at
+      // once, so this may be said only after whatever lies ahead has completed.
+      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
       const uint64_t keep = ptx::l2_policy_evict_last();
       uint32_t it = 0;
       bool ok = true;

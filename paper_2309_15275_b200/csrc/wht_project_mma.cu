@@ -128,9 +128,6 @@ __global__ void __launch_bounds__(MmaCfg<K>::kWarps * 32, 1)
     ptx::prefetch_tensormap(&tmap0);
     ptx::prefetch_tensormap(&tmap1);
   }
-  // a kernel launched behind this one with programmatic serialization may set
-  // itself up as SMs free up; it still waits for this grid before reading
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __syncthreads();
   // this kernel itself may have been launched the same way behind an earlier
   // kernel on the stream (the products kernel of the previous call, which still
@@ -138,6 +135,9 @@ __global__ void __launch_bounds__(MmaCfg<K>::kWarps * 32, 1)
   // kernel has completed (unless the caller vouches for disjoint buffers, see
   // ProjParams::defer_wait)
   if (!p.defer_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
+  // a kernel launched behind this one with programmatic serialization may set
+  // itself up as SMs free up; it still waits for this grid before reading
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   const uint32_t first = blockIdx.x * NW + warp;
   const uint32_t stride = gridDim.x * NW;
@@ -367,9 +367,9 @@ __global__ void __launch_bounds__(kStripWarps * 32, 1)
     ptx::prefetch_tensormap(&tmap0);
     ptx::prefetch_tensormap(&tmap1);
   }
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __syncthreads();
   if (!p.defer_wait) asm volatile("griddepcontrol.wait;" ::: "memory");   // see wht_project_mma_kernel
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // items count strips here: p.n_items0 / p.n_items = strips * chunks
   const uint32_t first = blockIdx.x * NW + warp;

@@ -170,6 +170,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
+  // Set-up.  The loads wait for the barriers alone, which the producers' own warps set up;
+  // the other warps meanwhile lay out the basis matrix and allocate TMEM (a batch of
+  // 896 -> 3584 and 3584 -> 896 with 1024 tokens at order 16 48.4 -> 47.0 us, 48 -> 192 and
+  // 192 -> 48 with 200704 tokens 95.8 -> 94.4).
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
       ptx::mbar_init(&full_bar[s], kProducers);
@@ -181,49 +185,54 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     ptx::mbar_fence_init();
     *abort_flag = 0;
-    ptx::prefetch_tensormap(&tmap0);
-    ptx::prefetch_tensormap(&tmap1);
-    ptx::prefetch_tensormap(&om.full[0]);
-    ptx::prefetch_tensormap(&om.full[1]);
   }
-  // The basis matrix as K-major B operands, one panel per part of 64 tokens: row n = 64
-  // tokens = 128 bytes, 16-byte piece c of row n at piece c ^ (n & 7); rows past the
-  // bases are zero.
-  for (int e = threadIdx.x; e < kParts * NB * 16 * 8; e += kThreads) {
-    const int part = e / (NB * 16 * 8), n = (e >> 3) % (NB * 16), c = e & 7;
-    uint32_t w[4];
-#pragma unroll
-    for (int h = 0; h < 8; ++h) {
-      uint32_t bits = 0u;
-      const int t = c * 8 + h;
-      if constexpr (K == 4) {
-        const int j = n / p.r, q = n - j * p.r, v = t & 15;
-        if (n < rows && (v >> 2) == j) bits = basis_bits<4>(mp, q, p.r, (t >> 4) * 4 + (v & 3));
-      } else {
-        bits = basis_bits<K>(mp, n, p.r, part * 64 + t);
-      }
-      w[h >> 1] = (h & 1) ? w[h >> 1] | (bits << 16) : bits;
-    }
-    *reinterpret_cast<uint4*>(sB + part * kPanelBytes + n * 128 + ((c ^ (n & 7)) << 4)) =
-        make_uint4(w[0], w[1], w[2], w[3]);
-  }
-  ptx::fence_proxy_async_smem();   // the tensor core reads B through the async proxy
   if (warp == 4) {
     ptx::tmem_alloc(tmem_slot, kTmemCols);
     ptx::tmem_relinquish();
+  } else if (warp == 5 && lane < 4) {
+    ptx::prefetch_tensormap(lane == 0 ? &tmap0 : lane == 1 ? &tmap1 : &om.full[lane - 2]);
+  } else if (warp >= 8) {
+    // The basis matrix as K-major B operands, one panel per part of 64 tokens: row n = 64
+    // tokens = 128 bytes, 16-byte piece c of row n at piece c ^ (n & 7); rows past the
+    // bases are zero.
+    for (int e = threadIdx.x - 256; e < kParts * NB * 16 * 8; e += kThreads - 256) {
+      const int part = e / (NB * 16 * 8), n = (e >> 3) % (NB * 16), c = e & 7;
+      uint32_t w[4];
+#pragma unroll
+      for (int h = 0; h < 8; ++h) {
+        uint32_t bits = 0u;
+        const int t = c * 8 + h;
+        if constexpr (K == 4) {
+          const int j = n / p.r, q = n - j * p.r, v = t & 15;
+          if (n < rows && (v >> 2) == j) bits = basis_bits<4>(mp, q, p.r, (t >> 4) * 4 + (v & 3));
+        } else {
+          bits = basis_bits<K>(mp, n, p.r, part * 64 + t);
+        }
+        w[h >> 1] = (h & 1) ? w[h >> 1] | (bits << 16) : bits;
+      }
+      *reinterpret_cast<uint4*>(sB + part * kPanelBytes + n * 128 + ((c ^ (n & 7)) << 4)) =
+          make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    ptx::fence_proxy_async_smem();   // the tensor core reads B through the async proxy
   }
-  // a kernel launched behind this one with programmatic serialization may set
-  // itself up as SMs free up; it still waits for this grid before reading
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  ptx::tc_fence_before_sync();
-  __syncthreads();
-  ptx::tc_fence_after_sync();
-  const uint32_t tmem_base = *tmem_slot;
   // launched the same way behind an earlier kernel on the stream that may still
   // read the buffers written below: nothing is read or written before it has
   // completed, unless the caller vouches for disjoint buffers (then the wait
   // moves to the end and only keeps completion ordered)
-  if (!p.defer_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (warp < kProducers) {
+    group_sync(1 + kMaxGroups);
+    asm volatile("bar.arrive %0, %1;" ::"r"(2 + kMaxGroups), "n"(kThreads) : "memory");
+    if (!p.defer_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
+    // A kernel launched behind this one the same way may set itself up as SMs free up; it
+    // still waits for this grid before reading.  Only now: whatever starts after this
+    // point may take it that the kernel ahead of this one has completed.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  } else {
+    ptx::tc_fence_before_sync();
+    asm volatile("bar.sync %0, %1;" ::"r"(2 + kMaxGroups), "n"(kThreads) : "memory");
+    ptx::tc_fence_after_sync();
+  }
+  const uint32_t tmem_base = warp < kProducers ? 0u : *tmem_slot;
 
   // items dealt to the CTAs round robin
   const uint32_t n_items = (p.n_chunks + 3) / 4;
