@@ -31,13 +31,17 @@ namespace {
 constexpr double kFeedGxBytesPerUs = 95e3, kFeedGwBytesPerUs = 76e3;
 constexpr double kTileFixedUs = 0.3;
 // The expansion writes g_x at about 43 GB/s per SM (bound by the stores in flight, up
-// to a 4 x 4 array); with an 8 x 8 array the epilogue warps bind.  It takes four blocks
-// at a time.
+// to a 4 x 4 array, so channels past the edge cost nothing until the warps bind: 12
+// blocks of 48 channels took 2.4 us in a tile of 128); with an 8 x 8 array the epilogue
+// warps bind.  It takes four blocks at a time.
 constexpr double kExpandBytesPerUs[3] = {43e3, 26e3, 18e3};
+constexpr double kExpandWarpsBytesPerUs = 90e3;
 constexpr double kGwStoreBytesPerUs = 45e3;
 // K slices of g_W go through fp32 planes and one more kernel.
 constexpr double kReduceFixedUs = 3.0;
 constexpr double kReduceBytesPerUs = 4e6;
+
+int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
 struct Costs {
   double mma_w, epi_w, mma_x, epi_x;
@@ -51,8 +55,16 @@ Costs tile_costs(const PlanShape& s, int bnw, int bnx, int kbps) {
   c.mma_w = kTileFixedUs + kbps * (a_bytes + bw) / kFeedGwBytesPerUs;
   c.mma_x = kTileFixedUs + s.num_kb_x * (a_bytes + bx) / kFeedGxBytesPerUs;
   c.epi_w = kTileFixedUs + 128.0 * bnw * 4 / kGwStoreBytesPerUs;
-  c.epi_x = 0.5 + (s.epi_kind < 0 ? bnx : (bnx / s.piece + 3) / 4 * 4) * s.expand_bytes * 128.0 /
-                    kExpandBytesPerUs[s.epi_kind < 0 ? 0 : s.epi_kind];
+  if (s.epi_kind < 0) {
+    c.epi_x = 0.5 + bnx * s.expand_bytes * 128.0 / kExpandBytesPerUs[0];
+  } else {
+    const double padded = (bnx / s.piece + 3) / 4 * 4 * static_cast<double>(s.expand_bytes) * 128.0;
+    const int row_tile = s.pair ? 256 : 128;
+    const double used = static_cast<double>(s.gx_side) / (ceil_div(s.gx_side, row_tile) * row_tile);
+    const double stores = padded * used / kExpandBytesPerUs[0];
+    const double warps = padded / (s.epi_kind == 0 ? kExpandWarpsBytesPerUs : kExpandBytesPerUs[s.epi_kind]);
+    c.epi_x = 0.5 + (stores > warps ? stores : warps);
+  }
   return c;
 }
 
@@ -108,8 +120,6 @@ bool same_shape(const PlanShape& a, const PlanShape& b) {
          a.bn_max == b.bn_max && a.max_splits == b.max_splits && a.expand_bytes == b.expand_bytes &&
          a.epi_kind == b.epi_kind && a.num_kb_w == b.num_kb_w && a.num_kb_x == b.num_kb_x;
 }
-
-int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
 // Tiles of this shape under given column tiles.
 int count_gx(const PlanShape& s, int row_tile, int bnx) {
