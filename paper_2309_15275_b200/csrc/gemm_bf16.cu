@@ -208,12 +208,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 template <int G>
 __global__ void __launch_bounds__(256)
     splitk_reduce_kernel(const float* __restrict__ part, void* __restrict__ D, long long mn,
-                         int splits, int d_bf16, float beta) {
+                         int splits, int d_bf16, float beta, int late) {
   constexpr int kCols = 256 / G;
   __shared__ float4 sums[G][kCols];
-  // at once: the kernels that write the planes said so themselves only after what lies
-  // ahead of them had completed
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // The next kernel may start (the kernels that write the planes said so themselves only
+  // after what lies ahead of them had completed): at once, or late, see launch_splitk_reduce.
+  if (!late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int c = threadIdx.x % kCols, g = threadIdx.x / kCols;
   const long long i4 = (static_cast<long long>(blockIdx.x) * kCols + c) * 4;
@@ -228,6 +228,7 @@ __global__ void __launch_bounds__(256)
       acc.w += v.w;
     }
   }
+  if (late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if constexpr (G > 1) {
     sums[g][c] = acc;
     __syncthreads();
@@ -325,7 +326,7 @@ Tiling choose_tiling(long long M, long long N, long long K, int sms) {
 }  // namespace
 
 int launch_splitk_reduce(const float* planes, void* D, long long mn, int splits, bool d_bf16,
-                         float beta, cudaStream_t stream) {
+                         float beta, bool late, cudaStream_t stream) {
   const long long threads = (mn + 3) / 4;
   // groups of planes: while that many threads leave SMs without a block of 256
   const int groups = threads >= 148 * 256 || splits < 4 ? 1 : threads >= 148 * 64 || splits < 16 ? 4 : 16;
@@ -341,7 +342,7 @@ int launch_splitk_reduce(const float* planes, void* D, long long mn, int splits,
   cfg.numAttrs = 1;
   const auto kernel = groups == 1 ? splitk_reduce_kernel<1> : groups == 4 ? splitk_reduce_kernel<4>
                                                                           : splitk_reduce_kernel<16>;
-  LBP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, planes, D, mn, splits, d_bf16 ? 1 : 0, beta));
+  LBP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, planes, D, mn, splits, d_bf16 ? 1 : 0, beta, late ? 1 : 0));
   count_launch();
   return LBP_OK;
 }
@@ -369,7 +370,7 @@ int launch_gemm(const void* A, bool a_mn_major, const void* Bm, void* D, int in_
     if (d_dtype != LBP_F32) return LBP_ERR_DTYPE;
     const GemmFp32 job{static_cast<const float*>(A), static_cast<const float*>(Bm), static_cast<float*>(D), M, N, K,
                        a_mn_major};
-    return launch_gemm_fp32(&job, 1, stream);
+    return launch_gemm_fp32(&job, 1, splitk_ws, splitk_ws_bytes, stream);
   }
   int dev = 0, sms = 0;
   LBP_CUDA_TRY(cudaGetDevice(&dev));
@@ -428,7 +429,7 @@ int launch_gemm(const void* A, bool a_mn_major, const void* Bm, void* D, int in_
   LBP_CUDA_TRY(cudaGetLastError());
 
   if (t.splits > 1)
-    return launch_splitk_reduce(splitk_ws, D, M * N, t.splits, d_dtype == LBP_BF16, 0.f, stream);
+    return launch_splitk_reduce(splitk_ws, D, M * N, t.splits, d_dtype == LBP_BF16, 0.f, false, stream);
   return LBP_OK;
 }
 

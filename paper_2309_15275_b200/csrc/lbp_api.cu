@@ -187,6 +187,14 @@ static ExtrasLayout plan_extras(const lbp_layer& L, size_t base_total, int r, co
 // separate product and expansion kernels instead.
 static bool fused_enabled() { return tune_options().fused; }
 
+// The two fp32 products of a layer: gx = gy W and g_W = gy^T xs over `rows` rows.
+static void products_fp32(const void* xs, const void* gy, const void* W, void* gx, void* g_W, const lbp_layer& L,
+                          long long rows, GemmFp32 (&jobs)[2]) {
+  const float* g = static_cast<const float*>(gy);
+  jobs[0] = {g, static_cast<const float*>(W), static_cast<float*>(gx), rows, L.Cin, L.Cout, false};
+  jobs[1] = {g, static_cast<const float*>(xs), static_cast<float*>(g_W), L.Cout, L.Cin, rows, true};
+}
+
 static Layout plan_layout(const lbp_layer& L, int r) {
   Layout w{};
   const long long T = static_cast<long long>(L.B) * L.H * L.W;
@@ -211,6 +219,11 @@ static Layout plan_layout(const lbp_layer& L, int r) {
     const size_t b = gemm_splitk_ws_bytes(T, L.Cin, L.Cout, L.dtype);
     w.splitk_bytes = a > b ? a : b;
   }
+  if (L.dtype == LBP_F32) {
+    GemmFp32 jobs[2];
+    products_fp32(nullptr, nullptr, nullptr, nullptr, nullptr, L, w.rows, jobs);
+    w.splitk_bytes = gemm_fp32_ws_bytes(jobs, 2);
+  }
   w.splitk = off = align_up(off, 1024);
   off += w.splitk_bytes;
   // scratch of the persistent products kernel (bf16, r <= 16): x_hat and
@@ -233,16 +246,6 @@ static int mark_phase(int i, cudaStream_t stream) {
   return LBP_OK;
 }
 
-// Both fp32 products of a layer, g_W = gy^T xs over `rows` rows and gx = gy W, in one launch.
-static int run_products_fp32(const void* xs, const void* gy, const void* W, void* gx, void* g_W,
-                             const lbp_layer& L, long long rows, cudaStream_t stream) {
-  const float* g = static_cast<const float*>(gy);
-  const GemmFp32 jobs[2] = {
-      {g, static_cast<const float*>(W), static_cast<float*>(gx), rows, L.Cin, L.Cout, false},
-      {g, static_cast<const float*>(xs), static_cast<float*>(g_W), L.Cout, L.Cin, rows, true}};
-  return launch_gemm_fp32(jobs, 2, stream);
-}
-
 static int run_fullrank(const void* x, const void* g_y, const void* W, void* g_x, void* g_W,
                         const lbp_layer& L, uint8_t* ws, cudaStream_t stream) {
   const Layout lay = plan_layout(L, L.k * L.k);
@@ -251,7 +254,9 @@ static int run_fullrank(const void* x, const void* g_y, const void* W, void* g_x
   float* sk = reinterpret_cast<float*>(ws + lay.splitk);
   if (int e = mark_phase(0, stream)) return e;
   if (L.dtype == LBP_F32) {   // Eq. 2, both products
-    if (int e = run_products_fp32(x, g_y, W, g_x, g_W, L, T, stream)) return e;
+    GemmFp32 jobs[2];
+    products_fp32(x, g_y, W, g_x, g_W, L, T, jobs);
+    if (int e = launch_gemm_fp32(jobs, 2, sk, lay.splitk_bytes, stream)) return e;
     if (int e = mark_phase(3, stream)) return e;
     return mark_phase(4, stream);
   }
@@ -777,7 +782,9 @@ static int run_core(const void* x, const void* x_hat_in, const void* g_y, const 
   if (int e = mark_phase(2, st)) return e;
   if (L.dtype == LBP_F32) {
     // steps 3 and 4
-    if (int e = run_products_fp32(x_hat, gy_hat, W, gx_hat, g_W, L, lay.rows, st)) return e;
+    GemmFp32 jobs[2];
+    products_fp32(x_hat, gy_hat, W, gx_hat, g_W, L, lay.rows, jobs);
+    if (int e = launch_gemm_fp32(jobs, 2, sk, lay.splitk_bytes, st)) return e;
     if (int e = mark_phase(3, st)) return e;
     if (int e = mark_phase(4, st)) return e;
     if (int e = launch_expand(gx_hat, /*in_f32=*/true, g_x, L.dtype, L.B, L.H, L.W, L.Cin, plan, dense, st,

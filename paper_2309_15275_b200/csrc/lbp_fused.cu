@@ -821,7 +821,7 @@ static int launch_products(const ProductsCall& c, cudaStream_t stream) {
   if (e != LBP_OK) return e;
   if (p.gw_splits > 1)
     return launch_splitk_reduce(p.gw_planes, c.g_W, static_cast<long long>(L.Cout) * L.Cin, p.gw_splits,
-                                p.gw_bf16 != 0, p.beta, stream);
+                                p.gw_bf16 != 0, p.beta, false, stream);
   return LBP_OK;
 }
 

@@ -163,12 +163,16 @@ struct GemmFp32 {
   long long M, N, K;
   bool a_mn;
 };
-int launch_gemm_fp32(const GemmFp32* jobs, int n, cudaStream_t stream);
+int launch_gemm_fp32(const GemmFp32* jobs, int n, float* ws, size_t ws_bytes, cudaStream_t stream);
+// Scratch for the K slices these take at best (with less, K is sliced less or not at all).
+size_t gemm_fp32_ws_bytes(const GemmFp32* jobs, int n);
 size_t gemm_splitk_ws_bytes(long long M, long long N, long long K, int in_dtype);
 // D[i] = beta * D[i] + sum over `splits` fp32 planes of mn elements each (mn a multiple
-// of 4), in plane order; D is not read when beta is 0.
+// of 4), in plane order; D is not read when beta is 0.  `late`: the next kernel on the
+// stream is one of many small CTAs (which would all settle on the SMs that are idle if they
+// came early), not one of a CTA per SM.
 int launch_splitk_reduce(const float* planes, void* D, long long mn, int splits, bool d_bf16,
-                         float beta, cudaStream_t stream);
+                         float beta, bool late, cudaStream_t stream);
 
 int check_device_arch();
 

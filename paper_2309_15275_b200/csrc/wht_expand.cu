@@ -60,6 +60,7 @@ __global__ void __launch_bounds__(256)
   const int lane = threadIdx.x & 31;
   const long long warp0 = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const long long n_warps = (static_cast<long long>(gridDim.x) * blockDim.x) >> 5;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // launched while the kernel ahead still runs
 
   for (long long item = warp0; item < p.n_items; item += n_warps) {
     const int chunk = static_cast<int>(item % p.n_chunks);
@@ -175,7 +176,16 @@ static int launch_one(const TI* t_hat, TO* t, const ExpandParams& p, const Devic
   long long want = (p.n_items + warps_per_cta - 1) / warps_per_cta;
   const long long cap = static_cast<long long>(sms) * 8;
   const int grid = static_cast<int>(want < cap ? want : cap);
-  wht_expand_kernel<TI, TO, K, LB><<<grid, 256, 0, stream>>>(t_hat, t, p, plan);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(256);
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  LBP_CUDA_TRY(cudaLaunchKernelEx(&cfg, wht_expand_kernel<TI, TO, K, LB>, t_hat, t, p, plan));
   count_launch();
   LBP_CUDA_TRY(cudaGetLastError());
   return LBP_OK;

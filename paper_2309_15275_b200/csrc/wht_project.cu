@@ -203,6 +203,8 @@ __global__ void __launch_bounds__(ProjCfg<K, sizeof(T) == 2>::kWarps * 32, 1)
       issue(idx + S, s);
     }
   }
+  // the next kernel may start (everything ahead of this one had completed before it began)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 template <typename T, int K, int LB>
@@ -262,14 +264,6 @@ int launch_project2(const void* t0, void* out0, int C0, const void* t1, void* ou
   const int es = dtype == LBP_BF16 ? 2 : 4;
   const int box_c = 128 / es;   // a box wider than C is legal: the excess is zero-filled
 
-  CUtensorMap tmaps[2];
-  if (int e = encode_block_tensor_map(&tmaps[0], t0, dtype, B, H, W, C0, K, box_c, false, view0)) return e;
-  if (t1 != nullptr) {
-    if (int e = encode_block_tensor_map(&tmaps[1], t1, dtype, B, H, W, C1, K, box_c, false, view1)) return e;
-  } else {
-    tmaps[1] = tmaps[0];
-  }
-
   ProjParams p;
   p.Hb = blocks_along(H, K);
   p.Wb = blocks_along(W, K);
@@ -323,6 +317,13 @@ int launch_project2(const void* t0, void* out0, int C0, const void* t1, void* ou
                               static_cast<__nv_bfloat16*>(out1), p, bp, sms, stream);
   }
 
+  CUtensorMap tmaps[2];
+  if (int e = encode_block_tensor_map(&tmaps[0], t0, dtype, B, H, W, C0, K, box_c, false, view0)) return e;
+  if (t1 != nullptr) {
+    if (int e = encode_block_tensor_map(&tmaps[1], t1, dtype, B, H, W, C1, K, box_c, false, view1)) return e;
+  } else {
+    tmaps[1] = tmaps[0];
+  }
   DevicePlan plan;
   for (int n = 0; n < 256; ++n) plan.qmap[n] = bp.qmap[n];
 
