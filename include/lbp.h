@@ -291,7 +291,7 @@ int lbp_backward_fullrank(const void* x, const void* g_y, const void* W,
  * memory until the process exits.
  *  - Same arguments, layouts and results as lbp_backward, minus ws / ws_bytes.
  *    The call allocates and frees nothing.
- *  - Layers with lbp_workspace_bytes(layer, r) > LBP_STATIC_SCRATCH_BYTES are
+ *  - Layers whose lbp_backward needs more scratch than LBP_STATIC_SCRATCH_BYTES are
  *    rejected with LBP_ERR_WORKSPACE before anything is enqueued.
  *  - The first call on a device looks up the array's device address (no
  *    allocation, but a runtime query): make that first call outside any stream

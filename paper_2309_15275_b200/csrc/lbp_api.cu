@@ -195,14 +195,17 @@ static void products_fp32(const void* xs, const void* gy, const void* W, void* g
   jobs[1] = {g, static_cast<const float*>(xs), static_cast<float*>(g_W), L.Cout, L.Cin, rows, true};
 }
 
-static Layout plan_layout(const lbp_layer& L, int r) {
+// from_coef: the call is handed x_hat.  At r = k^2 it then works on coefficients like any
+// other rank, where a call on x is Eq. 2 and needs none of them.
+static Layout plan_layout(const lbp_layer& L, int r, bool from_coef) {
+  const bool coef = r < L.k * L.k || from_coef;
   Layout w{};
   const long long T = static_cast<long long>(L.B) * L.H * L.W;
   // blocks of the grid extended with zero tokens to multiples of k
   const long long nb = static_cast<long long>(L.B) * blocks_along(L.H, L.k) * blocks_along(L.W, L.k);
   const int es = elem_size(L.dtype);
   size_t off = kStatusBytes;
-  if (r < L.k * L.k) {
+  if (coef) {
     w.rows = nb * r;
     w.x_hat = off = align_up(off, 1024);
     off += static_cast<size_t>(w.rows) * L.Cin * es;
@@ -229,7 +232,7 @@ static Layout plan_layout(const lbp_layer& L, int r) {
   // scratch of the persistent products kernel (bf16, r <= 16): x_hat and
   // g_y_hat with rows padded to 128-row groups
   w.fused = off = align_up(off, 1024);
-  if (r < L.k * L.k && L.dtype == LBP_BF16 && r <= fused_max_rank(L.k))
+  if (coef && L.dtype == LBP_BF16 && r <= fused_max_rank(L.k))
     off += fused_scratch_bytes(L, r, nullptr);
   w.total = align_up(off, 256);
   return w;
@@ -247,8 +250,7 @@ static int mark_phase(int i, cudaStream_t stream) {
 }
 
 static int run_fullrank(const void* x, const void* g_y, const void* W, void* g_x, void* g_W,
-                        const lbp_layer& L, uint8_t* ws, cudaStream_t stream) {
-  const Layout lay = plan_layout(L, L.k * L.k);
+                        const lbp_layer& L, const Layout& lay, uint8_t* ws, cudaStream_t stream) {
   const long long T = lay.rows;
   uint32_t* status = reinterpret_cast<uint32_t*>(ws);
   float* sk = reinterpret_cast<float*>(ws + lay.splitk);
@@ -286,7 +288,8 @@ extern "C" {
 size_t lbp_workspace_bytes(const lbp_layer* layer, int r) {
   if (check_layer(layer) != LBP_OK) return 0;
   if (r < 1 || r > layer->k * layer->k) return 0;
-  return plan_layout(*layer, r).total;
+  const size_t from_x = plan_layout(*layer, r, false).total, from_coef = plan_layout(*layer, r, true).total;
+  return from_x > from_coef ? from_x : from_coef;
 }
 
 int lbp_project(const void* t, void* t_hat, int B, int H, int W, int C, int k,
@@ -353,7 +356,8 @@ int lbp_expand(const void* t_hat, void* t, int B, int H, int W, int C, int k,
 // Host-side checks of one lbp_backward problem; nothing is enqueued.
 static int validate_backward(const void* x, const void* g_y, const void* W, const void* g_x,
                              const void* g_W, const lbp_layer* layer, const lbp_basis* set, int r,
-                             const void* ws, size_t ws_bytes, BasisPlan* plan, Layout* lay) {
+                             const void* ws, size_t ws_bytes, BasisPlan* plan, Layout* lay,
+                             bool from_coef = false) {
   if (x == nullptr || g_y == nullptr || W == nullptr || g_x == nullptr || g_W == nullptr)
     return LBP_ERR_NULL;
   if (int e = check_layer(layer)) return e;
@@ -361,7 +365,12 @@ static int validate_backward(const void* x, const void* g_y, const void* W, cons
   if (!aligned16(x) || !aligned16(g_y) || !aligned16(W) || !aligned16(g_x) || !aligned16(g_W) ||
       !aligned16(ws))
     return LBP_ERR_ALIGN;
-  *lay = plan_layout(*layer, r);
+  *lay = plan_layout(*layer, r, from_coef);
+  // the K slices of the fp32 products lie last and make do with what there is
+  if (layer->dtype == LBP_F32 && ws_bytes < lay->total && ws_bytes >= lay->splitk) {
+    lay->splitk_bytes = (ws_bytes - lay->splitk) / 256 * 256;
+    lay->total = lay->splitk + lay->splitk_bytes;
+  }
   if (ws == nullptr || ws_bytes < lay->total) return LBP_ERR_WORKSPACE;
   return LBP_OK;
 }
@@ -732,7 +741,7 @@ static int run_core(const void* x, const void* x_hat_in, const void* g_y, const 
                     const CallViews* views = nullptr, const FusedExtras* extras = nullptr) {
   const int r = plan.r;
   gy_loc->ptr = nullptr;
-  if (r == L.k * L.k && x_hat_in == nullptr) return run_fullrank(x, g_y, W, g_x, g_W, L, wsb, st);
+  if (r == L.k * L.k && x_hat_in == nullptr) return run_fullrank(x, g_y, W, g_x, g_W, L, lay, wsb, st);
 
   uint32_t* status = reinterpret_cast<uint32_t*>(wsb);
   if (runs_fused(L, plan)) {
@@ -990,7 +999,7 @@ int lbp_backward_ex(const void* x, const void* x_hat, const void* g_y, const voi
   const void* xin = x != nullptr ? x : x_hat;
   BasisPlan plan;
   Layout lay;
-  if (int e = validate_backward(xin, g_y, W, g_x, g_W, layer, set, r, ws, ws_bytes, &plan, &lay))
+  if (int e = validate_backward(xin, g_y, W, g_x, g_W, layer, set, r, ws, ws_bytes, &plan, &lay, x_hat != nullptr))
     return e;
   if (int e = check_extras(ex, layer)) return e;
   if (ws_bytes < lbp_workspace_bytes_ex(layer, r, ex)) return LBP_ERR_WORKSPACE;
@@ -1014,10 +1023,10 @@ int lbp_backward_fullrank(const void* x, const void* g_y, const void* W, void* g
   if (!aligned16(x) || !aligned16(g_y) || !aligned16(W) || !aligned16(g_x) || !aligned16(g_W) ||
       !aligned16(ws))
     return LBP_ERR_ALIGN;
-  const Layout lay = plan_layout(*layer, layer->k * layer->k);
+  const Layout lay = plan_layout(*layer, layer->k * layer->k, false);
   if (ws == nullptr || ws_bytes < lay.total) return LBP_ERR_WORKSPACE;
   if (int e = check_device_arch()) return e;
-  return run_fullrank(x, g_y, W, g_x, g_W, *layer, static_cast<uint8_t*>(ws),
+  return run_fullrank(x, g_y, W, g_x, g_W, *layer, lay, static_cast<uint8_t*>(ws),
                       static_cast<cudaStream_t>(stream));
 }
 

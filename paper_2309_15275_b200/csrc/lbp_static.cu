@@ -54,13 +54,11 @@ extern "C" int lbp_backward_static(const void* x, const void* g_y, const void* W
                                    void* g_W, const lbp_layer* layer, const lbp_basis* set, int r,
                                    void* stream) {
   if (layer == nullptr) return LBP_ERR_NULL;
-  // 0 means an invalid layer or rank: the validation below names the exact error
-  const size_t need = lbp_workspace_bytes(layer, r);
-  if (need > kStaticScratchBytes) return LBP_ERR_WORKSPACE;  // beyond the built-in scratch
   if (int e = lbp::check_device_arch()) return e;
   void* scratch = nullptr;
   if (int e = static_scratch_address(&scratch)) return e;
-  // every argument check of lbp_backward, before anything is enqueued
+  // every argument check of lbp_backward, before anything is enqueued (a layer whose
+  // scratch does not fit is one of them)
   if (int e = lbp::validate_backward_call(x, g_y, W, g_x, g_W, layer, set, r, scratch,
                                           kStaticScratchBytes))
     return e;

@@ -211,3 +211,13 @@ def test_binding_structs_have_the_size_the_library_was_compiled_with():
     for which, cls in ((0, B.Layer), (1, B.Extras), (2, B.View), (3, B.Basis)):
         assert lib.lbp_test_struct_size(which) == ctypes.sizeof(cls), cls.__name__
     assert lib.lbp_test_struct_size(99) == 0
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+def test_workspace_holds_the_coefficients_of_a_call_on_x_hat_at_full_rank(dtype):
+    # at r = k^2 a call on x is Eq. 2, one on x_hat still writes g_y_hat and g_x_hat
+    es = 2 if dtype == lbp.LBP_BF16 else 4
+    for H, k in ((8, 4), (9, 4), (16, 8)):
+        rows = 3 * (-(-H // k)) ** 2 * k * k
+        got = lbp.lbp_workspace_bytes(3, H, H, 64, 96, k, dtype, lbp.LBP_F32, k * k)
+        assert got >= rows * 96 * es + rows * 64 * 4
