@@ -12,6 +12,9 @@
 // per-thread sums; nothing but the k*k energies is written.
 #include <cuda_bf16.h>
 
+#include <atomic>
+
+
 #include "lbp_internal.h"
 #include "ptx_sm100.cuh"
 #include "wht_device.cuh"
@@ -164,6 +167,7 @@ __global__ void __launch_bounds__(MmaCfg<K>::kWarps * 32, 1)
   __syncthreads();
   // orthonormal coefficients: (1/k)^2 on the squares
   const double s2 = static_cast<double>(p.scale[0]) * static_cast<double>(p.scale[0]);
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // zero_energy_kernel has finished
   for (int i = threadIdx.x; i < R; i += NW * 32) atomicAdd(&energy[i], e_sm[i] * s2);
 }
 
@@ -297,7 +301,51 @@ __global__ void __launch_bounds__(MmaCfg<16>::kWarps * 32, 1)
     }
   __syncthreads();
   const double s2 = static_cast<double>(p.scale[0]) * static_cast<double>(p.scale[0]);
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // zero_energy_kernel has finished
   for (int i = threadIdx.x; i < R; i += NW * 32) atomicAdd(&energy[i], e_sm[i] * s2);
+}
+
+// The sums start from zero.  The kernel that adds to them is launched at once behind this
+// one and waits for it only before it adds, so the launch and the few stores lie under its
+// loads; what lies ahead of this kernel has completed before it starts.  Against a memset
+// ahead of the kernel: 64 x 16 x 16 tokens of 768 channels, order 8, 14.4 -> 12.4 us, order 4
+// 10.3 -> 8.4.  (Ahead of the two-pass form a memset is the faster one: 69 us against 72 for
+// 128 x 16 x 16 tokens of 768 fp32 channels.)
+__global__ void zero_energy_kernel(double* energy, int n) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (static_cast<int>(threadIdx.x) < n) energy[threadIdx.x] = 0.0;
+}
+static int launch_zero_energy(double* energy, int n, cudaStream_t stream) {
+  zero_energy_kernel<<<1, 256, 0, stream>>>(energy, n);
+  count_launch();
+  LBP_CUDA_TRY(cudaGetLastError());
+  return LBP_OK;
+}
+
+// A launch that may start while the kernel ahead of it on the stream still runs.
+template <class... Params, class... Args>
+static int launch_behind(void (*kern)(Params...), int grid, int threads, int smem, cudaStream_t stream,
+                         std::atomic<uint64_t>& configured, const Args&... args) {
+  int dev = 0;
+  LBP_CUDA_TRY(cudaGetDevice(&dev));
+  const uint64_t bit = 1ull << (dev & 63);
+  if (dev > 63 || (configured.load(std::memory_order_relaxed) & bit) == 0) {
+    LBP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    configured.fetch_or(bit, std::memory_order_relaxed);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  LBP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
+  count_launch();
+  return LBP_OK;
 }
 
 bool spectrum_mma_supported(int k, int dtype) {
@@ -308,14 +356,11 @@ template <int K>
 static int launch_spectrum_mma_k(const CUtensorMap& tmap, const ProjParams& p, const MmaPlan& mp,
                                  double* energy, int sms, cudaStream_t stream) {
   using Cfg = MmaCfg<K>;
-  auto kern = wht_spectrum_mma_kernel<K>;
-  LBP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
+  static std::atomic<uint64_t> configured{0};
   const uint32_t want = (p.n_items + Cfg::kWarps - 1) / Cfg::kWarps;
   const int grid = static_cast<int>(want < static_cast<uint32_t>(sms) ? want : sms);
-  kern<<<grid, Cfg::kWarps * 32, Cfg::kSmemBytes, stream>>>(tmap, p, mp, energy);
-  count_launch();
-  LBP_CUDA_TRY(cudaGetLastError());
-  return LBP_OK;
+  return launch_behind(wht_spectrum_mma_kernel<K>, grid, Cfg::kWarps * 32, Cfg::kSmemBytes, stream, configured,
+                       tmap, p, mp, energy);
 }
 
 // bp: the plan of all k*k pairs in raster order (i * k + j).
@@ -329,8 +374,6 @@ int launch_spectrum_mma(const void* t, int B, int H, int W, int C, const BasisPl
   p.Wb = blocks_along(W, K);
   p.nb = B * p.Hb * p.Wb;
   p.r = K * K;
-  p.bpt = 1;
-  p.tile_rows = p.r;
   p.C[0] = p.C[1] = C;
   p.n_chunks[0] = p.n_chunks[1] = (C + 63) / 64;
   const long long n0 = static_cast<long long>(p.nb) * p.n_chunks[0];
@@ -343,7 +386,7 @@ int launch_spectrum_mma(const void* t, int B, int H, int W, int C, const BasisPl
     mp.nat_i[q] = q < bp.r ? bp.nat_i[q] : 0;
     mp.nat_j[q] = q < bp.r ? bp.nat_j[q] : 0;
   }
-  LBP_CUDA_TRY(cudaMemsetAsync(energy, 0, static_cast<size_t>(K) * K * sizeof(double), stream));
+  if (int e = launch_zero_energy(energy, K * K, stream)) return e;
   int dev = 0, sms = 0;
   LBP_CUDA_TRY(cudaGetDevice(&dev));
   LBP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -351,14 +394,11 @@ int launch_spectrum_mma(const void* t, int B, int H, int W, int C, const BasisPl
     Seq16 sq;
     for (int sidx = 0; sidx < 16; ++sidx) sq.seq_of_nat[walsh_natural_index(16, sidx)] = static_cast<uint8_t>(sidx);
     using Cfg = MmaCfg<16>;
-    LBP_CUDA_TRY(cudaFuncSetAttribute(wht_spectrum16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      Cfg::kSmemBytes));
+    static std::atomic<uint64_t> configured{0};
     const uint32_t want = (p.n_items + Cfg::kWarps - 1) / Cfg::kWarps;
     const int grid = static_cast<int>(want < static_cast<uint32_t>(sms) ? want : sms);
-    wht_spectrum16_kernel<<<grid, Cfg::kWarps * 32, Cfg::kSmemBytes, stream>>>(tmap, p, sq, energy);
-    count_launch();
-    LBP_CUDA_TRY(cudaGetLastError());
-    return LBP_OK;
+    return launch_behind(wht_spectrum16_kernel, grid, Cfg::kWarps * 32, Cfg::kSmemBytes, stream, configured, tmap, p,
+                         sq, energy);
   }
   if (K == 4) return launch_spectrum_mma_k<4>(tmap, p, mp, energy, sms, stream);
   return launch_spectrum_mma_k<8>(tmap, p, mp, energy, sms, stream);
@@ -421,10 +461,8 @@ int launch_square_reduce(const void* t_hat, int dtype, long long rows, int C, in
   LBP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const long long want = (rows + kSqThreads / 32 - 1) / (kSqThreads / 32);
   const int grid = static_cast<int>(want < 4ll * sms ? want : 4ll * sms);
-  if (dtype == LBP_BF16)
-    square_reduce_kernel<true><<<grid, kSqThreads, 0, stream>>>(t_hat, rows, C, r, energy);
-  else
-    square_reduce_kernel<false><<<grid, kSqThreads, 0, stream>>>(t_hat, rows, C, r, energy);
+  const auto kern = dtype == LBP_BF16 ? square_reduce_kernel<true> : square_reduce_kernel<false>;
+  kern<<<grid, kSqThreads, 0, stream>>>(t_hat, rows, C, r, energy);
   count_launch();
   LBP_CUDA_TRY(cudaGetLastError());
   return LBP_OK;
