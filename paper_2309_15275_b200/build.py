@@ -14,7 +14,7 @@ LIB = os.path.join(HERE, "liblbp.so")
 BINDING = os.path.join(HERE, "_lbp_torch.so")
 BINDING_SOURCE = os.path.join(CSRC, "torch_binding.cpp")
 
-SOURCES = ["lbp_host.cpp", "lbp_api.cu", "wht_project.cu", "wht_project_mma.cu", "wht_expand.cu",
+SOURCES = ["lbp_host.cpp", "lbp_api.cu", "wht_project.cu", "wht_expand.cu",
            "gemm_fp32.cu", "gemm_bf16.cu", "lbp_fused.cu", "lbp_static.cu",
            "wht_spectrum.cu", "lbp_extras.cu", "lbp_fused_plan.cu", "wht_project_umma.cu"]
 

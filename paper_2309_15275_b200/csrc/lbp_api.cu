@@ -229,8 +229,7 @@ static Layout plan_layout(const lbp_layer& L, int r, bool from_coef) {
   }
   w.splitk = off = align_up(off, 1024);
   off += w.splitk_bytes;
-  // scratch of the persistent products kernel (bf16, r <= 16): x_hat and
-  // g_y_hat with rows padded to 128-row groups
+  // scratch of the persistent products kernel: x_hat, g_y_hat and K slices of g_W
   w.fused = off = align_up(off, 1024);
   if (coef && L.dtype == LBP_BF16 && r <= fused_max_rank(L.k))
     off += fused_scratch_bytes(L, r, nullptr);
@@ -301,7 +300,7 @@ int lbp_project(const void* t, void* t_hat, int B, int H, int W, int C, int k,
   if (!aligned16(t) || !aligned16(t_hat) || !aligned16(ws)) return LBP_ERR_ALIGN;
   if (ws == nullptr || ws_bytes < kStatusBytes) return LBP_ERR_WORKSPACE;
   if (int e = check_device_arch()) return e;
-  return launch_project(t, t_hat, dtype, B, H, W, C, plan, RowMap{1, r},
+  return launch_project(t, t_hat, dtype, B, H, W, C, plan,
                         static_cast<uint32_t*>(ws), static_cast<cudaStream_t>(stream));
 }
 
@@ -333,7 +332,7 @@ int lbp_spectrum(const void* t, double* energy, int B, int H, int W, int C, int 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (spectrum_mma_supported(k, dtype))   // one pass, nothing materialised
     return launch_spectrum_mma(t, B, H, W, C, plan, energy, static_cast<uint32_t*>(ws), st);
-  if (int e = launch_project(t, coef, dtype, B, H, W, C, plan, RowMap{1, r},
+  if (int e = launch_project(t, coef, dtype, B, H, W, C, plan,
                              static_cast<uint32_t*>(ws), st))
     return e;
   const long long rows = static_cast<long long>(B) * blocks_along(H, k) * blocks_along(W, k) * k * k;
@@ -350,7 +349,7 @@ int lbp_expand(const void* t_hat, void* t, int B, int H, int W, int C, int k,
   if (ws == nullptr || ws_bytes < kStatusBytes) return LBP_ERR_WORKSPACE;
   if (int e = check_device_arch()) return e;
   return launch_expand(t_hat, /*in_f32=*/dtype == LBP_F32, t, dtype, B, H, W, C, plan,
-                       RowMap{1, r}, static_cast<cudaStream_t>(stream));
+                       static_cast<cudaStream_t>(stream));
 }
 
 // Host-side checks of one lbp_backward problem; nothing is enqueued.
@@ -767,7 +766,6 @@ static int run_core(const void* x, const void* x_hat_in, const void* g_y, const 
   void* gy_hat = wsb + lay.gy_hat;
   float* gx_hat = reinterpret_cast<float*>(wsb + lay.gx_hat);
   float* sk = reinterpret_cast<float*>(wsb + lay.splitk);
-  const RowMap dense{1, r};
   gy_loc->ptr = gy_hat;
   gy_loc->dc_to_sum = static_cast<double>(L.k);   // orthonormal: coefficient = block sum / k
   gy_loc->dc_slot = -1;
@@ -777,13 +775,13 @@ static int run_core(const void* x, const void* x_hat_in, const void* g_y, const 
   if (int e = mark_phase(0, st)) return e;
   if (x_hat_in != nullptr) {
     // x_hat was taken at forward time: only g_y is projected
-    if (int e = launch_project(g_y, gy_hat, L.dtype, L.B, L.H, L.W, L.Cout, plan, dense, status, st,
+    if (int e = launch_project(g_y, gy_hat, L.dtype, L.B, L.H, L.W, L.Cout, plan, status, st,
                                0.f, views ? &views->gy : nullptr))
       return e;
   } else {
     // Algorithm 1, steps 1-2: x_hat = p(x), g_y_hat = p(g_y), one launch for both
     if (int e = launch_project2(g_y, gy_hat, L.Cout, x, wsb + lay.x_hat, L.Cin, L.dtype, L.B, L.H,
-                                L.W, plan, dense, status, st, 0.f, 0.f, views ? &views->gy : nullptr,
+                                L.W, plan, status, st, 0.f, 0.f, views ? &views->gy : nullptr,
                                 views ? &views->x : nullptr))
       return e;
   }
@@ -796,7 +794,7 @@ static int run_core(const void* x, const void* x_hat_in, const void* g_y, const 
     if (int e = launch_gemm_fp32(jobs, 2, sk, lay.splitk_bytes, st)) return e;
     if (int e = mark_phase(3, st)) return e;
     if (int e = mark_phase(4, st)) return e;
-    if (int e = launch_expand(gx_hat, /*in_f32=*/true, g_x, L.dtype, L.B, L.H, L.W, L.Cin, plan, dense, st,
+    if (int e = launch_expand(gx_hat, /*in_f32=*/true, g_x, L.dtype, L.B, L.H, L.W, L.Cin, plan, st,
                               views ? &views->gx : nullptr))
       return e;
     return mark_phase(5, st);
@@ -813,7 +811,7 @@ static int run_core(const void* x, const void* x_hat_in, const void* g_y, const 
   if (int e = mark_phase(4, st)) return e;
   // step 5: g_x = p^-1(g_x_hat)
   if (int e = launch_expand(gx_hat, /*in_f32=*/true, g_x, L.dtype, L.B, L.H, L.W, L.Cin, plan,
-                            dense, st, views ? &views->gx : nullptr))
+                            st, views ? &views->gx : nullptr))
     return e;
   return mark_phase(5, st);
 }

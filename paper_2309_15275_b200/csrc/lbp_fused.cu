@@ -609,18 +609,17 @@ double fused_projection_model_us(const lbp_layer& L, const BasisPlan& bp, int ct
 static int fused_project(const void* x, void* x_hat, const void* g_y, void* gy_hat, const lbp_layer& L,
                          const BasisPlan& bp, const CallViews* views, uint32_t* status,
                          cudaStream_t stream) {
-  const RowMap dense{1, bp.r};
   const FusedOverlap* ov = fused_overlap();
   cudaStream_t ps = ov != nullptr ? ov->proj_stream : stream;
   if (ov != nullptr) set_projection_launch(ProjLaunch{ov->proj_ctas, ov->proj_ctas > 0, false});
   const float sgy = fused_scale_gy(L.k, x == nullptr);
   int e = LBP_OK;
   if (x != nullptr)
-    e = launch_project2(g_y, gy_hat, L.Cout, x, x_hat, L.Cin, LBP_BF16, L.B, L.H, L.W, bp, dense, status,
+    e = launch_project2(g_y, gy_hat, L.Cout, x, x_hat, L.Cin, LBP_BF16, L.B, L.H, L.W, bp, status,
                         ps, sgy, fused_scale_x(L.k), views ? &views->gy : nullptr,
                         views ? &views->x : nullptr);
   else
-    e = launch_project(g_y, gy_hat, LBP_BF16, L.B, L.H, L.W, L.Cout, bp, dense, status, ps, sgy,
+    e = launch_project(g_y, gy_hat, LBP_BF16, L.B, L.H, L.W, L.Cout, bp, status, ps, sgy,
                        views ? &views->gy : nullptr);
   if (ov != nullptr) {
     set_projection_launch(ProjLaunch{0, false, true});

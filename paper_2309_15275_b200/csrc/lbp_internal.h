@@ -93,19 +93,13 @@ int encode_matrix_tensor_map(CUtensorMap* map, const void* base, long long rows,
                              int box_rows, long long pitch = 0);
 
 // ---- kernel launchers (each returns an lbp_status) ------------------------
-// Row q of block blk of a projected tensor lives at
-//   (blk / bpt) * tile_rows + (blk % bpt) * r + q ;   dense: bpt = 1, tile_rows = r.
-struct RowMap {
-  int32_t bpt;
-  int32_t tile_rows;
-};
-
+// Row q of block blk of a projected tensor is row blk * r + q.
 // `scale` multiplies the +-1 sums; 0 selects 1/k, the orthonormal coefficients of Eq. 6.
 int launch_project(const void* t, void* t_hat, int dtype, int B, int H, int W, int C,
-                   const BasisPlan& plan, RowMap rows, uint32_t* status, cudaStream_t stream,
+                   const BasisPlan& plan, uint32_t* status, cudaStream_t stream,
                    float scale = 0.f, const lbp_view* view = nullptr);
 
-// Per-thread switch read by the projection launchers (see ProjParams::defer_wait).
+// Per-thread switch read by the projection launchers (umma::Params::defer_wait).
 bool test_stall_projection();   // test hook (lbp_fused.cu)
 void set_projection_defer_wait(bool on);
 bool projection_defer_wait();
@@ -127,7 +121,7 @@ ProjLaunch projection_launch();
 
 // Projects two tensors that share the token grid (x and g_y) in one launch.
 int launch_project2(const void* t0, void* out0, int C0, const void* t1, void* out1, int C1,
-                    int dtype, int B, int H, int W, const BasisPlan& plan, RowMap rows,
+                    int dtype, int B, int H, int W, const BasisPlan& plan,
                     uint32_t* status, cudaStream_t stream, float scale0 = 0.f, float scale1 = 0.f,
                     const lbp_view* view0 = nullptr, const lbp_view* view1 = nullptr);
 
@@ -144,7 +138,7 @@ int launch_square_reduce(const void* t_hat, int dtype, long long rows, int C, in
 
 // t_hat is fp32 when `in_f32`, else of `dtype`; t is of `dtype`.
 int launch_expand(const void* t_hat, bool in_f32, void* t, int dtype, int B, int H, int W, int C,
-                  const BasisPlan& plan, RowMap rows, cudaStream_t stream,
+                  const BasisPlan& plan, cudaStream_t stream,
                   const lbp_view* view = nullptr);
 
 // D[M, N] = sum_k A(m, k) * B(k, n), fp32 accumulation.
@@ -211,7 +205,7 @@ int launch_bias_grad(const void* a, long long n_a, int r, int q, TokenMap ta, do
 //   LBP_FUSED=0          separate product and expansion kernels instead of the
 //                        persistent products kernel
 //   LBP_PAIR=0           one-CTA products kernel also on wide layers
-//   LBP_PROJECT_UMMA=0   projection of orders 8 and 16 on warp-level mma.sync instead of tcgen05
+//   LBP_PROJECT_UMMA=0   bf16 projection by additions on the CUDA cores instead of tcgen05
 //   LBP_FUSED_TILES=a,b,c  column tiles of the two products and K slices of g_W
 //   LBP_FUSED_VERBOSE=1  print the chosen tile plan
 //   LBP_BATCH_PROJ_SMS=n lbp_backward_batch: SMs given to the projection of the next

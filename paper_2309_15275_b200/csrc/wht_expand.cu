@@ -14,7 +14,6 @@ namespace lbp {
 
 struct ExpandParams {
   int32_t nb, Hb, Wb, H, W, C, r, n_chunks;
-  int32_t bpt, tile_rows;
   long long n_items;
   float scale;
   long long s_image, s_row, s_tok;   // element strides of t (dense: H*W*C, W*C, C)
@@ -68,8 +67,7 @@ __global__ void __launch_bounds__(256)
     const int c0 = (chunk * 32 + lane) * CH_PER_WORD;
     if (c0 >= p.C) continue;
     const int bw = blk % p.Wb, bh = (blk / p.Wb) % p.Hb, b = blk / (p.Wb * p.Hb);
-    const long long row0 =
-        static_cast<long long>(blk / p.bpt) * p.tile_rows + static_cast<long long>(blk % p.bpt) * p.r;
+    const long long row0 = static_cast<long long>(blk) * p.r;
     // offset of token (u, v) of this block: tok0 + u * s_row + v * s_tok
     const long long tok0 = static_cast<long long>(b) * p.s_image +
                            static_cast<long long>(bh * K) * p.s_row +
@@ -220,7 +218,7 @@ static int launch_t(const TI* t_hat, TO* t, const ExpandParams& p, const BasisPl
 }
 
 int launch_expand(const void* t_hat, bool in_f32, void* t, int dtype, int B, int H, int W, int C,
-                  const BasisPlan& bp, RowMap rows, cudaStream_t stream, const lbp_view* view) {
+                  const BasisPlan& bp, cudaStream_t stream, const lbp_view* view) {
   const int K = bp.k;
   ExpandParams p;
   const lbp_view sv = resolve_view(view, H, W, C);
@@ -236,8 +234,6 @@ int launch_expand(const void* t_hat, bool in_f32, void* t, int dtype, int B, int
   p.r = bp.r;
   const int ch_per_chunk = 32 * (dtype == LBP_BF16 ? 2 : 1);
   p.n_chunks = (C + ch_per_chunk - 1) / ch_per_chunk;
-  p.bpt = rows.bpt;
-  p.tile_rows = rows.tile_rows;
   p.n_items = static_cast<long long>(p.nb) * p.n_chunks;
   p.scale = 1.0f / static_cast<float>(K);
 

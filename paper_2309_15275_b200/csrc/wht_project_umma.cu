@@ -396,6 +396,30 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 }  // namespace umma
 
+// Grid size and launch attributes under the per-thread launch shape (see ProjLaunch):
+// `want` CTAs at most.
+static int projection_grid(uint32_t want, int sms, cudaLaunchAttribute* attr, unsigned* n_attr) {
+  const ProjLaunch shape = projection_launch();
+  int cap = shape.max_ctas > 0 && shape.max_ctas < sms ? shape.max_ctas : sms;
+  int grid = static_cast<int>(want < static_cast<uint32_t>(cap) ? want : cap);
+  unsigned n = 0;
+  if (shape.programmatic) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  if (shape.whole_tpcs && grid >= 2) {
+    grid &= ~1;
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = 2;
+    attr[n].val.clusterDim.y = 1;
+    attr[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  *n_attr = n;
+  return grid;
+}
+
 bool project_umma_supported(int k, int r) { return k == 4 || ((k == 8 || k == 16) && r <= 48); }
 
 int launch_project_umma(const void* t0, void* out0, int C0, const lbp_view* view0, const void* t1,
