@@ -1,0 +1,213 @@
+"""The kernels at the sizes where they can go wrong: edges of tiles, remainders, the
+smallest and the largest of each form's range, against the fp64 oracle.
+
+Bounds.  bf16: the two operands of a product and the output are rounded to 8 mantissa bits,
+at most 2^-9 per element each, sums are fp32: 3 * 2^-9 in the norm (BF16).  fp32: a sum of n
+terms in any order errs by about sqrt(n) * 2^-24 of its norm for these random signs, 4e-6 at
+the longest sum here (4096 terms), and the longest chain of kernels has three: F32 = 1.2e-5.
+"""
+import numpy as np
+import pytest
+import torch
+
+import paper_2309_15275_b200 as lbp
+from oracle import lbp_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+BF16 = 3 * 2.0 ** -9
+F32 = 1.2e-5
+
+
+@pytest.fixture(scope="module")
+def dev():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return torch.device("cuda:0")
+
+
+def f64(t):
+    return t.detach().cpu().to(torch.float64).numpy()
+
+
+def rel(got, want):
+    return O.rel_fro(f64(got), want)
+
+
+def draw(dev, seed, *shape, dtype=torch.bfloat16, scale=1.0):
+    g = torch.Generator().manual_seed(seed)
+    return (torch.randn(shape, generator=g) * scale).to(dtype).to(dev)
+
+
+def layer(dev, seed, B, H, W, ci, co, dtype=torch.bfloat16):
+    return (draw(dev, seed, B, H, W, ci, dtype=dtype), draw(dev, seed + 1, B, H, W, co, dtype=dtype, scale=0.01),
+            draw(dev, seed + 2, co, ci, dtype=dtype))
+
+
+def want_lowrank(x, gy, w, k, bases):
+    return O.backward_lowrank_padded(f64(x), f64(gy), f64(w), k, bases)
+
+
+def tri(n):
+    return [(i, j) for i in range(n) for j in range(n) if i + j < n]
+
+
+# one set per form of the expansion, with rows that start at j = 0 and without
+FORMS = {
+    "dc": [(0, 0)],
+    "2": [(0, 0), (1, 0), (0, 1)],
+    "2_holes": [(1, 1), (0, 1)],
+    "4": [(3, 0), (0, 0), (0, 3), (1, 2), (1, 0), (0, 1), (0, 2), (1, 1)],
+    "4_holes": [(0, 2), (3, 1), (2, 3)],
+    "sparse": tri(4) + [(4, 0), (0, 4), (1, 3)],
+    "sparse_holes": [(0, 0), (2, 5), (6, 1)],
+    "no_hh": tri(4) + [(0, 4), (0, 5), (4, 0), (5, 1)],
+    "8": tri(8),
+    "8_holes": [(7, 7), (0, 0), (4, 5), (2, 1)],
+}
+
+
+@pytest.mark.parametrize("form", list(FORMS))
+@pytest.mark.parametrize("k,ci,co,B,H,W", [
+    (8, 64, 64, 1, 8, 8),          # one block, half a channel tile
+    (8, 136, 72, 3, 17, 23),       # CTA pairs, 8 channels past a tile, ragged grid
+    (16, 264, 320, 5, 33, 16),     # 8 channels past a pair's tile
+    (4, 72, 200, 9, 7, 9),
+])
+def test_products_kernel_forms(dev, form, k, ci, co, B, H, W):
+    bases = FORMS[form]
+    if any(max(b) >= k for b in bases):
+        pytest.skip("the set needs a higher order")
+    x, gy, w = layer(dev, 11, B, H, W, ci, co)
+    ox, ow = want_lowrank(x, gy, w, k, bases)
+    ws = lbp.alloc_workspace(x, gy, k, len(bases))
+    gx, gw = lbp.lbp_backward(x, gy, w, k, bases, ws=ws)
+    assert lbp.lbp_poll_status(ws) == 0
+    assert rel(gx, ox) <= BF16 and rel(gw, ow) <= BF16
+    # from coefficients taken earlier, accumulating, with a token outside the grid
+    xe, ge = draw(dev, 5, B, ci), draw(dev, 6, B, co, scale=0.01)
+    oxe, owe = O.backward_extra_tokens(f64(xe), f64(ge), f64(w))
+    gw2, gxe = gw.clone(), torch.empty_like(xe)
+    gx2, _ = lbp.lbp_backward_ex(None, gy, w, k, bases, x_hat=lbp.lbp_project(x, k, bases), beta=0.5,
+                                 x_extra=xe, gy_extra=ge, gx_extra=gxe, g_W=gw2)
+    assert rel(gx2, ox) <= BF16 and rel(gxe, oxe) <= BF16
+    assert rel(gw2, ow + owe + 0.5 * f64(gw)) <= BF16
+
+
+@pytest.mark.parametrize("ci,co,T", [(64, 64, 1), (8, 8, 130), (136, 264, 65), (256, 128, 128), (128, 520, 2049)])
+def test_exact_mode_edges(dev, ci, co, T):
+    # one token; tiles with a few rows or channels past their edge; many K slices
+    x, gy, w = layer(dev, 21, 1, 4, 4 * T, ci, co)
+    bases = [(i, j) for i in range(4) for j in range(4)]
+    gx, gw = lbp.lbp_backward(x, gy, w, 4, bases)
+    ox, ow = O.backward_exact(f64(x), f64(gy), f64(w))
+    assert rel(gx, ox) <= 2.0 ** -9 and rel(gw, ow) <= F32   # operands are taken as they are
+
+
+@pytest.mark.parametrize("k,r", [(4, 1), (4, 4), (4, 5), (4, 9), (4, 15), (8, 1), (8, 16), (8, 17), (8, 33),
+                                 (8, 48), (16, 1), (16, 16), (16, 31), (16, 48)])
+@pytest.mark.parametrize("C,B,H,W", [(8, 1, 16, 16), (200, 3, 20, 36), (64, 70, 13, 12)])
+def test_projection_edges(dev, k, r, C, B, H, W):
+    # every width of the basis operand; less than a chunk of channels, a last chunk of 8,
+    # strips of four blocks that end early, more items than CTAs with a ragged last one
+    t = draw(dev, 31, B, H, W, C)
+    bases = lbp.lbp_select_bases(k, lbp.SEL_PREFIX, r)
+    got = lbp.lbp_project(t, k, bases)
+    want = O.project_padded(f64(t), k, bases)
+    assert rel(got, want) <= 2.0 ** -9
+    # a shift by one block or one channel leaves the norm alone, not the worst block
+    d = np.sqrt(((f64(got) - want) ** 2).sum(axis=(3, 4)))
+    assert np.all(d <= 2.0 ** -8 * np.sqrt((want ** 2).sum(axis=(3, 4))) + 1e-12)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("has_dc", [True, False])
+@pytest.mark.parametrize("B,H,C", [(1, 4, 8), (3, 7, 264), (70, 12, 136)])
+def test_bias_gradient_edges(dev, dtype, has_dc, B, H, C):
+    bases = [(0, 0), (0, 1)] if has_dc else [(0, 1), (1, 0)]
+    x, gy, w = layer(dev, 41, B, H, H, 64, C, dtype=dtype)
+    ge, xe = draw(dev, 44, B, C, dtype=dtype), draw(dev, 45, B, 64, dtype=dtype)
+    g_b = torch.full((C,), 3.0, dtype=torch.float32, device=dev)
+    gw = torch.zeros((C, 64), dtype=torch.float32, device=dev)
+    lbp.lbp_backward_ex(x, gy, w, 4, bases, beta=1.0, g_bias=g_b, x_extra=xe, gy_extra=ge,
+                        gx_extra=torch.empty_like(xe), g_W=gw)
+    want = O.bias_grad(f64(gy), f64(ge)) + 3.0
+    # read from the rounded (0, 0) coefficients where they exist, else from g_y itself
+    assert rel(g_b, want) <= (2.0 ** -9 if has_dc and dtype == torch.bfloat16 else F32)
+
+
+@pytest.mark.parametrize("ci,co,B,H,k,r", [
+    (4, 4, 1, 4, 4, 1),          # one tile of a few numbers
+    (68, 132, 1, 9, 8, 3),       # four rows and columns past the 64 x 64 tiles
+    (64, 64, 40, 32, 4, 3),      # g_W: one tile, hundreds of k-blocks
+    (448, 1344, 1, 8, 8, 10),    # g_x: few tiles, 42 k-blocks
+    (64, 192, 2, 33, 8, 64),     # exact, K no multiple of a k-block
+    (256, 256, 1, 8, 8, 63),
+])
+def test_fp32_products_edges(dev, ci, co, B, H, k, r):
+    x, gy, w = layer(dev, 51, B, H, H, ci, co, dtype=torch.float32)
+    bases = lbp.lbp_select_bases(k, lbp.SEL_PREFIX, r)
+    gx, gw = lbp.lbp_backward(x, gy, w, k, bases)
+    if r == k * k:
+        ox, ow = O.backward_exact(f64(x), f64(gy), f64(w))
+    else:
+        ox, ow = want_lowrank(x, gy, w, k, bases)
+    assert rel(gx, ox) <= F32 and rel(gw, ow) <= F32
+
+
+@pytest.mark.parametrize("co,ci,T,gw_dtype", [(64, 64, 512, torch.float32), (8, 8, 8192, torch.bfloat16),
+                                              (136, 264, 4096, torch.float32), (512, 512, 4096, torch.bfloat16)])
+def test_sum_of_k_slices(dev, co, ci, T, gw_dtype):
+    # few g_W tiles over many rows: from 2 to well over 16 planes, and onto a g_W
+    x, gy, w = layer(dev, 61, T // 64, 8, 8, ci, co)
+    bases = lbp.lbp_select_bases(8, lbp.SEL_PREFIX, 21)
+    _, ow = want_lowrank(x, gy, w, 8, bases)
+    for beta in (0.0, 1.0):
+        gw = torch.ones((co, ci), dtype=gw_dtype, device=dev)
+        lbp.lbp_backward_ex(x, gy, w, 8, bases, beta=beta, g_W=gw)
+        assert rel(gw, ow + beta) <= BF16
+
+
+@pytest.mark.parametrize("r", [16, 17, 48])
+def test_batch_equals_single_calls_at_high_rank(dev, r):
+    shapes = [(768, 2304), (768, 768), (2304, 768)]
+    bases = lbp.lbp_select_bases(8, lbp.SEL_PREFIX, r)
+    ins = [layer(dev, 71 + 3 * i, 8, 16, 16, ci, co) for i, (ci, co) in enumerate(shapes)]
+    xs, gys, ws_ = (list(v) for v in zip(*ins))
+    g_xs = [torch.empty_like(x) for x in xs]
+    g_Ws = [torch.empty(w.shape, dtype=torch.float32, device=dev) for w in ws_]
+    wss = [lbp.alloc_workspace(x, gy, 8, r) for x, gy in zip(xs, gys)]
+    for _ in range(2):
+        lbp.lbp_backward_batch(xs, gys, ws_, 8, bases, g_xs=g_xs, g_Ws=g_Ws, wss=wss)
+    for x, gy, w, gx, gw in zip(xs, gys, ws_, g_xs, g_Ws):
+        ox, ow = want_lowrank(x, gy, w, 8, bases)
+        assert rel(gx, ox) <= BF16 and rel(gw, ow) <= BF16
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("n_cls,bias", [(0, True), (1, True), (1, False)])
+def test_module_step_through_the_extension(dev, dtype, n_cls, bias):
+    # forward, backward and the bias gradient in the layer's dtype against the oracle
+    ci, co, B, H = 72, 136, 3, 12
+    bases = lbp.lbp_select_bases(4, lbp.SEL_L1, 2)
+    lin = lbp.LbpLinear(ci, co, 4, bases, bias=bias, device=dev, dtype=dtype, grid=(H, H) if n_cls else None)
+    if bias:
+        lin.bias.data.copy_(draw(dev, 83, co, dtype=dtype))
+    shape = (B, H, H) if n_cls == 0 else (B, n_cls + H * H)
+    x = draw(dev, 81, *shape, ci, dtype=dtype).requires_grad_()
+    gy = draw(dev, 82, *shape, co, dtype=dtype, scale=0.01)
+    y = lin(x)
+    y.backward(gy)
+    w = f64(lin.weight)
+    want_y = f64(x) @ w.T + (f64(lin.bias) if bias else 0.0)
+    grid = (lambda t: t) if n_cls == 0 else (lambda t: t[:, n_cls:].reshape(B, H, H, -1))
+    ox, ow = O.backward_lowrank_padded(grid(f64(x)), grid(f64(gy)), w, 4, bases)
+    if n_cls:
+        oxe, owe = O.backward_extra_tokens(f64(x)[:, :n_cls].reshape(-1, ci), f64(gy)[:, :n_cls].reshape(-1, co), w)
+        ow = ow + owe
+        assert rel(x.grad[:, :n_cls].reshape(-1, ci), oxe) <= (F32 if dtype == torch.float32 else BF16)
+    tol = F32 if dtype == torch.float32 else BF16
+    assert rel(y, want_y) <= tol and rel(grid(x.grad), ox) <= tol and rel(lin.weight.grad, ow) <= tol
+    if bias:
+        assert lin.bias.grad.dtype == dtype
+        assert rel(lin.bias.grad, O.bias_grad(f64(gy).reshape(-1, 1, 1, co))) <= tol
