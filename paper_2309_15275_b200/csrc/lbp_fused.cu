@@ -714,7 +714,7 @@ static int launch_products(const ProductsCall& c, cudaStream_t stream) {
   p.Cin = L.Cin;
   p.Cout = L.Cout;
   p.BNx = plan.BNx;
-  p.bpt = plan.BNx / c.r;
+  p.bpt = plan.bpt;
   p.n_ct = (L.Cin + ctas * BM - 1) / (ctas * BM);
   p.n_rt = (p.nb + p.bpt - 1) / p.bpt;
   p.num_kb_x = (L.Cout + BK - 1) / BK;

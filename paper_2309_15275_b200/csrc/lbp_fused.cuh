@@ -197,6 +197,7 @@ struct PlanShape {
 };
 struct TilePlan {
   int BNw, BNx, splits, kbps;
+  int bpt;           // blocks of a GX tile
   double model_us;   // time of the products kernel under the planner's cost model
   FusedSchedule sched;
 };

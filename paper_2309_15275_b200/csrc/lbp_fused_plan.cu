@@ -50,7 +50,7 @@ struct Costs {
   double mma_w, epi_w, mma_x, epi_x;
 };
 
-Costs tile_costs(const PlanShape& s, int bnw, int bnx, int kbps) {
+Costs tile_costs(const PlanShape& s, int bnw, int bnx, int bpt, int kbps) {
   const double a_bytes = 128.0 * 64 * 2;                       // a CTA's 128 rows of A per k-block
   const double bw = (s.pair ? bnw / 2 : bnw) * 64.0 * 2;       // its share of B
   const double bx = (s.pair ? bnx / 2 : bnx) * 64.0 * 2;
@@ -61,7 +61,7 @@ Costs tile_costs(const PlanShape& s, int bnw, int bnx, int kbps) {
   if (s.epi_kind < 0) {
     c.epi_x = 0.5 + bnx * s.expand_bytes * 128.0 / kExpandBytesPerUs[0];
   } else {
-    const double padded = (bnx / s.piece + 3) / 4 * 4 * static_cast<double>(s.expand_bytes) * 128.0;
+    const double padded = (bpt + 3) / 4 * 4 * static_cast<double>(s.expand_bytes) * 128.0;
     const int row_tile = s.pair ? 256 : 128;
     const double used = static_cast<double>(s.gx_side) / (ceil_div(s.gx_side, row_tile) * row_tile);
     const double stores = padded * used / kExpandBytesPerUs[0];
@@ -179,8 +179,8 @@ bool same_shape(const PlanShape& a, const PlanShape& b) {
 }
 
 // Tiles of this shape under given column tiles.
-int count_gx(const PlanShape& s, int row_tile, int bnx) {
-  return ceil_div(s.gx_side, row_tile) * (ceil_div(s.blocks, bnx / s.piece) + ceil_div(s.n_extra, bnx));
+int count_gx(const PlanShape& s, int row_tile, int bnx, int bpt) {
+  return ceil_div(s.gx_side, row_tile) * (ceil_div(s.blocks, bpt) + ceil_div(s.n_extra, bnx));
 }
 int count_gw(const PlanShape& s, int row_tile, int bnw, int splits) {
   return ceil_div(s.gw_rows, row_tile) * ceil_div(s.gw_cols, bnw) * splits;
@@ -212,25 +212,33 @@ const TilePlan& plan_products(const PlanShape& s) {
       // no wider than all pieces (or all single columns) together need
       const int less = bnx - s.bnx_step;
       if (less >= s.piece && less / s.piece >= s.blocks && less >= s.n_extra) continue;
-      for (int want : kSplitChoices) {
-        if (want > 1 && (want > s.max_splits || want > s.num_kb_w / 4)) continue;
-        if (tune.has_tiles &&
-            (bnw != tune.tiles_bnw || bnx != tune.tiles_bnx || want != tune.tiles_splits))
-          continue;
-        const int kbps = ceil_div(s.num_kb_w, want);
-        const int splits = ceil_div(s.num_kb_w, kbps);
-        const int n_gw = count_gw(s, row_tile, bnw, splits), n_gx = count_gx(s, row_tile, bnx);
-        const Costs c = tile_costs(s, bnw, bnx, kbps);
-        const int units = n_gw + n_gx < s.units ? n_gw + n_gx : s.units;
-        double t = deal(units, n_gx, n_gw, c, nullptr);
-        if (splits > 1)
-          t += kReduceFixedUs + (splits + 1.0) * s.gw_rows * static_cast<double>(s.gw_cols) * 4 / kReduceBytesPerUs;
-        if (best_t < 0 || t < best_t - 1e-9) {
-          best_t = t;
-          best.BNw = bnw;
-          best.BNx = bnx;
-          best.splits = splits;
-          best.kbps = kbps;
+      // Whole blocks that fit, or, in the narrowest tiles, fewer (what is left over is
+      // multiplied and dropped): a few large blocks at a low rank would otherwise lie in a
+      // handful of tiles (batch of 320 -> 1280 and 1280 -> 320, 36 blocks of 16 x 16 at rank
+      // 1: 32 to a tile 88 us, up to 8 37 us).
+      for (int bpt = bnx / s.piece; bpt > 0;
+           bpt = bnx == 32 && count_gx(s, row_tile, bnx, bpt) < 2 * s.units ? bpt / 8 * 4 : 0) {
+        for (int want : kSplitChoices) {
+          if (want > 1 && (want > s.max_splits || want > s.num_kb_w / 4)) continue;
+          if (tune.has_tiles &&
+              (bnw != tune.tiles_bnw || bnx != tune.tiles_bnx || want != tune.tiles_splits))
+            continue;
+          const int kbps = ceil_div(s.num_kb_w, want);
+          const int splits = ceil_div(s.num_kb_w, kbps);
+          const int n_gw = count_gw(s, row_tile, bnw, splits), n_gx = count_gx(s, row_tile, bnx, bpt);
+          const Costs c = tile_costs(s, bnw, bnx, bpt, kbps);
+          const int units = n_gw + n_gx < s.units ? n_gw + n_gx : s.units;
+          double t = deal(units, n_gx, n_gw, c, nullptr);
+          if (splits > 1)
+            t += kReduceFixedUs + (splits + 1.0) * s.gw_rows * static_cast<double>(s.gw_cols) * 4 / kReduceBytesPerUs;
+          if (best_t < 0 || t < best_t - 1e-9) {
+            best_t = t;
+            best.BNw = bnw;
+            best.BNx = bnx;
+            best.bpt = bpt;
+            best.splits = splits;
+            best.kbps = kbps;
+          }
         }
       }
     }
@@ -239,19 +247,20 @@ const TilePlan& plan_products(const PlanShape& s) {
   if (best_t < 0) {   // an override that fits nothing: the widest tiles, no slices
     best.BNw = bnw_top < s.bn_max ? bnw_top : s.bn_max;
     best.BNx = s.bn_max;
+    best.bpt = s.bn_max / s.piece;
     best.splits = 1;
     best.kbps = s.num_kb_w;
   }
 
   // per-unit tile lists of the chosen plan
   const int n_gw = count_gw(s, row_tile, best.BNw, best.splits);
-  const int n_gx = count_gx(s, row_tile, best.BNx);
+  const int n_gx = count_gx(s, row_tile, best.BNx, best.bpt);
   const int units = n_gw + n_gx < s.units ? n_gw + n_gx : s.units;
   FusedSchedule& sc = best.sched;
   sc.listed = 0;
   if (n_gw + n_gx <= kSchedMaxItems && units <= kSchedMaxUnits) {
     std::vector<int> owner;
-    deal(units, n_gx, n_gw, tile_costs(s, best.BNw, best.BNx, best.kbps), &owner);
+    deal(units, n_gx, n_gw, tile_costs(s, best.BNw, best.BNx, best.bpt, best.kbps), &owner);
     std::vector<std::vector<uint16_t>> lists(units);
     // tile ids as the kernels number them: the GW tiles come first
     for (int i = 0; i < n_gx; ++i) lists[owner[i]].push_back(static_cast<uint16_t>(n_gw + i));
@@ -265,9 +274,9 @@ const TilePlan& plan_products(const PlanShape& s) {
     sc.listed = 1;
   }
   if (tune.verbose)
-    fprintf(stderr, "lbp products plan (%s): BNw=%d BNx=%d gw_splits=%d kb/split=%d tiles=%d+%d "
+    fprintf(stderr, "lbp products plan (%s): BNw=%d BNx=%d (%d blocks) gw_splits=%d kb/split=%d tiles=%d+%d "
                     "units=%d listed=%d model=%.1f us\n",
-            s.pair ? "CTA pairs" : "CTAs", best.BNw, best.BNx, best.splits, best.kbps, n_gx, n_gw,
+            s.pair ? "CTA pairs" : "CTAs", best.BNw, best.BNx, best.bpt, best.splits, best.kbps, n_gx, n_gw,
             units, sc.listed, best_t);
 
   if (cache.capacity() < 128) cache.reserve(128);
