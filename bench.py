@@ -54,7 +54,7 @@ def _peaks():
 # DRAM traffic per step (sum over the four layers, bytes) of the two kernels, from
 # the ncu capture summarised in profiles/ (dram__bytes_read.sum + dram__bytes_write.sum);
 # None = not captured for the current kernels.
-NCU_TRAFFIC_PER_STEP = {"wht_project_umma_kernel": 824.0e6, "lbp_products_pair_kernel": 300.4e6}
+NCU_TRAFFIC_PER_STEP = {"wht_project_umma_kernel": 824.0e6, "lbp_products_kernel": 300.4e6}
 
 
 # ------------------------------------------------------------------ clocks ----
@@ -656,8 +656,8 @@ def _report_legs(args, torch, lbp, synth, dev, layers, k, bases, peaks, flush_bu
         ach = prod_bytes / (prod_us * 1e-6) / 1e9
         r_prod = {"bound": "hbm", "achieved": round(ach, 1), "peak": peaks["hbm_gbs"],
                   "unit": "GB/s", "frac": round(ach / peaks["hbm_gbs"], 4)}
-    r_prod.update({"kernel": "lbp_products_pair_kernel",
-                   "traffic": NCU_TRAFFIC_PER_STEP["lbp_products_pair_kernel"],
+    r_prod.update({"kernel": "lbp_products_kernel",
+                   "traffic": NCU_TRAFFIC_PER_STEP["lbp_products_kernel"],
                    "algorithmic_bytes": int(prod_bytes), "algorithmic_flops": prod_flops,
                    "launches_per_step": len(layers), "us_per_step": round(prod_us, 2),
                    "peak_source": peaks["source"], "share_of_step": round(prod_us / all_us, 4)})
