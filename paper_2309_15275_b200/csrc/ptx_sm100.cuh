@@ -208,7 +208,7 @@ __device__ __forceinline__ uint32_t tmem_ld_x1(uint32_t taddr) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(v) : "r"(taddr) : "memory");
   return v;
 }
-// N (2, 4, 8) consecutive fp32 columns from taddr on.
+// N (2, 4, 8, 16) consecutive fp32 columns from taddr on.
 template <int N>
 __device__ __forceinline__ void tmem_ld_xn(uint32_t taddr, uint32_t (&v)[N]) {
   if constexpr (N == 2) {
@@ -221,8 +221,10 @@ __device__ __forceinline__ void tmem_ld_xn(uint32_t taddr, uint32_t (&v)[N]) {
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
                  : "r"(taddr)
                  : "memory");
+  } else if constexpr (N == 16) {
+    tmem_ld_32x16(taddr, v);
   } else {
-    static_assert(N == 8, "2, 4 or 8 columns");
+    static_assert(N == 8, "2, 4, 8 or 16 columns");
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
                    "=r"(v[7])

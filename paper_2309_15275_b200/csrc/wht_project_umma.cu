@@ -19,8 +19,12 @@
 //   order 8   a block is one box (8 x 8 tokens);
 //   order 16  four parts of 64 tokens (four token rows each), every part a stage of its
 //             own against its own 64 columns of the basis matrix, accumulating;
-//   order 4   a "block" here is a strip of four along W (a box of 4 x 16 tokens); the
-//             basis matrix holds the bases of the four blocks one after the other.
+//   order 4   a "block" here is a strip of four along W, fetched as four boxes of 4 x 4
+//             tokens: every MMA then contracts the 16 tokens of one block, into 16 columns
+//             of its own.  (One 4 x 16 box has the four blocks' tokens in every MMA, zeros in
+//             the basis matrix keeping them apart, and zero times the infinity of a block is
+//             NaN in its neighbours; 128 x 16 x 16 tokens of 3072 channels took as long at
+//             rank 3, 49.2 us, and 56.4 against 57.4 at rank 8, 76.7 against 77.9 at rank 15.)
 // The accumulator holds one channel per TMEM lane and one coefficient per column: a
 // thread reads its r columns, rounds them and stores them to r rows of 64 channels in
 // shared memory, from where one TMA store per chunk writes them.
@@ -144,7 +148,7 @@ struct OutMaps {
   CUtensorMap full[2], tail[2];
 };
 
-// K: order; NB: N / 16
+// K: order; NB: N / 16 (order 4: what the epilogue reads of a block's 16 columns, / 4)
 template <int K, int NB>
 __global__ void __launch_bounds__(kThreads, 1)
     wht_project_umma_kernel(const __grid_constant__ CUtensorMap tmap0,
@@ -152,8 +156,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                             const __grid_constant__ OutMaps om, const __grid_constant__ Params p,
                             const __grid_constant__ MmaPlan mp) {
   constexpr int kParts = K == 16 ? 4 : 1;
-  constexpr int kPanelBytes = NB * 2048;   // 64 tokens x N rows
-  constexpr int kBoxH = K == 8 ? 8 : 4, kBoxW = K == 8 ? 8 : 16;
+  constexpr int kN = K == 4 ? 16 : NB * 16;   // columns of one MMA
+  constexpr int kPanelBytes = kN * 128;       // 64 tokens x N rows
+  constexpr int kBoxH = K == 8 ? 8 : 4, kBoxW = K == 8 ? 8 : 16;   // tokens of a chunk
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -194,17 +199,16 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp >= 8) {
     // The basis matrix as K-major B operands, one panel per part of 64 tokens: row n = 64
     // tokens = 128 bytes, 16-byte piece c of row n at piece c ^ (n & 7); rows past the
-    // bases are zero.
-    for (int e = threadIdx.x - 256; e < kParts * NB * 16 * 8; e += kThreads - 256) {
-      const int part = e / (NB * 16 * 8), n = (e >> 3) % (NB * 16), c = e & 7;
+    // bases are zero.  Order 4 uses the first 16 tokens of a row, those of a block.
+    for (int e = threadIdx.x - 256; e < kParts * kN * 8; e += kThreads - 256) {
+      const int part = e / (kN * 8), n = (e >> 3) % kN, c = e & 7;
       uint32_t w[4];
 #pragma unroll
       for (int h = 0; h < 8; ++h) {
         uint32_t bits = 0u;
         const int t = c * 8 + h;
         if constexpr (K == 4) {
-          const int j = n / p.r, q = n - j * p.r, v = t & 15;
-          if (n < rows && (v >> 2) == j) bits = basis_bits<4>(mp, q, p.r, (t >> 4) * 4 + (v & 3));
+          if (t < 16) bits = basis_bits<4>(mp, n, p.r, t);
         } else {
           bits = basis_bits<K>(mp, n, p.r, part * 64 + t);
         }
@@ -263,10 +267,14 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (have) {
             // the whole box counts, also where it hangs over the tensor (zero fill)
             ptx::mbar_expect_tx(&full_bar[s], kTileBytes);
-            ptx::tma_load_4d_hint(smem + s * kStageBytes + warp * kTileBytes, c.which ? &tmap1 : &tmap0,
-                                  &full_bar[s], ch, static_cast<int32_t>(c.bw * kBoxW),
-                                  static_cast<int32_t>(c.bh * (K == 16 ? 16 : kBoxH) + part * 4),
-                                  static_cast<int32_t>(c.b), stream_once);
+            constexpr int kBoxes = K == 4 ? 4 : 1;
+#pragma unroll
+            for (int j = 0; j < kBoxes; ++j)
+              ptx::tma_load_4d_hint(smem + s * kStageBytes + warp * kTileBytes + j * (kTileBytes / kBoxes),
+                                    c.which ? &tmap1 : &tmap0, &full_bar[s], ch,
+                                    static_cast<int32_t>(c.bw * kBoxW) + j * 4,
+                                    static_cast<int32_t>(c.bh * (K == 16 ? 16 : kBoxH) + part * 4),
+                                    static_cast<int32_t>(c.b), stream_once);
           } else {
             ptx::mbar_arrive(&full_bar[s]);   // no such chunk: what lies in the stage is multiplied and dropped
           }
@@ -282,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == 4) {
     // =========================== tcgen05 issuer ===========================
     if (ptx::elect_one()) {
-      constexpr uint32_t idesc = ptx::idesc_bf16(128, NB * 16, true, false);
+      constexpr uint32_t idesc = ptx::idesc_bf16(128, kN, true, false);
       const uint32_t b_addr = ptx::smem_u32(sB);
       bool ok = true;
       int s = 0;
@@ -305,11 +313,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
               // A: MN-major, 16 tokens = 16 rows of 128 bytes further per step, the two
-              // chunks 8 KB apart; B: K-major, 16 tokens = 32 bytes further
+              // chunks 8 KB apart; B: K-major, 16 tokens = 32 bytes further.  Order 4: a step
+              // is a block with the one basis matrix and columns of its own.
               const uint64_t da = ptx::smem_desc_sw128(sa + h * 2 * kTileBytes + kk * 2048, kTileBytes, 1024);
-              const uint64_t db = ptx::smem_desc_sw128(b_addr + part * kPanelBytes + kk * 32, 16, 1024);
-              ptx::mma_bf16_ss(tmem_base + slot * kSlotCols + h * kHalfCols, da, db, idesc,
-                               (part == 0 && kk == 0) ? 0u : 1u);
+              const uint64_t db =
+                  ptx::smem_desc_sw128(b_addr + part * kPanelBytes + (K == 4 ? 0 : kk * 32), 16, 1024);
+              ptx::mma_bf16_ss(tmem_base + slot * kSlotCols + h * kHalfCols + (K == 4 ? kk * kN : 0), da, db, idesc,
+                               (K == 4 || (part == 0 && kk == 0)) ? 0u : 1u);
             }
           }
           ptx::mma_commit(&empty_bar[s]);
@@ -350,18 +360,42 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int i = 2 * h + (quarter >> 1);
           const float sc = p.scale[chunk0 + i >= p.n_chunks0 ? 1 : 0];
           uint16_t* const o = reinterpret_cast<uint16_t*>(out + i * out_bytes) + (quarter & 1) * 32 + lane;
+          const uint32_t acc =
+              tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + slot * kSlotCols + h * kHalfCols;
+          auto put = [&](uint16_t* at, uint32_t v0, uint32_t v1, int left) {   // rows 0 and 1 of `left`
+            const uint32_t pk = pack_bf16x2(__uint_as_float(v0) * sc, __uint_as_float(v1) * sc);
+            if (0 < left) at[0] = static_cast<uint16_t>(pk);
+            if (1 < left) at[64] = static_cast<uint16_t>(pk >> 16);
+          };
+          if constexpr (K == 4) {
+            constexpr int kCols = 4 * NB;   // columns read of a block
+            uint16_t* oj = o;
+            // (unrolled, the wide forms run out of registers)
+#pragma unroll(kCols <= 8 ? 4 : 1)
+            for (int j = 0; j < 4; ++j, oj += p.r * 64) {
+              uint32_t v[kCols];
+              if constexpr (kCols == 12) {
+                uint32_t lo[8], hi[4];
+                ptx::tmem_ld_xn<8>(acc + j * kN, lo);
+                ptx::tmem_ld_xn<4>(acc + j * kN + 8, hi);
+                ptx::tmem_ld_wait();
 #pragma unroll
-          for (int nb = 0; nb < NB; ++nb) {
-            uint32_t v[16];
-            ptx::tmem_ld_32x16(tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + slot * kSlotCols +
-                                   h * kHalfCols + nb * 16,
-                               v);
-            ptx::tmem_ld_wait();
+                for (int q = 0; q < 12; ++q) v[q] = q < 8 ? lo[q & 7] : hi[q & 3];
+              } else {
+                ptx::tmem_ld_xn<kCols>(acc + j * kN, v);
+                ptx::tmem_ld_wait();
+              }
 #pragma unroll
-            for (int q = 0; q < 16; q += 2) {
-              const uint32_t pk = pack_bf16x2(__uint_as_float(v[q]) * sc, __uint_as_float(v[q + 1]) * sc);
-              if (nb * 16 + q < rows) o[(nb * 16 + q) * 64] = static_cast<uint16_t>(pk);
-              if (nb * 16 + q + 1 < rows) o[(nb * 16 + q + 1) * 64] = static_cast<uint16_t>(pk >> 16);
+              for (int q = 0; q < kCols; q += 2) put(oj + q * 64, v[q], v[q + 1], p.r - q);
+            }
+          } else {
+#pragma unroll
+            for (int nb = 0; nb < NB; ++nb) {
+              uint32_t v[16];
+              ptx::tmem_ld_xn<16>(acc + nb * 16, v);
+              ptx::tmem_ld_wait();
+#pragma unroll
+              for (int q = 0; q < 16; q += 2) put(o + (nb * 16 + q) * 64, v[q], v[q + 1], rows - nb * 16 - q);
             }
           }
         }
@@ -428,7 +462,7 @@ int launch_project_umma(const void* t0, void* out0, int C0, const lbp_view* view
                         cudaStream_t stream) {
   using namespace umma;
   const int K = bp.k, r = bp.r;
-  const int box_w = K == 8 ? 8 : 16, box_h = K == 8 ? 8 : 4;
+  const int box_w = K, box_h = K == 16 ? 4 : K;
   Params p{};
   p.per_strip = K == 4 ? 4 : 1;
   p.Hb = blocks_along(H, K);
@@ -481,8 +515,9 @@ int launch_project_umma(const void* t0, void* out0, int C0, const lbp_view* view
     om.tail[1] = om.tail[0];
   }
 
-  const int rows = r * p.per_strip, nb = (rows + 15) / 16, parts = K == 16 ? 4 : 1;
-  const int fixed = 1024 + kBarBytes + parts * nb * 2048;
+  const int rows = r * p.per_strip, parts = K == 16 ? 4 : 1;
+  const int nb = K == 4 ? (r + 3) / 4 : (r + 15) / 16;
+  const int fixed = 1024 + kBarBytes + parts * (K == 4 ? 1 : nb) * 2048;
   auto ring = [&](int groups) { return (kSmemMax - fixed - 4 * groups * rows * 128) / kStageBytes; };
   p.groups = kMaxGroups;
   while (p.groups > 2 && ring(p.groups) < 4) --p.groups;

@@ -211,3 +211,31 @@ def test_module_step_through_the_extension(dev, dtype, n_cls, bias):
     if bias:
         assert lin.bias.grad.dtype == dtype
         assert rel(lin.bias.grad, O.bias_grad(f64(gy).reshape(-1, 1, 1, co))) <= tol
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("k,r", [(4, 1), (4, 3), (4, 4), (4, 5), (4, 8), (4, 9), (4, 15), (8, 10), (8, 36), (16, 21)])
+def test_infinities_stay_in_their_block_and_channel(dev, dtype, k, r):
+    # a block's coefficients and its part of g_x are functions of that block alone: a token
+    # that is not finite changes nothing elsewhere, bit for bit
+    B, H, W, ci, co = 2, 3 * k, 6 * k + 1, 72, 136
+    bases = lbp.lbp_select_bases(k, lbp.SEL_PREFIX, r)
+    x, gy, w = layer(dev, 91, B, H, W, ci, co, dtype=dtype)
+    bad = gy.clone()
+    at = [(0, 1, k, 5, np.inf), (0, H - 1, 4 * k + 1, 70, np.nan), (1, k, 0, 135, -np.inf), (1, 0, W - 1, 64, np.inf)]
+    clean_blocks = torch.ones((B, H // k, -(-W // k)), dtype=torch.bool)
+    for b, h, v, c, val in at:
+        bad[b, h, v, c] = val
+        clean_blocks[b, h // k, v // k] = False
+    want, got = lbp.lbp_project(gy, k, bases), lbp.lbp_project(bad, k, bases)
+    keep = clean_blocks[..., None, None].expand(want.shape).clone()
+    for b, h, v, c, _ in at:
+        keep[b, h // k, v // k] = True
+    for b, h, v, c, _ in at:
+        keep[b, h // k, v // k, :, c] = False
+    keep = keep.to(dev)
+    assert torch.equal(got[keep], want[keep]) and not torch.isfinite(got[~keep]).any()
+    g_x, _ = lbp.lbp_backward(x, gy, w, k, bases)
+    g_x_bad, _ = lbp.lbp_backward(x, bad, w, k, bases)
+    tokens = clean_blocks.repeat_interleave(k, 1).repeat_interleave(k, 2)[:, :, :W].to(dev)
+    assert torch.equal(g_x_bad[tokens], g_x[tokens])
