@@ -12,6 +12,7 @@
 #include <Python.h>
 
 #include <ATen/ATen.h>
+#include <ATen/autocast_mode.h>
 #include <c10/cuda/CUDAFunctions.h>
 #include <c10/cuda/CUDAStream.h>
 #include <dlfcn.h>
@@ -444,7 +445,14 @@ struct LinearFunction : public torch::autograd::Function<LinearFunction> {
     } else {
       ctx->save_for_backward({x, weight});
     }
-    return at::linear(x, weight, bias);
+    // The bias rides in the product's epilogue where that is all one type.  Otherwise (a bias
+    // of another type, autocast, which casts the product's operands but not the sum's) torch's
+    // rules for the two operations decide the type of y.
+    const at::ScalarType dt = x.scalar_type();
+    if (!bias.has_value() || (weight.scalar_type() == dt && bias->scalar_type() == dt &&
+                              !at::autocast::is_autocast_enabled(x.device().type())))
+      return at::linear(x, weight, bias);
+    return at::matmul(x, weight.t()) + *bias;
   }
 
   static torch::autograd::variable_list backward(torch::autograd::AutogradContext* ctx,

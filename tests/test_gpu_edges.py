@@ -239,3 +239,19 @@ def test_infinities_stay_in_their_block_and_channel(dev, dtype, k, r):
     g_x_bad, _ = lbp.lbp_backward(x, bad, w, k, bases)
     tokens = clean_blocks.repeat_interleave(k, 1).repeat_interleave(k, 2)[:, :, :W].to(dev)
     assert torch.equal(g_x_bad[tokens], g_x[tokens])
+
+
+def test_module_step_under_autocast(dev):
+    # the product runs in bf16, the sum with the fp32 bias in fp32: y and the backward pass are fp32
+    ci, co, B, H = 64, 96, 2, 8
+    bases = lbp.lbp_select_bases(4, lbp.SEL_L1, 2)
+    lin = lbp.LbpLinear(ci, co, 4, bases, bias=True, device=dev)
+    x = draw(dev, 101, B, H, H, ci, dtype=torch.float32).requires_grad_()
+    gy = draw(dev, 102, B, H, H, co, dtype=torch.float32, scale=0.01)
+    with torch.autocast("cuda", dtype=torch.bfloat16):
+        y = lin(x)
+    assert y.dtype == torch.float32
+    y.backward(gy)
+    ox, ow = want_lowrank(x, gy, lin.weight, 4, bases)
+    assert rel(x.grad, ox) <= F32 and rel(lin.weight.grad, ow) <= F32
+    assert rel(lin.bias.grad, O.bias_grad(f64(gy))) <= F32

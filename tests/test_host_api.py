@@ -221,3 +221,20 @@ def test_workspace_holds_the_coefficients_of_a_call_on_x_hat_at_full_rank(dtype)
         rows = 3 * (-(-H // k)) ** 2 * k * k
         got = lbp.lbp_workspace_bytes(3, H, H, 64, 96, k, dtype, lbp.LBP_F32, k * k)
         assert got >= rows * 96 * es + rows * 64 * 4
+
+
+def test_module_forward_keeps_torch_dtype_rules():
+    # y is matmul(x, W^T) + b under torch's own rules, also where the three types differ
+    import torch
+    lin = lbp.LbpLinear(16, 24, 4, [(0, 0)], bias=True)
+    x = torch.randn(2, 4, 4, 16)
+
+    def plain(x):
+        return torch.matmul(x, lin.weight.t()) + lin.bias
+    with torch.autocast("cpu", dtype=torch.bfloat16):
+        y, want = lin(x), plain(x)
+    assert y.dtype == want.dtype == torch.float32 and torch.equal(y, want)
+    with torch.no_grad():
+        lin.weight.data = lin.weight.data.bfloat16()   # bf16 weights and inputs, fp32 bias
+        y, want = lin(x.bfloat16()), plain(x.bfloat16())
+    assert y.dtype == want.dtype == torch.float32 and torch.equal(y, want)
