@@ -60,22 +60,34 @@ struct Bases {
   lbp_basis v[256];
   int r = 0;
 };
-// A list or tuple of pairs of ints.
+// int(o), where that is an int32; false otherwise (no error is left behind).
+bool index_of(PyObject* o, int32_t* v) {
+  int over = 0;
+  long l = 0;
+  if (PyLong_Check(o)) {
+    l = PyLong_AsLongAndOverflow(o, &over);
+  } else {   // a numpy or torch scalar, a float
+    PyObject* n = PyNumber_Long(o);
+    if (n == nullptr) {
+      PyErr_Clear();
+      return false;
+    }
+    l = PyLong_AsLongAndOverflow(n, &over);
+    Py_DECREF(n);
+  }
+  *v = static_cast<int32_t>(l);
+  return over == 0 && *v == l;
+}
+// A list or tuple of pairs; whether a pair is a basis is the library's to say.
 bool parse_bases(PyObject* o, Bases* out) {
   if (!PyList_Check(o) && !PyTuple_Check(o)) return false;
   const Py_ssize_t n = PySequence_Fast_GET_SIZE(o);
-  if (n < 1 || n > 256) return false;
+  if (n > 256) return false;
   for (Py_ssize_t q = 0; q < n; ++q) {
     PyObject* p = PySequence_Fast_GET_ITEM(o, q);
     if (!PyTuple_Check(p) || PyTuple_GET_SIZE(p) != 2) return false;
-    PyObject *i = PyTuple_GET_ITEM(p, 0), *j = PyTuple_GET_ITEM(p, 1);
-    if (!PyLong_Check(i) || !PyLong_Check(j)) return false;
-    int over = 0;
-    const long a = PyLong_AsLongAndOverflow(i, &over);
-    if (over != 0 || a < 0 || a > 255) return false;
-    const long b = PyLong_AsLongAndOverflow(j, &over);
-    if (over != 0 || b < 0 || b > 255) return false;
-    out->v[q] = lbp_basis{static_cast<int32_t>(a), static_cast<int32_t>(b)};
+    if (!index_of(PyTuple_GET_ITEM(p, 0), &out->v[q].i) || !index_of(PyTuple_GET_ITEM(p, 1), &out->v[q].j))
+      return false;
   }
   out->r = static_cast<int>(n);
   return true;

@@ -238,3 +238,16 @@ def test_module_forward_keeps_torch_dtype_rules():
         lin.weight.data = lin.weight.data.bfloat16()   # bf16 weights and inputs, fp32 bias
         y, want = lin(x.bfloat16()), plain(x.bfloat16())
     assert y.dtype == want.dtype == torch.float32 and torch.equal(y, want)
+
+
+@pytest.mark.parametrize("kind", ["numpy rows", "numpy scalars", "lists", "tensors", "floats", "none"])
+def test_module_takes_bases_in_any_form_int_takes(kind):
+    import numpy as np
+    import torch
+    pairs = [(0, 0), (0, 1), (1, 0)]
+    bases = {"numpy rows": np.array(pairs), "numpy scalars": [(np.int64(i), np.int32(j)) for i, j in pairs],
+             "lists": [list(p) for p in pairs], "tensors": [(torch.tensor(i), torch.tensor(j)) for i, j in pairs],
+             "floats": [(float(i), float(j)) for i, j in pairs], "none": []}[kind]
+    lin = lbp.LbpLinear(16, 24, 4, bases)
+    x = torch.randn(2, 4, 4, 16)
+    assert torch.equal(lin(x), torch.matmul(x, lin.weight.t()))
