@@ -44,6 +44,11 @@ int lbp_test_tile_plan(int Cin, int Cout, int G, int bpt, int k, int units, int 
  * the switches select.  Returns LBP_OK. */
 int lbp_test_reload_env(void);
 
+/* Calls inside(arg) in the section in which lbp_backward_batch uses the stream and the
+ * events that the library keeps for `device` (0..63), and returns its result.  No
+ * device needed. */
+int lbp_test_side_section(int device, int (*inside)(void*), void* arg);
+
 /* sizeof of the structs of include/lbp.h as the library was compiled (which: 0
  * lbp_layer, 1 lbp_extras, 2 lbp_view, 3 lbp_basis; anything else: 0), so that a
  * binding in another language can check its own declarations against them. */

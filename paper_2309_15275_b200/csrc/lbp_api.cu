@@ -385,14 +385,18 @@ struct SideStream {
   cudaEvent_t fork;
   cudaEvent_t done[64];
 };
-static int side_stream(SideStream** out) {
+// One set serves every host thread, so a call keeps the device's section from its first
+// event record to its last wait: a wait takes an event as it stands when it is enqueued,
+// and another thread's record in between would order the call behind that thread's work
+// instead of its own.
+static std::mutex& side_section(int dev) {
+  static std::mutex mu[64];
+  return mu[dev];
+}
+// (with the device's section held)
+static int side_stream(int dev, SideStream** out) {
   static SideStream per_device[64];
   static bool ready[64] = {};
-  static std::mutex mu;
-  int dev = 0;
-  LBP_CUDA_TRY(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64) return LBP_ERR_ARCH;
-  std::lock_guard<std::mutex> lock(mu);
   if (!ready[dev]) {
     SideStream& s = per_device[dev];
     LBP_CUDA_TRY(cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking));
@@ -608,6 +612,12 @@ size_t lbp_test_struct_size(int which) {
   return 0;
 }
 
+int lbp_test_side_section(int device, int (*inside)(void*), void* arg) {
+  if (device < 0 || device >= 64 || inside == nullptr) return LBP_ERR_SHAPE;
+  std::lock_guard<std::mutex> lock(side_section(device));
+  return inside(arg);
+}
+
 int lbp_test_reload_env(void) {
   reload_tune_options();
   return LBP_OK;
@@ -674,8 +684,13 @@ int lbp_backward_batch(int n, const void* const* x, const void* const* g_y, cons
   if (int e = plan_batch(n, layers, set, r, &bplan)) return e;
   const bool side = bplan.side;
   SideStream* ss = nullptr;
+  std::unique_lock<std::mutex> section;
   if (side) {
-    if (int e = side_stream(&ss)) return e;
+    int dev = 0;
+    LBP_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return LBP_ERR_ARCH;
+    section = std::unique_lock<std::mutex>(side_section(dev));
+    if (int e = side_stream(dev, &ss)) return e;
     // everything enqueued so far on the caller's stream comes before the first projection
     LBP_CUDA_TRY(cudaEventRecord(ss->fork, st));
     LBP_CUDA_TRY(cudaStreamWaitEvent(ss->stream, ss->fork, 0));
@@ -710,6 +725,10 @@ int lbp_backward_batch(int n, const void* const* x, const void* const* g_y, cons
     }
   }
   set_projection_defer_wait(false);
+  if (side && status != LBP_OK) {   // projections may be under way that nothing waits for yet
+    (void)cudaEventRecord(ss->fork, ss->stream);
+    (void)cudaStreamWaitEvent(st, ss->fork, 0);
+  }
   return status;
 }
 

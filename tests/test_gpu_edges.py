@@ -6,6 +6,10 @@ at most 2^-9 per element each, sums are fp32: 3 * 2^-9 in the norm (BF16).  fp32
 terms in any order errs by about sqrt(n) * 2^-24 of its norm for these random signs, 4e-6 at
 the longest sum here (4096 terms), and the longest chain of kernels has three: F32 = 1.2e-5.
 """
+import ctypes
+import threading
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -255,3 +259,61 @@ def test_module_step_under_autocast(dev):
     ox, ow = want_lowrank(x, gy, lin.weight, 4, bases)
     assert rel(x.grad, ox) <= F32 and rel(lin.weight.grad, ow) <= F32
     assert rel(lin.bias.grad, O.bias_grad(f64(gy))) <= F32
+
+
+def batch_of(dev, seed, shapes, B=8, r=8):
+    ins = [layer(dev, seed + 3 * i, B, 16, 16, ci, co) for i, (ci, co) in enumerate(shapes)]
+    xs, gys, ws_ = (list(v) for v in zip(*ins))
+    return dict(xs=xs, g_ys=gys, Ws=ws_, k=8, bases=lbp.lbp_select_bases(8, lbp.SEL_PREFIX, r),
+                g_xs=[torch.empty_like(x) for x in xs],
+                g_Ws=[torch.empty(w.shape, dtype=torch.float32, device=dev) for w in ws_],
+                wss=[lbp.alloc_workspace(x, gy, 8, r) for x, gy in zip(xs, gys)])
+
+
+def test_batch_call_waits_for_the_section_of_the_side_stream(dev):
+    a = batch_of(dev, 111, [(768, 768), (256, 1024)])
+    events = [None, None]
+    lbp.lbp_backward_batch(**a, done_events=events)
+    torch.cuda.synchronize()
+    usleep = ctypes.cast(ctypes.CDLL(None).usleep, ctypes.c_void_p)
+    held = threading.Thread(target=lambda: lbp.binding._lib().lbp_test_side_section(dev.index, usleep, 400000))
+    held.start()
+    time.sleep(0.1)
+    t0 = time.perf_counter()
+    lbp.lbp_backward_batch(**a, done_events=events)
+    waited = time.perf_counter() - t0
+    held.join()
+    assert 0.1 < waited < 5.0
+
+
+def test_batch_calls_of_two_threads_on_two_streams(dev):
+    # every call's projections follow its own inputs, its products its own projections
+    sets = [batch_of(dev, 131, [(768, 768), (256, 1024), (1024, 256)]), batch_of(dev, 151, [(384, 1536), (768, 384)])]
+    want = []
+    for s in sets:
+        lbp.lbp_backward_batch(**s)
+        torch.cuda.synchronize()
+        want.append([t.clone() for t in s["g_xs"] + s["g_Ws"]])
+    clean = [[t.clone() for t in s["xs"] + s["g_ys"]] for s in sets]
+    failed = []
+
+    def work(s, src, want):
+        torch.cuda.set_device(dev)
+        stream = torch.cuda.Stream(device=dev)
+        with torch.cuda.stream(stream):
+            for _ in range(40):
+                for t in s["xs"] + s["g_ys"]:
+                    t.zero_()
+                for t, c in zip(s["xs"] + s["g_ys"], src):
+                    t.copy_(c)
+                lbp.lbp_backward_batch(**s, done_events=[None] * len(s["xs"]))
+                got = s["g_xs"] + s["g_Ws"]
+                if not all(torch.equal(g, w) for g, w in zip(got, want)):
+                    failed.append(1)
+    threads = [threading.Thread(target=work, args=v) for v in zip(sets, clean, want)]
+    torch.cuda.synchronize()
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed

@@ -251,3 +251,30 @@ def test_module_takes_bases_in_any_form_int_takes(kind):
     lin = lbp.LbpLinear(16, 24, 4, bases)
     x = torch.randn(2, 4, 4, 16)
     assert torch.equal(lin(x), torch.matmul(x, lin.weight.t()))
+
+
+def test_batch_section_admits_one_thread_per_device():
+    # the library's one stream and event set per device: what one batch call enqueues on
+    # them is not interleaved with another thread's
+    import threading
+    import time
+    lib = lbp.binding._lib()
+    inside, most, order = [0, 0], [0, 0], threading.Lock()
+
+    def enter(dev):
+        def body(_):
+            with order:
+                inside[dev] += 1
+                most[dev] = max(most[dev], inside[dev])
+            time.sleep(0.02)
+            with order:
+                inside[dev] -= 1
+            return 40 + dev
+        cb = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p)(body)
+        assert lib.lbp_test_side_section(dev, ctypes.cast(cb, ctypes.c_void_p), None) == 40 + dev
+    threads = [threading.Thread(target=enter, args=(i % 2,)) for i in range(8)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert most == [1, 1]
