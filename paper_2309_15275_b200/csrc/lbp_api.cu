@@ -409,6 +409,20 @@ static int side_stream(int dev, SideStream** out) {
   return LBP_OK;
 }
 
+// Whether `side` belongs to a stream capture that `st` is no part of: it joined the capture
+// of an earlier batch call and stays in it until that capture ends.  An event of any other
+// stream would be an error on it and spoil the capture.
+static int in_another_capture(cudaStream_t side, cudaStream_t st, bool* out) {
+  cudaStreamCaptureStatus a, b;
+  unsigned long long id_a = 0, id_b = 0;
+  LBP_CUDA_TRY(cudaStreamGetCaptureInfo(side, &a, &id_a));
+  *out = false;
+  if (a == cudaStreamCaptureStatusNone) return LBP_OK;
+  LBP_CUDA_TRY(cudaStreamGetCaptureInfo(st, &b, &id_b));
+  *out = b == cudaStreamCaptureStatusNone || id_a != id_b;
+  return LBP_OK;
+}
+
 // How lbp_backward_batch runs its problems: in which order, whether the
 // projections go to the side stream, and how many SMs the projection at each
 // position gets beside the products kernel before it.
@@ -682,7 +696,7 @@ int lbp_backward_batch(int n, const void* const* x, const void* const* g_y, cons
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   BatchPlan bplan;
   if (int e = plan_batch(n, layers, set, r, &bplan)) return e;
-  const bool side = bplan.side;
+  bool side = bplan.side;
   SideStream* ss = nullptr;
   std::unique_lock<std::mutex> section;
   if (side) {
@@ -691,6 +705,14 @@ int lbp_backward_batch(int n, const void* const* x, const void* const* g_y, cons
     if (dev < 0 || dev >= 64) return LBP_ERR_ARCH;
     section = std::unique_lock<std::mutex>(side_section(dev));
     if (int e = side_stream(dev, &ss)) return e;
+    bool taken = false;
+    if (int e = in_another_capture(ss->stream, st, &taken)) return e;
+    if (taken) {   // on one stream then
+      side = false;
+      section.unlock();
+    }
+  }
+  if (side) {
     // everything enqueued so far on the caller's stream comes before the first projection
     LBP_CUDA_TRY(cudaEventRecord(ss->fork, st));
     LBP_CUDA_TRY(cudaStreamWaitEvent(ss->stream, ss->fork, 0));

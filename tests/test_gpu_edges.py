@@ -317,3 +317,31 @@ def test_batch_calls_of_two_threads_on_two_streams(dev):
     for t in threads:
         t.join()
     assert not failed
+
+
+def test_batch_call_beside_the_capture_of_another(dev):
+    # the library's stream stays in a capture it has joined until that ends: a call on a
+    # stream outside it runs on its own stream alone, and leaves the capture intact
+    a = batch_of(dev, 171, [(768, 768), (256, 1024)])
+    b = batch_of(dev, 181, [(384, 1536), (768, 384)])
+    want = []
+    for s in (a, b):
+        lbp.lbp_backward_batch(**s)
+        want.append([t.clone() for t in s["g_xs"] + s["g_Ws"]])
+    for t in a["g_xs"] + a["g_Ws"] + b["g_xs"] + b["g_Ws"]:
+        t.zero_()
+    torch.cuda.synchronize()
+    graph, inner, outer = torch.cuda.CUDAGraph(), torch.cuda.Stream(device=dev), torch.cuda.Stream(device=dev)
+    with torch.cuda.stream(inner):
+        graph.capture_begin(capture_error_mode="thread_local")
+        lbp.lbp_backward_batch(**a)
+        with torch.cuda.stream(outer):
+            lbp.lbp_backward_batch(**b)
+        graph.capture_end()
+    graph.replay()
+    torch.cuda.synchronize()
+    for s, w in zip((a, b), want):
+        n = len(s["g_xs"])
+        assert all(torch.equal(g, v) for g, v in zip(s["g_xs"], w[:n]))
+        # other K slices of g_W on one stream: fp32 sums in another order
+        assert all(rel(g, f64(v)) <= F32 for g, v in zip(s["g_Ws"], w[n:]))
