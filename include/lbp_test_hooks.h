@@ -49,6 +49,10 @@ int lbp_test_reload_env(void);
  * device needed. */
 int lbp_test_side_section(int device, int (*inside)(void*), void* arg);
 
+/* What the library does once on each device (the opt-in of a kernel to more shared
+ * memory): done[i] = 1 where a run over devices[0..n-1] would have done it at i. */
+int lbp_test_per_device(const int* devices, int n, uint8_t* done);
+
 /* sizeof of the structs of include/lbp.h as the library was compiled (which: 0
  * lbp_layer, 1 lbp_extras, 2 lbp_view, 3 lbp_basis; anything else: 0), so that a
  * binding in another language can check its own declarations against them. */

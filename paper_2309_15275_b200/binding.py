@@ -124,6 +124,8 @@ def _lib() -> C.CDLL:
         lib.lbp_test_struct_size.restype = sz
         lib.lbp_test_side_section.argtypes = [i32, vp, vp]
         lib.lbp_test_side_section.restype = i32
+        lib.lbp_test_per_device.argtypes = [C.POINTER(i32), i32, C.POINTER(C.c_uint8)]
+        lib.lbp_test_per_device.restype = i32
         lib.lbp_test_stall_products.argtypes = [i32]
         lib.lbp_test_stall_products.restype = i32
         lib.lbp_launch_count.argtypes = []
@@ -169,7 +171,7 @@ EXPORTED = ("lbp_select_bases", "lbp_basis_matrix", "lbp_flops", "lbp_status_str
             "lbp_backward_batch", "lbp_test_stall_products",
             "lbp_test_reload_env", "lbp_workspace_bytes_ex", "lbp_backward_ex",
             "lbp_backward_projected", "lbp_test_tile_plan", "lbp_test_struct_size",
-            "lbp_test_side_section")
+            "lbp_test_side_section", "lbp_test_per_device")
 
 
 def _check(status: int, where: str) -> None:

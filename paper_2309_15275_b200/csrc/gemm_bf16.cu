@@ -409,22 +409,10 @@ int launch_gemm(const void* A, bool a_mn_major, const void* Bm, void* D, int in_
 
   dim3 grid(static_cast<unsigned>((N + t.BN - 1) / t.BN), static_cast<unsigned>((M + BM - 1) / BM),
             static_cast<unsigned>(t.splits));
-  static bool configured[2] = {false, false};
-  if (a_mn_major) {
-    if (!configured[1]) {
-      LBP_CUDA_TRY(cudaFuncSetAttribute(gemm_bf16_kernel<true>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-      configured[1] = true;
-    }
-    gemm_bf16_kernel<true><<<grid, kThreads, kSmemBytes, stream>>>(tmap_a, tmap_b, p);
-  } else {
-    if (!configured[0]) {
-      LBP_CUDA_TRY(cudaFuncSetAttribute(gemm_bf16_kernel<false>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-      configured[0] = true;
-    }
-    gemm_bf16_kernel<false><<<grid, kThreads, kSmemBytes, stream>>>(tmap_a, tmap_b, p);
-  }
+  static PerDevice configured[2];
+  const auto kernel = a_mn_major ? gemm_bf16_kernel<true> : gemm_bf16_kernel<false>;
+  if (int e = allow_dynamic_smem(configured[a_mn_major], reinterpret_cast<const void*>(kernel), kSmemBytes)) return e;
+  kernel<<<grid, kThreads, kSmemBytes, stream>>>(tmap_a, tmap_b, p);
   count_launch();
   LBP_CUDA_TRY(cudaGetLastError());
 

@@ -17,8 +17,6 @@
 // alone 0.54).  8 x 8 sums in 64 threads read less but leave the latency bare: 3.1 us for a
 // CTA alone.  64 blocks of 448 -> 1792 at rank 10 with both products (7840 k-blocks of
 // tiles) 64 -> 58 us, 48 rows of 2880 -> 960 at order 16 (2700) 140 -> 25.
-#include <atomic>
-
 #include "lbp_internal.h"
 #include "ptx_sm100.cuh"
 
@@ -241,14 +239,8 @@ int launch_gemm_fp32(const GemmFp32* job, int n, float* ws, size_t ws_bytes, cud
     if (i == 0) js.items0 = static_cast<int32_t>(items);
   }
   js.per = static_cast<int32_t>(per);
-  int dev = 0;
-  LBP_CUDA_TRY(cudaGetDevice(&dev));
-  static std::atomic<uint64_t> configured{0};
-  const uint64_t bit = 1ull << (dev & 63);
-  if (dev > 63 || (configured.load(std::memory_order_relaxed) & bit) == 0) {
-    LBP_CUDA_TRY(cudaFuncSetAttribute(gemm_fp32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-    configured.fetch_or(bit, std::memory_order_relaxed);
-  }
+  static PerDevice configured;
+  if (int e = allow_dynamic_smem(configured, reinterpret_cast<const void*>(gemm_fp32_kernel), kSmemBytes)) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -45,8 +45,8 @@ using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t
 // The driver entry point is resolved at run time so that the library loads
 // (for its host-only functions) on machines without a CUDA driver.
 static int get_encode_fn(EncodeTiledFn* out) {
-  static EncodeTiledFn cached = nullptr;
-  if (cached == nullptr) {
+  static std::atomic<EncodeTiledFn> cached{nullptr};
+  if (cached.load(std::memory_order_relaxed) == nullptr) {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult qres;
     LBP_CUDA_TRY(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
@@ -55,9 +55,9 @@ static int get_encode_fn(EncodeTiledFn* out) {
       set_last_cuda_error(cudaErrorNotSupported);
       return LBP_ERR_CUDA;
     }
-    cached = reinterpret_cast<EncodeTiledFn>(fn);
+    cached.store(reinterpret_cast<EncodeTiledFn>(fn), std::memory_order_relaxed);
   }
-  *out = cached;
+  *out = cached.load(std::memory_order_relaxed);
   return LBP_OK;
 }
 
@@ -630,6 +630,16 @@ int lbp_test_side_section(int device, int (*inside)(void*), void* arg) {
   if (device < 0 || device >= 64 || inside == nullptr) return LBP_ERR_SHAPE;
   std::lock_guard<std::mutex> lock(side_section(device));
   return inside(arg);
+}
+
+int lbp_test_per_device(const int* devices, int n, uint8_t* done) {
+  if (devices == nullptr || done == nullptr) return LBP_ERR_NULL;
+  PerDevice once;
+  for (int i = 0; i < n; ++i) {
+    done[i] = 0;
+    if (int e = once(devices[i], [&] { return done[i] = 1, LBP_OK; })) return e;
+  }
+  return LBP_OK;
 }
 
 int lbp_test_reload_env(void) {

@@ -39,7 +39,6 @@
 // reported through the status block.
 #include <cuda_bf16.h>
 
-#include <atomic>
 #include <cstdio>
 #include <cstdlib>
 
@@ -674,16 +673,11 @@ struct ProductsCall {
 };
 
 template <int K, int CORE, bool PAIR>
-static int launch_kernel(const cudaLaunchConfig_t& cfg, int dev, const fused::OperandMaps& tm,
-                         const fused::StoreMaps& sm, const FusedParams& p, const FusedBasis& fb,
-                         const FusedSchedule& sc) {
+static int launch_kernel(const cudaLaunchConfig_t& cfg, const fused::OperandMaps& tm, const fused::StoreMaps& sm,
+                         const FusedParams& p, const FusedBasis& fb, const FusedSchedule& sc) {
   auto kern = fused::lbp_products_kernel<K, CORE, PAIR>;
-  static std::atomic<uint64_t> configured{0};   // one bit per device
-  const uint64_t bit = 1ull << (dev & 63);
-  if (dev > 63 || (configured.load(std::memory_order_relaxed) & bit) == 0) {
-    LBP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, fused::kSmemBytes));
-    configured.fetch_or(bit, std::memory_order_relaxed);
-  }
+  static PerDevice configured;
+  if (int e = allow_dynamic_smem(configured, reinterpret_cast<const void*>(kern), fused::kSmemBytes)) return e;
   LBP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, tm, sm, p, fb, sc));
   count_launch();
   return LBP_OK;
@@ -799,8 +793,8 @@ static int launch_products(const ProductsCall& c, cudaStream_t stream) {
   int e = LBP_ERR_BASIS;
 #define LBP_CASE(KK, CC)                                                                          \
   case KK * 100 + CC:                                                                             \
-    e = pair ? launch_kernel<KK, CC, true>(cfg, dev, tm, sm, p, c.fb, plan.sched)                 \
-             : launch_kernel<KK, CC, false>(cfg, dev, tm, sm, p, c.fb, plan.sched);               \
+    e = pair ? launch_kernel<KK, CC, true>(cfg, tm, sm, p, c.fb, plan.sched)                      \
+             : launch_kernel<KK, CC, false>(cfg, tm, sm, p, c.fb, plan.sched);                    \
     break
   switch (K * 100 + c.core) {
     LBP_CASE(4, 2);

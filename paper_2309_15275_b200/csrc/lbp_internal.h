@@ -7,6 +7,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "lbp.h"
 
 namespace lbp {
@@ -69,6 +71,32 @@ void note_cuda_failure(cudaError_t e, const char* file, int line);   // LBP_VERB
       return LBP_ERR_CUDA;                                 \
     }                                                      \
   } while (0)
+
+// What is to be done once on each device, from whichever thread comes first (twice when two
+// come at the same time, so it must bear that); on devices past the 63rd every time.
+class PerDevice {
+ public:
+  template <class Action>
+  int operator()(int dev, Action action) {
+    const uint64_t bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;
+    if ((done_.load(std::memory_order_relaxed) & bit) != 0) return LBP_OK;
+    if (int e = action()) return e;
+    done_.fetch_or(bit, std::memory_order_relaxed);
+    return LBP_OK;
+  }
+
+ private:
+  std::atomic<uint64_t> done_{0};
+};
+// The opt-in to more than 48 KB of dynamic shared memory is a kernel's on one device.
+inline int allow_dynamic_smem(PerDevice& per_device, const void* kernel, int bytes) {
+  int dev = 0;
+  LBP_CUDA_TRY(cudaGetDevice(&dev));
+  return per_device(dev, [&]() -> int {
+    LBP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    return LBP_OK;
+  });
+}
 
 // ---- tensor maps (TMA descriptors), encoded on the host ------------------
 // 4-D channels-last tensor (B, H, W, C): box = one k x k block x box_c

@@ -202,14 +202,8 @@ static int launch_one(const CUtensorMap* tmaps, T* out0, T* out1, const ProjPara
                       const DevicePlan& plan, int sms, cudaStream_t stream) {
   using Cfg = ProjCfg<K, sizeof(T) == 2>;
   auto kern = wht_project_kernel<T, K, LB>;
-  static bool configured[64] = {};
-  int dev = 0;
-  LBP_CUDA_TRY(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64 || !configured[dev]) {
-    LBP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      Cfg::kSmemBytes));
-    if (dev >= 0 && dev < 64) configured[dev] = true;
-  }
+  static PerDevice configured;
+  if (int e = allow_dynamic_smem(configured, reinterpret_cast<const void*>(kern), Cfg::kSmemBytes)) return e;
   const uint32_t want = (p.n_items + Cfg::kWarps - 1) / Cfg::kWarps;
   const int grid = static_cast<int>(want < static_cast<uint32_t>(sms) ? want : sms);
   kern<<<grid, Cfg::kWarps * 32, Cfg::kSmemBytes, stream>>>(tmaps[0], tmaps[1], out0, out1, p, plan);

@@ -36,8 +36,6 @@
 // the exit.
 #include <cuda_bf16.h>
 
-#include <atomic>
-
 #include "lbp_internal.h"
 #include "ptx_sm100.cuh"
 #include "wht_device.cuh"
@@ -542,19 +540,13 @@ int launch_project_umma(const void* t0, void* out0, int C0, const lbp_view* view
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = stream;
   cfg.attrs = attr;
-  int dev = 0;
-  LBP_CUDA_TRY(cudaGetDevice(&dev));
-  auto launch = [&](auto kern, std::atomic<uint64_t>& configured) -> int {
-    const uint64_t bit = 1ull << (dev & 63);
-    if (dev > 63 || (configured.load(std::memory_order_relaxed) & bit) == 0) {
-      LBP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
-      configured.fetch_or(bit, std::memory_order_relaxed);
-    }
+  auto launch = [&](auto kern, PerDevice& configured) -> int {
+    if (int e = allow_dynamic_smem(configured, reinterpret_cast<const void*>(kern), kSmemMax)) return e;
     LBP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, in[0], in[1], om, p, mp));
     count_launch();
     return LBP_OK;
   };
-  static std::atomic<uint64_t> configured[3][4];
+  static PerDevice configured[3][4];
 #define LBP_CASE(KK, NB) \
   case KK * 10 + NB: return launch(wht_project_umma_kernel<KK, NB>, configured[KK / 8][NB - 1])
   switch (K * 10 + nb) {

@@ -12,9 +12,6 @@
 // per-thread sums; nothing but the k*k energies is written.
 #include <cuda_bf16.h>
 
-#include <atomic>
-
-
 #include "lbp_internal.h"
 #include "ptx_sm100.cuh"
 #include "wht_device.cuh"
@@ -325,14 +322,8 @@ static int launch_zero_energy(double* energy, int n, cudaStream_t stream) {
 // A launch that may start while the kernel ahead of it on the stream still runs.
 template <class... Params, class... Args>
 static int launch_behind(void (*kern)(Params...), int grid, int threads, int smem, cudaStream_t stream,
-                         std::atomic<uint64_t>& configured, const Args&... args) {
-  int dev = 0;
-  LBP_CUDA_TRY(cudaGetDevice(&dev));
-  const uint64_t bit = 1ull << (dev & 63);
-  if (dev > 63 || (configured.load(std::memory_order_relaxed) & bit) == 0) {
-    LBP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    configured.fetch_or(bit, std::memory_order_relaxed);
-  }
+                         PerDevice& configured, const Args&... args) {
+  if (int e = allow_dynamic_smem(configured, reinterpret_cast<const void*>(kern), smem)) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -356,7 +347,7 @@ template <int K>
 static int launch_spectrum_mma_k(const CUtensorMap& tmap, const ProjParams& p, const MmaPlan& mp,
                                  double* energy, int sms, cudaStream_t stream) {
   using Cfg = MmaCfg<K>;
-  static std::atomic<uint64_t> configured{0};
+  static PerDevice configured;
   const uint32_t want = (p.n_items + Cfg::kWarps - 1) / Cfg::kWarps;
   const int grid = static_cast<int>(want < static_cast<uint32_t>(sms) ? want : sms);
   return launch_behind(wht_spectrum_mma_kernel<K>, grid, Cfg::kWarps * 32, Cfg::kSmemBytes, stream, configured,
@@ -394,7 +385,7 @@ int launch_spectrum_mma(const void* t, int B, int H, int W, int C, const BasisPl
     Seq16 sq;
     for (int sidx = 0; sidx < 16; ++sidx) sq.seq_of_nat[walsh_natural_index(16, sidx)] = static_cast<uint8_t>(sidx);
     using Cfg = MmaCfg<16>;
-    static std::atomic<uint64_t> configured{0};
+    static PerDevice configured;
     const uint32_t want = (p.n_items + Cfg::kWarps - 1) / Cfg::kWarps;
     const int grid = static_cast<int>(want < static_cast<uint32_t>(sms) ? want : sms);
     return launch_behind(wht_spectrum16_kernel, grid, Cfg::kWarps * 32, Cfg::kSmemBytes, stream, configured, tmap, p,

@@ -278,3 +278,16 @@ def test_batch_section_admits_one_thread_per_device():
     for t in threads:
         t.join()
     assert most == [1, 1]
+
+
+def test_kernel_attributes_are_set_on_every_device():
+    import glob
+    import os
+    # the one place that sets them remembers the devices one by one
+    devices = [0, 0, 1, 1, 0, 63, 63, 70, 70]
+    done = (ctypes.c_uint8 * len(devices))()
+    assert lbp.binding._lib().lbp_test_per_device((ctypes.c_int * len(devices))(*devices), len(devices), done) == 0
+    assert list(done) == [1, 0, 1, 0, 0, 1, 0, 1, 1]
+    csrc = os.path.join(os.path.dirname(lbp.__file__), "csrc")
+    sites = [f for f in glob.glob(os.path.join(csrc, "*")) for _ in range(open(f).read().count("cudaFuncSetAttribute("))]
+    assert [os.path.basename(f) for f in sites] == ["lbp_internal.h"]
