@@ -124,9 +124,10 @@ int lbp_last_cuda_error(void);
 
 /* ---- device entry points ------------------------------------------------- */
 
-/* Bytes of scratch the calls below need for this layer at rank r (Algorithm 1
+/* Bytes of scratch the calls on x below need for this layer at rank r (Algorithm 1
  * materialises x_hat and g_y_hat; the status word lives there too).  Returns 0
- * for an invalid layer.  lbp_project / lbp_expand need lbp_status_bytes(). */
+ * for an invalid layer.  lbp_project / lbp_expand need lbp_status_bytes(); calls on
+ * x_hat: lbp_workspace_bytes_projected. */
 size_t lbp_workspace_bytes(const lbp_layer* layer, int r);
 size_t lbp_status_bytes(void);
 
@@ -249,8 +250,12 @@ typedef struct {
   int32_t g_bias_dtype;
 } lbp_extras;
 
-/* Scratch for lbp_backward_ex (>= lbp_workspace_bytes; 0 = invalid arguments). */
+/* Scratch for lbp_backward_ex on x (>= lbp_workspace_bytes; 0 = invalid arguments). */
 size_t lbp_workspace_bytes_ex(const lbp_layer* layer, int r, const lbp_extras* ex);
+/* Scratch for lbp_backward_ex and lbp_backward_projected on x_hat (ex may be NULL; 0 =
+ * invalid arguments).  It differs from the above at r = k*k only: there a call on x is
+ * Eq. 2 and needs no coefficients, one on x_hat works on them as at any other rank. */
+size_t lbp_workspace_bytes_projected(const lbp_layer* layer, int r, const lbp_extras* ex);
 
 /* Algorithm 1 with the parts above.  Exactly one of x and x_hat is given:
  *  - x (B,H,W,Cin): as lbp_backward;
@@ -260,14 +265,15 @@ size_t lbp_workspace_bytes_ex(const lbp_layer* layer, int r, const lbp_extras* e
  *    at its second step (g_y_hat = p(g_y)).  The result equals lbp_backward on
  *    x up to the rounding of x_hat to `dtype` that both take.
  * ex may be NULL (then this is lbp_backward / lbp_backward_projected).
- * ws: >= lbp_workspace_bytes_ex(layer, r, ex). */
+ * ws: >= lbp_workspace_bytes_ex(layer, r, ex), on x_hat lbp_workspace_bytes_projected. */
 int lbp_backward_ex(const void* x, const void* x_hat, const void* g_y, const void* W,
                     void* g_x, void* g_W, const lbp_layer* layer,
                     const lbp_basis* set, int r, const lbp_extras* ex,
                     void* ws, size_t ws_bytes, void* stream);
 
 /* Algorithm 1 from its second step on (Eq. 3 applied to x beforehand):
- * lbp_backward_ex with x = NULL and no extras.  ws: >= lbp_workspace_bytes. */
+ * lbp_backward_ex with x = NULL and no extras.
+ * ws: >= lbp_workspace_bytes_projected(layer, r, NULL). */
 int lbp_backward_projected(const void* x_hat, const void* g_y, const void* W,
                            void* g_x, void* g_W, const lbp_layer* layer,
                            const lbp_basis* set, int r,

@@ -95,8 +95,10 @@ def _lib() -> C.CDLL:
         lib.lbp_backward.argtypes = [vp, vp, vp, vp, vp, C.POINTER(Layer), C.POINTER(Basis), i32,
                                      vp, sz, vp]
         lib.lbp_backward.restype = i32
-        lib.lbp_workspace_bytes_ex.argtypes = [C.POINTER(Layer), i32, C.POINTER(Extras)]
-        lib.lbp_workspace_bytes_ex.restype = sz
+        for name in ("lbp_workspace_bytes_ex", "lbp_workspace_bytes_projected"):
+            f = getattr(lib, name)
+            f.argtypes = [C.POINTER(Layer), i32, C.POINTER(Extras)]
+            f.restype = sz
         lib.lbp_backward_ex.argtypes = [vp, vp, vp, vp, vp, vp, C.POINTER(Layer), C.POINTER(Basis),
                                         i32, C.POINTER(Extras), vp, sz, vp]
         lib.lbp_backward_ex.restype = i32
@@ -169,7 +171,7 @@ EXPORTED = ("lbp_select_bases", "lbp_basis_matrix", "lbp_flops", "lbp_status_str
             "lbp_backward_static", "lbp_launch_count", "lbp_set_phase_events", "lbp_phase_count",
             "lbp_phase_name", "lbp_select_lhe", "lbp_spectrum_workspace_bytes", "lbp_spectrum",
             "lbp_backward_batch", "lbp_test_stall_products",
-            "lbp_test_reload_env", "lbp_workspace_bytes_ex", "lbp_backward_ex",
+            "lbp_test_reload_env", "lbp_workspace_bytes_ex", "lbp_workspace_bytes_projected", "lbp_backward_ex",
             "lbp_backward_projected", "lbp_test_tile_plan", "lbp_test_struct_size",
             "lbp_test_side_section", "lbp_test_per_device")
 
@@ -271,9 +273,19 @@ def _layer(B, H, W, Cin, Cout, k, dtype, gw_dtype) -> Layer:
     return Layer(B, H, W, Cin, Cout, k, dtype, gw_dtype)
 
 
-def lbp_workspace_bytes(B, H, W, Cin, Cout, k, dtype: int, gw_dtype: int, r: int) -> int:
-    lay = _layer(B, H, W, Cin, Cout, k, dtype, gw_dtype)
-    return int(_lib().lbp_workspace_bytes(C.byref(lay), r))
+def _workspace_bytes(lay: Layer, r: int, ex: Extras | None, x_hat: bool | None) -> int:
+    on = lambda f: int(f(C.byref(lay), r, None if ex is None else C.byref(ex)))  # noqa: E731
+    lib = _lib()
+    if x_hat is None:
+        return max(on(lib.lbp_workspace_bytes_ex), on(lib.lbp_workspace_bytes_projected))
+    return on(lib.lbp_workspace_bytes_projected if x_hat else lib.lbp_workspace_bytes_ex)
+
+
+def lbp_workspace_bytes(B, H, W, Cin, Cout, k, dtype: int, gw_dtype: int, r: int,
+                        x_hat: bool | None = None) -> int:
+    """Scratch of a call on x (x_hat=False), on x_hat (True), or enough for either (None).
+    At r = k*k, and only there, a call on x needs much less."""
+    return _workspace_bytes(_layer(B, H, W, Cin, Cout, k, dtype, gw_dtype), r, None, x_hat)
 
 
 # ---------------------------------------------------------- device calls ----
@@ -356,9 +368,10 @@ def lbp_expand(t_hat: torch.Tensor, k: int, bases, out: torch.Tensor | None = No
 
 def alloc_workspace(x: torch.Tensor, g_y: torch.Tensor, k: int, r: int,
                     gw_dtype: torch.dtype = torch.float32) -> torch.Tensor:
+    """A workspace for calls on x."""
     B, H, W, Cin = x.shape
     n = lbp_workspace_bytes(B, H, W, Cin, g_y.shape[-1], k, _dtype_code(x.dtype),
-                            _dtype_code(gw_dtype), r)
+                            _dtype_code(gw_dtype), r, x_hat=False)
     if n == 0:
         raise ValueError("invalid layer for lbp_workspace_bytes")
     return torch.empty(n, dtype=torch.uint8, device=x.device)
@@ -448,9 +461,10 @@ def _extras(g_y, Cin, beta, g_bias, x_extra, gy_extra, gx_extra):
 
 def lbp_workspace_bytes_ex(B, H, W, Cin, Cout, k, dtype: int, gw_dtype: int, r: int, *, beta=0.0,
                            bias=False, n_extra=0, x_view=None, gy_view=None, gx_view=None,
-                           extra_pitches=None) -> int:
+                           extra_pitches=None, x_hat: bool | None = None) -> int:
     """Scratch of lbp_backward_ex.  Views are (image, row, token) element strides,
-    extra_pitches the (x, g_y, g_x) row pitches of the extra tokens."""
+    extra_pitches the (x, g_y, g_x) row pitches of the extra tokens; x_hat as in
+    lbp_workspace_bytes."""
     lay = _layer(B, H, W, Cin, Cout, k, dtype, gw_dtype)
     ex = Extras()
     ex.beta, ex.n_extra = float(beta), 0
@@ -463,7 +477,7 @@ def lbp_workspace_bytes_ex(B, H, W, Cin, Cout, k, dtype: int, gw_dtype: int, r: 
     for name, v in (("x_view", x_view), ("gy_view", gy_view), ("gx_view", gx_view)):
         if v is not None:
             setattr(ex, name, View(*[int(a) for a in v]))
-    return int(_lib().lbp_workspace_bytes_ex(C.byref(lay), r, C.byref(ex)))
+    return _workspace_bytes(lay, r, ex, x_hat)
 
 
 def lbp_backward_ex(x, g_y, W, k: int, bases, *, x_hat=None, beta: float = 0.0, g_bias=None,
@@ -501,7 +515,7 @@ def lbp_backward_ex(x, g_y, W, k: int, bases, *, x_hat=None, beta: float = 0.0, 
     ex.gx_view = View(*v)
     lay = _layer(B, H, Wd, Cin, Cout, k, _dtype_code(g_y.dtype), _dtype_code(g_W.dtype))
     if ws is None:
-        n = int(_lib().lbp_workspace_bytes_ex(C.byref(lay), r, C.byref(ex)))
+        n = _workspace_bytes(lay, r, ex, x_hat is not None)
         if n == 0:
             raise ValueError("invalid layer, strides or extras for lbp_workspace_bytes_ex")
         ws = torch.empty(n, dtype=torch.uint8, device=g_y.device)
@@ -527,9 +541,9 @@ def lbp_backward_projected(x_hat, g_y, W, k: int, bases, *, gw_dtype: torch.dtyp
         g_W = torch.empty((Cout, Cin), dtype=gw_dtype, device=g_y.device)
     lay = _layer(B, H, Wd, Cin, Cout, k, _dtype_code(g_y.dtype), _dtype_code(g_W.dtype))
     if ws is None:
-        n = int(_lib().lbp_workspace_bytes(C.byref(lay), r))
+        n = _workspace_bytes(lay, r, None, True)
         if n == 0:
-            raise ValueError("invalid layer for lbp_workspace_bytes")
+            raise ValueError("invalid layer for lbp_workspace_bytes_projected")
         ws = torch.empty(n, dtype=torch.uint8, device=g_y.device)
     _check(_lib().lbp_backward_projected(_dev(x_hat, "x_hat"), _dev(g_y, "g_y"), _dev(W, "W"),
                                          _dev(g_x, "g_x"), _dev(g_W, "g_W"), C.byref(lay),

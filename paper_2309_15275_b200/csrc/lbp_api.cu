@@ -287,8 +287,7 @@ extern "C" {
 size_t lbp_workspace_bytes(const lbp_layer* layer, int r) {
   if (check_layer(layer) != LBP_OK) return 0;
   if (r < 1 || r > layer->k * layer->k) return 0;
-  const size_t from_x = plan_layout(*layer, r, false).total, from_coef = plan_layout(*layer, r, true).total;
-  return from_x > from_coef ? from_x : from_coef;
+  return plan_layout(*layer, r, false).total;
 }
 
 int lbp_project(const void* t, void* t_hat, int B, int H, int W, int C, int k,
@@ -908,6 +907,18 @@ static int check_extras(const lbp_extras* ex, const lbp_layer* L) {
   return LBP_OK;
 }
 
+// Scratch of a call with these extras on top of the layout of the call without.
+static size_t total_with_extras(const lbp_layer& L, const Layout& lay, int r, const lbp_extras* ex) {
+  if (ex == nullptr) return lay.total;
+  const bool strided = !is_dense(&ex->x_view) || !is_dense(&ex->gy_view) || !is_dense(&ex->gx_view);
+  if (ex->beta == 0.f && ex->n_extra == 0 && ex->g_bias == nullptr && !strided) return lay.total;
+  return plan_extras(L, lay.total, r, ex).total;
+}
+static size_t bytes_of_call(const lbp_layer* L, int r, const lbp_extras* ex, bool from_coef) {
+  if (check_extras(ex, L) != LBP_OK) return 0;
+  return total_with_extras(*L, plan_layout(*L, r, from_coef), r, ex);
+}
+
 // lbp_backward_ex after validation.
 static int run_backward_ex(const void* x, const void* x_hat, const void* g_y, const void* W,
                            void* g_x, void* g_W, const lbp_layer& L, const BasisPlan& plan,
@@ -1033,12 +1044,11 @@ int lbp_backward(const void* x, const void* g_y, const void* W, void* g_x, void*
 }
 
 size_t lbp_workspace_bytes_ex(const lbp_layer* layer, int r, const lbp_extras* ex) {
-  const size_t base = lbp_workspace_bytes(layer, r);
-  if (base == 0 || check_extras(ex, layer) != LBP_OK) return 0;
-  if (ex == nullptr) return base;
-  const bool strided = !is_dense(&ex->x_view) || !is_dense(&ex->gy_view) || !is_dense(&ex->gx_view);
-  if (ex->beta == 0.f && ex->n_extra == 0 && ex->g_bias == nullptr && !strided) return base;
-  return plan_extras(*layer, base, r, ex).total;
+  return lbp_workspace_bytes(layer, r) == 0 ? 0 : lbp::bytes_of_call(layer, r, ex, false);
+}
+
+size_t lbp_workspace_bytes_projected(const lbp_layer* layer, int r, const lbp_extras* ex) {
+  return lbp_workspace_bytes(layer, r) == 0 ? 0 : lbp::bytes_of_call(layer, r, ex, true);
 }
 
 int lbp_backward_ex(const void* x, const void* x_hat, const void* g_y, const void* W, void* g_x,
@@ -1051,7 +1061,14 @@ int lbp_backward_ex(const void* x, const void* x_hat, const void* g_y, const voi
   if (int e = validate_backward(xin, g_y, W, g_x, g_W, layer, set, r, ws, ws_bytes, &plan, &lay, x_hat != nullptr))
     return e;
   if (int e = check_extras(ex, layer)) return e;
-  if (ws_bytes < lbp_workspace_bytes_ex(layer, r, ex)) return LBP_ERR_WORKSPACE;
+  // the K slices of the fp32 products make do with what there is behind the rest
+  const size_t need = total_with_extras(*layer, lay, r, ex);
+  if (ws_bytes < need) {
+    const size_t over = align_up(need - ws_bytes, 1024);
+    if (layer->dtype != LBP_F32 || over > lay.splitk_bytes) return LBP_ERR_WORKSPACE;
+    lay.splitk_bytes -= over;
+    lay.total -= over;
+  }
   if (int e = check_device_arch()) return e;
   return run_backward_ex(x, x_hat, g_y, W, g_x, g_W, *layer, plan, lay, ex,
                          static_cast<uint8_t*>(ws), static_cast<cudaStream_t>(stream));

@@ -39,6 +39,7 @@ struct Library {
   decltype(&lbp_status_bytes) status_bytes;
   decltype(&lbp_workspace_bytes) workspace_bytes;
   decltype(&lbp_workspace_bytes_ex) workspace_bytes_ex;
+  decltype(&lbp_workspace_bytes_projected) workspace_bytes_projected;
   decltype(&lbp_spectrum_workspace_bytes) spectrum_workspace_bytes;
   decltype(&lbp_project) project;
   decltype(&lbp_spectrum) spectrum;
@@ -336,7 +337,7 @@ int run_ex(ExCall* c, const lbp_basis* set, int r) {
       !view_of(c->g_x, dev, &ex.gx_view))
     return -1;
   if (!c->ws.defined()) {
-    const size_t bytes = lib.workspace_bytes_ex(&L, r, &ex);
+    const size_t bytes = (c->x_hat.defined() ? lib.workspace_bytes_projected : lib.workspace_bytes_ex)(&L, r, &ex);
     if (bytes == 0) return -1;
     c->ws = bytes_on(c->g_y, bytes);
   }
@@ -597,6 +598,7 @@ PyObject* py_load(PyObject*, PyObject* args) {
                   resolve(h, "lbp_status_bytes", &lib.status_bytes) &&
                   resolve(h, "lbp_workspace_bytes", &lib.workspace_bytes) &&
                   resolve(h, "lbp_workspace_bytes_ex", &lib.workspace_bytes_ex) &&
+                  resolve(h, "lbp_workspace_bytes_projected", &lib.workspace_bytes_projected) &&
                   resolve(h, "lbp_spectrum_workspace_bytes", &lib.spectrum_workspace_bytes) &&
                   resolve(h, "lbp_project", &lib.project) && resolve(h, "lbp_spectrum", &lib.spectrum) &&
                   resolve(h, "lbp_backward", &lib.backward) && resolve(h, "lbp_backward_ex", &lib.backward_ex) &&

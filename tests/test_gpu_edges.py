@@ -345,3 +345,26 @@ def test_batch_call_beside_the_capture_of_another(dev):
         assert all(torch.equal(g, v) for g, v in zip(s["g_xs"], w[:n]))
         # other K slices of g_W on one stream: fp32 sums in another order
         assert all(rel(g, f64(v)) <= F32 for g, v in zip(s["g_Ws"], w[n:]))
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_each_call_asks_for_the_workspace_it_needs(dev, dtype):
+    # r = k*k: a call on x runs in the room of Eq. 2, one on x_hat wants that of its coefficients;
+    # fp32: with no room for K slices at all as well
+    B, H, ci, co, k = 4, 16, 64, 96, 4
+    x, gy, w = layer(dev, 191, B, H, H, ci, co, dtype=dtype)
+    bases = lbp.lbp_select_bases(k, lbp.SEL_LINF, k)
+    code = lbp.LBP_BF16 if dtype == torch.bfloat16 else lbp.LBP_F32
+    size = lambda form, **kw: lbp.lbp_workspace_bytes_ex(B, H, H, ci, co, k, code, lbp.LBP_F32, k * k,  # noqa: E731
+                                                         bias=True, x_hat=form)
+    ox, ow = O.backward_exact(f64(x), f64(gy), f64(w))
+    for n in [size(False)] + ([256 + 2 * 4 * ci * co + 4096] if dtype == torch.float32 else []):
+        ws, g_b = torch.empty(n, dtype=torch.uint8, device=dev), torch.empty(co, device=dev)
+        gx, gw = lbp.lbp_backward_ex(x, gy, w, k, bases, g_bias=g_b, ws=ws)
+        assert rel(gx, ox) <= BF16 and rel(gw, ow) <= F32 and rel(g_b, O.bias_grad(f64(gy))) <= F32
+        with pytest.raises(lbp.LbpError) as err:
+            lbp.lbp_backward_ex(None, gy, w, k, bases, x_hat=lbp.lbp_project(x, k, bases), g_bias=g_b, ws=ws)
+        assert err.value.status == 7
+    ws = torch.empty(size(True), dtype=torch.uint8, device=dev)
+    gx, gw = lbp.lbp_backward_ex(None, gy, w, k, bases, x_hat=lbp.lbp_project(x, k, bases), g_bias=g_b, ws=ws)
+    assert rel(gx, ox) <= BF16 and rel(gw, ow) <= BF16

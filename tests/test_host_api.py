@@ -291,3 +291,20 @@ def test_kernel_attributes_are_set_on_every_device():
     csrc = os.path.join(os.path.dirname(lbp.__file__), "csrc")
     sites = [f for f in glob.glob(os.path.join(csrc, "*")) for _ in range(open(f).read().count("cudaFuncSetAttribute("))]
     assert [os.path.basename(f) for f in sites] == ["lbp_internal.h"]
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+@pytest.mark.parametrize("ci,co,k,B,H", [(768, 3072, 8, 128, 16), (1024, 4096, 4, 128, 32), (64, 96, 4, 3, 9)])
+def test_exact_backpropagation_on_x_needs_no_room_for_coefficients(dtype, ci, co, k, B, H):
+    es = 2 if dtype == lbp.LBP_BF16 else 4
+    rows = B * (-(-H // k) * k) ** 2
+    size = lambda r, form: lbp.lbp_workspace_bytes(B, H, H, ci, co, k, dtype, lbp.LBP_F32, r, x_hat=form)  # noqa: E731
+    ex = lambda form, **kw: lbp.lbp_workspace_bytes_ex(B, H, H, ci, co, k, dtype, lbp.LBP_F32, k * k, x_hat=form, **kw)  # noqa: E731
+    # the status block and the fp32 planes of the K slices: 48 MiB for both at the most, beside g_W itself
+    assert 256 <= size(k * k, False) <= 1024 + max(48 << 20, 192 * ci * co * 4 // max(1, (ci // 64) * (co // 128)))
+    assert size(k * k, True) >= rows * (co * es + ci * 4)
+    assert size(k * k, None) == max(size(k * k, False), size(k * k, True))
+    assert size(2, False) == size(2, True) == size(2, None)
+    # with extras: the same room on top of either
+    assert ex(False, beta=1.0) - size(k * k, False) < 2 * ci * co * 4 + 8192
+    assert ex(True, beta=1.0) - ex(False, beta=1.0) >= size(k * k, True) - size(k * k, False) - 4096
