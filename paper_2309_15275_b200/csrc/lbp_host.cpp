@@ -110,9 +110,7 @@ static bool prefix_less(const PairKey& a, const PairKey& b) {
 using namespace lbp;
 
 namespace lbp {
-static TuneOptions g_tune;
-static bool g_tune_loaded = false;
-void reload_tune_options() {
+static TuneOptions read_tune_options() {
   TuneOptions t{};
   const char* e = std::getenv("LBP_FUSED");
   t.fused = !(e != nullptr && e[0] == '0');
@@ -127,13 +125,14 @@ void reload_tune_options() {
                 std::sscanf(e, "%d,%d,%d", &t.tiles_bnw, &t.tiles_bnx, &t.tiles_splits) == 3;
   e = std::getenv("LBP_BATCH_PROJ_SMS");
   t.batch_proj_sms = e != nullptr ? std::atoi(e) : -1;
-  g_tune = t;
-  g_tune_loaded = true;
+  return t;
 }
-const TuneOptions& tune_options() {
-  if (!g_tune_loaded) reload_tune_options();
-  return g_tune;
+static TuneOptions& tune_options_slot() {
+  static TuneOptions options = read_tune_options();   // by whichever thread comes first
+  return options;
 }
+void reload_tune_options() { tune_options_slot() = read_tune_options(); }
+const TuneOptions& tune_options() { return tune_options_slot(); }
 }  // namespace lbp
 
 extern "C" {

@@ -166,6 +166,14 @@ PyObject* pair(const Tensor& a, const Tensor& b) {
 }
 PyObject* not_handled() { Py_RETURN_NONE; }
 
+// A call into the library: other Python threads run meanwhile (it may search a tile plan, wait
+// for the batch section of another thread, or for room in a full launch queue).
+template <class F>
+auto without_gil(F call) {
+  pybind11::gil_scoped_release no_gil;
+  return call();
+}
+
 // One problem's shapes, dtypes and devices, as binding._check_layer_tensors has them.
 struct Problem {
   lbp_layer L;
@@ -224,8 +232,10 @@ PyObject* py_project(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return not_handled();
   if (!ws.defined()) ws = bytes_on(t, lib.status_bytes());
   if (!dense_on(ws, dev)) return not_handled();
-  const int e = lib.project(t.data_ptr(), out.data_ptr(), t.size(0), t.size(1), t.size(2), t.size(3), k, b.v, b.r,
-                            dt, ws.data_ptr(), ws.numel(), current_stream(dev));
+  const int e = without_gil([&] {
+    return lib.project(t.data_ptr(), out.data_ptr(), t.size(0), t.size(1), t.size(2), t.size(3), k, b.v, b.r, dt,
+                       ws.data_ptr(), ws.numel(), current_stream(dev));
+  });
   return e != LBP_OK ? PyLong_FromLong(e) : THPVariable_Wrap(out);
   END_HANDLE_TH_ERRORS
 }
@@ -252,8 +262,10 @@ PyObject* py_spectrum(PyObject*, PyObject* const* a, Py_ssize_t n) {
     ws = bytes_on(t, bytes);
   }
   if (!dense_on(ws, dev)) return not_handled();
-  const int e = lib.spectrum(t.data_ptr(), out.data_ptr<double>(), t.size(0), t.size(1), t.size(2), t.size(3), k,
-                             dt, ws.data_ptr(), ws.numel(), current_stream(dev));
+  const int e = without_gil([&] {
+    return lib.spectrum(t.data_ptr(), out.data_ptr<double>(), t.size(0), t.size(1), t.size(2), t.size(3), k, dt,
+                        ws.data_ptr(), ws.numel(), current_stream(dev));
+  });
   return e != LBP_OK ? PyLong_FromLong(e) : THPVariable_Wrap(out);
   END_HANDLE_TH_ERRORS
 }
@@ -279,12 +291,13 @@ PyObject* py_backward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     ws = bytes_on(g_y, bytes);
   }
   if (!dense_on(ws, dev)) return not_handled();
-  const int e =
-      a[4] == Py_None
-          ? lib.backward_fullrank(x.data_ptr(), g_y.data_ptr(), W.data_ptr(), g_x.data_ptr(), g_W.data_ptr(), &p.L,
-                                  ws.data_ptr(), ws.numel(), current_stream(dev))
-          : lib.backward(x.data_ptr(), g_y.data_ptr(), W.data_ptr(), g_x.data_ptr(), g_W.data_ptr(), &p.L, b.v, b.r,
-                         ws.data_ptr(), ws.numel(), current_stream(dev));
+  const bool exact = a[4] == Py_None;
+  const int e = without_gil([&] {
+    return exact ? lib.backward_fullrank(x.data_ptr(), g_y.data_ptr(), W.data_ptr(), g_x.data_ptr(), g_W.data_ptr(),
+                                         &p.L, ws.data_ptr(), ws.numel(), current_stream(dev))
+                 : lib.backward(x.data_ptr(), g_y.data_ptr(), W.data_ptr(), g_x.data_ptr(), g_W.data_ptr(), &p.L, b.v,
+                                b.r, ws.data_ptr(), ws.numel(), current_stream(dev));
+  });
   return e != LBP_OK ? PyLong_FromLong(e) : pair(g_x, g_W);
   END_HANDLE_TH_ERRORS
 }
@@ -361,7 +374,7 @@ PyObject* py_backward_ex(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return not_handled();
   c.beta = PyFloat_AS_DOUBLE(a[6]);
   c.gw_code = parse_dtype(a[11]);
-  const int e = run_ex(&c, b.v, b.r);
+  const int e = without_gil([&] { return run_ex(&c, b.v, b.r); });
   if (e < 0) return not_handled();
   return e != LBP_OK ? PyLong_FromLong(e) : pair(c.g_x, c.g_W);
   END_HANDLE_TH_ERRORS
@@ -382,6 +395,8 @@ PyObject* py_backward_batch(PyObject*, PyObject* const* a, Py_ssize_t n) {
     count = m;
   }
   if (count < 1 || count > 64) return not_handled();
+  std::vector<Tensor> held;   // the lists are the caller's to change once the lock is released
+  held.reserve(6 * count);
   void* ptr[6][64];
   lbp_layer layers[64];
   size_t sizes[64];
@@ -397,12 +412,15 @@ PyObject* py_backward_batch(PyObject*, PyObject* const* a, Py_ssize_t n) {
     for (int l = 0; l < 6; ++l) {
       if (!dense_on(t[l], dev)) return not_handled();
       ptr[l][i] = t[l].data_ptr();
+      held.push_back(t[l]);
     }
     layers[i] = p.L;
     sizes[i] = static_cast<size_t>(t[5].numel());
   }
-  const int e = lib.backward_batch(static_cast<int>(count), ptr[0], ptr[1], ptr[2], ptr[3], ptr[4], layers, b.v, b.r,
-                                   ptr[5], sizes, nullptr, current_stream(dev));
+  const int e = without_gil([&] {
+    return lib.backward_batch(static_cast<int>(count), ptr[0], ptr[1], ptr[2], ptr[3], ptr[4], layers, b.v, b.r, ptr[5],
+                              sizes, nullptr, current_stream(dev));
+  });
   return PyLong_FromLong(e);
   END_HANDLE_TH_ERRORS
 }

@@ -368,3 +368,28 @@ def test_each_call_asks_for_the_workspace_it_needs(dev, dtype):
     ws = torch.empty(size(True), dtype=torch.uint8, device=dev)
     gx, gw = lbp.lbp_backward_ex(None, gy, w, k, bases, x_hat=lbp.lbp_project(x, k, bases), g_bias=g_b, ws=ws)
     assert rel(gx, ox) <= BF16 and rel(gw, ow) <= BF16
+
+
+def test_other_threads_run_during_a_call(dev):
+    # a call that waits (here for the section of the side stream) does not hold the interpreter
+    a = batch_of(dev, 201, [(768, 768), (256, 1024)])
+    lbp.lbp_backward_batch(**a)
+    torch.cuda.synchronize()
+    usleep = ctypes.cast(ctypes.CDLL(None).usleep, ctypes.c_void_p)
+    held = threading.Thread(target=lambda: lbp.binding._lib().lbp_test_side_section(dev.index, usleep, 500000))
+    ticks, stop = [], threading.Event()
+
+    def tick():
+        while not stop.is_set():
+            ticks.append(time.perf_counter())
+            time.sleep(0.005)
+    ticker = threading.Thread(target=tick)
+    held.start(), ticker.start()
+    time.sleep(0.1)
+    t0 = time.perf_counter()
+    lbp.lbp_backward_batch(**a)
+    t1 = time.perf_counter()
+    stop.set()
+    held.join(), ticker.join()
+    assert t1 - t0 > 0.1
+    assert sum(t0 < t < t1 - 0.05 for t in ticks) >= 5
