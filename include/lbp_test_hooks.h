@@ -38,6 +38,14 @@ int lbp_test_stall_products(int on);
 int lbp_test_tile_plan(int Cin, int Cout, int G, int bpt, int k, int units, int pair,
                        int max_splits, int epi_kind, int32_t* out6, uint16_t* first, uint16_t* ids);
 
+/* The plan that a call with this bf16 layer, basis list and number of tokens outside the
+ * grid runs on `units` CTAs (pair = 0) or CTA pairs (1); set = NULL: exact backpropagation
+ * of the whole grid.  out8 = {BNw, BNx, blocks of a GX tile, K slices of g_W, k-blocks of a
+ * slice, listed, k-blocks of g_W, K slices there is room for}; first and ids as above (where
+ * listed).  No device needed. */
+int lbp_test_products_plan(const lbp_layer* layer, const lbp_basis* set, int r, int n_extra, int units, int pair,
+                           int32_t* out8, uint16_t* first, uint16_t* ids);
+
 /* The library reads its tuning switches (LBP_FUSED, LBP_PAIR, LBP_FUSED_TILES,
  * LBP_FUSED_VERBOSE) from the environment once, at first use.  This reads them
  * again, so that one test process can run the same layer through the paths

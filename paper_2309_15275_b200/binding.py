@@ -120,6 +120,10 @@ def _lib() -> C.CDLL:
         lib.lbp_test_tile_plan.argtypes = [i32] * 9 + [C.POINTER(C.c_int32), C.POINTER(C.c_uint16),
                                                        C.POINTER(C.c_uint16)]
         lib.lbp_test_tile_plan.restype = i32
+        lib.lbp_test_products_plan.argtypes = [C.POINTER(Layer), C.POINTER(Basis), i32, i32, i32, i32,
+                                               C.POINTER(C.c_int32), C.POINTER(C.c_uint16),
+                                               C.POINTER(C.c_uint16)]
+        lib.lbp_test_products_plan.restype = i32
         lib.lbp_test_reload_env.argtypes = []
         lib.lbp_test_reload_env.restype = i32
         lib.lbp_test_struct_size.argtypes = [i32]
@@ -173,7 +177,7 @@ EXPORTED = ("lbp_select_bases", "lbp_basis_matrix", "lbp_flops", "lbp_status_str
             "lbp_backward_batch", "lbp_test_stall_products",
             "lbp_test_reload_env", "lbp_workspace_bytes_ex", "lbp_workspace_bytes_projected", "lbp_backward_ex",
             "lbp_backward_projected", "lbp_test_tile_plan", "lbp_test_struct_size",
-            "lbp_test_side_section", "lbp_test_per_device")
+            "lbp_test_side_section", "lbp_test_per_device", "lbp_test_products_plan")
 
 
 def _check(status: int, where: str) -> None:
@@ -645,6 +649,20 @@ def lbp_test_tile_plan(Cin, Cout, G, bpt, k, units, pair, max_splits=1, epi_kind
     _check(_lib().lbp_test_tile_plan(Cin, Cout, G, bpt, k, units, 1 if pair else 0, max_splits,
                                      epi_kind, out, first, ids), "lbp_test_tile_plan")
     info = {"BNw": out[0], "BNx": out[1], "splits": out[2], "kbps": out[3], "listed": bool(out[4])}
+    if not info["listed"]:
+        return info, None
+    return info, [[ids[j] for j in range(first[u], first[u + 1])] for u in range(units)]
+
+
+def lbp_test_products_plan(B, H, W, Cin, Cout, k, bases, *, n_extra=0, units=74, pair=True):
+    """Test hook: the tile plan of a call with this bf16 layer (bases None: exact).  Returns
+    (dict, list of per-unit tile-id lists or None when not listed)."""
+    out, first, ids = (C.c_int32 * 8)(), (C.c_uint16 * 161)(), (C.c_uint16 * 1536)()
+    lay = _layer(B, H, W, Cin, Cout, k, LBP_BF16, LBP_F32)
+    _check(_lib().lbp_test_products_plan(C.byref(lay), None if bases is None else _bases(bases),
+                                         0 if bases is None else len(bases), n_extra, units,
+                                         1 if pair else 0, out, first, ids), "lbp_test_products_plan")
+    info = dict(zip(("BNw", "BNx", "bpt", "splits", "kbps", "listed", "num_kb_w", "room"), out))
     if not info["listed"]:
         return info, None
     return info, [[ids[j] for j in range(first[u], first[u + 1])] for u in range(units)]

@@ -452,14 +452,14 @@ static int plan_batch(int n, const lbp_layer* layers, const lbp_basis* set, int 
   // recent answers (the search below evaluates the cost models many times)
   struct Key {
     int n, r, sms, want;
-    lbp_layer layers[8];
+    lbp_layer layers[64];
     lbp_basis set[48];   // r <= 48 here
     BatchPlan plan;
   };
   static thread_local Key cache[8];
   static thread_local int cache_n = 0, cache_next = 0;
   const char* env_order = std::getenv("LBP_BATCH_ORDER");   // tuning override: "1,3,2,0"
-  const bool keyed = n <= 8 && env_order == nullptr;
+  const bool keyed = env_order == nullptr;
   auto same = [&](const Key& k) {
     if (k.n != n || k.r != r || k.sms != sms || k.want != want) return false;
     for (int i = 0; i < n; ++i)
@@ -612,6 +612,34 @@ int lbp_test_tile_plan(int Cin, int Cout, int G, int bpt, int k, int units, int 
   out6[5] = t.sched.listed ? t.sched.first[kSchedMaxUnits] : 0;
   for (int i = 0; i <= kSchedMaxUnits; ++i) first[i] = t.sched.first[i];
   for (int i = 0; i < kSchedMaxItems; ++i) ids[i] = t.sched.ids[i];
+  return LBP_OK;
+}
+
+int lbp_test_products_plan(const lbp_layer* layer, const lbp_basis* set, int r, int n_extra, int units, int pair,
+                           int32_t* out8, uint16_t* first, uint16_t* ids) {
+  if (out8 == nullptr || first == nullptr || ids == nullptr) return LBP_ERR_NULL;
+  if (int e = check_layer(layer)) return e;
+  if (units < 1 || units > kSchedMaxUnits || n_extra < 0 || layer->dtype != LBP_BF16) return LBP_ERR_SHAPE;
+  BasisPlan bp;
+  const bool exact = set == nullptr;
+  size_t planes = 0;
+  if (exact) {
+    planes = plan_layout(*layer, layer->k * layer->k, false).splitk_bytes;
+    n_extra = layer->B * layer->H * layer->W;
+  } else {
+    if (int e = make_basis_plan(layer->k, set, r, &bp)) return e;
+    if (!fused_supported(*layer, bp)) return LBP_ERR_BASIS;
+    FusedLayout fl;
+    fused_scratch_bytes(*layer, r, &fl);
+    planes = fl.planes_bytes;
+  }
+  PlanShape s;
+  const TilePlan& t = fused_tile_plan(*layer, exact ? nullptr : &bp, n_extra, planes, units, pair != 0, &s);
+  const int32_t out[8] = {t.BNw, t.BNx, t.bpt, t.splits, t.kbps, t.sched.listed, s.num_kb_w,
+                          static_cast<int32_t>(planes / (static_cast<size_t>(layer->Cout) * layer->Cin * 4))};
+  std::copy(out, out + 8, out8);
+  std::copy(t.sched.first, t.sched.first + kSchedMaxUnits + 1, first);
+  std::copy(t.sched.ids, t.sched.ids + kSchedMaxItems, ids);
   return LBP_OK;
 }
 

@@ -584,6 +584,13 @@ static PlanShape plan_shape(const lbp_layer& L, long long blocks, int piece, int
   return s;
 }
 
+const TilePlan& fused_tile_plan(const lbp_layer& L, const BasisPlan* bp, int n_extra, size_t planes_bytes, int units,
+                                bool pair, PlanShape* shape) {
+  *shape = bp != nullptr ? plan_shape(L, grid_blocks(L), bp->r, expand_core(*bp), n_extra, planes_bytes, units, pair)
+                         : plan_shape(L, 0, 1, 4, n_extra, planes_bytes, units, pair);
+  return plan_products(*shape);
+}
+
 double fused_products_model_us(const lbp_layer& L, const BasisPlan& bp, int pairs) {
   FusedLayout lay;
   fused_scratch_bytes(L, bp.r, &lay);

@@ -244,6 +244,10 @@ int launch_exact(const void* x, const void* g_y, const void* W, void* g_x, void*
 // measurements); lbp_backward_batch balances the two when it runs the
 // projection of one layer beside the products kernel of another.
 double fused_products_model_us(const lbp_layer& L, const BasisPlan& bp, int pairs);
+// The plan of a call on `units` CTAs or CTA pairs; bp null: exact backpropagation.  `shape`
+// receives what was planned.
+const TilePlan& fused_tile_plan(const lbp_layer& L, const BasisPlan* bp, int n_extra, size_t planes_bytes, int units,
+                                bool pair, PlanShape* shape);
 double fused_projection_model_us(const lbp_layer& L, const BasisPlan& bp, int ctas);
 
 // Whether the products kernel runs on CTA pairs (tcgen05 cta_group::2): Cin >= 128

@@ -17,7 +17,11 @@
 // first under the cost model below (measured on B200): greedily, each to the unit that
 // would finish it first; or the GW tiles spread evenly and the GX tiles filled in around
 // them, which is better where most units get both kinds (exact 768 -> 3072 with 8192
-// tokens 63 -> 55 us: greedily, the units without a GW tile idled at the end).
+// tokens: greedily, the units without a GW tile idled at the end).  All tiles of a kind
+// cost the same, so both ways are worked out by classes of units, and a candidate whose even
+// share alone is longer than the best so far is not dealt at all: a first plan of 768 -> 3072
+// with 512 blocks at rank 8 takes 0.2 ms of a host core instead of 5, exact 256 -> 256 with
+// two million tokens 1 instead of 1500.
 #include <cstdio>
 #include <vector>
 
@@ -76,11 +80,6 @@ struct Unit {
   double mma_free = 0, epi_free = 0;
   double slot_free[2] = {0, 0};   // when the epilogue has read the accumulator slot
   int n = 0;
-  double finish_if(double mma, double epi) const {
-    const double start = mma_free > slot_free[n & 1] ? mma_free : slot_free[n & 1];
-    const double mend = start + mma;
-    return (mend > epi_free ? mend : epi_free) + epi;
-  }
   void take(double mma, double epi) {
     const double start = mma_free > slot_free[n & 1] ? mma_free : slot_free[n & 1];
     mma_free = start + mma;
@@ -91,28 +90,61 @@ struct Unit {
   }
 };
 
-// Hands out n_gx GX tiles, then n_gw GW tiles greedily; returns the time the last unit
-// finishes.  `owner` (optional) receives the unit of every tile, GX ids first.
+// Hands out n_gx GX tiles, then n_gw GW tiles greedily, each to the unit that would finish it
+// first (the lowest numbered of several); returns the time the last unit finishes.  `owner`
+// (optional) receives the unit of every tile, GX ids first.
+//
+// The units start alike and the tiles of a kind are alike, so the GX tiles go round the
+// units, and from then on there are two classes of units, those that got one GX tile more
+// and the others.  Within a class the next tile always goes to the next unit that has had
+// the fewest, and which class it goes to changes only when all its units have had as many:
+// the work is one step per tile of a unit, not one per tile and unit (a layer of 524288
+// tokens took a second).
 double deal_greedily(int units, int n_gx, int n_gw, const Costs& c, std::vector<int>* owner) {
-  std::vector<Unit> u(units);
-  if (owner) owner->assign(n_gx + n_gw, 0);
-  auto place = [&](int idx, double mma, double epi) {
-    int best = 0;
-    double best_t = u[0].finish_if(mma, epi);
-    for (int i = 1; i < units; ++i) {
-      const double t = u[i].finish_if(mma, epi);
-      if (t < best_t - 1e-9) {
-        best_t = t;
-        best = i;
-      }
-    }
-    u[best].take(mma, epi);
-    if (owner) (*owner)[idx] = best;
+  if (owner) {
+    owner->assign(n_gx + n_gw, 0);
+    for (int i = 0; i < n_gx; ++i) (*owner)[i] = i % units;
+  }
+  struct Class {
+    int first, size;   // its units
+    int dealt;         // how many of them have had a GW tile more than the others
+    Unit now, next;    // the others, and those
+    double finish;     // the next GW tile here
+  } cls[2];
+  cls[0].first = 0;
+  cls[0].size = n_gx % units;
+  cls[1].first = cls[0].size;
+  cls[1].size = units - cls[0].size;
+  Unit u;
+  for (int i = 0; i < n_gx / units; ++i) u.take(c.mma_x, c.epi_x);
+  cls[1].now = u;
+  u.take(c.mma_x, c.epi_x);
+  cls[0].now = u;
+  auto look_ahead = [&](Class& k) {
+    k.dealt = 0;
+    k.next = k.now;
+    k.next.take(c.mma_w, c.epi_w);
+    k.finish = k.next.epi_free;
   };
-  for (int i = 0; i < n_gx; ++i) place(i, c.mma_x, c.epi_x);
-  for (int i = 0; i < n_gw; ++i) place(n_gx + i, c.mma_w, c.epi_w);
+  for (Class& k : cls) look_ahead(k);
+  for (int i = 0; i < n_gw;) {
+    Class& k = cls[0].size == 0 || cls[1].finish < cls[0].finish - 1e-9 ? cls[1] : cls[0];
+    const int left = n_gw - i, n = k.size - k.dealt < left ? k.size - k.dealt : left;
+    if (owner)
+      for (int q = 0; q < n; ++q) (*owner)[n_gx + i + q] = k.first + k.dealt + q;
+    i += n;
+    k.dealt += n;
+    if (k.dealt == k.size) {
+      k.now = k.next;
+      look_ahead(k);
+    }
+  }
   double last = 0;
-  for (const Unit& x : u) last = x.epi_free > last ? x.epi_free : last;
+  for (const Class& k : cls) {
+    if (k.size == 0) continue;
+    const double t = k.dealt > 0 ? k.next.epi_free : k.now.epi_free;
+    last = t > last ? t : last;
+  }
   return last;
 }
 
@@ -122,20 +154,37 @@ double deal_greedily(int units, int n_gx, int n_gw, const Costs& c, std::vector<
 // on at the same time.
 double deal_evenly(int units, int n_gx, int n_gw, const Costs& c, std::vector<int>* owner) {
   const int gw = n_gw / units, more = n_gw % units, less = units - more;
+  std::vector<Unit> after_gx(1);   // a unit behind its first, second, ... GX tile
   auto unit_time = [&](int gx, int n) {
-    Unit u;
-    for (int i = 0; i < gx; ++i) u.take(c.mma_x, c.epi_x);
+    while (static_cast<int>(after_gx.size()) <= gx) {
+      after_gx.push_back(after_gx.back());
+      after_gx.back().take(c.mma_x, c.epi_x);
+    }
+    Unit u = after_gx[gx];
     for (int i = 0; i < n; ++i) u.take(c.mma_w, c.epi_w);
     return u.epi_free;
   };
+  auto gx_of_less = [&](int x) {   // GX tiles of the units with fewer GW tiles
+    const long long rest = n_gx - static_cast<long long>(more) * x;
+    const int y = rest <= 0 ? 0 : static_cast<int>((rest + less - 1) / less);
+    return y == 0 && gw == 0 ? 1 : y;   // no unit without work
+  };
+  // Start where the units with fewer GW tiles could finish in the time that an even split of
+  // the GX tiles takes (a unit needs at least the longer stage of each).
+  int x0 = 0;
+  if (more > 0) {
+    const int x = n_gx / units;
+    const double t0 = unit_time(x, gw + 1), t1 = unit_time(gx_of_less(x), gw), t = t0 > t1 ? t0 : t1;
+    const long long y_most = static_cast<long long>(t / (c.mma_x > c.epi_x ? c.mma_x : c.epi_x)) + 1;
+    const long long over = n_gx - y_most * less;
+    if (over > 0) x0 = static_cast<int>((over + more - 1) / more);
+  }
   double best = -1.0;
   int gx_more = 0, gx_less = 0;
-  for (int x = 0; more == 0 ? x == 0 : x <= (n_gx + more - 1) / more; ++x) {
+  for (int x = x0; more == 0 ? x == 0 : x <= (n_gx + more - 1) / more; ++x) {
     const double t0 = more > 0 ? unit_time(x, gw + 1) : 0.0;
     if (best >= 0 && t0 > best) break;
-    const int rest = n_gx - more * x;
-    int y = rest <= 0 ? 0 : (rest + less - 1) / less;
-    if (y == 0 && gw == 0) y = 1;   // no unit without work
+    const int y = gx_of_less(x);
     const double t1 = unit_time(y, gw), t = t0 > t1 ? t0 : t1;
     if (best < 0 || t < best - 1e-9) {
       best = t;
@@ -228,9 +277,14 @@ const TilePlan& plan_products(const PlanShape& s) {
           const int n_gw = count_gw(s, row_tile, bnw, splits), n_gx = count_gx(s, row_tile, bnx, bpt);
           const Costs c = tile_costs(s, bnw, bnx, bpt, kbps);
           const int units = n_gw + n_gx < s.units ? n_gw + n_gx : s.units;
-          double t = deal(units, n_gx, n_gw, c, nullptr);
-          if (splits > 1)
-            t += kReduceFixedUs + (splits + 1.0) * s.gw_rows * static_cast<double>(s.gw_cols) * 4 / kReduceBytesPerUs;
+          const double reduce =
+              splits > 1 ? kReduceFixedUs +
+                               (splits + 1.0) * s.gw_rows * static_cast<double>(s.gw_cols) * 4 / kReduceBytesPerUs
+                         : 0.0;
+          // an even share of either stage is the least it can take: most candidates end here
+          const double mma = n_gx * c.mma_x + n_gw * c.mma_w, epi = n_gx * c.epi_x + n_gw * c.epi_w;
+          if (best_t >= 0 && (mma > epi ? mma : epi) / units + reduce >= best_t) continue;
+          const double t = deal(units, n_gx, n_gw, c, nullptr) + reduce;
           if (best_t < 0 || t < best_t - 1e-9) {
             best_t = t;
             best.BNw = bnw;
