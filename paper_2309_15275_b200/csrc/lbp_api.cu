@@ -1048,7 +1048,8 @@ static int run_backward_ex(const void* x, const void* x_hat, const void* g_y, co
     if (int e = launch_bias_grad(dc ? gy_loc.ptr : gy_tokens, dc ? blocks : T, dc ? plan.r : 0,
                                  dc ? gy_loc.dc_slot : 0, gy_map, dc ? gy_loc.dc_to_sum : 1.0, ex->gy_extra,
                                  ex->n_extra, gye_map, L.Cout, L.dtype, ex->g_bias,
-                                 ex->g_bias_dtype == LBP_BF16, ex->beta, st))
+                                 ex->g_bias_dtype == LBP_BF16, ex->beta, reinterpret_cast<double*>(gw0),
+                                 el.gw1 - el.gw0 + static_cast<size_t>(L.Cout) * L.Cin * 4, st))
       return e;
   }
   return LBP_OK;

@@ -3,6 +3,8 @@
 // dense copies of strided token tensors.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "lbp_internal.h"
 #include "wht_device.cuh"
 
@@ -56,12 +58,29 @@ __global__ void __launch_bounds__(256)
 // memory in a fixed order.  What bounds it: latency (a few hundred rows), so rows are
 // fetched four at a time and the cluster grows with their number; the three launches it
 // replaces (column sums of 256 rows per CTA, of the extra tokens, and a finish) took
-// 11.4 + 4.7 + 2.1 us on 256 blocks of 3072 channels and 64 class tokens.
+// 11.4 + 4.7 + 2.1 us on 256 blocks of 3072 channels and 64 class tokens.  Over many rows
+// (all tokens of g_y) a few CTAs would be bound by their own loads: there are several
+// clusters then, each leaves its sums in a row of `partial`, and bias_finish_kernel adds
+// those up in order.  What that takes beside the call without a bias, against one cluster
+// and against the three launches: 200704 tokens of 192 bf16 channels 45 us (479, 260), 32768
+// of 768 32 (84, 102), 802816 of 16 129 (1149, 693).
+__device__ __forceinline__ void store_bias(void* g_bias, int c, double s, int out_bf16, float beta) {
+  if (out_bf16) {
+    __nv_bfloat16* o = static_cast<__nv_bfloat16*>(g_bias) + c;
+    if (beta != 0.f) s += static_cast<double>(beta) * static_cast<double>(__bfloat162float(*o));
+    *o = __float2bfloat16_rn(static_cast<float>(s));
+  } else {
+    float* o = static_cast<float*>(g_bias) + c;
+    if (beta != 0.f) s += static_cast<double>(beta) * static_cast<double>(*o);
+    *o = static_cast<float>(s);
+  }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256)
     bias_grad_kernel(const T* __restrict__ a, long long n_a, int r, int q, TokenMap ta, double scale,
-                     const T* __restrict__ b, long long n_b, TokenMap tb, int C, void* __restrict__ g_bias,
-                     int out_bf16, float beta) {
+                     const T* __restrict__ b, long long n_b, TokenMap tb, int C, int slabs,
+                     double* __restrict__ partial, void* __restrict__ g_bias, int out_bf16, float beta) {
   constexpr int V = 16 / sizeof(T);          // channels per thread
   constexpr int kCols = 8 * V;
   __shared__ double sm[32][kCols + 1];
@@ -69,7 +88,6 @@ __global__ void __launch_bounds__(256)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int col = threadIdx.x & 7, ph = threadIdx.x >> 3;
   const int c = blockIdx.x * kCols + col * V;
-  const int slabs = gridDim.y;
   double acc[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) acc[v] = 0.0;
@@ -89,7 +107,7 @@ __global__ void __launch_bounds__(256)
     }
   };
   if (c < C) {   // C is a multiple of V
-    const long long first = static_cast<long long>(blockIdx.y) * 32 + ph, step = 32ll * slabs;
+    const long long first = static_cast<long long>(blockIdx.y) * 32 + ph, step = 32ll * gridDim.y;
     constexpr int U = 4;
     for (long long i = first; i < n_a; i += U * step) {
       uint4 w[U];
@@ -122,7 +140,7 @@ __global__ void __launch_bounds__(256)
     __syncthreads();
   }
   const int cc = blockIdx.x * kCols + threadIdx.x;
-  if (blockIdx.y == 0 && threadIdx.x < kCols && cc < C) {
+  if (blockIdx.y % slabs == 0 && threadIdx.x < kCols && cc < C) {
     double s = part[threadIdx.x];
     for (int j = 1; j < slabs; ++j) {
       uint32_t at = static_cast<uint32_t>(__cvta_generic_to_shared(&part[threadIdx.x]));
@@ -134,18 +152,31 @@ __global__ void __launch_bounds__(256)
           : "memory");
       s += o;
     }
-    if (out_bf16) {
-      __nv_bfloat16* o = static_cast<__nv_bfloat16*>(g_bias) + cc;
-      if (beta != 0.f) s += static_cast<double>(beta) * static_cast<double>(__bfloat162float(*o));
-      *o = __float2bfloat16_rn(static_cast<float>(s));
-    } else {
-      float* o = static_cast<float*>(g_bias) + cc;
-      if (beta != 0.f) s += static_cast<double>(beta) * static_cast<double>(*o);
-      *o = static_cast<float>(s);
-    }
+    if (partial != nullptr)
+      partial[static_cast<long long>(blockIdx.y / slabs) * C + cc] = s;
+    else
+      store_bias(g_bias, cc, s, out_bf16, beta);
   }
   if (slabs > 1)   // no CTA leaves while its sums may still be read
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// g_bias <- beta * g_bias + the sum of `rows` rows of partial sums: 32 channels a block, eight
+// threads a channel.
+__global__ void __launch_bounds__(256)
+    bias_finish_kernel(const double* __restrict__ partial, int rows, int C, void* __restrict__ g_bias, int out_bf16,
+                       float beta) {
+  __shared__ double sm[8][32];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int lane = threadIdx.x & 31, ph = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
+  double s = 0.0;
+  if (c < C)
+    for (int i = ph; i < rows; i += 8) s += partial[static_cast<long long>(i) * C + c];
+  sm[ph][lane] = s;
+  __syncthreads();
+  if (ph != 0 || c >= C) return;
+  for (int j = 1; j < 8; ++j) s += sm[j][lane];
+  store_bias(g_bias, c, s, out_bf16, beta);
 }
 
 // Moves n_tok tokens of C channels between a tensor laid out as `tm` says and a
@@ -193,13 +224,22 @@ int launch_gw_combine(void* g_W, bool gw_bf16, const float* a, const float* b, f
 
 int launch_bias_grad(const void* a, long long n_a, int r, int q, TokenMap ta, double scale,
                      const void* b, long long n_b, TokenMap tb, int C, int dtype, void* g_bias,
-                     bool out_bf16, float beta, cudaStream_t stream) {
-  const int cols = dtype == LBP_BF16 ? 64 : 32;
+                     bool out_bf16, float beta, double* scratch, size_t scratch_bytes, cudaStream_t stream) {
+  const int cols = dtype == LBP_BF16 ? 64 : 32, tiles = (C + cols - 1) / cols;
   // a slab of at least 128 rows: four fetches per thread
   int slabs = 1;
   while (slabs < 8 && 128ll * slabs < n_a + n_b) slabs *= 2;
+  // Clusters that share the rows: up to four CTAs an SM in all, 2048 rows a cluster at the least
+  // (with fewer the second launch costs more than it gives).
+  long long clusters = 1;
+  if (slabs == 8 && n_a + n_b >= 4096) {
+    const long long fit = static_cast<long long>(scratch_bytes / (static_cast<size_t>(C) * 8));
+    clusters = std::min({(n_a + n_b) / 2048, (4ll * 148 + 8 * tiles - 1) / (8 * tiles), fit});
+    if (clusters < 2) clusters = 1;
+  }
+  double* const partial = clusters > 1 ? scratch : nullptr;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>((C + cols - 1) / cols), static_cast<unsigned>(slabs));
+  cfg.gridDim = dim3(static_cast<unsigned>(tiles), static_cast<unsigned>(slabs * clusters));
   cfg.blockDim = dim3(256);
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
@@ -214,12 +254,19 @@ int launch_bias_grad(const void* a, long long n_a, int r, int q, TokenMap ta, do
   if (dtype == LBP_BF16)
     LBP_CUDA_TRY(cudaLaunchKernelEx(&cfg, bias_grad_kernel<__nv_bfloat16>, static_cast<const __nv_bfloat16*>(a),
                                     n_a, r, q, ta, scale, static_cast<const __nv_bfloat16*>(b), n_b, tb, C,
-                                    g_bias, out_bf16 ? 1 : 0, beta));
+                                    slabs, partial, g_bias, out_bf16 ? 1 : 0, beta));
   else
     LBP_CUDA_TRY(cudaLaunchKernelEx(&cfg, bias_grad_kernel<float>, static_cast<const float*>(a), n_a, r, q, ta,
-                                    scale, static_cast<const float*>(b), n_b, tb, C, g_bias, out_bf16 ? 1 : 0,
-                                    beta));
+                                    scale, static_cast<const float*>(b), n_b, tb, C, slabs, partial, g_bias,
+                                    out_bf16 ? 1 : 0, beta));
   count_launch();
+  if (partial != nullptr) {
+    cfg.gridDim = dim3(static_cast<unsigned>((C + 31) / 32));
+    cfg.numAttrs = 1;
+    LBP_CUDA_TRY(cudaLaunchKernelEx(&cfg, bias_finish_kernel, static_cast<const double*>(partial),
+                                    static_cast<int>(clusters), C, g_bias, out_bf16 ? 1 : 0, beta));
+    count_launch();
+  }
   return LBP_OK;
 }
 

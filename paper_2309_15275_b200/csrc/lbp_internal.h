@@ -209,7 +209,8 @@ struct TokenMap {
   int32_t HW, W;
   long long s_image, s_row, s_tok;
   __host__ __device__ long long offset(long long i) const {
-    const long long b = i / HW;
+    // (a 64-bit division costs a kernel more than what it addresses)
+    const long long b = i < (1ll << 31) ? static_cast<int>(i) / HW : i / HW;
     const int t = static_cast<int>(i - b * HW);
     return b * s_image + (t / W) * s_row + (t % W) * s_tok;
   }
@@ -225,9 +226,10 @@ int launch_copy_tokens(const void* src, void* dst, bool to_dense, long long n_to
 // g_bias <- beta * g_bias + scale * (sum of n_a rows of a) + (sum of n_b rows of b), fp64
 // sums.  r > 0: the rows of a are the coefficients of slot q of its blocks (dense, r
 // per block); r == 0: tokens under `ta`.  b: tokens under `tb`.  g_bias is fp32 or bf16.
+// scratch: for the sums of parts of the rows, as many as fit.
 int launch_bias_grad(const void* a, long long n_a, int r, int q, TokenMap ta, double scale,
                      const void* b, long long n_b, TokenMap tb, int C, int dtype, void* g_bias,
-                     bool out_bf16, float beta, cudaStream_t stream);
+                     bool out_bf16, float beta, double* scratch, size_t scratch_bytes, cudaStream_t stream);
 
 // Tuning switches, read from the environment once (first use):
 //   LBP_FUSED=0          separate product and expansion kernels instead of the

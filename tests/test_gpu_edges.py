@@ -393,3 +393,19 @@ def test_other_threads_run_during_a_call(dev):
     held.join(), ticker.join()
     assert t1 - t0 > 0.1
     assert sum(t0 < t < t1 - 0.05 for t in ticks) >= 5
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("B,H,W,C,ci", [(1, 63, 65, 8, 8), (3, 64, 64, 72, 64), (5, 61, 67, 200, 16), (2, 128, 128, 1544, 8)])
+def test_bias_gradient_over_many_tokens(dev, dtype, B, H, W, C, ci):
+    # g_y itself is summed, by one cluster of CTAs, by several, by as many as the scratch has rows for
+    x, gy, w = layer(dev, 211, B, H, W, ci, C, dtype=dtype)
+    gy += 0.01     # sums that do not cancel: every row counts
+    ge, xe = draw(dev, 214, B, C, dtype=dtype), draw(dev, 215, B, ci, dtype=dtype)
+    for beta in (0.0, 0.5):
+        g_b = torch.full((C,), 3.0, dtype=torch.float32, device=dev)
+        gw = torch.zeros((C, ci), dtype=torch.float32, device=dev)
+        lbp.lbp_backward_ex(x, gy, w, 4, [(0, 1)], beta=beta, g_bias=g_b, x_extra=xe, gy_extra=ge,
+                            gx_extra=torch.empty_like(xe), g_W=gw)
+        # fp64 sums, one rounding to fp32
+        assert rel(g_b, O.bias_grad(f64(gy), f64(ge)) + 3.0 * beta) <= 2.0 ** -23
