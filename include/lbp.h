@@ -228,6 +228,10 @@ typedef struct {
    * x_extra (n_extra, Cin), gy_extra (n_extra, Cout), gx_extra (n_extra, Cin),
    * of the layer's dtype. */
   int32_t n_extra;
+  /* lbp_dtype of g_bias: LBP_F32 (0), or LBP_BF16 with bf16 data; not read without g_bias.  (In the four bytes that
+   * the alignment of the pointers leaves here: size and offsets are those of the struct
+   * without it, so a zeroed one compiled before there was the field reads as LBP_F32.) */
+  int32_t g_bias_dtype;
   const void* x_extra;
   const void* gy_extra;
   void* gx_extra;
@@ -246,8 +250,6 @@ typedef struct {
    * same rules as a view's strides.  With one class token per image in a
    * (B, 1 + H*W, C) sequence this is (1 + H*W) * C. */
   int64_t x_extra_pitch, gy_extra_pitch, gx_extra_pitch;
-  /* lbp_dtype of g_bias: LBP_F32 (0), or LBP_BF16 with bf16 data. */
-  int32_t g_bias_dtype;
 } lbp_extras;
 
 /* Scratch for lbp_backward_ex on x (>= lbp_workspace_bytes; 0 = invalid arguments). */

@@ -49,11 +49,11 @@ class View(C.Structure):
 
 
 class Extras(C.Structure):
-    _fields_ = [("beta", C.c_float), ("g_bias", C.c_void_p), ("n_extra", C.c_int32),
+    _fields_ = [("beta", C.c_float), ("g_bias", C.c_void_p), ("n_extra", C.c_int32), ("g_bias_dtype", C.c_int32),
                 ("x_extra", C.c_void_p), ("gy_extra", C.c_void_p), ("gx_extra", C.c_void_p),
                 ("x_view", View), ("gy_view", View), ("gx_view", View),
                 ("x_extra_pitch", C.c_int64), ("gy_extra_pitch", C.c_int64),
-                ("gx_extra_pitch", C.c_int64), ("g_bias_dtype", C.c_int32)]
+                ("gx_extra_pitch", C.c_int64)]
 
 
 _LIB = None

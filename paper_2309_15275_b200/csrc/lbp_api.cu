@@ -927,7 +927,8 @@ static int check_extras(const lbp_extras* ex, const lbp_layer* L) {
     if (int e = check_pitch(ex->gx_extra_pitch, L->Cin, es)) return e;
   }
   if (ex->g_bias != nullptr && !aligned16(ex->g_bias)) return LBP_ERR_ALIGN;
-  if (ex->g_bias_dtype != LBP_F32 && (ex->g_bias_dtype != LBP_BF16 || L->dtype != LBP_BF16))
+  if (ex->g_bias != nullptr && ex->g_bias_dtype != LBP_F32 &&
+      (ex->g_bias_dtype != LBP_BF16 || L->dtype != LBP_BF16))
     return LBP_ERR_DTYPE;
   if (int e = check_view(ex->x_view, L->Cin, es)) return e;
   if (int e = check_view(ex->gy_view, L->Cout, es)) return e;

@@ -355,3 +355,18 @@ def test_planning_a_new_shape_is_quick(Cin, Cout, B, H, k, r):
         lbp.lbp_test_products_plan(B, H, H, Cin, Cout, k, bases, units=units)
         spent.append(time.process_time() - t0)
     assert min(spent) < (0.015 if r is not None else 0.1), spent
+
+
+def test_extras_keep_their_layout():
+    # compiled callers: the size and the offsets of every field since the struct was first released
+    from paper_2309_15275_b200 import binding as B
+    at = {"beta": 0, "g_bias": 8, "n_extra": 16, "x_extra": 24, "gy_extra": 32, "gx_extra": 40, "x_view": 48,
+          "gy_view": 72, "gx_view": 96, "x_extra_pitch": 120, "gy_extra_pitch": 128, "gx_extra_pitch": 136}
+    assert {n: getattr(B.Extras, n).offset for n in at} == at
+    assert B._lib().lbp_test_struct_size(1) == 144
+    # what lies in the padding of such a caller's struct counts only with a bias
+    lay = B._layer(1, 8, 8, 64, 64, 8, lbp.LBP_BF16, lbp.LBP_F32)
+    ex = B.Extras(beta=1.0, g_bias_dtype=12345)
+    assert B._lib().lbp_workspace_bytes_ex(ctypes.byref(lay), 8, ctypes.byref(ex)) > 0
+    ex.g_bias = 16
+    assert B._lib().lbp_workspace_bytes_ex(ctypes.byref(lay), 8, ctypes.byref(ex)) == 0
