@@ -270,7 +270,9 @@ int launch_project2(const void* t0, void* out0, int C0, const void* t1, void* ou
   LBP_CUDA_TRY(cudaGetDevice(&dev));
   LBP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
 
-  if (dtype == LBP_BF16 && tune_options().umma && project_umma_supported(K, bp.r))
+  // (the tcgen05 form addresses coefficient rows with 32 bits)
+  const bool rows_fit = static_cast<long long>(p.nb) * bp.r < (1ll << 31);
+  if (dtype == LBP_BF16 && tune_options().umma && project_umma_supported(K, bp.r) && rows_fit)
     return launch_project_umma(t0, out0, C0, view0, t1, out1, C1, view1, B, H, W, bp, p.scale[0], p.scale[1],
                                sms, status, stream);
   CUtensorMap tmaps[2];

@@ -473,9 +473,8 @@ int launch_project_umma(const void* t0, void* out0, int C0, const lbp_view* view
   p.cols[1] = (p.C[1] + 63) / 64;
   const long long cells = static_cast<long long>(B) * p.Hb * p.Wb;
   const long long n0 = cells * p.cols[0], n1 = t1 != nullptr ? cells * p.cols[1] : 0;
-  // chunk numbers, and one stride past the last, fit 32 bits
-  if (n0 + n1 >= (1ll << 31) || static_cast<long long>(B) * p.Hb * p.Wblocks * r >= (1ll << 31))
-    return LBP_ERR_SHAPE;
+  // chunk numbers, and one stride past the last, fit 32 bits; so do the rows (the caller)
+  if (n0 + n1 >= (1ll << 31)) return LBP_ERR_SHAPE;
   p.n_chunks0 = static_cast<uint32_t>(n0);
   p.n_chunks = static_cast<uint32_t>(n0 + n1);
   p.status = status;
