@@ -2,6 +2,7 @@
 _lbp_torch.so (the native part of the Python binding) with the host compiler."""
 from __future__ import annotations
 
+import importlib.metadata
 import os
 import shutil
 import subprocess
@@ -13,6 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblbp.so")
 BINDING = os.path.join(HERE, "_lbp_torch.so")
 BINDING_SOURCE = os.path.join(CSRC, "torch_binding.cpp")
+TORCH_STAMP = os.path.join(HERE, "_build", "torch_version")
 
 SOURCES = ["lbp_host.cpp", "lbp_api.cu", "wht_project.cu", "wht_expand.cu",
            "gemm_fp32.cu", "gemm_bf16.cu", "lbp_fused.cu", "lbp_static.cu",
@@ -26,8 +28,15 @@ def _nvcc() -> str:
     return exe
 
 
+def _torch_version() -> str:
+    return importlib.metadata.version("torch")
+
+
 def _stale() -> bool:
     if not os.path.exists(LIB) or not os.path.exists(BINDING):
+        return True
+    # the binding is good for the torch it was compiled against only
+    if not os.path.exists(TORCH_STAMP) or open(TORCH_STAMP).read() != _torch_version():
         return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
@@ -88,6 +97,9 @@ def build_library(force: bool = False, verbose: bool = False, extra_flags=(), ou
         raise RuntimeError("nvcc failed")
     link = [_nvcc(), "-shared", "-o", lib, *objs, "-lcudart_static", "-ldl", "-lrt", "-lpthread"]
     subprocess.run(link, check=True)
+    if out is None:
+        with open(TORCH_STAMP, "w") as f:
+            f.write(_torch_version())
     return lib
 
 

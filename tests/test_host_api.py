@@ -370,3 +370,11 @@ def test_extras_keep_their_layout():
     assert B._lib().lbp_workspace_bytes_ex(ctypes.byref(lay), 8, ctypes.byref(ex)) > 0
     ex.g_bias = 16
     assert B._lib().lbp_workspace_bytes_ex(ctypes.byref(lay), 8, ctypes.byref(ex)) == 0
+
+
+def test_another_torch_makes_the_binding_stale(monkeypatch):
+    from paper_2309_15275_b200 import build
+    build.build_library()
+    assert not build._stale()
+    monkeypatch.setattr(build, "_torch_version", lambda: "0.0.0+other")
+    assert build._stale()
