@@ -1,10 +1,12 @@
 """The kernels at the sizes where they can go wrong: edges of tiles, remainders, the
 smallest and the largest of each form's range, against the fp64 oracle.
 
-Bounds.  bf16: the two operands of a product and the output are rounded to 8 mantissa bits,
-at most 2^-9 per element each, sums are fp32: 3 * 2^-9 in the norm (BF16).  fp32: a sum of n
-terms in any order errs by about sqrt(n) * 2^-24 of its norm for these random signs, 4e-6 at
-the longest sum here (4096 terms), and the longest chain of kernels has three: F32 = 1.2e-5.
+Bounds.  bf16: the two operands of a product and the output are rounded to 8 significant bits,
+each by at most 2^-8 of an element and, over many, by 1.7e-3 < 2^-9 of the norm; sums are
+fp32: 3 * 2^-9 in the norm (BF16).  fp32: a sum of n
+terms in any order errs by about sqrt(n) * 2^-24 of its norm for these random signs: 4e-6 for
+4096 terms, through the three kernels of the longest chain, and 1.1e-5 for the one sum of
+32784 terms in the exact mode: F32 = 1.2e-5.
 """
 import ctypes
 import threading
@@ -100,12 +102,24 @@ def test_products_kernel_forms(dev, form, k, ci, co, B, H, W):
 
 @pytest.mark.parametrize("ci,co,T", [(64, 64, 1), (8, 8, 130), (136, 264, 65), (256, 128, 128), (128, 520, 2049)])
 def test_exact_mode_edges(dev, ci, co, T):
-    # one token; tiles with a few rows or channels past their edge; many K slices
+    # 16 tokens; tiles with a few rows or channels past their edge; many K slices
     x, gy, w = layer(dev, 21, 1, 4, 4 * T, ci, co)
     bases = [(i, j) for i in range(4) for j in range(4)]
     gx, gw = lbp.lbp_backward(x, gy, w, 4, bases)
     ox, ow = O.backward_exact(f64(x), f64(gy), f64(w))
     assert rel(gx, ox) <= 2.0 ** -9 and rel(gw, ow) <= F32   # operands are taken as they are
+
+
+@pytest.mark.parametrize("ci,co,B,H,W", [(64, 64, 1, 1, 1), (136, 264, 1, 1, 1), (72, 200, 1, 3, 5), (264, 72, 7, 3, 3),
+                                         (128, 128, 1, 7, 37)])
+def test_exact_mode_with_odd_token_counts(dev, ci, co, B, H, W):
+    # 1, 15, 63 and 259 tokens: tiles of one row, k-blocks that end early or hold one token more
+    x, gy, w = layer(dev, 23, B, H, W, ci, co)
+    gx, gw = lbp.lbp_backward_fullrank(x, gy, w, 8)
+    ox, ow = O.backward_exact(f64(x), f64(gy), f64(w))
+    # a product of two bf16 numbers is exact in fp32: of one token g_W holds nothing else; g_x is
+    # rounded once, with as few elements as here to be held to the bound of each
+    assert rel(gx, ox) <= 2.0 ** -8 and rel(gw, ow) <= (0.0 if B * H * W == 1 else F32)
 
 
 @pytest.mark.parametrize("k,r", [(4, 1), (4, 4), (4, 5), (4, 9), (4, 15), (8, 1), (8, 16), (8, 17), (8, 33),
@@ -186,6 +200,9 @@ def test_batch_equals_single_calls_at_high_rank(dev, r):
     for x, gy, w, gx, gw in zip(xs, gys, ws_, g_xs, g_Ws):
         ox, ow = want_lowrank(x, gy, w, 8, bases)
         assert rel(gx, ox) <= BF16 and rel(gw, ow) <= BF16
+        # g_x has one order of summation whatever the tile plan; the K slices of g_W may differ
+        gx1, gw1 = lbp.lbp_backward(x, gy, w, 8, bases)
+        assert torch.equal(gx, gx1) and rel(gw, f64(gw1)) <= F32
 
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
