@@ -140,7 +140,9 @@ __global__ void __launch_bounds__(256)
     __syncthreads();
   }
   const int cc = blockIdx.x * kCols + threadIdx.x;
-  if (blockIdx.y % slabs == 0 && threadIdx.x < kCols && cc < C) {
+  uint32_t rank;   // in the cluster
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  if (rank == 0 && threadIdx.x < kCols && cc < C) {
     double s = part[threadIdx.x];
     for (int j = 1; j < slabs; ++j) {
       uint32_t at = static_cast<uint32_t>(__cvta_generic_to_shared(&part[threadIdx.x]));
