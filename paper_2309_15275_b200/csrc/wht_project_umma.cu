@@ -23,8 +23,8 @@
 //             tokens: every MMA then contracts the 16 tokens of one block, into 16 columns
 //             of its own.  (One 4 x 16 box has the four blocks' tokens in every MMA, zeros in
 //             the basis matrix keeping them apart, and zero times the infinity of a block is
-//             NaN in its neighbours; 128 x 16 x 16 tokens of 3072 channels took as long at
-//             rank 3, 49.2 us, and 56.4 against 57.4 at rank 8, 76.7 against 77.9 at rank 15.)
+//             NaN in its neighbours; it took as long: 128 x 16 x 16 tokens of 3072 channels 48
+//             us at rank 3, 57 at rank 8, 75 at rank 15.)
 // The accumulator holds one channel per TMEM lane and one coefficient per column: a
 // thread reads its r columns, rounds them and stores them to r rows of 64 channels in
 // shared memory, from where one TMA store per chunk writes them.
@@ -360,11 +360,6 @@ __global__ void __launch_bounds__(kThreads, 1)
           uint16_t* const o = reinterpret_cast<uint16_t*>(out + i * out_bytes) + (quarter & 1) * 32 + lane;
           const uint32_t acc =
               tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + slot * kSlotCols + h * kHalfCols;
-          auto put = [&](uint16_t* at, uint32_t v0, uint32_t v1, int left) {   // rows 0 and 1 of `left`
-            const uint32_t pk = pack_bf16x2(__uint_as_float(v0) * sc, __uint_as_float(v1) * sc);
-            if (0 < left) at[0] = static_cast<uint16_t>(pk);
-            if (1 < left) at[64] = static_cast<uint16_t>(pk >> 16);
-          };
           if constexpr (K == 4) {
             constexpr int kCols = 4 * NB;   // columns read of a block
             uint16_t* oj = o;
@@ -384,7 +379,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 ptx::tmem_ld_wait();
               }
 #pragma unroll
-              for (int q = 0; q < kCols; q += 2) put(oj + q * 64, v[q], v[q + 1], p.r - q);
+              for (int q = 0; q < kCols; q += 2) {
+                const uint32_t pk = pack_bf16x2(__uint_as_float(v[q]) * sc, __uint_as_float(v[q + 1]) * sc);
+                if (q < p.r) oj[q * 64] = static_cast<uint16_t>(pk);
+                if (q + 1 < p.r) oj[(q + 1) * 64] = static_cast<uint16_t>(pk >> 16);
+              }
             }
           } else {
 #pragma unroll
@@ -393,7 +392,11 @@ __global__ void __launch_bounds__(kThreads, 1)
               ptx::tmem_ld_xn<16>(acc + nb * 16, v);
               ptx::tmem_ld_wait();
 #pragma unroll
-              for (int q = 0; q < 16; q += 2) put(o + (nb * 16 + q) * 64, v[q], v[q + 1], rows - nb * 16 - q);
+              for (int q = 0; q < 16; q += 2) {
+                const uint32_t pk = pack_bf16x2(__uint_as_float(v[q]) * sc, __uint_as_float(v[q + 1]) * sc);
+                if (nb * 16 + q < rows) o[(nb * 16 + q) * 64] = static_cast<uint16_t>(pk);
+                if (nb * 16 + q + 1 < rows) o[(nb * 16 + q + 1) * 64] = static_cast<uint16_t>(pk >> 16);
+              }
             }
           }
         }
