@@ -328,7 +328,7 @@ Tiling choose_tiling(long long M, long long N, long long K, int sms) {
 int launch_splitk_reduce(const float* planes, void* D, long long mn, int splits, bool d_bf16,
                          float beta, bool late, cudaStream_t stream) {
   const long long threads = (mn + 3) / 4;
-  // groups of planes: while that many threads leave SMs without a block of 256
+  // groups of planes: while that many threads leave SMs (148 on a B200) without a block of 256
   const int groups = threads >= 148 * 256 || splits < 4 ? 1 : threads >= 148 * 64 || splits < 16 ? 4 : 16;
   const int cols = 256 / groups;
   cudaLaunchConfig_t cfg = {};

@@ -205,7 +205,9 @@ double deal_evenly(int units, int n_gx, int n_gw, const Costs& c, std::vector<in
 }
 
 // Evenly only where that promises a clear gain: nearer than the model is accurate, the
-// greedy order has the advantage that the units' lists differ in length.
+// greedy order has the advantage that the units' lists differ in length.  (3 % is fitted, as
+// the rates above are, to some dozen layers of 256 to 4096 channels: exact layers with as many
+// GW tiles as units gain 14 % from the even deal, ties lose a few per cent.)
 double deal(int units, int n_gx, int n_gw, const Costs& c, std::vector<int>* owner) {
   const double even = deal_evenly(units, n_gx, n_gw, c, nullptr);
   const double greedy = deal_greedily(units, n_gx, n_gw, c, nullptr);
