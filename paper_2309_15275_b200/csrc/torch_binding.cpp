@@ -79,27 +79,36 @@ bool index_of(PyObject* o, int32_t* v) {
   *v = static_cast<int32_t>(l);
   return over == 0 && *v == l;
 }
-// A list or tuple of pairs; whether a pair is a basis is the library's to say.
+// A sequence of pairs; whether a pair is a basis is the library's to say.
+bool parse_pair(PyObject* p, lbp_basis* out) {
+  if (PyTuple_Check(p) && PyTuple_GET_SIZE(p) == 2)
+    return index_of(PyTuple_GET_ITEM(p, 0), &out->i) && index_of(PyTuple_GET_ITEM(p, 1), &out->j);
+  PyObject* t = PySequence_Check(p) ? PySequence_Tuple(p) : nullptr;   // a list, a row of an array
+  const bool ok = t != nullptr && PyTuple_GET_SIZE(t) == 2 && index_of(PyTuple_GET_ITEM(t, 0), &out->i) &&
+                  index_of(PyTuple_GET_ITEM(t, 1), &out->j);
+  Py_XDECREF(t);
+  PyErr_Clear();
+  return ok;
+}
 bool parse_bases(PyObject* o, Bases* out) {
-  if (!PyList_Check(o) && !PyTuple_Check(o)) return false;
-  const Py_ssize_t n = PySequence_Fast_GET_SIZE(o);
-  if (n > 256) return false;
-  for (Py_ssize_t q = 0; q < n; ++q) {
-    PyObject* p = PySequence_Fast_GET_ITEM(o, q);
-    if (!PyTuple_Check(p) || PyTuple_GET_SIZE(p) != 2) return false;
-    if (!index_of(PyTuple_GET_ITEM(p, 0), &out->v[q].i) || !index_of(PyTuple_GET_ITEM(p, 1), &out->v[q].j))
-      return false;
+  if (!PySequence_Check(o)) return false;
+  PyObject* s = PySequence_Fast(o, "");
+  if (s == nullptr) {
+    PyErr_Clear();
+    return false;
   }
+  const Py_ssize_t n = PySequence_Fast_GET_SIZE(s);
+  bool ok = n <= 256;
+  for (Py_ssize_t q = 0; q < n && ok; ++q) ok = parse_pair(PySequence_Fast_GET_ITEM(s, q), &out->v[q]);
+  Py_DECREF(s);
   out->r = static_cast<int>(n);
-  return true;
+  return ok;
 }
 
 bool parse_int(PyObject* o, int* v) {
-  if (!PyLong_Check(o)) return false;
-  int over = 0;
-  const long a = PyLong_AsLongAndOverflow(o, &over);
-  if (over != 0 || a < 0 || a > (1l << 30)) return false;
-  *v = static_cast<int>(a);
+  int32_t a = 0;
+  if (!PyIndex_Check(o) || !index_of(o, &a) || a < 0 || a > (1 << 30)) return false;   // no floats
+  *v = a;
   return true;
 }
 
@@ -545,6 +554,13 @@ struct LinearFunction : public torch::autograd::Function<LinearFunction> {
   }
 };
 
+// Whether torch's functions on a tensor of this type give tensors of it (unless the class has
+// switched that off).
+bool makes_subclasses(PyTypeObject* type) {
+  const pybind11::object off = pybind11::module_::import("torch._C").attr("_disabled_torch_function_impl");
+  return !pybind11::getattr(reinterpret_cast<PyObject*>(type), "__torch_function__", off).is(off);
+}
+
 // linear(x, weight, bias | None, k, bases, save_projected, H, W) -> y
 PyObject* py_linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
   HANDLE_TH_ERRORS
@@ -571,7 +587,15 @@ PyObject* py_linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
                               static_cast<int64_t>(k), flat, projected, static_cast<int64_t>(H),
                               static_cast<int64_t>(W));
   }
-  return THPVariable_Wrap(y);
+  PyObject* out = THPVariable_Wrap(y);
+  // a subclass among the operands makes the result one, as under torch's own functions
+  for (int i = 0; i < 3 && out != nullptr && THPVariable_CheckExact(out); ++i)
+    if (THPVariable_Check(a[i]) && !THPVariable_CheckExact(a[i]) && makes_subclasses(Py_TYPE(a[i]))) {
+      PyObject* as = PyObject_CallMethod(out, "as_subclass", "O", Py_TYPE(a[i]));
+      Py_DECREF(out);
+      out = as;
+    }
+  return out;
   END_HANDLE_TH_ERRORS
 }
 

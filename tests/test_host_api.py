@@ -378,3 +378,26 @@ def test_another_torch_makes_the_binding_stale(monkeypatch):
     assert not build._stale()
     monkeypatch.setattr(build, "_torch_version", lambda: "0.0.0+other")
     assert build._stale()
+
+
+def test_module_attributes_and_operands_as_torch_takes_them():
+    import torch
+
+    class Tagged(torch.Tensor):
+        pass
+    lin = lbp.LbpLinear(16, 24, 4, [(0, 0)], bias=True)
+    x = torch.randn(2, 4, 4, 16)
+    want = lin(x)
+    for bases in ([[0, 0], [0, 1]], np.array([[0, 0], [0, 1]]), ((0, 0),)):    # set after construction
+        lin.bases = bases
+        assert torch.equal(lin(x), want)
+    lin.k = np.int64(4)
+    assert torch.equal(lin(x), want)
+    y = lin(x.as_subclass(Tagged))
+    assert type(y) is Tagged and torch.equal(y.as_subclass(torch.Tensor), want)
+    lin.grid = (np.int64(4), 4)
+    assert torch.equal(lin(x.flatten(1, 2)), want.flatten(1, 2))
+    for wrong in ([(0,)], [0, 1], 7, None, [("a", "b")]):
+        lin.bases = wrong
+        with pytest.raises(ValueError):
+            lin(x.flatten(1, 2))
