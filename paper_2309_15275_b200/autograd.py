@@ -2,8 +2,9 @@
 Algorithm 1 (low-rank backpropagation on the selected Walsh-Hadamard bases).
 
 Only the backward pass is the library's: the forward product `y = x W^T + b` is a
-plain matrix product and is left to torch (one call: the bias is added in the product's
-epilogue instead of in a pass over y of its own).  The layer takes the token grid
+plain matrix product and is left to torch (in one call, the bias added in the product's
+epilogue, where x, weight and bias are of one type and autocast is off; else as a product
+and a sum).  The layer takes the token grid
 explicit, x of shape (B, H, W, Cin), or, with `grid=(H, W)`, a token sequence
 (B, n + H*W, Cin) whose first n tokens (class tokens) are not part of the grid:
 those take exact backpropagation (Eq. 2), and the grid tokens are handed to the
