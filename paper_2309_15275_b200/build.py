@@ -17,7 +17,7 @@ BINDING_SOURCE = os.path.join(CSRC, "torch_binding.cpp")
 TORCH_STAMP = os.path.join(HERE, "_build", "torch_version")
 
 SOURCES = ["lbp_host.cpp", "lbp_api.cu", "wht_project.cu", "wht_expand.cu",
-           "gemm_fp32.cu", "gemm_bf16.cu", "lbp_fused.cu", "lbp_static.cu",
+           "gemm_fp32.cu", "gemm_fp32_split.cu", "gemm_bf16.cu", "lbp_fused.cu", "lbp_static.cu",
            "wht_spectrum.cu", "lbp_extras.cu", "lbp_fused_plan.cu", "wht_project_umma.cu"]
 
 

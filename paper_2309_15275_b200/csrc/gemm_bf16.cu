@@ -370,7 +370,7 @@ int launch_gemm(const void* A, bool a_mn_major, const void* Bm, void* D, int in_
     if (d_dtype != LBP_F32) return LBP_ERR_DTYPE;
     const GemmFp32 job{static_cast<const float*>(A), static_cast<const float*>(Bm), static_cast<float*>(D), M, N, K,
                        a_mn_major};
-    return launch_gemm_fp32(&job, 1, splitk_ws, splitk_ws_bytes, stream);
+    return launch_gemm_fp32(&job, 1, splitk_ws, splitk_ws_bytes, status, stream);
   }
   int dev = 0, sms = 0;
   LBP_CUDA_TRY(cudaGetDevice(&dev));

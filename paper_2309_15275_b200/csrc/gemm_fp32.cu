@@ -1,22 +1,24 @@
-// fp32 products (Algorithm 1's two in the low-rank space, Eq. 2's two) on the FFMA pipe.
+// fp32 products (Algorithm 1's two in the low-rank space, Eq. 2's two): the plan, and the
+// kernel on the FFMA pipe for the smallest of them (the others: gemm_fp32_split.cu).
 //
-// fp32 data must meet a 1e-5 relative error, which a single-pass TF32 tensor
-// product (10-bit mantissa) cannot.
 //   D[M, N] = sum_k A(m, k) * B(k, n),  B stored (K, N) row-major,
 //   A stored (M, K) row-major or, when A_MN, (K, M) row-major.
 //
 // Both products of a call go out in one launch: they are independent, and either alone
-// leaves SMs idle.  An item of work is a 64 x 64 tile over at most `per` k-blocks of 32; a
-// CTA takes one item, and where K needs several, each writes its sums to a plane of its
-// own, which one more kernel adds up in order.  So the items of a small M x N with a long
-// K and of a large one with a short K last equally long, and fill the chip together
-// (plan(): slices through planes are taken only where they pay for themselves).
-// A thread holds 8 x 4 sums; operands come by cp.async into three stages of 32 k's (A as
-// it lies: from (M, K) a thread reads four k's of a row at once, from (K, M) four rows).
-// What bounds it: shared-memory reads (a k-block of a tile takes an SM about 1 us, FFMA
-// alone 0.54).  8 x 8 sums in 64 threads read less but leave the latency bare: 3.1 us for a
-// CTA alone.  64 blocks of 448 -> 1792 at rank 10 with both products (7840 k-blocks of
-// tiles) 64 -> 58 us, 48 rows of 2880 -> 960 at order 16 (2700) 140 -> 25.
+// leaves SMs idle.  An item of work is a tile over a run of k-blocks; a CTA takes one item,
+// and where K needs several, each writes its sums to a plane of its own, which one more
+// kernel adds up in order.  So the items of a small M x N with a long K and of a large one
+// with a short K last equally long, and fill the chip together (plan(): slices through planes
+// are taken only where they pay for themselves).
+//
+// FFMA kernel: tiles of 64 x 64, k-blocks of 32.  A thread holds 8 x 4 sums; operands come by
+// cp.async into three stages (A as it lies: from (M, K) a thread reads four k's of a row at
+// once, from (K, M) four rows).  What bounds it: shared-memory reads (a k-block of a tile takes
+// an SM about 1 us, FFMA alone 0.54).  8 x 8 sums in 64 threads read less but leave the latency
+// bare: 3.1 us for a CTA alone.
+#include <cstdio>
+
+#include "gemm_fp32.cuh"
 #include "lbp_internal.h"
 #include "ptx_sm100.cuh"
 
@@ -31,18 +33,6 @@ constexpr int kSmemBytes = kStages * kStageFloats * 4;
 constexpr int kResident = 4;          // CTAs of an SM at a time
 constexpr int kSms = 148;             // of a B200 (the scratch is sized without a device)
 
-struct Job {
-  const float *A, *B;
-  float* D;                       // chunks > 1: the planes [chunks][M][N]
-  long long M, N, K;
-  int32_t a_mn, tiles_n, tiles;   // tiles of D along N, in all
-  int32_t kb, chunks;             // k-blocks; items per tile
-};
-struct Jobs {
-  Job j[2];
-  int32_t n, per, items0;         // k-blocks of an item; items of the first job
-};
-
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool valid) {
   const int bytes = valid ? 16 : 0;   // 0: the 16 bytes are filled with zeros, nothing is read
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ptx::smem_u32(smem)), "l"(gmem), "r"(bytes)
@@ -54,7 +44,7 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool va
 __device__ __forceinline__ int row_of(int ty, int i) { return (i >> 2) * 32 + ty * 4 + (i & 3); }
 
 template <bool A_MN>
-__device__ __forceinline__ void tile_sums(const Job& g, long long m0, long long n0, int kb0, int kb1,
+__device__ __forceinline__ void tile_sums(const GemmFp32Job& g, long long m0, long long n0, int kb0, int kb1,
                                           float* smem, float (&acc)[8][4]) {
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   // what this thread fetches of a k-block: four 16-byte pieces of A and of B, each a fixed
@@ -136,22 +126,22 @@ __device__ __forceinline__ void tile_sums(const Job& g, long long m0, long long 
   }
 }
 
-__global__ void __launch_bounds__(kThreads, kResident) gemm_fp32_kernel(const __grid_constant__ Jobs jobs) {
+__global__ void __launch_bounds__(kThreads, kResident) gemm_fp32_kernel(const __grid_constant__ GemmFp32Jobs jobs) {
   extern __shared__ __align__(16) float smem[];
   asm volatile("griddepcontrol.wait;" ::: "memory");   // launched as the kernel ahead ends
   int t = blockIdx.x;
-  const Job& g = jobs.j[t >= jobs.items0 ? 1 : 0];
+  const GemmFp32Job& g = jobs.j[t >= jobs.items0 ? 1 : 0];
   if (t >= jobs.items0) t -= jobs.items0;
   const int chunk = t % g.chunks;
   t /= g.chunks;
-  const long long m0 = static_cast<long long>(t / g.tiles_n) * kTile, n0 = static_cast<long long>(t % g.tiles_n) * kTile;
+  const long long m0 = static_cast<long long>(t / g.tiles_c) * kTile, n0 = static_cast<long long>(t % g.tiles_c) * kTile;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   float acc[8][4];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  const int kb0 = chunk * jobs.per, kb1 = kb0 + jobs.per < g.kb ? kb0 + jobs.per : g.kb;
+  const int kb0 = chunk * g.per, kb1 = kb0 + g.per < g.kb ? kb0 + g.per : g.kb;
   if (g.a_mn)
     tile_sums<true>(g, m0, n0, kb0, kb1, smem, acc);
   else
@@ -168,95 +158,194 @@ __global__ void __launch_bounds__(kThreads, kResident) gemm_fp32_kernel(const __
   }
 }
 
-long long tiles_of(const GemmFp32& g) {
-  return ((g.M + kTile - 1) / kTile) * ((g.N + kTile - 1) / kTile);
-}
-long long kblocks(const GemmFp32& g) { return (g.K + kBK - 1) / kBK; }
+// The forms a product can take: tile, k-block, and what a k-block and an item take an SM (us),
+// as measured.  FFMA: an SM works off a k-block in about a microsecond however many CTAs it
+// holds.  Split operands (one CTA to an SM): 6 us for an item of one k-block of 128 x 128 x 64
+// alone on the chip, 12.4 of four, 23.6 of twelve; 5 us, 8.6 of four, 30 of twenty-four of 128 x 64.
+// Both sides of the line (us a call): 8 x 7 x 7 tokens of 64 -> 256 at order 4, rank 6, FFMA
+// 10.8, split 11.5; 2 x 16 x 16 of 64 -> 64, order 8, rank 4 10.4 and 10.7; 4 x 56 x 56 of 48 ->
+// 192, order 4, rank 3 17.8 and 16.5; 8 x 28 x 28 of 192 -> 768, order 8, rank 21 64 and 38; 64 x
+// 7 x 7 of 448 -> 1792, order 8, rank 10 69 and 31; 392 tokens of 768 -> 3072, exact 105 and 31.
+struct Form {
+  int lanes, cols, bk;   // (split operands: lanes of TMEM, of the operand stored (K, lanes))
+  double kb_us, item_us, launch_us;
+};
+constexpr Form kForms[] = {
+    {kTile, kTile, kBK, 1.0, 0.2, 0.0},
+    {128, 64, 64, 1.05, 2.5, 2.0},
+    {128, 128, 64, 1.45, 3.5, 2.0},
+};
 
-// k-blocks of an item, and the bytes of planes that takes (at most `room`).  An SM works
-// off a k-block in about a microsecond however many CTAs it holds (its shared-memory reads
-// bind: 12 of 16 bytes per 32 FFMA), so what counts is how many k-blocks the fullest SM
-// gets, and short items share out best: 2 to 5 k-blocks, or K left whole.  (Longer ones only
-// with many items per SM: with two or three, 6 to 12 k-blocks measured up to half as slow
-// again as 3 or 4.)  Planes cost their bytes and about 1.5 us of the kernel that adds them
-// up.  28 tiles of 42 k-blocks and 147 of 8 (256 tokens, exact, 448 -> 1344): 53 us whole,
-// 23 at 4, 34 at 8; 212 of 8 and 16 of 105: 133 whole, 50 at 4; 15 of 90 and 675 of 2: 121
-// and 42; 12 of 12 and 12 of 11: 14 whole, 16 at 4.
-long long plan(const GemmFp32* job, int n, size_t room, size_t* planes) {
+struct Plan {
+  int form, per;
+  size_t planes;   // bytes
+};
+
+long long ceil_div(long long a, long long b) { return (a + b - 1) / b; }
+long long lanes_of(const GemmFp32& g, const Form& f) { return ceil_div(g.a_mn ? g.M : g.N, f.lanes); }
+long long cols_of(const GemmFp32& g, const Form& f) { return ceil_div(g.a_mn ? g.N : g.M, f.cols); }
+long long tiles_of(const GemmFp32& g, const Form& f) { return lanes_of(g, f) * cols_of(g, f); }
+
+// Time until the last of n0 items of t0 and then n1 of t1 ends, each taken by the first SM that is free.
+double makespan(long long n0, double t0, long long n1, double t1) {
+  const long long q = n0 / kSms, more = n0 % kSms;
+  double low = q * t0, high = low + (more > 0 ? t0 : 0.0);   // `more` SMs are free at `high`, the others at `low`
+  double end = high;
+  long long at_low = kSms - more, at_high = more;
+  while (n1 > 0) {
+    if (at_high > 0 && high < low) {
+      const double d = high;
+      high = low, low = d;
+      const long long n = at_high;
+      at_high = at_low, at_low = n;
+    }
+    n1 -= at_low;
+    low += t1;
+    end = low > end ? low : end;
+  }
+  return end;
+}
+
+// Items of a product of kb k-blocks at `per` an item, evenly long.
+long long chunks_of(long long kb, long long per) { return ceil_div(kb, ceil_div(kb, ceil_div(kb, per))); }
+
+// The form, k-blocks of an item, and the bytes of planes that takes (at most `room`).  FFMA:
+// what counts is how many k-blocks the fullest SM gets, and short items share out best: 2 to 5
+// k-blocks, or K left whole.  (Longer ones only with many items per SM: with two or three, 6
+// to 12 k-blocks measured up to half as slow again as 3 or 4.)  Planes cost their bytes and
+// about 1.5 us of the kernel that adds them up.
+Plan make_plan(const GemmFp32* job, int n, size_t room) {
   constexpr size_t kRoom = 48u << 20;
   if (room > kRoom) room = kRoom;
-  long long most = 1;
-  for (int i = 0; i < n; ++i) most = kblocks(job[i]) > most ? kblocks(job[i]) : most;
-  long long best = most;
+  Plan best{};
   double best_t = -1.0;
-  *planes = 0;
-  for (long long per : {most, 64ll, 32ll, 16ll, 8ll, 5ll, 4ll, 3ll, 2ll}) {
-    if (per > most) continue;
-    double items = 0, t = 0;
-    size_t bytes = 0;
+  const int forced = tune_options().fp32_form;
+  for (int f = 0; f < 3; ++f) {
+    const Form& form = kForms[f];
+    if (forced >= 0 && f != forced) continue;
+    bool fits = true;   // TMA coordinates are 32-bit
+    for (int i = 0; i < n; ++i)
+      for (long long d : {job[i].M, job[i].N, job[i].K}) fits &= d < (1ll << 31) - 256;
+    if (f > 0 && !fits) continue;
+    long long kb[2] = {0, 0}, most = 1;
     for (int i = 0; i < n; ++i) {
-      const long long chunks = (kblocks(job[i]) + per - 1) / per;
-      items += static_cast<double>(tiles_of(job[i])) * chunks;
-      if (chunks > 1) {
-        const size_t b = static_cast<size_t>(chunks) * job[i].M * job[i].N * 4;
-        bytes += b;
-        t += 1.5 + 2.0 * b / 8e6;
-      }
+      kb[i] = ceil_div(job[i].K, form.bk);
+      most = kb[i] > most ? kb[i] : most;
     }
-    if (bytes > room || (per > 5 && per < most && items < 8.0 * kSms)) continue;
-    t += static_cast<double>(static_cast<long long>((items + kSms - 1) / kSms)) * (per + 0.2);
-    if (best_t < 0 || t < best_t) {
-      best_t = t;
-      best = per;
-      *planes = bytes;
+    for (long long per : {most, 64ll, 48ll, 32ll, 24ll, 16ll, 12ll, 10ll, 8ll, 7ll, 6ll, 5ll, 4ll, 3ll, 2ll, 1ll}) {
+      if (per > most || (f == 0 && per == 1 && per < most)) continue;
+      double t = 0, item_t[2] = {0, 0};
+      long long items[2] = {0, 0};
+      size_t bytes = 0;
+      for (int i = 0; i < n; ++i) {
+        const long long chunks = chunks_of(kb[i], per);
+        items[i] = tiles_of(job[i], form) * chunks;
+        item_t[i] = ceil_div(kb[i], chunks) * form.kb_us + form.item_us;
+        if (chunks > 1) {
+          const size_t b = static_cast<size_t>(chunks) * job[i].M * job[i].N * 4;
+          bytes += b;
+          t += 1.5 + 2.0 * b / 8e6;
+        }
+      }
+      const double all = static_cast<double>(items[0] + items[1]);
+      if (bytes > room || (f == 0 && per > 5 && per < most && all < 8.0 * kSms)) continue;
+      t += f == 0 ? static_cast<double>(ceil_div(items[0] + items[1], kSms)) * (per + form.item_us)
+           : item_t[0] < item_t[1] ? form.launch_us + makespan(items[1], item_t[1], items[0], item_t[0])
+                                    : form.launch_us + makespan(items[0], item_t[0], items[1], item_t[1]);
+      if (best_t < 0 || t < best_t) {
+        best_t = t;
+        best = Plan{f, static_cast<int>(per), bytes};
+      }
     }
   }
   return best;
 }
 
+// (remembered per calling thread for recent shapes)
+Plan plan(const GemmFp32* job, int n, size_t room) {
+  struct Entry {
+    long long dims[6];
+    size_t room;
+    int forced;
+    Plan plan;
+  };
+  static thread_local Entry cache[16];
+  static thread_local int filled = 0, next = 0;
+  const GemmFp32 &a = job[0], &b = job[n - 1];
+  const long long dims[6] = {a.M, a.N, a.K, n > 1 ? b.M : 0, n > 1 ? b.N : 0, n > 1 ? b.K : 0};
+  for (int c = 0; c < filled; ++c) {
+    const Entry& e = cache[c];
+    bool same = e.room == room && e.forced == tune_options().fp32_form;
+    for (int i = 0; i < 6; ++i) same &= e.dims[i] == dims[i];
+    if (same) return e.plan;
+  }
+  Entry& e = cache[next];
+  for (int i = 0; i < 6; ++i) e.dims[i] = dims[i];
+  e.room = room;
+  e.forced = tune_options().fp32_form;
+  e.plan = make_plan(job, n, room);
+  if (tune_options().verbose)
+    fprintf(stderr, "lbp fp32 products plan: %lldx%lldx%lld, %lldx%lldx%lld: form %d, %d k-blocks an item, planes %zu\n",
+            dims[0], dims[1], dims[2], dims[3], dims[4], dims[5], e.plan.form, e.plan.per, e.plan.planes);
+  next = (next + 1) % 16;
+  filled = filled < 16 ? filled + 1 : 16;
+  return e.plan;
+}
+
 }  // namespace
 
 size_t gemm_fp32_ws_bytes(const GemmFp32* job, int n) {
-  size_t planes = 0;
-  plan(job, n, static_cast<size_t>(-1), &planes);
-  return planes;
+  return plan(job, n, static_cast<size_t>(-1)).planes;
 }
 
-int launch_gemm_fp32(const GemmFp32* job, int n, float* ws, size_t ws_bytes, cudaStream_t stream) {
-  Jobs js{};
-  js.n = n;
-  size_t planes = 0;
-  const long long per = plan(job, n, ws != nullptr ? ws_bytes : 0, &planes);
+int launch_gemm_fp32(const GemmFp32* job, int n, float* ws, size_t ws_bytes, uint32_t* status, cudaStream_t stream) {
+  GemmFp32Jobs js{};
+  js.status = status;
+  const Plan pl = plan(job, n, ws != nullptr ? ws_bytes : 0);
+  const Form& form = kForms[pl.form];
+  // split operands: the longer items first
+  const auto per_of = [&](int i) {
+    const long long kb = ceil_div(job[i].K, form.bk);
+    return ceil_div(kb, chunks_of(kb, pl.per));
+  };
+  const bool swap = n > 1 && pl.form > 0 && per_of(0) < per_of(1);
   long long items = 0;
-  for (int i = 0; i < n; ++i) {
-    const long long tiles = tiles_of(job[i]), kb = kblocks(job[i]), chunks = (kb + per - 1) / per;
+  for (int at = 0; at < n; ++at) {
+    const GemmFp32& g = job[swap ? 1 - at : at];
+    const long long tiles = tiles_of(g, form), kb = ceil_div(g.K, form.bk), chunks = chunks_of(kb, pl.per);
     if (tiles >= (1ll << 30) || kb >= (1ll << 30) || items + tiles * chunks >= (1ll << 31)) return LBP_ERR_SHAPE;
-    js.j[i] = Job{job[i].A, job[i].B, chunks > 1 ? ws : job[i].D, job[i].M, job[i].N, job[i].K, job[i].a_mn ? 1 : 0,
-                  static_cast<int32_t>((job[i].N + kTile - 1) / kTile), static_cast<int32_t>(tiles),
-                  static_cast<int32_t>(kb), static_cast<int32_t>(chunks)};
-    if (chunks > 1) ws += chunks * job[i].M * job[i].N;
+    js.j[at] = GemmFp32Job{g.A, g.B, chunks > 1 ? ws : g.D, g.M, g.N, g.K, g.a_mn ? 1 : 0,
+                           static_cast<int32_t>(pl.form > 0 ? cols_of(g, form) : ceil_div(g.N, form.cols)),
+                           static_cast<int32_t>(tiles), static_cast<int32_t>(kb),
+                           static_cast<int32_t>(ceil_div(kb, chunks)), static_cast<int32_t>(chunks)};
+    if (chunks > 1) ws += chunks * g.M * g.N;
     items += tiles * chunks;
-    if (i == 0) js.items0 = static_cast<int32_t>(items);
+    if (at == 0) js.items0 = static_cast<int32_t>(items);
   }
-  js.per = static_cast<int32_t>(per);
-  static PerDevice configured;
-  if (int e = allow_dynamic_smem(configured, reinterpret_cast<const void*>(gemm_fp32_kernel), kSmemBytes)) return e;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.gridDim = dim3(static_cast<unsigned>(items));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kSmemBytes;
-  cfg.stream = stream;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  LBP_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_fp32_kernel, js));
-  count_launch();
-  for (int i = 0; i < n; ++i)
-    if (js.j[i].chunks > 1)
-      if (int e = launch_splitk_reduce(js.j[i].D, job[i].D, job[i].M * job[i].N, js.j[i].chunks, false, 0.f, true, stream))
-        return e;
+  js.items = static_cast<int32_t>(items);
+  if (pl.form > 0) {
+    if (int e = launch_gemm_fp32_split(js, n, form.cols, stream)) return e;
+  } else {
+    static PerDevice configured;
+    if (int e = allow_dynamic_smem(configured, reinterpret_cast<const void*>(gemm_fp32_kernel), kSmemBytes)) return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(static_cast<unsigned>(items));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    LBP_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_fp32_kernel, js));
+    count_launch();
+  }
+  for (int at = 0; at < n; ++at) {
+    const GemmFp32& g = job[swap ? 1 - at : at];
+    if (js.j[at].chunks > 1)
+      if (int e = launch_splitk_reduce(js.j[at].D, g.D, g.M * g.N, js.j[at].chunks, false, 0.f, true, stream)) return e;
+  }
   return LBP_OK;
 }
 

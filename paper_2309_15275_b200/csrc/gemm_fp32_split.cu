@@ -1,0 +1,331 @@
+// fp32 products on the tcgen05 tensor cores, by splitting every operand into three bf16 parts.
+//
+//   D(l, c) = sum_k L(k, l) * C(k, c)
+//
+// L, stored (K, lanes) row-major, becomes the A operand, a TMEM lane per l; C, stored (K,
+// columns) or (columns, K) row-major, the B operand.  g_W = g_y_hat^T x_hat is this with L =
+// g_y_hat and C = x_hat, g_x_hat = g_y_hat W with L = W and C = g_y_hat (D transposed).
+//
+// x = hi + mid + lo, each part the bf16 nearest to what the parts before it leave: 8
+// significant bits a part and a sign each, so the three hold x to 2^-27 of itself.  Of the
+// nine products of parts the six largest are formed; the rest is below 2^-26 of a term.
+// A product of two bf16 numbers is exact in fp32, so what is left is the summation.  The
+// tensor core drops bits of the smaller addend when it adds to an accumulator, so a
+// k-block of 64 starts from an accumulator of its own, its small products go first, and the
+// sums of k-blocks are added up in registers, rounding to nearest.
+//
+// An item is a tile of 128 lanes x BN columns over a run of k-blocks of 64.  TMA brings a block's
+// fp32 operands to shared memory, two blocks ahead.  Of a CTA's 16 warps eight split L (a
+// thread the k's of its lane) and write the parts to TMEM, the others split C and store the
+// parts to shared memory in the 128-byte-swizzled layout the tensor core reads.  One thread
+// of a warp of its own issues the 24 MMAs of 128 x BN x 16; under them all warps add the
+// accumulator of the block before to their sums.  Two stages of everything.
+//
+// A 128 x 128 x 64 block takes 1.4 us: its MMAs 0.8, splitting 0.7 (conversions and shifts at
+// half rate), one partly under the other; an item's start and end another 4.5.  Tried
+// before: loads into registers, issued as these become free, make every use wait for the
+// latest load (2.1 us a block, from 8 or 16 warps, also with persistent CTAs, two CTAs to an SM
+// or the parts of L in TMEM).  64 blocks of 448 -> 1792 at rank 10: both products 55 us on FFMA
+// (37 TFLOP/s), 20.6 here (100, six times that in bf16); error against 64 bits of g_x and g_W
+// 2.4e-7 and 2.5e-7 there, 1.3e-7 and 1.4e-7 here.
+//
+// Infinities, NaN and values next to the largest float leave the parts meaningless
+// (inf - inf, 0 * inf), but they always show as a sum that is not finite: such sums are
+// computed again, term by term with fp32 FMAs.
+#include "gemm_fp32.cuh"
+#include "lbp_internal.h"
+#include "ptx_sm100.cuh"
+#include "wht_device.cuh"
+
+namespace lbp {
+namespace split {
+
+constexpr int kLanes = 128, kBK = 64;
+constexpr int kWarps = 16;                       // 8 for L, 8 for C
+constexpr int kThreads = (kWarps + 1) * 32;      // and one that issues loads and MMAs
+constexpr int kChunkBytes = 64 * kBK * 2;        // 64 columns of an MN-major operand
+constexpr uint32_t kTmemCols = 512, kTmemL = 256, kPartCols = kBK / 2;   // L: two stages of three parts behind the accumulators
+
+template <int BN>
+struct Cfg {
+  static constexpr int kPart = BN * kBK * 2;                  // of C
+  static constexpr int kStage = 3 * kPart;
+  static constexpr int kRawL = kLanes * kBK * 4, kRaw = kRawL + BN * kBK * 4;   // as TMA brings them
+  static constexpr int kOut = 16 * 32 * (BN / 4) * 4;         // the sums on their way out
+  static constexpr int kSmem = 2 * (kStage + kRaw) + 1024 + 64;
+  static_assert(kOut <= 2 * kStage && kSmem <= 227 * 1024, "shared memory");
+  static constexpr int kPieces = BN * kBK / 4 / 256;          // of four numbers, per thread
+  static constexpr int kCols = BN / 4;                        // accumulator columns of a warp
+};
+
+struct Maps {
+  CUtensorMap l[2], c[2];   // of either job
+};
+
+__device__ __forceinline__ void tmem_st_x8(uint32_t taddr, const uint32_t (&v)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(v[0]),
+               "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
+// D[tmem] (+)= A[tmem] * B[smem desc]
+__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                            uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// The next part of two numbers; what it leaves of them.
+__device__ __forceinline__ uint32_t take_part(float& a, float& b) {
+  const uint32_t w = pack_bf16x2(a, b);
+  a -= bf16_lo(w);   // exact
+  b -= bf16_hi(w);
+  return w;
+}
+
+template <int BN>
+__global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __grid_constant__ GemmFp32Jobs jobs,
+                                                                    const __grid_constant__ Maps maps) {
+  using C = Cfg<BN>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  uint8_t* const raw = smem + 2 * C::kStage;
+  uint64_t* full = reinterpret_cast<uint64_t*>(raw + 2 * C::kRaw);   // [2]: a block's operands have arrived
+  uint64_t* ready = full + 2;                                        // [2]: its parts are written
+  uint64_t* done = ready + 2;                                        // [2]: its MMAs have completed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 2);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  int t = blockIdx.x;
+  const int which = t >= jobs.items0 ? 1 : 0;
+  const GemmFp32Job& g = jobs.j[which];
+  if (which) t -= jobs.items0;
+  const int chunk = t % g.chunks;
+  t /= g.chunks;
+  const bool wt = g.a_mn == 0;   // L = B, C = A stored (columns, K), D transposed
+  const long long lanes = wt ? g.N : g.M, cols = wt ? g.M : g.N;
+  const float* const L = wt ? g.B : g.A;
+  const float* const Cm = wt ? g.A : g.B;
+  const long long l0 = static_cast<long long>(t / g.tiles_c) * kLanes, c0 = static_cast<long long>(t % g.tiles_c) * BN;
+  const int kb0 = chunk * g.per, kb1 = kb0 + g.per < g.kb ? kb0 + g.per : g.kb, n_kb = kb1 - kb0;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 2; ++i) {
+      ptx::mbar_init(&full[i], 1);
+      ptx::mbar_init(&ready[i], kWarps);
+      ptx::mbar_init(&done[i], 1);
+    }
+    ptx::mbar_fence_init();
+    ptx::prefetch_tensormap(&maps.l[which]);
+    ptx::prefetch_tensormap(&maps.c[which]);
+  }
+  if (warp == 0) {
+    ptx::tmem_alloc(tmem_slot, kTmemCols);
+    ptx::tmem_relinquish();
+  }
+  ptx::tc_fence_before_sync();
+  __syncthreads();
+  ptx::tc_fence_after_sync();
+  const uint32_t tmem_base = *tmem_slot;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // launched as the kernel ahead ends
+
+  auto load = [&](int i) {   // one thread: block i of the item
+    uint8_t* const dst = raw + (i & 1) * C::kRaw;
+    const int k = (kb0 + i) * kBK;
+    ptx::mbar_expect_tx(&full[i & 1], C::kRaw);   // boxes count in full, also where they hang over an edge (zeros)
+    ptx::tma_load_2d(dst, &maps.l[which], &full[i & 1], static_cast<int32_t>(l0), k);
+    ptx::tma_load_2d(dst + C::kRawL, &maps.c[which], &full[i & 1], wt ? k : static_cast<int32_t>(c0),
+                     wt ? static_cast<int32_t>(c0) : k);
+  };
+  // L: a thread has its lane's k's of one half of the block.  C: pieces of four numbers, a
+  // warp whole 128-byte lines; row `row` + q * rows of the block, in shared memory `hop` apart.
+  const bool is_l = warp < 8;
+  const int quarter = warp & 3, tid = threadIdx.x & 255;
+  const int c_row = wt ? tid >> 4 : tid / (BN / 4), c_pc = wt ? tid & 15 : tid % (BN / 4);
+  const int hop = (wt ? 16 : 256 / (BN / 4)) * 128;
+  const int to = (wt ? 0 : (c_pc >> 4) * kChunkBytes) + c_row * 128 + ((((c_pc & 15) >> 1) ^ (c_row & 7)) << 4) + (c_pc & 1) * 8;
+  const long long l = l0 + quarter * 32 + lane;
+
+  float sum[C::kCols];
+#pragma unroll
+  for (int j = 0; j < C::kCols; ++j) sum[j] = 0.f;
+  const int group = warp >> 2;
+  const uint32_t lane_bits = static_cast<uint32_t>(quarter * 32) << 16;
+  const uint32_t acc_at = tmem_base + lane_bits + group * C::kCols;
+  bool ok = true;
+  auto drain = [&](int i) {
+    ok = __all_sync(0xffffffffu,
+                    ptx::mbar_wait(&done[i & 1], static_cast<uint32_t>(i >> 1) & 1u, jobs.status, (7u << 16) | 1u));
+    ptx::tc_fence_after_sync();
+#pragma unroll
+    for (int c = 0; c < C::kCols; c += 16) {
+      uint32_t a[16];
+      ptx::tmem_ld_xn<16>(acc_at + (i & 1) * BN + c, a);
+      ptx::tmem_ld_wait();
+#pragma unroll
+      for (int j = 0; j < 16; ++j) sum[c + j] += __uint_as_float(a[j]);
+    }
+  };
+
+  if (warp == kWarps) {
+    if (ptx::elect_one()) {
+      const uint32_t idesc = ptx::idesc_bf16(kLanes, BN, false, !wt);
+      load(0);
+      if (n_kb > 1) load(1);
+      for (int i = 0; i < n_kb; ++i) {
+        const int s = i & 1;
+        if (!ptx::mbar_wait(&ready[s], static_cast<uint32_t>(i >> 1) & 1u, jobs.status, (7u << 16) | 3u)) break;
+        if (i + 2 < n_kb) load(i + 2);   // everyone has read block i
+        ptx::tc_fence_after_sync();
+        const uint32_t a = tmem_base + kTmemL + s * 3 * kPartCols, b = ptx::smem_u32(smem + s * C::kStage);
+        const uint32_t d = tmem_base + s * BN;
+        // parts 0 hi, 1 mid, 2 lo: the small products first, hi * hi last
+        constexpr int kPl[6] = {2, 0, 1, 1, 0, 0}, kPc[6] = {0, 2, 1, 0, 1, 0};
+#pragma unroll
+        for (int q = 0; q < 6; ++q)
+#pragma unroll
+          for (int kk = 0; kk < kBK / 16; ++kk) {
+            const uint32_t bp = b + kPc[q] * C::kPart;
+            const uint64_t db = wt ? ptx::smem_desc_sw128(bp + kk * 32, 16, 1024)
+                                   : ptx::smem_desc_sw128(bp + kk * 2048, kChunkBytes, 1024);
+            mma_bf16_ts(d, a + kPl[q] * kPartCols + kk * 8, db, idesc, (q == 0 && kk == 0) ? 0u : 1u);
+          }
+        ptx::mma_commit(&done[s]);
+      }
+    }
+    __syncwarp();
+  }
+  for (int i = 0; i < n_kb && ok && warp < kWarps; ++i) {
+    // (the MMAs that read this stage of parts have completed: their accumulator was drained)
+    const int s = i & 1;
+    ok = __all_sync(0xffffffffu,
+                    ptx::mbar_wait(&full[s], static_cast<uint32_t>(i >> 1) & 1u, jobs.status, (7u << 16) | 2u));
+    if (!ok) break;
+    if (is_l) {
+      const float* const src = reinterpret_cast<const float*>(raw + s * C::kRaw) + (warp >> 2) * 32 * kLanes + quarter * 32 + lane;
+      const uint32_t dst = tmem_base + lane_bits + kTmemL + s * 3 * kPartCols + (warp >> 2) * 16;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {   // 16 k's
+        float v[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = src[(16 * h + j) * kLanes];
+#pragma unroll
+        for (int part = 0; part < 3; ++part) {
+          uint32_t w[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) w[j] = take_part(v[2 * j], v[2 * j + 1]);
+          tmem_st_x8(dst + part * kPartCols + h * 8, w);
+        }
+      }
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    } else {
+      const float4* const src = reinterpret_cast<const float4*>(raw + s * C::kRaw + C::kRawL) + tid;
+      uint8_t* const dst = smem + s * C::kStage + to;
+#pragma unroll
+      for (int q = 0; q < C::kPieces; ++q) {
+        float4 v = src[q * 256];
+#pragma unroll
+        for (int part = 0; part < 3; ++part) {
+          const uint32_t w0 = take_part(v.x, v.y), w1 = take_part(v.z, v.w);
+          *reinterpret_cast<uint2*>(dst + q * hop + part * C::kPart) = make_uint2(w0, w1);
+        }
+      }
+      ptx::fence_proxy_async_smem();   // the tensor core reads the parts through the async proxy
+    }
+    ptx::tc_fence_before_sync();
+    __syncwarp();
+    if (lane == 0) ptx::mbar_arrive(&ready[s]);
+    if (i > 0) drain(i - 1);   // under the MMAs just issued
+  }
+  if (ok && warp < kWarps) drain(n_kb - 1);
+
+  const long long n0 = c0 + group * C::kCols;   // this thread's columns
+  bool bad = false;
+#pragma unroll
+  for (int j = 0; j < C::kCols; ++j) bad |= !(fabsf(sum[j]) <= 3.402823466e38f);
+  if (bad && ok && l < lanes && warp < kWarps) {
+    const long long k00 = static_cast<long long>(kb0) * kBK;
+    const long long k1 = static_cast<long long>(kb1) * kBK < g.K ? static_cast<long long>(kb1) * kBK : g.K;
+    const long long ck = wt ? 1 : cols, cc = wt ? g.K : 1;
+#pragma unroll
+    for (int j = 0; j < C::kCols; ++j) {
+      float again = 0.f;
+      if (n0 + j < cols)
+        for (long long k = k00; k < k1; ++k) again = fmaf(L[k * lanes + l], Cm[k * ck + (n0 + j) * cc], again);
+      sum[j] = again;
+    }
+  }
+  ptx::tc_fence_before_sync();
+  __syncthreads();   // every read of TMEM and, the MMAs being done, of shared memory has ended
+  if (warp == 0) ptx::tmem_dealloc(tmem_base, kTmemCols);
+  // The next kernel may start, as late as this: CTAs that come early, while some SMs are
+  // idle, would all settle on those.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (warp == kWarps) return;
+  float* const D = g.D + chunk * g.M * g.N;
+  if (wt) {   // a warp 32 numbers of a row at a time
+#pragma unroll
+    for (int j = 0; j < C::kCols; ++j)
+      if (l < lanes && n0 + j < cols) D[(n0 + j) * lanes + l] = sum[j];
+  } else {    // through shared memory, a warp its own 32 rows, so that a store covers whole rows
+    constexpr int kRowPieces = C::kCols / 4;
+    float4* const mine = reinterpret_cast<float4*>(smem) + warp * 32 * kRowPieces;
+#pragma unroll
+    for (int c = 0; c < kRowPieces; ++c)
+      mine[lane * kRowPieces + (c ^ (lane & (kRowPieces - 1)))] =
+          make_float4(sum[4 * c], sum[4 * c + 1], sum[4 * c + 2], sum[4 * c + 3]);
+    __syncwarp();
+    const int c = lane % kRowPieces;
+#pragma unroll
+    for (int r0 = 0; r0 < 32; r0 += 32 / kRowPieces) {
+      const int row = r0 + lane / kRowPieces;
+      const long long gm = l0 + quarter * 32 + row, gn = n0 + 4 * c;
+      if (gm < lanes && gn < cols)
+        *reinterpret_cast<float4*>(D + gm * cols + gn) = mine[row * kRowPieces + (c ^ (row & (kRowPieces - 1)))];
+    }
+  }
+}
+
+}  // namespace split
+
+template <int BN>
+static int launch_bn(const GemmFp32Jobs& js, int n, cudaStream_t stream) {
+  using C = split::Cfg<BN>;
+  split::Maps maps;
+  for (int i = 0; i < n; ++i) {
+    const GemmFp32Job& g = js.j[i];
+    if (g.a_mn) {
+      if (int e = encode_f32_matrix_map(&maps.l[i], g.A, g.K, g.M, split::kBK, split::kLanes)) return e;
+      if (int e = encode_f32_matrix_map(&maps.c[i], g.B, g.K, g.N, split::kBK, BN)) return e;
+    } else {
+      if (int e = encode_f32_matrix_map(&maps.l[i], g.B, g.K, g.N, split::kBK, split::kLanes)) return e;
+      if (int e = encode_f32_matrix_map(&maps.c[i], g.A, g.M, g.K, BN, split::kBK)) return e;
+    }
+  }
+  static PerDevice configured;
+  const auto kern = split::gemm_fp32_split_kernel<BN>;
+  if (int e = allow_dynamic_smem(configured, reinterpret_cast<const void*>(kern), C::kSmem)) return e;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3(js.items);
+  cfg.blockDim = dim3(split::kThreads);
+  cfg.dynamicSmemBytes = C::kSmem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  LBP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, js, maps));
+  count_launch();
+  return LBP_OK;
+}
+
+int launch_gemm_fp32_split(const GemmFp32Jobs& js, int n, int bn, cudaStream_t stream) {
+  return bn == 64 ? launch_bn<64>(js, n, stream) : launch_bn<128>(js, n, stream);
+}
+
+}  // namespace lbp

@@ -117,6 +117,25 @@ int encode_matrix_tensor_map(CUtensorMap* map, const void* base, long long rows,
   return LBP_OK;
 }
 
+int encode_f32_matrix_map(CUtensorMap* map, const void* base, long long rows, long long cols, int box_rows,
+                          int box_cols) {
+  EncodeTiledFn enc;
+  if (int e = get_encode_fn(&enc)) return e;
+  const cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
+  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(cols) * 4};
+  const cuuint32_t box[2] = {static_cast<cuuint32_t>(box_cols), static_cast<cuuint32_t>(box_rows)};
+  const cuuint32_t estr[2] = {1u, 1u};
+  const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims, strides, box, estr,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    set_last_cuda_error(static_cast<cudaError_t>(r));
+    note_cuda_failure(static_cast<cudaError_t>(r), __FILE__, __LINE__);
+    return LBP_ERR_CUDA;
+  }
+  return LBP_OK;
+}
+
 static int check_grid(int B, int H, int W, int C, int k, int dtype) {
   if (int e = check_order(k)) return e;
   if (dtype != LBP_F32 && dtype != LBP_BF16) return LBP_ERR_DTYPE;
@@ -257,7 +276,7 @@ static int run_fullrank(const void* x, const void* g_y, const void* W, void* g_x
   if (L.dtype == LBP_F32) {   // Eq. 2, both products
     GemmFp32 jobs[2];
     products_fp32(x, g_y, W, g_x, g_W, L, T, jobs);
-    if (int e = launch_gemm_fp32(jobs, 2, sk, lay.splitk_bytes, stream)) return e;
+    if (int e = launch_gemm_fp32(jobs, 2, sk, lay.splitk_bytes, status, stream)) return e;
     if (int e = mark_phase(3, stream)) return e;
     return mark_phase(4, stream);
   }
@@ -869,7 +888,7 @@ static int run_core(const void* x, const void* x_hat_in, const void* g_y, const 
     // steps 3 and 4
     GemmFp32 jobs[2];
     products_fp32(x_hat, gy_hat, W, gx_hat, g_W, L, lay.rows, jobs);
-    if (int e = launch_gemm_fp32(jobs, 2, sk, lay.splitk_bytes, st)) return e;
+    if (int e = launch_gemm_fp32(jobs, 2, sk, lay.splitk_bytes, status, st)) return e;
     if (int e = mark_phase(3, st)) return e;
     if (int e = mark_phase(4, st)) return e;
     if (int e = launch_expand(gx_hat, /*in_f32=*/true, g_x, L.dtype, L.B, L.H, L.W, L.Cin, plan, st,

@@ -125,6 +125,8 @@ static TuneOptions read_tune_options() {
                 std::sscanf(e, "%d,%d,%d", &t.tiles_bnw, &t.tiles_bnx, &t.tiles_splits) == 3;
   e = std::getenv("LBP_BATCH_PROJ_SMS");
   t.batch_proj_sms = e != nullptr ? std::atoi(e) : -1;
+  e = std::getenv("LBP_FP32_FORM");
+  t.fp32_form = e != nullptr ? std::atoi(e) : -1;
   return t;
 }
 static TuneOptions& tune_options_slot() {

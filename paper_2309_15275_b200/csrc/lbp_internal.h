@@ -120,6 +120,10 @@ inline bool is_dense(const lbp_view* v) { return v == nullptr || v->token == 0; 
 int encode_matrix_tensor_map(CUtensorMap* map, const void* base, long long rows, long long cols,
                              int box_rows, long long pitch = 0);
 
+// 2-D row-major fp32 matrix (rows, cols), no swizzle.
+int encode_f32_matrix_map(CUtensorMap* map, const void* base, long long rows, long long cols, int box_rows,
+                          int box_cols);
+
 // ---- kernel launchers (each returns an lbp_status) ------------------------
 // Row q of block blk of a projected tensor is row blk * r + q.
 // `scale` multiplies the +-1 sums; 0 selects 1/k, the orthonormal coefficients of Eq. 6.
@@ -185,7 +189,7 @@ struct GemmFp32 {
   long long M, N, K;
   bool a_mn;
 };
-int launch_gemm_fp32(const GemmFp32* jobs, int n, float* ws, size_t ws_bytes, cudaStream_t stream);
+int launch_gemm_fp32(const GemmFp32* jobs, int n, float* ws, size_t ws_bytes, uint32_t* status, cudaStream_t stream);
 // Scratch for the K slices these take at best (with less, K is sliced less or not at all).
 size_t gemm_fp32_ws_bytes(const GemmFp32* jobs, int n);
 size_t gemm_splitk_ws_bytes(long long M, long long N, long long K, int in_dtype);
@@ -237,6 +241,8 @@ int launch_bias_grad(const void* a, long long n_a, int r, int q, TokenMap ta, do
 //   LBP_PAIR=0           one-CTA products kernel also on wide layers
 //   LBP_PROJECT_UMMA=0   bf16 projection by additions on the CUDA cores instead of tcgen05
 //   LBP_FUSED_TILES=a,b,c  column tiles of the two products and K slices of g_W
+//   LBP_FP32_FORM=n      fp32 products: 0 on FFMA, 1 / 2 split operands on tcgen05 in tiles
+//                        of 128 x 64 / 128 x 128 (unset = chosen by size)
 //   LBP_FUSED_VERBOSE=1  print the chosen tile plan
 //   LBP_BATCH_PROJ_SMS=n lbp_backward_batch: SMs given to the projection of the next
 //                        layer while the products kernel of a layer runs (0 = one
@@ -247,6 +253,7 @@ struct TuneOptions {
   bool fused, pair, umma, verbose, has_tiles;
   int tiles_bnw, tiles_bnx, tiles_splits;
   int batch_proj_sms;   // -1 = library default
+  int fp32_form;        // -1 = chosen by size
 };
 const TuneOptions& tune_options();
 void reload_tune_options();   // test hook: read the environment again

@@ -426,3 +426,44 @@ def test_bias_gradient_over_many_tokens(dev, dtype, B, H, W, C, ci):
                             gx_extra=torch.empty_like(xe), g_W=gw)
         # fp64 sums, one rounding to fp32
         assert rel(g_b, O.bias_grad(f64(gy), f64(ge)) + 3.0 * beta) <= 2.0 ** -23
+
+
+@pytest.fixture
+def fp32_form(request, monkeypatch):
+    monkeypatch.setenv("LBP_FP32_FORM", str(request.param))
+    lbp.lbp_test_reload_env()
+    yield request.param
+    monkeypatch.undo()
+    lbp.lbp_test_reload_env()
+
+
+@pytest.mark.parametrize("fp32_form", [0, 1, 2], indirect=True)
+@pytest.mark.parametrize("ci,co,T", [(4, 4, 1), (132, 68, 65), (64, 260, 1000), (320, 128, 256), (128, 1028, 60)])
+def test_fp32_product_forms(dev, fp32_form, ci, co, T):
+    # tiles and k-blocks of every form with 4 lanes, columns or k's past an edge, K slices of
+    # unequal length.  Exact mode: D of either product is the result itself
+    x, gy, w = layer(dev, 81, 1, 1, T, ci, co, dtype=torch.float32)
+    for scale in (1.0, 2.0 ** -100, 2.0 ** 120):   # the parts down to subnormal, the sums up to 2^124
+        gys = gy * scale
+        gx, gw = lbp.lbp_backward_fullrank(x, gys, w, 8)
+        ox, ow = O.backward_exact(f64(x), f64(gys), f64(w))
+        assert rel(gx, ox) <= F32 and rel(gw, ow) <= F32
+
+
+@pytest.mark.parametrize("fp32_form", [1, 2], indirect=True)
+def test_fp32_infinities_as_term_by_term(dev, fp32_form):
+    # infinities and NaN reach the sums they belong to and no others; numbers whose bf16
+    # neighbour is infinite stay finite
+    x, gy, w = layer(dev, 91, 1, 1, 200, 136, 200, dtype=torch.float32)
+    x[0, 0, 3, 5] = float("inf")
+    gy[0, 0, 150, 131] = float("nan")
+    w[7, 130] = -float("inf")
+    gy[0, 0, 70, :] = 0.0
+    x[0, 0, 70, 9] = 3.4e38
+    gx, gw = lbp.lbp_backward_fullrank(x, gy, w, 8)
+    X, G, Wd = x.reshape(-1, 136).double(), gy.reshape(-1, 200).double(), w.double()
+    for got, want in ((gx.reshape(-1, 136).double(), G @ Wd), (gw.double(), G.t() @ X)):
+        fin = torch.isfinite(want)
+        assert torch.equal(torch.isfinite(got), fin) and torch.equal(torch.isnan(got), torch.isnan(want))
+        assert torch.equal(got[~fin & ~torch.isnan(want)], want[~fin & ~torch.isnan(want)])
+        assert ((got - want)[fin].norm() / want[fin].norm()).item() <= F32
