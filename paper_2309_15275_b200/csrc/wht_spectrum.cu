@@ -38,6 +38,9 @@ __global__ void __launch_bounds__(MmaCfg<K>::kWarps * 32, 1)
 
   extern __shared__ uint8_t smem_raw[];
   __shared__ double e_sm[R];
+  // the +-1 basis matrix, two tokens a word; rows so far apart that a fragment's 8 rows x 4
+  // words lie in different banks
+  __shared__ uint32_t basis[R][K * K / 2 + 4];
   uint8_t* tiles = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(tiles + NW * S * Cfg::kTileBytes);
@@ -52,11 +55,13 @@ __global__ void __launch_bounds__(MmaCfg<K>::kWarps * 32, 1)
     for (int s = 0; s < S; ++s) ptx::mbar_init(&my_bars[s], 1);
     ptx::mbar_fence_init();
   }
+  // the next call's small kernel may come as early as this (it waits for this one)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (threadIdx.x == 0) ptx::prefetch_tensormap(&tmap);
   for (int i = threadIdx.x; i < R; i += NW * 32) e_sm[i] = 0.0;
   __syncthreads();
 
-  const uint32_t first = blockIdx.x * NW + warp;
+  const uint32_t first = warp * gridDim.x + blockIdx.x;   // a last round that is not full falls to every SM
   const uint32_t stride = gridDim.x * NW;
   const uint32_t n_my = first < p.n_items ? (p.n_items - first + stride - 1) / stride : 0;
   const uint32_t nch = static_cast<uint32_t>(p.n_chunks[0]);
@@ -74,7 +79,14 @@ __global__ void __launch_bounds__(MmaCfg<K>::kWarps * 32, 1)
     for (uint32_t i = 0; i < S && i < n_my; ++i) issue(i, i);
   }
 
-  // A fragments (rows of the +-1 basis matrix), as in the projection kernel
+  // A fragments: rows of the basis matrix, laid out once for all warps under the first loads
+  // (every warp by itself, a thread works out 128 signs: 128 x 16 x 16 tokens of 768 channels
+  // 15.0 us a call, so 14.1: 3.6 TB/s, the pass itself about 10 us of it)
+  for (int i = threadIdx.x; i < R * (K * K / 2); i += NW * 32) {
+    const int q = i / (K * K / 2), w = i % (K * K / 2);
+    basis[q][w] = basis_bits<K>(mp, q, R, 2 * w) | (basis_bits<K>(mp, q, R, 2 * w + 1) << 16);
+  }
+  __syncthreads();
   uint32_t afrag[NG][GM][KS][4];
 #pragma unroll
   for (int ng = 0; ng < NG; ++ng)
@@ -83,11 +95,8 @@ __global__ void __launch_bounds__(MmaCfg<K>::kWarps * 32, 1)
 #pragma unroll
       for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int q = (ng * GM + mt) * 16 + g + (j & 1) * 8;
-          const int tok = ks * 16 + 2 * tq + (j >> 1) * 8;
-          afrag[ng][mt][ks][j] = basis_bits<K>(mp, q, R, tok) | (basis_bits<K>(mp, q, R, tok + 1) << 16);
-        }
+        for (int j = 0; j < 4; ++j)
+          afrag[ng][mt][ks][j] = basis[(ng * GM + mt) * 16 + g + (j & 1) * 8][ks * 8 + tq + (j >> 1) * 4];
 
   // per-thread sums of squared responses: rows g and g + 8 of every m16 tile
   float e[NG][GM][2];
@@ -210,11 +219,13 @@ __global__ void __launch_bounds__(MmaCfg<16>::kWarps * 32, 1)
     for (int s = 0; s < S; ++s) ptx::mbar_init(&my_bars[s], 1);
     ptx::mbar_fence_init();
   }
+  // the next call's small kernel may come as early as this (it waits for this one)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (threadIdx.x == 0) ptx::prefetch_tensormap(&tmap);
   for (int i = threadIdx.x; i < R; i += NW * 32) e_sm[i] = 0.0;
   __syncthreads();
 
-  const uint32_t first = blockIdx.x * NW + warp;
+  const uint32_t first = warp * gridDim.x + blockIdx.x;   // a last round that is not full falls to every SM
   const uint32_t stride = gridDim.x * NW;
   const uint32_t n_my = first < p.n_items ? (p.n_items - first + stride - 1) / stride : 0;
   const uint32_t nch = static_cast<uint32_t>(p.n_chunks[0]);
@@ -304,19 +315,17 @@ __global__ void __launch_bounds__(MmaCfg<16>::kWarps * 32, 1)
 
 // The sums start from zero.  The kernel that adds to them is launched at once behind this
 // one and waits for it only before it adds, so the launch and the few stores lie under its
-// loads; what lies ahead of this kernel has completed before it starts.  Against a memset
-// ahead of the kernel: 64 x 16 x 16 tokens of 768 channels, order 8, 14.4 -> 12.4 us, order 4
-// 10.3 -> 8.4.  (Ahead of the two-pass form a memset is the faster one: 69 us against 72 for
-// 128 x 16 x 16 tokens of 768 fp32 channels.)
+// loads.  This one lets it start only after its own wait: what lies ahead of it (whatever
+// wrote the tensor, and an earlier call that still adds to the same sums) has then completed.
+// It is itself launched under the end of what lies ahead.  128 x 16 x 16 tokens of 768 channels
+// (50 MB), order 8, call behind call, with an even last round of items: 16.4 -> 15.0 us.
+// Against a memset ahead of the kernel: 64 x 16 x 16 tokens of 768 channels, order 8, 14.4 ->
+// 12.4 us, order 4 10.3 -> 8.4.  (Ahead of the two-pass form a memset is the faster one: 69 us
+// against 72 for 128 x 16 x 16 tokens of 768 fp32 channels.)
 __global__ void zero_energy_kernel(double* energy, int n) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (static_cast<int>(threadIdx.x) < n) energy[threadIdx.x] = 0.0;
-}
-static int launch_zero_energy(double* energy, int n, cudaStream_t stream) {
-  zero_energy_kernel<<<1, 256, 0, stream>>>(energy, n);
-  count_launch();
-  LBP_CUDA_TRY(cudaGetLastError());
-  return LBP_OK;
 }
 
 // A launch that may start while the kernel ahead of it on the stream still runs.
@@ -337,6 +346,11 @@ static int launch_behind(void (*kern)(Params...), int grid, int threads, int sme
   LBP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
   count_launch();
   return LBP_OK;
+}
+
+static int launch_zero_energy(double* energy, int n, cudaStream_t stream) {
+  static PerDevice configured;
+  return launch_behind(zero_energy_kernel, 1, 256, 0, stream, configured, energy, n);
 }
 
 bool spectrum_mma_supported(int k, int dtype) {
