@@ -502,14 +502,6 @@ static int plan_batch(int n, const lbp_layer* layers, const lbp_basis* set, int 
   }
   bp.side = true;
 
-  // What the side stream has to hide, under the model, to be worth its events and the launches
-  // in plain stream order.  Hidden, and a call on the side stream and on one (us, B200): 768 ->
-  // 3072 and 3072 -> 768 with 1024 tokens 8 47.4 and 43.5, 8192 tokens 16 71.8 and 67.3, 16384
-  // tokens 24 106.9 and 109.5; 192 -> 768 and 768 -> 192 with 1568 tokens 6 28.9 and 20.8; 256 ->
-  // 1024 and 1024 -> 256, 25088 tokens, 17 70.2 and 68.7; four layers of 768 with 2048 tokens 24
-  // 74.7 and 75.9, of 192 with 50176 tokens 56 133 and 148.
-  constexpr double kHideUs = 17.0;
-  double in_turn = 0, beside = 0;
   // cost of running problem a's products kernel beside problem b's projection,
   // and the SM split that gives it
   auto pair_cost = [&](int a, int b, int* ps_out) {
@@ -569,25 +561,10 @@ static int plan_batch(int n, const lbp_layer* layers, const lbp_basis* set, int 
       if (ok)
         for (int i = 0; i < n; ++i) best_perm[i] = o[i];
     }
-    beside = best;
-    for (int i = 0; i < n; ++i) in_turn += first[i] + last[i];
     for (int i = 0; i < n; ++i) bp.order[i] = best_perm[i];
     for (int i = 1; i < n; ++i) bp.proj_sms[i] = pps[best_perm[i - 1]][best_perm[i]];
   } else {
-    for (int i = 0; i < n; ++i) {
-      const double proj = fused_projection_model_us(layers[i], plans[i], sms);
-      const double prod = fused_products_model_us(layers[i], plans[i], sms / 2);
-      in_turn += proj + prod;
-      beside += i == 0 ? proj : pair_cost(i - 1, i, &bp.proj_sms[i]);
-      if (i == n - 1) beside += prod;
-    }
-  }
-  if (want < 0 && keyed && in_turn - beside < kHideUs) {
-    bp.side = false;
-    for (int i = 0; i < n; ++i) {
-      bp.order[i] = i;
-      bp.proj_sms[i] = 0;
-    }
+    for (int i = 1; i < n; ++i) pair_cost(i - 1, i, &bp.proj_sms[i]);
   }
   if (tune_options().verbose) {
     fprintf(stderr, "lbp batch: order");
