@@ -177,7 +177,8 @@ constexpr Form kForms[] = {
 };
 
 struct Plan {
-  int form, per;
+  int form;
+  long long per;
   size_t planes;   // bytes
 };
 
@@ -219,14 +220,13 @@ Plan make_plan(const GemmFp32* job, int n, size_t room) {
   if (room > kRoom) room = kRoom;
   Plan best{};
   double best_t = -1.0;
-  const int forced = tune_options().fp32_form;
+  bool fits = true;   // TMA coordinates are 32-bit
+  for (int i = 0; i < n; ++i)
+    for (long long d : {job[i].M, job[i].N, job[i].K}) fits &= d < (1ll << 31) - 256;
+  const int forced = fits ? tune_options().fp32_form : 0;
   for (int f = 0; f < 3; ++f) {
     const Form& form = kForms[f];
     if (forced >= 0 && f != forced) continue;
-    bool fits = true;   // TMA coordinates are 32-bit
-    for (int i = 0; i < n; ++i)
-      for (long long d : {job[i].M, job[i].N, job[i].K}) fits &= d < (1ll << 31) - 256;
-    if (f > 0 && !fits) continue;
     long long kb[2] = {0, 0}, most = 1;
     for (int i = 0; i < n; ++i) {
       kb[i] = ceil_div(job[i].K, form.bk);
@@ -254,7 +254,7 @@ Plan make_plan(const GemmFp32* job, int n, size_t room) {
                                     : form.launch_us + makespan(items[0], item_t[0], items[1], item_t[1]);
       if (best_t < 0 || t < best_t) {
         best_t = t;
-        best = Plan{f, static_cast<int>(per), bytes};
+        best = Plan{f, per, bytes};
       }
     }
   }
@@ -285,7 +285,7 @@ Plan plan(const GemmFp32* job, int n, size_t room) {
   e.forced = tune_options().fp32_form;
   e.plan = make_plan(job, n, room);
   if (tune_options().verbose)
-    fprintf(stderr, "lbp fp32 products plan: %lldx%lldx%lld, %lldx%lldx%lld: form %d, %d k-blocks an item, planes %zu\n",
+    fprintf(stderr, "lbp fp32 products plan: %lldx%lldx%lld, %lldx%lldx%lld: form %d, %lld k-blocks an item, planes %zu\n",
             dims[0], dims[1], dims[2], dims[3], dims[4], dims[5], e.plan.form, e.plan.per, e.plan.planes);
   next = (next + 1) % 16;
   filled = filled < 16 ? filled + 1 : 16;
@@ -296,6 +296,17 @@ Plan plan(const GemmFp32* job, int n, size_t room) {
 
 size_t gemm_fp32_ws_bytes(const GemmFp32* job, int n) {
   return plan(job, n, static_cast<size_t>(-1)).planes;
+}
+
+void gemm_fp32_plan(const GemmFp32 (&job)[2], size_t room, int64_t* out6) {
+  const Plan pl = plan(job, 2, room);
+  out6[0] = pl.form;
+  out6[1] = static_cast<int64_t>(pl.planes);
+  for (int i = 0; i < 2; ++i) {
+    const long long kb = ceil_div(job[i].K, kForms[pl.form].bk), chunks = chunks_of(kb, pl.per);
+    out6[2 + 2 * i] = ceil_div(kb, chunks);
+    out6[3 + 2 * i] = chunks;
+  }
 }
 
 int launch_gemm_fp32(const GemmFp32* job, int n, float* ws, size_t ws_bytes, uint32_t* status, cudaStream_t stream) {

@@ -688,6 +688,16 @@ int lbp_test_per_device(const int* devices, int n, uint8_t* done) {
   return LBP_OK;
 }
 
+int lbp_test_fp32_plan(int Cin, int Cout, long long rows, size_t room, int64_t* out6) {
+  lbp_layer L{};
+  L.Cin = Cin;
+  L.Cout = Cout;
+  GemmFp32 jobs[2];
+  products_fp32(nullptr, nullptr, nullptr, nullptr, nullptr, L, rows, jobs);
+  gemm_fp32_plan(jobs, room, out6);
+  return LBP_OK;
+}
+
 int lbp_test_reload_env(void) {
   reload_tune_options();
   return LBP_OK;

@@ -192,6 +192,7 @@ struct GemmFp32 {
 int launch_gemm_fp32(const GemmFp32* jobs, int n, float* ws, size_t ws_bytes, uint32_t* status, cudaStream_t stream);
 // Scratch for the K slices these take at best (with less, K is sliced less or not at all).
 size_t gemm_fp32_ws_bytes(const GemmFp32* jobs, int n);
+void gemm_fp32_plan(const GemmFp32 (&jobs)[2], size_t room, int64_t* out6);   // test hook
 size_t gemm_splitk_ws_bytes(long long M, long long N, long long K, int in_dtype);
 // D[i] = beta * D[i] + sum over `splits` fp32 planes of mn elements each (mn a multiple
 // of 4), in plane order; D is not read when beta is 0.  `late`: the next kernel on the
@@ -242,7 +243,7 @@ int launch_bias_grad(const void* a, long long n_a, int r, int q, TokenMap ta, do
 //   LBP_PROJECT_UMMA=0   bf16 projection by additions on the CUDA cores instead of tcgen05
 //   LBP_FUSED_TILES=a,b,c  column tiles of the two products and K slices of g_W
 //   LBP_FP32_FORM=n      fp32 products: 0 on FFMA, 1 / 2 split operands on tcgen05 in tiles
-//                        of 128 x 64 / 128 x 128 (unset = chosen by size)
+//                        of 128 x 64 / 128 x 128 (unset or anything else = chosen by size)
 //   LBP_FUSED_VERBOSE=1  print the chosen tile plan
 //   LBP_BATCH_PROJ_SMS=n lbp_backward_batch: SMs given to the projection of the next
 //                        layer while the products kernel of a layer runs (0 = one

@@ -401,3 +401,30 @@ def test_module_attributes_and_operands_as_torch_takes_them():
         lin.bases = wrong
         with pytest.raises(ValueError):
             lin(x.flatten(1, 2))
+
+
+@pytest.mark.parametrize("ci,co,rows", [(64, 64, 5), (448, 1792, 640), (768, 3072, 32768), (8, 8, 2 ** 31 - 256),
+                                        (8, 8, 2 ** 38)])
+def test_fp32_products_are_planned_whatever_the_switch_says(monkeypatch, ci, co, rows):
+    def plan(form, room):
+        if form is None:
+            monkeypatch.delenv("LBP_FP32_FORM", raising=False)
+        else:
+            monkeypatch.setenv("LBP_FP32_FORM", form)
+        lbp.lbp_test_reload_env()
+        return lbp.lbp_test_fp32_plan(ci, co, rows, room)
+    try:
+        for room in (0, 1 << 20, 2 ** 63):
+            free = plan(None, room)
+            assert all(plan(form, room) == free for form in ("3", "-1", "", "x", "1x", "10"))
+            for form in range(3):
+                got = plan(str(form), room)
+                # sizes beyond a tensor map's coordinates are left to the form without one
+                assert got["form"] == (form if rows < 2 ** 31 - 256 else 0)
+                bk = 64 if got["form"] else 32
+                for kb, items, K in ((got["gx_kb"], got["gx_items"], co), (got["gw_kb"], got["gw_items"], rows)):
+                    assert kb >= 1 and items >= 1 and kb * items >= -(-K // bk) > kb * (items - 1)
+                    assert items == 1 or room > 0
+    finally:
+        monkeypatch.undo()
+        lbp.lbp_test_reload_env()
