@@ -683,11 +683,12 @@ def lbp_test_reload_env() -> None:
     _check(_lib().lbp_test_reload_env(), "lbp_test_reload_env")
 
 
-def lbp_test_stall_products(on, projection: bool = False) -> None:
+def lbp_test_stall_products(on, projection: bool = False, fp32: bool = False) -> None:
     """Test hook (include/lbp_test_hooks.h): while on, the products kernel's TMA
-    producers (with `projection`: those of the tcgen05 projection kernel) issue
-    nothing, so the call ends in LBP_ERR_TIMEOUT (lbp_poll_status)."""
-    mode = (2 if projection else 1) if on else 0
+    producers (with `projection`: those of the tcgen05 projection kernel; with `fp32`:
+    those of the fp32 products on the tensor cores) issue nothing, so the call ends in
+    LBP_ERR_TIMEOUT (lbp_poll_status)."""
+    mode = (2 if projection else 4 if fp32 else 1) if on else 0
     _check(_lib().lbp_test_stall_products(mode), "lbp_test_stall_products")
 
 

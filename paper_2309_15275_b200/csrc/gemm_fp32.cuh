@@ -19,9 +19,10 @@ struct GemmFp32Jobs {
   GemmFp32Job j[2];
   int32_t items0, items;          // items of the first job, of both
   uint32_t* status;
+  int32_t test_stall;             // failure injection (lbp_test_stall_products): no loads
 };
 
 // n: one job or two; bn: columns of a tile, 64 or 128.
-int launch_gemm_fp32_split(const GemmFp32Jobs& js, int n, int bn, cudaStream_t stream);
+int launch_gemm_fp32_split(GemmFp32Jobs& js, int n, int bn, cudaStream_t stream);
 
 }  // namespace lbp

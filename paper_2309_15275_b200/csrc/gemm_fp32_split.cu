@@ -174,12 +174,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
   if (warp == kWarps) {
     if (ptx::elect_one()) {
       const uint32_t idesc = ptx::idesc_bf16(kLanes, BN, false, !wt);
-      load(0);
-      if (n_kb > 1) load(1);
+      const int n = jobs.test_stall ? 0 : n_kb;
+      int loads = 0, begun = 0;   // blocks fetched, blocks whose MMAs have been issued
+      for (; loads < 2 && loads < n; ++loads) load(loads);
       for (int i = 0; i < n_kb; ++i) {
         const int s = i & 1;
         if (!ptx::mbar_wait(&ready[s], static_cast<uint32_t>(i >> 1) & 1u, jobs.status, (7u << 16) | 3u)) break;
-        if (i + 2 < n_kb) load(i + 2);   // everyone has read block i
+        if (i + 2 < n_kb) load(loads++);   // everyone has read block i
         ptx::tc_fence_after_sync();
         const uint32_t a = tmem_base + kTmemL + s * 3 * kPartCols, b = ptx::smem_u32(smem + s * C::kStage);
         const uint32_t d = tmem_base + s * BN;
@@ -195,7 +196,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
             mma_bf16_ts(d, a + kPl[q] * kPartCols + kk * 8, db, idesc, (q == 0 && kk == 0) ? 0u : 1u);
           }
         ptx::mma_commit(&done[s]);
+        begun = i + 1;
       }
+      // whatever made the others leave: nothing is under way in this CTA's memories when it ends
+      for (int i = begun; i < loads; ++i)
+        ptx::mbar_wait(&full[i & 1], static_cast<uint32_t>(i >> 1) & 1u, jobs.status, (7u << 16) | 4u);
+      if (begun > 0)
+        ptx::mbar_wait(&done[(begun - 1) & 1], static_cast<uint32_t>((begun - 1) >> 1) & 1u, jobs.status, (7u << 16) | 5u);
     }
     __syncwarp();
   }
@@ -260,7 +267,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
     }
   }
   ptx::tc_fence_before_sync();
-  __syncthreads();   // every read of TMEM and, the MMAs being done, of shared memory has ended
+  __syncthreads();   // every load, MMA and read of TMEM and shared memory has ended
   if (warp == 0) ptx::tmem_dealloc(tmem_base, kTmemCols);
   // The next kernel may start, as late as this: CTAs that come early, while some SMs are
   // idle, would all settle on those.
@@ -291,6 +298,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
 }
 
 }  // namespace split
+
+static thread_local bool g_test_stall = false;
+void set_test_stall_fp32(bool on) { g_test_stall = on; }
 
 template <int BN>
 static int launch_bn(const GemmFp32Jobs& js, int n, cudaStream_t stream) {
@@ -324,7 +334,8 @@ static int launch_bn(const GemmFp32Jobs& js, int n, cudaStream_t stream) {
   return LBP_OK;
 }
 
-int launch_gemm_fp32_split(const GemmFp32Jobs& js, int n, int bn, cudaStream_t stream) {
+int launch_gemm_fp32_split(GemmFp32Jobs& js, int n, int bn, cudaStream_t stream) {
+  js.test_stall = g_test_stall ? 1 : 0;
   return bn == 64 ? launch_bn<64>(js, n, stream) : launch_bn<128>(js, n, stream);
 }
 

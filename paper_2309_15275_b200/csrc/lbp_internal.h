@@ -192,6 +192,7 @@ struct GemmFp32 {
 int launch_gemm_fp32(const GemmFp32* jobs, int n, float* ws, size_t ws_bytes, uint32_t* status, cudaStream_t stream);
 // Scratch for the K slices these take at best (with less, K is sliced less or not at all).
 size_t gemm_fp32_ws_bytes(const GemmFp32* jobs, int n);
+void set_test_stall_fp32(bool on);   // test hook (gemm_fp32_split.cu)
 void gemm_fp32_plan(const GemmFp32 (&jobs)[2], size_t room, int64_t* out6);   // test hook
 size_t gemm_splitk_ws_bytes(long long M, long long N, long long K, int in_dtype);
 // D[i] = beta * D[i] + sum over `splits` fp32 planes of mn elements each (mn a multiple

@@ -70,3 +70,34 @@ def test_expired_wait_in_the_projection_kernel():
     got = lbp.lbp_project(t, k, bases, ws=ws)
     assert lbp.lbp_poll_status(ws) == 0
     assert O.rel_fro(f64(got), O.project(f64(t), k, bases)) <= 2e-2
+
+
+@pytest.mark.parametrize("form,Cin,Cout,T", [(1, 64, 128, 100), (2, 448, 256, 640)])
+def test_expired_wait_in_the_fp32_products(monkeypatch, form, Cin, Cout, T):
+    # one k-block an item, and several: no load is issued, both kinds of warp and the issuer
+    # of the MMAs give up, the CTA frees its TMEM, the next call is clean
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    dev = torch.device("cuda:0")
+    monkeypatch.setenv("LBP_FP32_FORM", str(form))
+    lbp.lbp_test_reload_env()
+    try:
+        x = synth.make_tensor((1, 1, T, Cin), ("normal", 1.0), "f32", case_key=2600).to(dev)
+        gy = synth.make_tensor((1, 1, T, Cout), ("normal", 1.0), "f32", case_key=2601).to(dev)
+        w = synth.make_tensor((Cout, Cin), ("normal", 1.0), "f32", case_key=2602).to(dev)
+        ws = lbp.alloc_workspace(x, gy, 8, 64)
+        ws.zero_()
+        lbp.lbp_test_stall_products(True, fp32=True)
+        try:
+            lbp.lbp_backward_fullrank(x, gy, w, 8, ws=ws)
+        finally:
+            lbp.lbp_test_stall_products(False)
+        assert lbp.lbp_poll_status(ws) == LBP_ERR_TIMEOUT
+        assert lbp.lbp_poll_status(ws) == 0
+        gx, gw = lbp.lbp_backward_fullrank(x, gy, w, 8, ws=ws)
+        assert lbp.lbp_poll_status(ws) == 0
+        ox, ow = O.backward_exact(f64(x), f64(gy), f64(w))
+        assert O.rel_fro(f64(gx), ox) <= 1e-6 and O.rel_fro(f64(gw), ow) <= 1e-6
+    finally:
+        monkeypatch.undo()
+        lbp.lbp_test_reload_env()
