@@ -30,8 +30,12 @@
 // 2.4e-7 and 2.5e-7 there, 1.3e-7 and 1.4e-7 here.
 //
 // Infinities, NaN and values next to the largest float leave the parts meaningless
-// (inf - inf, 0 * inf), but they always show as a sum that is not finite: such sums are
-// computed again, term by term with fp32 FMAs.
+// (inf - inf, 0 * inf), but they always show as a sum that is not finite.  A CTA that has one
+// fetches the item's operands once more and its warps form their sums from them with fp32
+// FMAs, term by term; only those that were not finite are replaced.  640 x 448 -> 1792, both
+// products: 22 us, with one NaN in g_y 118, with nothing but NaN 128 (FFMA kernel 60 whatever
+// the values; a serial sum per thread from global memory 980 and 1120); 2048 x 768 -> 3072: 115,
+// 247 and 748 (436; 1690 and 6850).
 #include "gemm_fp32.cuh"
 #include "lbp_internal.h"
 #include "ptx_sm100.cuh"
@@ -108,8 +112,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
   t /= g.chunks;
   const bool wt = g.a_mn == 0;   // L = B, C = A stored (columns, K), D transposed
   const long long lanes = wt ? g.N : g.M, cols = wt ? g.M : g.N;
-  const float* const L = wt ? g.B : g.A;
-  const float* const Cm = wt ? g.A : g.B;
   const long long l0 = static_cast<long long>(t / g.tiles_c) * kLanes, c0 = static_cast<long long>(t % g.tiles_c) * BN;
   const int kb0 = chunk * g.per, kb1 = kb0 + g.per < g.kb ? kb0 + g.per : g.kb, n_kb = kb1 - kb0;
 
@@ -133,13 +135,17 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
   const uint32_t tmem_base = *tmem_slot;
   asm volatile("griddepcontrol.wait;" ::: "memory");   // launched as the kernel ahead ends
 
-  auto load = [&](int i) {   // one thread: block i of the item
-    uint8_t* const dst = raw + (i & 1) * C::kRaw;
-    const int k = (kb0 + i) * kBK;
-    ptx::mbar_expect_tx(&full[i & 1], C::kRaw);   // boxes count in full, also where they hang over an edge (zeros)
-    ptx::tma_load_2d(dst, &maps.l[which], &full[i & 1], static_cast<int32_t>(l0), k);
-    ptx::tma_load_2d(dst + C::kRawL, &maps.c[which], &full[i & 1], wt ? k : static_cast<int32_t>(c0),
+  // One thread: the u-th load of this CTA, block u of the item (and u - n_kb once more from there on).
+  auto load = [&](int u) {
+    uint8_t* const dst = raw + (u & 1) * C::kRaw;
+    const int k = (kb0 + (u < n_kb ? u : u - n_kb)) * kBK;
+    ptx::mbar_expect_tx(&full[u & 1], C::kRaw);   // boxes count in full, also where they hang over an edge (zeros)
+    ptx::tma_load_2d(dst, &maps.l[which], &full[u & 1], static_cast<int32_t>(l0), k);
+    ptx::tma_load_2d(dst + C::kRawL, &maps.c[which], &full[u & 1], wt ? k : static_cast<int32_t>(c0),
                      wt ? static_cast<int32_t>(c0) : k);
+  };
+  auto arrived = [&](int u, uint32_t site) {
+    return ptx::mbar_wait(&full[u & 1], static_cast<uint32_t>(u >> 1) & 1u, jobs.status, (7u << 16) | site);
   };
   // L: a thread has its lane's k's of one half of the block.  C: pieces of four numbers, a
   // warp whole 128-byte lines; row `row` + q * rows of the block, in shared memory `hop` apart.
@@ -171,6 +177,62 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
     }
   };
 
+  // A warp's sums by FMAs from a raw stage, term by term, one k after the other: a thread has
+  // kCols / 4 lanes (in runs of four) by 4 columns, which reads less than a lane by kCols.
+  constexpr int kRuns = C::kCols / 16, kAlong = 8 / kRuns;   // runs of a thread; threads along the lanes
+  const int run = (lane % kAlong) * 4, four = lane / kAlong * 4;
+  auto finite = [](float v) { return fabsf(v) <= 3.402823466e38f; };
+  auto add_terms = [&](int stage, int nk) {
+    const float* const ls = reinterpret_cast<const float*>(raw + stage * C::kRaw) + quarter * 32 + run;
+    const float* const cs = reinterpret_cast<const float*>(raw + stage * C::kRaw + C::kRawL) +
+                            (group * C::kCols + four) * (wt ? kBK : 1);
+#pragma unroll 1
+    for (int k = 0; k < nk; k += 4) {
+      float c[4][4];   // [k][column]
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 v = *reinterpret_cast<const float4*>(wt ? cs + q * kBK + k : cs + (k + q) * BN);
+        if (wt)
+          c[0][q] = v.x, c[1][q] = v.y, c[2][q] = v.z, c[3][q] = v.w;
+        else
+          c[q][0] = v.x, c[q][1] = v.y, c[q][2] = v.z, c[q][3] = v.w;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int h = 0; h < kRuns; ++h) {
+          const float4 v = *reinterpret_cast<const float4*>(ls + (k + q) * kLanes + h * 4 * kAlong);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            sum[h * 16 + j] = fmaf(v.x, c[q][j], sum[h * 16 + j]);
+            sum[h * 16 + 4 + j] = fmaf(v.y, c[q][j], sum[h * 16 + 4 + j]);
+            sum[h * 16 + 8 + j] = fmaf(v.z, c[q][j], sum[h * 16 + 8 + j]);
+            sum[h * 16 + 12 + j] = fmaf(v.w, c[q][j], sum[h * 16 + 12 + j]);
+          }
+        }
+    }
+  };
+  // They replace what the warp's plane in the place of the parts holds (all of it, or what is
+  // not finite there), which then becomes a lane by kCols a thread once more.
+  float* const plane = reinterpret_cast<float*>(smem) + warp * 32;   // [kCols][all lanes of all warps]
+  auto put_terms = [&](bool all) {
+#pragma unroll
+    for (int h = 0; h < kRuns; ++h)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float4* const at = reinterpret_cast<float4*>(plane + (four + j) * kWarps * 32 + h * 4 * kAlong + run);
+        float4 v = *at;
+        if (all || !finite(v.x)) v.x = sum[h * 16 + j];
+        if (all || !finite(v.y)) v.y = sum[h * 16 + 4 + j];
+        if (all || !finite(v.z)) v.z = sum[h * 16 + 8 + j];
+        if (all || !finite(v.w)) v.w = sum[h * 16 + 12 + j];
+        *at = v;
+      }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < C::kCols; ++j) sum[j] = plane[j * kWarps * 32 + lane];
+  };
+
   if (warp == kWarps) {
     if (ptx::elect_one()) {
       const uint32_t idesc = ptx::idesc_bf16(kLanes, BN, false, !wt);
@@ -199,8 +261,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
         begun = i + 1;
       }
       // whatever made the others leave: nothing is under way in this CTA's memories when it ends
-      for (int i = begun; i < loads; ++i)
-        ptx::mbar_wait(&full[i & 1], static_cast<uint32_t>(i >> 1) & 1u, jobs.status, (7u << 16) | 4u);
+      for (int i = begun; i < loads; ++i) arrived(i, 4u);
       if (begun > 0)
         ptx::mbar_wait(&done[(begun - 1) & 1], static_cast<uint32_t>((begun - 1) >> 1) & 1u, jobs.status, (7u << 16) | 5u);
     }
@@ -209,8 +270,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
   for (int i = 0; i < n_kb && ok && warp < kWarps; ++i) {
     // (the MMAs that read this stage of parts have completed: their accumulator was drained)
     const int s = i & 1;
-    ok = __all_sync(0xffffffffu,
-                    ptx::mbar_wait(&full[s], static_cast<uint32_t>(i >> 1) & 1u, jobs.status, (7u << 16) | 2u));
+    ok = __all_sync(0xffffffffu, arrived(i, 2u));
     if (!ok) break;
     if (is_l) {
       const float* const src = reinterpret_cast<const float*>(raw + s * C::kRaw) + (warp >> 2) * 32 * kLanes + quarter * 32 + lane;
@@ -253,21 +313,35 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
   const long long n0 = c0 + group * C::kCols;   // this thread's columns
   bool bad = false;
 #pragma unroll
-  for (int j = 0; j < C::kCols; ++j) bad |= !(fabsf(sum[j]) <= 3.402823466e38f);
-  if (bad && ok && l < lanes && warp < kWarps) {
-    const long long k00 = static_cast<long long>(kb0) * kBK;
-    const long long k1 = static_cast<long long>(kb1) * kBK < g.K ? static_cast<long long>(kb1) * kBK : g.K;
-    const long long ck = wt ? 1 : cols, cc = wt ? g.K : 1;
-#pragma unroll
-    for (int j = 0; j < C::kCols; ++j) {
-      float again = 0.f;
-      if (n0 + j < cols)
-        for (long long k = k00; k < k1; ++k) again = fmaf(L[k * lanes + l], Cm[k * ck + (n0 + j) * cc], again);
-      sum[j] = again;
-    }
-  }
+  for (int j = 0; j < C::kCols; ++j) bad |= !finite(sum[j]) && l < lanes && n0 + j < cols;
   ptx::tc_fence_before_sync();
-  __syncthreads();   // every load, MMA and read of TMEM and shared memory has ended
+  // every load, MMA and read of TMEM and shared memory has ended
+  if (__syncthreads_or(bad || !ok) && __syncthreads_and(ok)) {
+    // the operands once more, for the warps that have sums to replace
+    bad = __any_sync(0xffffffffu, bad);
+    if (bad) {
+#pragma unroll
+      for (int j = 0; j < C::kCols; ++j) {
+        plane[j * kWarps * 32 + lane] = sum[j];
+        sum[j] = 0.f;
+      }
+      __syncwarp();
+    }
+    if (threadIdx.x == 0)
+      for (int i = 0; i < 2 && i < n_kb; ++i) load(n_kb + i);
+    for (int i = 0; i < n_kb; ++i) {
+      const int u = n_kb + i;
+      if (!__syncthreads_and(arrived(u, 6u))) {
+        if (i + 1 < n_kb) arrived(u + 1, 7u);   // (under way too)
+        break;
+      }
+      if (bad) add_terms(u & 1, kBK);
+      __syncthreads();
+      if (threadIdx.x == 0 && i + 2 < n_kb) load(u + 2);
+    }
+    if (bad) put_terms(false);
+    __syncthreads();   // the sums' way out lies there too
+  }
   if (warp == 0) ptx::tmem_dealloc(tmem_base, kTmemCols);
   // The next kernel may start, as late as this: CTAs that come early, while some SMs are
   // idle, would all settle on those.
