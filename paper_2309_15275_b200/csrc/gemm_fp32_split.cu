@@ -29,6 +29,10 @@
 // (37 TFLOP/s), 20.6 here (100, six times that in bf16); error against 64 bits of g_x and g_W
 // 2.4e-7 and 2.5e-7 there, 1.3e-7 and 1.4e-7 here.
 //
+// An item of one to five k's is summed by FMAs instead: these round once per term, which is
+// less than the tensor core drops from six products (relative error at 1, 2, 3, 4, 5, 6 and 8
+// terms: FMAs 2.5, 3.1, 3.6, 4.0, 4.4, 4.7 and 5.4e-8, split 4.5 to 4.7e-8 at all of them).
+//
 // Infinities, NaN and values next to the largest float leave the parts meaningless
 // (inf - inf, 0 * inf), but they always show as a sum that is not finite.  A CTA that has one
 // fetches the item's operands once more and its warps form their sums from them with fp32
@@ -47,6 +51,7 @@ namespace split {
 constexpr int kLanes = 128, kBK = 64;
 constexpr int kWarps = 16;                       // 8 for L, 8 for C
 constexpr int kThreads = (kWarps + 1) * 32;      // and one that issues loads and MMAs
+constexpr int kFewTerms = 5;                     // an item of no more k's is left to FMAs
 constexpr int kChunkBytes = 64 * kBK * 2;        // 64 columns of an MN-major operand
 constexpr uint32_t kTmemCols = 512, kTmemL = 256, kPartCols = kBK / 2;   // L: two stages of three parts behind the accumulators
 
@@ -90,30 +95,159 @@ __device__ __forceinline__ uint32_t take_part(float& a, float& b) {
   return w;
 }
 
+// The item of this CTA.
+template <int BN>
+struct Item {
+  const CUtensorMap *map_l, *map_c;
+  uint8_t *smem, *raw;
+  uint64_t* full;        // [2]: a block's operands have arrived
+  uint32_t* status;
+  float* D;
+  long long lanes, cols, K;
+  int32_t l0, c0, kb0, n_kb;
+  bool wt;               // L = B, C = A stored (columns, K), D transposed
+
+  __device__ __forceinline__ Item(const GemmFp32Jobs& jobs, const Maps& maps) {
+    extern __shared__ uint8_t smem_raw[];
+    smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    raw = smem + 2 * Cfg<BN>::kStage;
+    full = reinterpret_cast<uint64_t*>(raw + 2 * Cfg<BN>::kRaw);
+    status = jobs.status;
+    int t = blockIdx.x;
+    const int which = t >= jobs.items0 ? 1 : 0;
+    const GemmFp32Job& g = jobs.j[which];
+    map_l = &maps.l[which];
+    map_c = &maps.c[which];
+    if (which) t -= jobs.items0;
+    const int chunk = t % g.chunks;
+    t /= g.chunks;
+    wt = g.a_mn == 0;
+    lanes = wt ? g.N : g.M;
+    cols = wt ? g.M : g.N;
+    K = g.K;
+    l0 = (t / g.tiles_c) * kLanes;   // (coordinates of a tensor map: below 2^31)
+    c0 = (t % g.tiles_c) * BN;
+    kb0 = chunk * g.per;
+    n_kb = (kb0 + g.per < g.kb ? kb0 + g.per : g.kb) - kb0;
+    D = g.D + chunk * g.M * g.N;
+  }
+
+  // One thread: the u-th load of this CTA, block u of the item (and u - n_kb once more from there on).
+  __device__ __forceinline__ void load(int u) const {
+    using C = Cfg<BN>;
+    uint8_t* const dst = raw + (u & 1) * C::kRaw;
+    const int k = (kb0 + (u < n_kb ? u : u - n_kb)) * kBK;
+    ptx::mbar_expect_tx(&full[u & 1], C::kRaw);   // boxes count in full, also where they hang over an edge (zeros)
+    ptx::tma_load_2d(dst, map_l, &full[u & 1], l0, k);
+    ptx::tma_load_2d(dst + C::kRawL, map_c, &full[u & 1], wt ? k : c0, wt ? c0 : k);
+  }
+  __device__ __forceinline__ bool arrived(int u, uint32_t site) const {
+    return ptx::mbar_wait(&full[u & 1], static_cast<uint32_t>(u >> 1) & 1u, status, (7u << 16) | site);
+  }
+};
+
+__device__ __forceinline__ bool finite(float v) { return fabsf(v) <= 3.402823466e38f; }
+
+// The rest of an item by FMAs, with all threads of the CTA: its sums term by term, one k after
+// the other.  few: its only block has been fetched.  Otherwise the item is fetched once more,
+// and of the sums in smem = [kCols][threads] what is not finite is replaced, in warps with
+// `mine` set.  A thread has kCols / 4 lanes (in runs of four) by 4 columns, which reads less
+// than a lane by kCols.  Not inlined, and with nothing handed over: registers that the kernel
+// spills for this path cost every item of one block 0.5 us.
+template <int BN>
+__device__ __noinline__ void finish_by_fma(const GemmFp32Jobs& jobs, const Maps& maps, bool few, bool mine) {
+  using C = Cfg<BN>;
+  const Item<BN> item(jobs, maps);
+  const float* const old = reinterpret_cast<const float*>(item.smem);
+  constexpr int kRuns = C::kCols / 16, kAlong = 8 / kRuns;   // runs of a thread; threads along the lanes
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int run = (lane % kAlong) * 4, four = lane / kAlong * 4;
+  const bool wt = item.wt;
+  const int l_at = (warp & 3) * 32 + run, c_at = C::kRawL / 4 + ((warp >> 2) * C::kCols + four) * (wt ? kBK : 1);
+  float sum[C::kCols];
+#pragma unroll
+  for (int j = 0; j < C::kCols; ++j) sum[j] = 0.f;
+  const int first = few ? 0 : item.n_kb;
+  if (threadIdx.x == 0 && !few)
+    for (int i = 0; i < 2 && i < item.n_kb; ++i) item.load(first + i);
+  for (int i = 0; i < item.n_kb; ++i) {
+    const int u = first + i;
+    if (!__syncthreads_and(item.arrived(u, 6u))) {
+      if (i + 1 < item.n_kb) item.arrived(u + 1, 7u);   // (under way too)
+      break;
+    }
+    const float* const at = reinterpret_cast<const float*>(item.raw + (u & 1) * C::kRaw);
+    if (mine) {
+#pragma unroll 1
+      for (int k = 0; k < (few ? 8 : kBK); k += 4) {   // (beyond K a block is zero)
+        float c[4][4];   // [k][column]
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float4 v = *reinterpret_cast<const float4*>(at + c_at + (wt ? q * kBK + k : (k + q) * BN));
+          if (wt)
+            c[0][q] = v.x, c[1][q] = v.y, c[2][q] = v.z, c[3][q] = v.w;
+          else
+            c[q][0] = v.x, c[q][1] = v.y, c[q][2] = v.z, c[q][3] = v.w;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int h = 0; h < kRuns; ++h) {
+            const float4 v = *reinterpret_cast<const float4*>(at + l_at + (k + q) * kLanes + h * 4 * kAlong);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              sum[h * 16 + j] = fmaf(v.x, c[q][j], sum[h * 16 + j]);
+              sum[h * 16 + 4 + j] = fmaf(v.y, c[q][j], sum[h * 16 + 4 + j]);
+              sum[h * 16 + 8 + j] = fmaf(v.z, c[q][j], sum[h * 16 + 8 + j]);
+              sum[h * 16 + 12 + j] = fmaf(v.w, c[q][j], sum[h * 16 + 12 + j]);
+            }
+          }
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && i + 2 < item.n_kb) item.load(u + 2);
+  }
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (warp == kWarps) return;
+  const long long l = item.l0 + (warp & 3) * 32 + run, n = item.c0 + (warp >> 2) * C::kCols + four;
+#pragma unroll
+  for (int h = 0; h < kRuns; ++h) {
+    float v[4][4];   // [lane][column]
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        v[i][j] = sum[h * 16 + 4 * i + j];
+        if (!few) {
+          const float was = old[(four + j) * kWarps * 32 + warp * 32 + h * 4 * kAlong + run + i];
+          if (finite(was)) v[i][j] = was;
+        }
+      }
+    if (l + h * 4 * kAlong >= item.lanes) continue;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {   // (lanes are a multiple of four, and columns where they lie together)
+      if (wt && n + i < item.cols)
+        *reinterpret_cast<float4*>(item.D + (n + i) * item.lanes + l + h * 4 * kAlong) = make_float4(v[0][i], v[1][i], v[2][i], v[3][i]);
+      if (!wt && n < item.cols)
+        *reinterpret_cast<float4*>(item.D + (l + h * 4 * kAlong + i) * item.cols + n) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+    }
+  }
+}
+
 template <int BN>
 __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __grid_constant__ GemmFp32Jobs jobs,
                                                                     const __grid_constant__ Maps maps) {
   using C = Cfg<BN>;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint8_t* const raw = smem + 2 * C::kStage;
-  uint64_t* full = reinterpret_cast<uint64_t*>(raw + 2 * C::kRaw);   // [2]: a block's operands have arrived
-  uint64_t* ready = full + 2;                                        // [2]: its parts are written
+  const Item<BN> item(jobs, maps);
+  uint8_t *const smem = item.smem, *const raw = item.raw;
+  uint64_t* const full = item.full;
+  uint64_t* ready = full + 2;                                        // [2]: a block's parts are written
   uint64_t* done = ready + 2;                                        // [2]: its MMAs have completed
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 2);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-  int t = blockIdx.x;
-  const int which = t >= jobs.items0 ? 1 : 0;
-  const GemmFp32Job& g = jobs.j[which];
-  if (which) t -= jobs.items0;
-  const int chunk = t % g.chunks;
-  t /= g.chunks;
-  const bool wt = g.a_mn == 0;   // L = B, C = A stored (columns, K), D transposed
-  const long long lanes = wt ? g.N : g.M, cols = wt ? g.M : g.N;
-  const long long l0 = static_cast<long long>(t / g.tiles_c) * kLanes, c0 = static_cast<long long>(t % g.tiles_c) * BN;
-  const int kb0 = chunk * g.per, kb1 = kb0 + g.per < g.kb ? kb0 + g.per : g.kb, n_kb = kb1 - kb0;
+  const bool wt = item.wt;
+  const int n_kb = item.n_kb;
+  const bool few = n_kb == 1 && item.K - static_cast<long long>(item.kb0) * kBK <= kFewTerms;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) {
@@ -122,31 +256,24 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
       ptx::mbar_init(&done[i], 1);
     }
     ptx::mbar_fence_init();
-    ptx::prefetch_tensormap(&maps.l[which]);
-    ptx::prefetch_tensormap(&maps.c[which]);
+    ptx::prefetch_tensormap(item.map_l);
+    ptx::prefetch_tensormap(item.map_c);
   }
-  if (warp == 0) {
+  if (warp == 0 && !few) {
     ptx::tmem_alloc(tmem_slot, kTmemCols);
     ptx::tmem_relinquish();
   }
   ptx::tc_fence_before_sync();
   __syncthreads();
   ptx::tc_fence_after_sync();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = *tmem_slot;   // (few: none)
   asm volatile("griddepcontrol.wait;" ::: "memory");   // launched as the kernel ahead ends
 
-  // One thread: the u-th load of this CTA, block u of the item (and u - n_kb once more from there on).
-  auto load = [&](int u) {
-    uint8_t* const dst = raw + (u & 1) * C::kRaw;
-    const int k = (kb0 + (u < n_kb ? u : u - n_kb)) * kBK;
-    ptx::mbar_expect_tx(&full[u & 1], C::kRaw);   // boxes count in full, also where they hang over an edge (zeros)
-    ptx::tma_load_2d(dst, &maps.l[which], &full[u & 1], static_cast<int32_t>(l0), k);
-    ptx::tma_load_2d(dst + C::kRawL, &maps.c[which], &full[u & 1], wt ? k : static_cast<int32_t>(c0),
-                     wt ? static_cast<int32_t>(c0) : k);
-  };
-  auto arrived = [&](int u, uint32_t site) {
-    return ptx::mbar_wait(&full[u & 1], static_cast<uint32_t>(u >> 1) & 1u, jobs.status, (7u << 16) | site);
-  };
+  if (few) {
+    if (threadIdx.x == 0) item.load(0);
+    finish_by_fma<BN>(jobs, maps, true, true);
+    return;
+  }
   // L: a thread has its lane's k's of one half of the block.  C: pieces of four numbers, a
   // warp whole 128-byte lines; row `row` + q * rows of the block, in shared memory `hop` apart.
   const bool is_l = warp < 8;
@@ -154,7 +281,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
   const int c_row = wt ? tid >> 4 : tid / (BN / 4), c_pc = wt ? tid & 15 : tid % (BN / 4);
   const int hop = (wt ? 16 : 256 / (BN / 4)) * 128;
   const int to = (wt ? 0 : (c_pc >> 4) * kChunkBytes) + c_row * 128 + ((((c_pc & 15) >> 1) ^ (c_row & 7)) << 4) + (c_pc & 1) * 8;
-  const long long l = l0 + quarter * 32 + lane;
 
   float sum[C::kCols];
 #pragma unroll
@@ -177,72 +303,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
     }
   };
 
-  // A warp's sums by FMAs from a raw stage, term by term, one k after the other: a thread has
-  // kCols / 4 lanes (in runs of four) by 4 columns, which reads less than a lane by kCols.
-  constexpr int kRuns = C::kCols / 16, kAlong = 8 / kRuns;   // runs of a thread; threads along the lanes
-  const int run = (lane % kAlong) * 4, four = lane / kAlong * 4;
-  auto finite = [](float v) { return fabsf(v) <= 3.402823466e38f; };
-  auto add_terms = [&](int stage, int nk) {
-    const float* const ls = reinterpret_cast<const float*>(raw + stage * C::kRaw) + quarter * 32 + run;
-    const float* const cs = reinterpret_cast<const float*>(raw + stage * C::kRaw + C::kRawL) +
-                            (group * C::kCols + four) * (wt ? kBK : 1);
-#pragma unroll 1
-    for (int k = 0; k < nk; k += 4) {
-      float c[4][4];   // [k][column]
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float4 v = *reinterpret_cast<const float4*>(wt ? cs + q * kBK + k : cs + (k + q) * BN);
-        if (wt)
-          c[0][q] = v.x, c[1][q] = v.y, c[2][q] = v.z, c[3][q] = v.w;
-        else
-          c[q][0] = v.x, c[q][1] = v.y, c[q][2] = v.z, c[q][3] = v.w;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int h = 0; h < kRuns; ++h) {
-          const float4 v = *reinterpret_cast<const float4*>(ls + (k + q) * kLanes + h * 4 * kAlong);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            sum[h * 16 + j] = fmaf(v.x, c[q][j], sum[h * 16 + j]);
-            sum[h * 16 + 4 + j] = fmaf(v.y, c[q][j], sum[h * 16 + 4 + j]);
-            sum[h * 16 + 8 + j] = fmaf(v.z, c[q][j], sum[h * 16 + 8 + j]);
-            sum[h * 16 + 12 + j] = fmaf(v.w, c[q][j], sum[h * 16 + 12 + j]);
-          }
-        }
-    }
-  };
-  // They replace what the warp's plane in the place of the parts holds (all of it, or what is
-  // not finite there), which then becomes a lane by kCols a thread once more.
-  float* const plane = reinterpret_cast<float*>(smem) + warp * 32;   // [kCols][all lanes of all warps]
-  auto put_terms = [&](bool all) {
-#pragma unroll
-    for (int h = 0; h < kRuns; ++h)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float4* const at = reinterpret_cast<float4*>(plane + (four + j) * kWarps * 32 + h * 4 * kAlong + run);
-        float4 v = *at;
-        if (all || !finite(v.x)) v.x = sum[h * 16 + j];
-        if (all || !finite(v.y)) v.y = sum[h * 16 + 4 + j];
-        if (all || !finite(v.z)) v.z = sum[h * 16 + 8 + j];
-        if (all || !finite(v.w)) v.w = sum[h * 16 + 12 + j];
-        *at = v;
-      }
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < C::kCols; ++j) sum[j] = plane[j * kWarps * 32 + lane];
-  };
-
   if (warp == kWarps) {
     if (ptx::elect_one()) {
       const uint32_t idesc = ptx::idesc_bf16(kLanes, BN, false, !wt);
       const int n = jobs.test_stall ? 0 : n_kb;
       int loads = 0, begun = 0;   // blocks fetched, blocks whose MMAs have been issued
-      for (; loads < 2 && loads < n; ++loads) load(loads);
+      for (; loads < 2 && loads < n; ++loads) item.load(loads);
       for (int i = 0; i < n_kb; ++i) {
         const int s = i & 1;
         if (!ptx::mbar_wait(&ready[s], static_cast<uint32_t>(i >> 1) & 1u, jobs.status, (7u << 16) | 3u)) break;
-        if (i + 2 < n_kb) load(loads++);   // everyone has read block i
+        if (i + 2 < n_kb) item.load(loads++);   // everyone has read block i
         ptx::tc_fence_after_sync();
         const uint32_t a = tmem_base + kTmemL + s * 3 * kPartCols, b = ptx::smem_u32(smem + s * C::kStage);
         const uint32_t d = tmem_base + s * BN;
@@ -261,7 +331,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
         begun = i + 1;
       }
       // whatever made the others leave: nothing is under way in this CTA's memories when it ends
-      for (int i = begun; i < loads; ++i) arrived(i, 4u);
+      for (int i = begun; i < loads; ++i) item.arrived(i, 4u);
       if (begun > 0)
         ptx::mbar_wait(&done[(begun - 1) & 1], static_cast<uint32_t>((begun - 1) >> 1) & 1u, jobs.status, (7u << 16) | 5u);
     }
@@ -270,7 +340,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
   for (int i = 0; i < n_kb && ok && warp < kWarps; ++i) {
     // (the MMAs that read this stage of parts have completed: their accumulator was drained)
     const int s = i & 1;
-    ok = __all_sync(0xffffffffu, arrived(i, 2u));
+    ok = __all_sync(0xffffffffu, item.arrived(i, 2u));
     if (!ok) break;
     if (is_l) {
       const float* const src = reinterpret_cast<const float*>(raw + s * C::kRaw) + (warp >> 2) * 32 * kLanes + quarter * 32 + lane;
@@ -310,44 +380,28 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
   }
   if (ok && warp < kWarps) drain(n_kb - 1);
 
-  const long long n0 = c0 + group * C::kCols;   // this thread's columns
+  const long long lanes = item.lanes, cols = item.cols;
+  const long long l = item.l0 + quarter * 32 + lane, n0 = item.c0 + group * C::kCols;   // this thread's lane, its columns
   bool bad = false;
 #pragma unroll
-  for (int j = 0; j < C::kCols; ++j) bad |= !finite(sum[j]) && l < lanes && n0 + j < cols;
+  for (int j = 0; j < C::kCols; ++j) bad |= !finite(sum[j]);
   ptx::tc_fence_before_sync();
-  // every load, MMA and read of TMEM and shared memory has ended
+  // past this barrier every load, MMA and read of TMEM and shared memory has ended
   if (__syncthreads_or(bad || !ok) && __syncthreads_and(ok)) {
-    // the operands once more, for the warps that have sums to replace
-    bad = __any_sync(0xffffffffu, bad);
-    if (bad) {
+    if (warp == 0) ptx::tmem_dealloc(tmem_base, kTmemCols);
+    if (warp < kWarps) {
 #pragma unroll
-      for (int j = 0; j < C::kCols; ++j) {
-        plane[j * kWarps * 32 + lane] = sum[j];
-        sum[j] = 0.f;
-      }
-      __syncwarp();
+      for (int j = 0; j < C::kCols; ++j) reinterpret_cast<float*>(smem)[j * kWarps * 32 + threadIdx.x] = sum[j];
     }
-    if (threadIdx.x == 0)
-      for (int i = 0; i < 2 && i < n_kb; ++i) load(n_kb + i);
-    for (int i = 0; i < n_kb; ++i) {
-      const int u = n_kb + i;
-      if (!__syncthreads_and(arrived(u, 6u))) {
-        if (i + 1 < n_kb) arrived(u + 1, 7u);   // (under way too)
-        break;
-      }
-      if (bad) add_terms(u & 1, kBK);
-      __syncthreads();
-      if (threadIdx.x == 0 && i + 2 < n_kb) load(u + 2);
-    }
-    if (bad) put_terms(false);
-    __syncthreads();   // the sums' way out lies there too
+    finish_by_fma<BN>(jobs, maps, false, __any_sync(0xffffffffu, bad));
+    return;
   }
   if (warp == 0) ptx::tmem_dealloc(tmem_base, kTmemCols);
   // The next kernel may start, as late as this: CTAs that come early, while some SMs are
   // idle, would all settle on those.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (warp == kWarps) return;
-  float* const D = g.D + chunk * g.M * g.N;
+  float* const D = item.D;
   if (wt) {   // a warp 32 numbers of a row at a time
 #pragma unroll
     for (int j = 0; j < C::kCols; ++j)
@@ -364,7 +418,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
 #pragma unroll
     for (int r0 = 0; r0 < 32; r0 += 32 / kRowPieces) {
       const int row = r0 + lane / kRowPieces;
-      const long long gm = l0 + quarter * 32 + row, gn = n0 + 4 * c;
+      const long long gm = item.l0 + quarter * 32 + row, gn = n0 + 4 * c;
       if (gm < lanes && gn < cols)
         *reinterpret_cast<float4*>(D + gm * cols + gn) = mine[row * kRowPieces + (c ^ (row & (kRowPieces - 1)))];
     }

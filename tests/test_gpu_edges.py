@@ -512,3 +512,25 @@ def test_fp32_nan_costs_a_few_times_ffma_at_most(dev, monkeypatch):
     finally:
         monkeypatch.undo()
         lbp.lbp_test_reload_env()
+
+
+@pytest.mark.parametrize("ci,co,T", [(264, 136, 1), (136, 4, 200), (128, 260, 2), (64, 64, 3), (320, 128, 4), (132, 516, 5)])
+def test_fp32_products_of_few_terms_round_once_a_term(dev, monkeypatch, ci, co, T):
+    # sums of one to five terms: the same numbers from every form, of one term the rounded product
+    x, gy, w = layer(dev, 99, 1, 1, T, ci, co, dtype=torch.float32)
+    got = []
+    try:
+        for form in range(3):
+            monkeypatch.setenv("LBP_FP32_FORM", str(form))
+            lbp.lbp_test_reload_env()
+            got.append(lbp.lbp_backward_fullrank(x, gy, w, 8))
+    finally:
+        monkeypatch.undo()
+        lbp.lbp_test_reload_env()
+    for gx, gw in got[1:]:
+        if T <= 5:
+            assert torch.equal(gw, got[0][1])
+        if co <= 5:
+            assert torch.equal(gx, got[0][0])
+    if T == 1:
+        assert torch.equal(got[1][1], gy.reshape(-1, 1) * x.reshape(1, -1))
