@@ -51,7 +51,7 @@ int lbp_test_products_plan(const lbp_layer* layer, const lbp_basis* set, int r, 
  * `room` bytes for planes (gemm_fp32.cu).  out6 = {form, bytes of planes,
  * k-blocks of an item of g_x and items of K per tile of it, the same of g_W}.  No device
  * needed. */
-int lbp_test_fp32_plan(int Cin, int Cout, long long rows, size_t room, int64_t* out6);
+int lbp_test_float_plan(int Cin, int Cout, long long rows, size_t room, int64_t* out6);
 
 /* The library reads its tuning switches (LBP_FUSED, LBP_PAIR, LBP_FUSED_TILES,
  * LBP_FUSED_VERBOSE) from the environment once, at first use.  This reads them

@@ -124,8 +124,8 @@ def _lib() -> C.CDLL:
                                                C.POINTER(C.c_int32), C.POINTER(C.c_uint16),
                                                C.POINTER(C.c_uint16)]
         lib.lbp_test_products_plan.restype = i32
-        lib.lbp_test_fp32_plan.argtypes = [i32, i32, C.c_longlong, sz, C.POINTER(C.c_int64)]
-        lib.lbp_test_fp32_plan.restype = i32
+        lib.lbp_test_float_plan.argtypes = [i32, i32, C.c_longlong, sz, C.POINTER(C.c_int64)]
+        lib.lbp_test_float_plan.restype = i32
         lib.lbp_test_reload_env.argtypes = []
         lib.lbp_test_reload_env.restype = i32
         lib.lbp_test_struct_size.argtypes = [i32]
@@ -180,7 +180,7 @@ EXPORTED = ("lbp_select_bases", "lbp_basis_matrix", "lbp_flops", "lbp_status_str
             "lbp_test_reload_env", "lbp_workspace_bytes_ex", "lbp_workspace_bytes_projected", "lbp_backward_ex",
             "lbp_backward_projected", "lbp_test_tile_plan", "lbp_test_struct_size",
             "lbp_test_side_section", "lbp_test_per_device", "lbp_test_products_plan",
-            "lbp_test_fp32_plan")
+            "lbp_test_float_plan")
 
 
 def _check(status: int, where: str) -> None:
@@ -671,10 +671,10 @@ def lbp_test_products_plan(B, H, W, Cin, Cout, k, bases, *, n_extra=0, units=74,
     return info, [[ids[j] for j in range(first[u], first[u + 1])] for u in range(units)]
 
 
-def lbp_test_fp32_plan(Cin, Cout, rows, room=2 ** 63):
+def lbp_test_float_plan(Cin, Cout, rows, room=2 ** 63):
     """Test hook: the plan of the two fp32 products over this many rows."""
     out = (C.c_int64 * 6)()
-    _check(_lib().lbp_test_fp32_plan(Cin, Cout, rows, room, out), "lbp_test_fp32_plan")
+    _check(_lib().lbp_test_float_plan(Cin, Cout, rows, room, out), "lbp_test_float_plan")
     return dict(zip(("form", "planes", "gx_kb", "gx_items", "gw_kb", "gw_items"), out))
 
 

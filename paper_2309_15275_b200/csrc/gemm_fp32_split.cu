@@ -37,9 +37,9 @@
 // (inf - inf, 0 * inf), but they always show as a sum that is not finite.  A CTA that has one
 // fetches the item's operands once more and its warps form their sums from them with fp32
 // FMAs, term by term; only those that were not finite are replaced.  640 x 448 -> 1792, both
-// products: 22 us, with one NaN in g_y 118, with nothing but NaN 128 (FFMA kernel 60 whatever
+// products: 22 us, with one NaN in g_y 120, with nothing but NaN 141 (FFMA kernel 60 whatever
 // the values; a serial sum per thread from global memory 980 and 1120); 2048 x 768 -> 3072: 115,
-// 247 and 748 (436; 1690 and 6850).
+// 250 and 803 (436; 1690 and 6850).
 #include "gemm_fp32.cuh"
 #include "lbp_internal.h"
 #include "ptx_sm100.cuh"

@@ -688,7 +688,7 @@ int lbp_test_per_device(const int* devices, int n, uint8_t* done) {
   return LBP_OK;
 }
 
-int lbp_test_fp32_plan(int Cin, int Cout, long long rows, size_t room, int64_t* out6) {
+int lbp_test_float_plan(int Cin, int Cout, long long rows, size_t room, int64_t* out6) {
   lbp_layer L{};
   L.Cin = Cin;
   L.Cout = Cout;

@@ -507,7 +507,7 @@ def test_fp32_nan_costs_a_few_times_ffma_at_most(dev, monkeypatch):
         ffma = us(0, gy)
         for form in (1, 2):
             for g in (one, every):
-                # measured: 1.2 to 2.4 of it (with a serial sum per thread 6.6 to 19)
+                # measured: 1.3 to 2.7 of it (with a serial sum per thread 6.6 to 19)
                 assert us(form, g) <= 4 * ffma
     finally:
         monkeypatch.undo()

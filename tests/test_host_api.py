@@ -412,7 +412,7 @@ def test_fp32_products_are_planned_whatever_the_switch_says(monkeypatch, ci, co,
         else:
             monkeypatch.setenv("LBP_FP32_FORM", form)
         lbp.lbp_test_reload_env()
-        return lbp.lbp_test_fp32_plan(ci, co, rows, room)
+        return lbp.lbp_test_float_plan(ci, co, rows, room)
     try:
         for room in (0, 1 << 20, 2 ** 63):
             free = plan(None, room)
