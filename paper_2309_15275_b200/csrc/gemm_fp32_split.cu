@@ -7,8 +7,13 @@
 // g_y_hat and C = x_hat, g_x_hat = g_y_hat W with L = W and C = g_y_hat (D transposed).
 //
 // x = hi + mid + lo, each part the bf16 nearest to what the parts before it leave: 8
-// significant bits a part and a sign each, so the three hold x to 2^-27 of itself.  Of the
-// nine products of parts the six largest are formed; the rest is below 2^-26 of a term.
+// significant bits a part and a sign each, so the three hold x to 2^-27 of itself.  mid and lo
+// are held times 2^15, which keeps them clear of the end of bf16's range (2^-133) for every
+// normal x: held as they are, they lose bits of numbers below 2^-110 (g_y of 2^-114: error
+// 5.7e-7, of 2^-120: 3.6e-5; now 0.9e-7 down to 2^-124, FFMA 1.8e-7.  Where the sums themselves
+// are subnormal the tensor core cuts at 2^-149 where FMAs round there: g_y of 2^-130 times W of
+// 1, 1.4e-6 against 5.6e-7).  The scaling costs 0.02 of 1.4 us a block.  Of the nine products of parts the six largest are formed; the
+// rest is below 2^-26 of a term.
 // A product of two bf16 numbers is exact in fp32, so what is left is the summation.  The
 // tensor core drops bits of the smaller addend when it adds to an accumulator, so a
 // k-block of 64 starts from an accumulator of its own, its small products go first, and the
@@ -51,6 +56,7 @@ namespace split {
 constexpr int kLanes = 128, kBK = 64;
 constexpr int kWarps = 16;                       // 8 for L, 8 for C
 constexpr int kThreads = (kWarps + 1) * 32;      // and one that issues loads and MMAs
+constexpr int kShift = 15;                       // mid and lo are held times 2^15
 constexpr int kFewTerms = 5;                     // an item of no more k's is left to FMAs
 constexpr int kChunkBytes = 64 * kBK * 2;        // 64 columns of an MN-major operand
 constexpr uint32_t kTmemCols = 512, kTmemL = 256, kPartCols = kBK / 2;   // L: two stages of three parts behind the accumulators
@@ -86,12 +92,25 @@ __device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, ui
       "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// D = 2^-kShift D + A * B
+__device__ __forceinline__ void mma_bf16_ts_down(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.eq.b32 p, 0, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p, %4;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b_desc), "r"(idesc), "n"(kShift)
+      : "memory");
+}
 
-// The next part of two numbers; what it leaves of them.
-__device__ __forceinline__ uint32_t take_part(float& a, float& b) {
+// The next part of two numbers (0 hi, 1 mid, 2 lo); what it leaves of them.
+__device__ __forceinline__ uint32_t take_part(float& a, float& b, int part) {
   const uint32_t w = pack_bf16x2(a, b);
   a -= bf16_lo(w);   // exact
   b -= bf16_hi(w);
+  if (part == 0) {
+    a *= 1 << kShift;
+    b *= 1 << kShift;
+  }
   return w;
 }
 
@@ -316,8 +335,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
         ptx::tc_fence_after_sync();
         const uint32_t a = tmem_base + kTmemL + s * 3 * kPartCols, b = ptx::smem_u32(smem + s * C::kStage);
         const uint32_t d = tmem_base + s * BN;
-        // parts 0 hi, 1 mid, 2 lo: the small products first, hi * hi last
-        constexpr int kPl[6] = {2, 0, 1, 1, 0, 0}, kPc[6] = {0, 2, 1, 0, 1, 0};
+        // parts 0 hi, 1 mid, 2 lo.  mid * mid comes out times 2^30, the products of one of them
+        // times 2^15, hi * hi as it is: the accumulator is taken down between them
+        constexpr int kPl[6] = {1, 2, 0, 1, 0, 0}, kPc[6] = {1, 0, 2, 0, 1, 0};
 #pragma unroll
         for (int q = 0; q < 6; ++q)
 #pragma unroll
@@ -325,7 +345,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
             const uint32_t bp = b + kPc[q] * C::kPart;
             const uint64_t db = wt ? ptx::smem_desc_sw128(bp + kk * 32, 16, 1024)
                                    : ptx::smem_desc_sw128(bp + kk * 2048, kChunkBytes, 1024);
-            mma_bf16_ts(d, a + kPl[q] * kPartCols + kk * 8, db, idesc, (q == 0 && kk == 0) ? 0u : 1u);
+            const uint32_t al = a + kPl[q] * kPartCols + kk * 8;
+            if (kk == 0 && (q == 1 || q == 5))
+              mma_bf16_ts_down(d, al, db, idesc);
+            else
+              mma_bf16_ts(d, al, db, idesc, (q == 0 && kk == 0) ? 0u : 1u);
           }
         ptx::mma_commit(&done[s]);
         begun = i + 1;
@@ -354,7 +378,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
         for (int part = 0; part < 3; ++part) {
           uint32_t w[8];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) w[j] = take_part(v[2 * j], v[2 * j + 1]);
+          for (int j = 0; j < 8; ++j) w[j] = take_part(v[2 * j], v[2 * j + 1], part);
           tmem_st_x8(dst + part * kPartCols + h * 8, w);
         }
       }
@@ -367,7 +391,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
         float4 v = src[q * 256];
 #pragma unroll
         for (int part = 0; part < 3; ++part) {
-          const uint32_t w0 = take_part(v.x, v.y), w1 = take_part(v.z, v.w);
+          const uint32_t w0 = take_part(v.x, v.y, part), w1 = take_part(v.z, v.w, part);
           *reinterpret_cast<uint2*>(dst + q * hop + part * C::kPart) = make_uint2(w0, w1);
         }
       }

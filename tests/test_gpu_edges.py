@@ -534,3 +534,18 @@ def test_fp32_products_of_few_terms_round_once_a_term(dev, monkeypatch, ci, co, 
             assert torch.equal(gx, got[0][0])
     if T == 1:
         assert torch.equal(got[1][1], gy.reshape(-1, 1) * x.reshape(1, -1))
+
+
+@pytest.mark.parametrize("fp32_form", [0, 1, 2], indirect=True)
+@pytest.mark.parametrize("exponent", [-104, -112, -118, -122, -124])
+def test_fp32_products_of_small_numbers(dev, fp32_form, exponent):
+    # g_y down to the smallest normal numbers: 320 and 256 terms of random signs err by
+    # sqrt(320) * 2^-24 at most in any order, wherever in the range they lie (x and W times 64, so
+    # that sums and most products of parts are normal; below 2^-120 a step of 2^-149 beside it)
+    x, gy, w = layer(dev, 103, 1, 1, 320, 256, 256, dtype=torch.float32)
+    x, w = x * 64, w * 64
+    gy = gy * 100 * 2.0 ** exponent
+    gx, gw = lbp.lbp_backward_fullrank(x, gy, w, 8)
+    ox, ow = O.backward_exact(f64(x), f64(gy), f64(w))
+    bound = 320 ** 0.5 * 2.0 ** -24 + (2.0 ** -149 / 2.0 ** exponent if exponent < -120 else 0)
+    assert rel(gx, ox) <= bound and rel(gw, ow) <= bound
