@@ -224,6 +224,7 @@ Plan make_plan(const GemmFp32* job, int n, size_t room) {
   for (int i = 0; i < n; ++i)
     for (long long d : {job[i].M, job[i].N, job[i].K}) fits &= d < (1ll << 31) - 256;
   const int forced = fits ? tune_options().fp32_form : 0;
+  const long long wanted = tune_options().fp32_per;
   for (int f = 0; f < 3; ++f) {
     const Form& form = kForms[f];
     if (forced >= 0 && f != forced) continue;
@@ -232,8 +233,8 @@ Plan make_plan(const GemmFp32* job, int n, size_t room) {
       kb[i] = ceil_div(job[i].K, form.bk);
       most = kb[i] > most ? kb[i] : most;
     }
-    for (long long per : {most, 64ll, 48ll, 32ll, 24ll, 16ll, 12ll, 10ll, 8ll, 7ll, 6ll, 5ll, 4ll, 3ll, 2ll, 1ll}) {
-      if (per > most || (f == 0 && per == 1 && per < most)) continue;
+    for (long long per : {most, wanted, 64ll, 48ll, 32ll, 24ll, 16ll, 12ll, 10ll, 8ll, 7ll, 6ll, 5ll, 4ll, 3ll, 2ll, 1ll}) {
+      if (per == 0 || per > most || (f == 0 && per == 1 && per < most)) continue;
       double t = 0, item_t[2] = {0, 0};
       long long items[2] = {0, 0};
       size_t bytes = 0;
@@ -252,6 +253,10 @@ Plan make_plan(const GemmFp32* job, int n, size_t room) {
       t += f == 0 ? static_cast<double>(ceil_div(items[0] + items[1], kSms)) * (per + form.item_us)
            : item_t[0] < item_t[1] ? form.launch_us + makespan(items[1], item_t[1], items[0], item_t[0])
                                     : form.launch_us + makespan(items[0], item_t[0], items[1], item_t[1]);
+      if (per == wanted) {   // whatever it takes
+        best = Plan{f, per, bytes};
+        break;
+      }
       if (best_t < 0 || t < best_t) {
         best_t = t;
         best = Plan{f, per, bytes};
@@ -266,7 +271,7 @@ Plan plan(const GemmFp32* job, int n, size_t room) {
   struct Entry {
     long long dims[6];
     size_t room;
-    int forced;
+    int forced, wanted;
     Plan plan;
   };
   static thread_local Entry cache[16];
@@ -275,7 +280,7 @@ Plan plan(const GemmFp32* job, int n, size_t room) {
   const long long dims[6] = {a.M, a.N, a.K, n > 1 ? b.M : 0, n > 1 ? b.N : 0, n > 1 ? b.K : 0};
   for (int c = 0; c < filled; ++c) {
     const Entry& e = cache[c];
-    bool same = e.room == room && e.forced == tune_options().fp32_form;
+    bool same = e.room == room && e.forced == tune_options().fp32_form && e.wanted == tune_options().fp32_per;
     for (int i = 0; i < 6; ++i) same &= e.dims[i] == dims[i];
     if (same) return e.plan;
   }
@@ -283,6 +288,7 @@ Plan plan(const GemmFp32* job, int n, size_t room) {
   for (int i = 0; i < 6; ++i) e.dims[i] = dims[i];
   e.room = room;
   e.forced = tune_options().fp32_form;
+  e.wanted = tune_options().fp32_per;
   e.plan = make_plan(job, n, room);
   if (tune_options().verbose)
     fprintf(stderr, "lbp fp32 products plan: %lldx%lldx%lld, %lldx%lldx%lld: form %d, %lld k-blocks an item, planes %zu\n",

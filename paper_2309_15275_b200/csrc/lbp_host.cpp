@@ -127,7 +127,10 @@ static TuneOptions read_tune_options() {
   t.batch_proj_sms = e != nullptr ? std::atoi(e) : -1;
   e = std::getenv("LBP_FP32_FORM");
   t.fp32_form = -1;
-  if (e != nullptr && e[0] >= '0' && e[0] <= '2' && e[1] == 0) t.fp32_form = e[0] - '0';
+  if (e != nullptr && e[0] >= '0' && e[0] <= '2' && (e[1] == 0 || e[1] == ',')) {
+    t.fp32_form = e[0] - '0';
+    if (e[1] == ',') t.fp32_per = std::max(0, std::atoi(e + 2));
+  }
   return t;
 }
 static TuneOptions& tune_options_slot() {

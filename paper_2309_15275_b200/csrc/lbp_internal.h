@@ -244,7 +244,8 @@ int launch_bias_grad(const void* a, long long n_a, int r, int q, TokenMap ta, do
 //   LBP_PROJECT_UMMA=0   bf16 projection by additions on the CUDA cores instead of tcgen05
 //   LBP_FUSED_TILES=a,b,c  column tiles of the two products and K slices of g_W
 //   LBP_FP32_FORM=n      fp32 products: 0 on FFMA, 1 / 2 split operands on tcgen05 in tiles
-//                        of 128 x 64 / 128 x 128 (unset or anything else = chosen by size)
+//                        of 128 x 64 / 128 x 128 (unset or anything else = chosen by size);
+//                        n,p: in items of p k-blocks, where the workspace has room
 //   LBP_FUSED_VERBOSE=1  print the chosen tile plan
 //   LBP_BATCH_PROJ_SMS=n lbp_backward_batch: SMs given to the projection of the next
 //                        layer while the products kernel of a layer runs (0 = one
@@ -256,6 +257,7 @@ struct TuneOptions {
   int tiles_bnw, tiles_bnx, tiles_splits;
   int batch_proj_sms;   // -1 = library default
   int fp32_form;        // -1 = chosen by size
+  int fp32_per;         // 0 = chosen by size
 };
 const TuneOptions& tune_options();
 void reload_tune_options();   // test hook: read the environment again
