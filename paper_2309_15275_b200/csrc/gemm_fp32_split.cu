@@ -10,10 +10,8 @@
 // significant bits a part and a sign each, so the three hold x to 2^-27 of itself.  mid and lo
 // are held times 2^15, which keeps them clear of the end of bf16's range (2^-133) for every
 // normal x: held as they are, they lose bits of numbers below 2^-110 (g_y of 2^-114: error
-// 5.7e-7, of 2^-120: 3.6e-5; now 0.9e-7 down to 2^-124, FFMA 1.8e-7.  Where the sums themselves
-// are subnormal the tensor core cuts at 2^-149 where FMAs round there: g_y of 2^-130 times W of
-// 1, 1.4e-6 against 5.6e-7).  The scaling costs 0.02 of 1.4 us a block.  Of the nine products of parts the six largest are formed; the
-// rest is below 2^-26 of a term.
+// 5.7e-7, of 2^-120: 3.6e-5; now 0.9e-7 throughout).  The scaling makes a block 2 % longer.  Of
+// the nine products of parts the six largest are formed; the rest is below 2^-26 of a term.
 // A product of two bf16 numbers is exact in fp32, so what is left is the summation.  The
 // tensor core drops bits of the smaller addend when it adds to an accumulator, so a
 // k-block of 64 starts from an accumulator of its own, its small products go first, and the
@@ -39,9 +37,11 @@
 // terms: FMAs 2.5, 3.1, 3.6, 4.0, 4.4, 4.7 and 5.4e-8, split 4.5 to 4.7e-8 at all of them).
 //
 // Infinities, NaN and values next to the largest float leave the parts meaningless
-// (inf - inf, 0 * inf), but they always show as a sum that is not finite.  A CTA that has one
-// fetches the item's operands once more and its warps form their sums from them with fp32
-// FMAs, term by term; only those that were not finite are replaced.  640 x 448 -> 1792, both
+// (inf - inf, 0 * inf), but they always show as a sum that is not finite; and where a sum is
+// next to subnormal the tensor core's cut at 2^-149 shows, where FMAs round (g_y of 2^-130, W of
+// 1: 1.4e-6 against 5.6e-7).  A CTA that has a sum not finite or below 2^-120 fetches the item's
+// operands once more and its warps form their sums from them with fp32 FMAs, term by term;
+// only such sums are replaced.  640 x 448 -> 1792, both
 // products: 22 us, with one NaN in g_y 120, with nothing but NaN 141 (FFMA kernel 60 whatever
 // the values; a serial sum per thread from global memory 980 and 1120); 2048 x 768 -> 3072: 115,
 // 250 and 803 (436; 1690 and 6850).
@@ -165,11 +165,16 @@ struct Item {
   }
 };
 
-__device__ __forceinline__ bool finite(float v) { return fabsf(v) <= 3.402823466e38f; }
+// A sum that stays: zero, or a finite one of 2^-120 and more.
+__device__ __forceinline__ bool stays(float v) {
+  constexpr uint32_t kLeast = (127 - 120) << 23, kMost = 0x7f7fffff;
+  const uint32_t u = __float_as_uint(v) & 0x7fffffffu;
+  return u == 0 || u - kLeast <= kMost - kLeast;
+}
 
 // The rest of an item by FMAs, with all threads of the CTA: its sums term by term, one k after
 // the other.  few: its only block has been fetched.  Otherwise the item is fetched once more,
-// and of the sums in smem = [kCols][threads] what is not finite is replaced, in warps with
+// and of the sums in smem = [kCols][threads] those that do not stay are replaced, in warps with
 // `mine` set.  A thread has kCols / 4 lanes (in runs of four) by 4 columns, which reads less
 // than a lane by kCols.  Not inlined, and with nothing handed over: registers that the kernel
 // spills for this path cost every item of one block 0.5 us.
@@ -239,7 +244,7 @@ __device__ __noinline__ void finish_by_fma(const GemmFp32Jobs& jobs, const Maps&
         v[i][j] = sum[h * 16 + 4 * i + j];
         if (!few) {
           const float was = old[(four + j) * kWarps * 32 + warp * 32 + h * 4 * kAlong + run + i];
-          if (finite(was)) v[i][j] = was;
+          if (stays(was)) v[i][j] = was;
         }
       }
     if (l + h * 4 * kAlong >= item.lanes) continue;
@@ -408,7 +413,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
   const long long l = item.l0 + quarter * 32 + lane, n0 = item.c0 + group * C::kCols;   // this thread's lane, its columns
   bool bad = false;
 #pragma unroll
-  for (int j = 0; j < C::kCols; ++j) bad |= !finite(sum[j]);
+  for (int j = 0; j < C::kCols; ++j) bad |= !stays(sum[j]);
   ptx::tc_fence_before_sync();
   // past this barrier every load, MMA and read of TMEM and shared memory has ended
   if (__syncthreads_or(bad || !ok) && __syncthreads_and(ok)) {

@@ -574,3 +574,24 @@ def test_fp32_products_of_small_numbers(dev, fp32_form, exponent):
     ox, ow = O.backward_exact(f64(x), f64(gy), f64(w))
     bound = 320 ** 0.5 * 2.0 ** -24 + (2.0 ** -149 / 2.0 ** exponent if exponent < -120 else 0)
     assert rel(gx, ox) <= bound and rel(gw, ow) <= bound
+
+
+@pytest.mark.parametrize("exponent", [-124, -130, -134])
+def test_fp32_sums_below_the_normal_numbers(dev, monkeypatch, exponent):
+    # sums around 2^(exponent + 4): whatever the form, as near as FMAs come, which round at 2^-149
+    # (the tensor core cuts there)
+    x, gy, w = layer(dev, 107, 1, 1, 320, 256, 256, dtype=torch.float32)
+    gy = gy * 100 * 2.0 ** exponent
+    ox, ow = O.backward_exact(f64(x), f64(gy), f64(w))
+    err = []
+    try:
+        for form in range(3):
+            monkeypatch.setenv("LBP_FP32_FORM", str(form))
+            lbp.lbp_test_reload_env()
+            gx, gw = lbp.lbp_backward_fullrank(x, gy, w, 8)
+            err.append((rel(gx, ox), rel(gw, ow)))
+    finally:
+        monkeypatch.undo()
+        lbp.lbp_test_reload_env()
+    for ex, ew in err[1:]:
+        assert ex <= 1.1 * err[0][0] and ew <= 1.1 * err[0][1]
