@@ -158,14 +158,18 @@ __global__ void __launch_bounds__(kThreads, kResident) gemm_fp32_kernel(const __
   }
 }
 
-// The forms a product can take: tile, k-block, and what a k-block and an item take an SM (us),
-// as measured.  FFMA: an SM works off a k-block in about a microsecond however many CTAs it
-// holds.  Split operands (one CTA to an SM): 6 us for an item of one k-block of 128 x 128 x 64
-// alone on the chip, 12.4 of four, 23.6 of twelve; 5 us, 8.6 of four, 30 of twenty-four of 128 x 64.
-// Both sides of the line (us a call): 8 x 7 x 7 tokens of 64 -> 256 at order 4, rank 6, FFMA
-// 10.8, split 11.5; 2 x 16 x 16 of 64 -> 64, order 8, rank 4 10.4 and 10.7; 4 x 56 x 56 of 48 ->
-// 192, order 4, rank 3 17.8 and 16.5; 8 x 28 x 28 of 192 -> 768, order 8, rank 21 64 and 38; 64 x
-// 7 x 7 of 448 -> 1792, order 8, rank 10 69 and 31; 392 tokens of 768 -> 3072, exact 105 and 31.
+// The forms a product can take: tile, k-block, and what a k-block and an item take an SM (us).
+// FFMA: an SM works off a k-block in about a microsecond however many CTAs it holds.  Split
+// operands (one CTA to an SM): fitted to whole calls, in which all SMs fetch at once; alone on
+// the chip a block takes 1.04 and 1.3 us, an item's start and end with the launch 5.6 and 7.
+// Both sides of the line (us a call, replayed from a graph; FFMA / split, its better tile): 2 x
+// 16 x 16 tokens of 64 -> 64, order 8, rank 4: 8.8 / 10.1; 8 x 7 x 7 of 64 -> 256, order 4, rank 6:
+// 11.5 / 13.1; 2 x 56 x 56 of 64 -> 64, order 4, rank 6: 11.2 / 12.2; 8 x 28 x 28 of 96 -> 384, order
+// 4, rank 3: 20.6 / 16.8; 8 x 56 x 56 of 48 -> 192, order 4, rank 3: 24.2 / 19.9; 8 x 28 x 28 of 192
+// -> 768, order 8, rank 21: 65 / 36; 64 x 7 x 7 of 448 -> 1792, order 8, rank 10: 69 / 32; 392 tokens
+// of 448 -> 1792, exact: 45 / 18.  Close to the line, where planes decide, the model is off by up
+// to 2 us: it takes FFMA for 4 x 56 x 56 of 48 -> 192, rank 3 (18.0 / 16.4) and 16 x 28 x 28 of 96
+// -> 96, rank 3 (15.7 / 14.1).
 struct Form {
   int lanes, cols, bk;   // (split operands: lanes of TMEM, of the operand stored (K, lanes))
   double kb_us, item_us, launch_us;

@@ -24,9 +24,10 @@
 // of a warp of its own issues the 24 MMAs of 128 x BN x 16; under them all warps add the
 // accumulator of the block before to their sums.  Two stages of everything.
 //
-// A 128 x 128 x 64 block takes 1.4 us: its MMAs 0.8, splitting 0.7 (conversions and shifts at
-// half rate), one partly under the other; an item's start and end another 4.5.  Tried
-// before: loads into registers, issued as these become free, make every use wait for the
+// A 128 x 128 x 64 block takes 1.3 us (128 x 64 x 64: 1.04): its MMAs 0.8, splitting 0.7
+// (conversions and shifts at half rate), one partly under the other; an item's start and end,
+// with the launch, another 7 (5.6): 8.3, 9.4, 12.2, 22.4 and 37.7 us for one of 1, 2, 4, 12 and 24
+// blocks alone on the chip and from cold caches (7.0, 7.5, 9.2, 17.4 and 30.0).  Tried before: loads into registers, issued as these become free, make every use wait for the
 // latest load (2.1 us a block, from 8 or 16 warps, also with persistent CTAs, two CTAs to an SM
 // or the parts of L in TMEM).  64 blocks of 448 -> 1792 at rank 10: both products 55 us on FFMA
 // (37 TFLOP/s), 20.6 here (100, six times that in bf16); error against 64 bits of g_x and g_W
