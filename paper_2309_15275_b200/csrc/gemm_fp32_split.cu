@@ -167,10 +167,9 @@ struct Item {
 };
 
 // A sum that stays: zero, or a finite one of 2^-120 and more.
+constexpr float kLeastSum = 0x1p-120f, kMostSum = 3.402823466e38f;
 __device__ __forceinline__ bool stays(float v) {
-  constexpr uint32_t kLeast = (127 - 120) << 23, kMost = 0x7f7fffff;
-  const uint32_t u = __float_as_uint(v) & 0x7fffffffu;
-  return u == 0 || u - kLeast <= kMost - kLeast;
+  return v == 0.f || (fabsf(v) >= kLeastSum && fabsf(v) <= kMostSum);
 }
 
 // The rest of an item by FMAs, with all threads of the CTA: its sums term by term, one k after
@@ -328,11 +327,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
     }
   };
 
+  int begun = 0;   // blocks whose MMAs this thread has issued
   if (warp == kWarps) {
     if (ptx::elect_one()) {
       const uint32_t idesc = ptx::idesc_bf16(kLanes, BN, false, !wt);
       const int n = jobs.test_stall ? 0 : n_kb;
-      int loads = 0, begun = 0;   // blocks fetched, blocks whose MMAs have been issued
+      int loads = 0;   // blocks fetched
       for (; loads < 2 && loads < n; ++loads) item.load(loads);
       for (int i = 0; i < n_kb; ++i) {
         const int s = i & 1;
@@ -360,10 +360,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
         ptx::mma_commit(&done[s]);
         begun = i + 1;
       }
-      // whatever made the others leave: nothing is under way in this CTA's memories when it ends
+      // (after an expired wait: no load is under way when the CTA ends)
       for (int i = begun; i < loads; ++i) item.arrived(i, 4u);
-      if (begun > 0)
-        ptx::mbar_wait(&done[(begun - 1) & 1], static_cast<uint32_t>((begun - 1) >> 1) & 1u, jobs.status, (7u << 16) | 5u);
+      ok = begun == n_kb;
     }
     __syncwarp();
   }
@@ -412,19 +411,30 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_fp32_split_kernel(const __gr
 
   const long long lanes = item.lanes, cols = item.cols;
   const long long l = item.l0 + quarter * 32 + lane, n0 = item.c0 + group * C::kCols;   // this thread's lane, its columns
-  bool bad = false;
+  float most = 0.f;
+  uint32_t least = ~0u;
 #pragma unroll
-  for (int j = 0; j < C::kCols; ++j) bad |= !stays(sum[j]);
+  for (int j = 0; j < C::kCols; j += 2) {
+    // (a NaN stays; zero becomes the largest)
+    asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(most) : "f"(sum[j]), "f"(sum[j + 1]));
+    least = __vimin3_u32(least, __float_as_uint(sum[j]) * 2u - 1u, __float_as_uint(sum[j + 1]) * 2u - 1u);
+  }
+  const bool bad = !(most <= kMostSum) || least < __float_as_uint(kLeastSum) * 2u - 1u;
   ptx::tc_fence_before_sync();
-  // past this barrier every load, MMA and read of TMEM and shared memory has ended
-  if (__syncthreads_or(bad || !ok) && __syncthreads_and(ok)) {
-    if (warp == 0) ptx::tmem_dealloc(tmem_base, kTmemCols);
-    if (warp < kWarps) {
+  // past this barrier every load, MMA and read of TMEM and shared memory has ended, unless a wait ran out
+  if (__syncthreads_or(bad || !ok)) {
+    if (__syncthreads_and(ok)) {
+      if (warp == 0) ptx::tmem_dealloc(tmem_base, kTmemCols);
+      if (warp < kWarps) {
 #pragma unroll
-      for (int j = 0; j < C::kCols; ++j) reinterpret_cast<float*>(smem)[j * kWarps * 32 + threadIdx.x] = sum[j];
+        for (int j = 0; j < C::kCols; ++j) reinterpret_cast<float*>(smem)[j * kWarps * 32 + threadIdx.x] = sum[j];
+      }
+      finish_by_fma<BN>(jobs, maps, false, __any_sync(0xffffffffu, bad));
+      return;
     }
-    finish_by_fma<BN>(jobs, maps, false, __any_sync(0xffffffffu, bad));
-    return;
+    if (begun > 0)
+      ptx::mbar_wait(&done[(begun - 1) & 1], static_cast<uint32_t>((begun - 1) >> 1) & 1u, jobs.status, (7u << 16) | 5u);
+    __syncthreads();
   }
   if (warp == 0) ptx::tmem_dealloc(tmem_base, kTmemCols);
   // The next kernel may start, as late as this: CTAs that come early, while some SMs are
