@@ -27,9 +27,10 @@
 // A 128 x 128 x 64 block takes 1.3 us (128 x 64 x 64: 1.04): its MMAs 0.8, splitting 0.7
 // (conversions and shifts at half rate), one partly under the other; an item's start and end,
 // with the launch, another 7 (5.6): 8.3, 9.4, 12.2, 22.4 and 37.7 us for one of 1, 2, 4, 12 and 24
-// blocks alone on the chip and from cold caches (7.0, 7.5, 9.2, 17.4 and 30.0).  Tried before: loads into registers, issued as these become free, make every use wait for the
-// latest load (2.1 us a block, from 8 or 16 warps, also with persistent CTAs, two CTAs to an SM
-// or the parts of L in TMEM).  64 blocks of 448 -> 1792 at rank 10: both products 55 us on FFMA
+// blocks alone on the chip and from cold caches (7.0, 7.5, 9.2, 17.4 and 30.0).  Tried before:
+// loads into registers, issued as these become free, make every use wait for the latest load
+// (2.1 us a block, from 8 or 16 warps, also with persistent CTAs, two CTAs to an SM or the parts
+// of L in TMEM).  64 blocks of 448 -> 1792 at rank 10: both products 55 us on FFMA
 // (37 TFLOP/s), 20.6 here (100, six times that in bf16); error against 64 bits of g_x and g_W
 // 2.4e-7 and 2.5e-7 there, 1.3e-7 and 1.4e-7 here.
 //
@@ -38,14 +39,14 @@
 // terms: FMAs 2.5, 3.1, 3.6, 4.0, 4.4, 4.7 and 5.4e-8, split 4.5 to 4.7e-8 at all of them).
 //
 // Infinities, NaN and values next to the largest float leave the parts meaningless
-// (inf - inf, 0 * inf), but they always show as a sum that is not finite; and where a sum is
-// next to subnormal the tensor core's cut at 2^-149 shows, where FMAs round (g_y of 2^-130, W of
-// 1: 1.4e-6 against 5.6e-7).  A CTA that has a sum not finite or below 2^-120 fetches the item's
-// operands once more and its warps form their sums from them with fp32 FMAs, term by term;
-// only such sums are replaced.  640 x 448 -> 1792, both
-// products: 22 us, with one NaN in g_y 120, with nothing but NaN 141 (FFMA kernel 60 whatever
-// the values; a serial sum per thread from global memory 980 and 1120); 2048 x 768 -> 3072: 115,
-// 250 and 803 (436; 1690 and 6850).
+// (inf - inf, 0 * inf), and the scaled products of terms of 2^113 and more overflow, but all
+// that always shows as a sum that is not finite; and where a sum is next to subnormal the
+// tensor core's cut at 2^-149 shows, where FMAs round (g_y of 2^-130, W of 1: 1.4e-6 against
+// 5.6e-7).  A CTA that has a sum not finite or below 2^-120 fetches the item's operands once more
+// and its warps form their sums from them with fp32 FMAs, term by term; only such sums are
+// replaced.  640 x 448 -> 1792, both products: 22 us, with one NaN in g_y 120, with nothing but
+// NaN 141 (FFMA kernel 60 whatever the values; a serial sum per thread from global memory 980
+// and 1120); 2048 x 768 -> 3072: 115, 250 and 803 (436; 1690 and 6850).
 #include "gemm_fp32.cuh"
 #include "lbp_internal.h"
 #include "ptx_sm100.cuh"
